@@ -680,8 +680,8 @@ def main():
                                "kernel": "loca_kspace_accumulate (prep, X A on tcgen05, stats, final)",
                                "bytes_per_launch": xbytes}}
 
-    # the same pass with the targets generated inside the statistics kernel (T never written):
-    # error -> ||T||^2 in closed form -> fused Gram / cross at alpha = 1 -> step -> solve
+    # the same pass from the targets' factors (T never formed): error -> ||T||^2 in closed form ->
+    # Gram and Q^T ((E P)^T X) at alpha = 1 -> step -> solve
     fused = None
     if not args.no_fused and X.dtype == torch.bfloat16:
         tsq_f = torch.empty((L,), dtype=torch.float64, device=dev)
@@ -726,14 +726,16 @@ def main():
             raise SystemExit("the fused-targets steps reported a device error or a non-PD system")
         fst = {n: statistics.mean(e[i].elapsed_time(e[i + 1]) for e in fev)
                for i, n in enumerate(["error", "targets_sq", "gram_cross_fused", "step", "ridge_solve"])}
-        ach_f = flops / (fst["gram_cross_fused"] / 1e3) / 1e12
+        flops_f = float(L) * N * (d * (d + 1) + 2.0 * r * d) + 2.0 * L * d * d * r
+        ach_f = flops_f / (fst["gram_cross_fused"] / 1e3) / 1e12
         fused = {"value": world * N * L / (ms_f / 1e3), "unit": UNIT, "ms_per_step": ms_f, "stages_ms": fst,
                  "vs_split": {"targets_plus_gram_ms": stages["targets"] + stages["gram_cross"],
                               "targets_sq_plus_fused_ms": fst["targets_sq"] + fst["gram_cross_fused"]},
                  "roofline": {"bound": "tensor", "achieved": ach_f, "peak": peak, "unit": "TFLOP/s",
-                              "frac": ach_f / peak, "kernel": "k_gram_cross_tc<fused> (+ k_gram_mirror)",
-                              "flops_per_launch": flops, "note": "useful flops of the statistics only; the "
-                              "generation of T adds 6 N d r flops per block on the tensor cores"}}
+                              "frac": ach_f / peak, "kernel": "k_gram_cross_tc (factored), k_expand_cross (+ k_factor_u, "
+                              "k_gram_mirror)",
+                              "flops_per_launch": flops_f, "note": "useful flops of the upper Gram triangle and the "
+                              "factored cross product"}}
         del ws_q, ws_f
 
     # the head error where it is HBM-bound: the Qwen2.5-14B row of the workloads (N = 131072 tokens,

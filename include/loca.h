@@ -298,10 +298,9 @@ int loca_gram_cross(const void* X, const void* T, int dtype, int32_t L, int64_t 
                     size_t workspace_bytes, void* stream);
 
 /*
- * Fused targets: the Gram / cross statistics with each block's targets generated inside the
- * tensor-core kernel instead of read from memory (S3: Q_l := F_l E; S11: F e applied through
- * the factors).  Together with loca_targets_sq they replace loca_targets + loca_gram_cross; T is
- * never written, so the statistics read only X from HBM.
+ * Fused targets: the Gram / cross statistics from the factors of the targets, T never formed
+ * (S3: Q_l := F_l E; S11: F e applied through the factors).  Together with loca_targets_sq they
+ * replace loca_targets + loca_gram_cross; the statistics read only X from HBM.
  *
  * loca_targets_sq (S3, S11; the ||Q_l||^2 of the step in Eq. 10):
  *   tsq[l] = ||E P_l Q_l||_F^2 = < P_l (Q_l Q_l^T) P_l^T , E^T E >, without forming T.
@@ -309,16 +308,16 @@ int loca_gram_cross(const void* X, const void* T, int dtype, int32_t L, int64_t 
  *   1 <= C <= 64, 1 <= r <= 32.  fp32 products summed in fp64; deterministic.
  *   Workspace: loca_targets_sq_workspace_size(N, C) bytes (partial sums of E^T E).
  * loca_gram_cross_fused (Eq. 9; S7): gram_l (+)= X_l^T X_l, cross_l (+)= alpha[l] T_l^T X_l with
- *   T_l = (E P_l) Q_l formed tile by tile on the tensor cores (bf16 hi / lo parts of U = E P_l and
- *   of Q_l, three products, ~2^-17 per element) and rounded once to bf16 before it meets X, as
- *   loca_gram_cross does with a T from loca_targets.  X: L x N x d bf16 only (dtype LOCA_BF16),
+ *   T_l = (E P_l) Q_l, as T_l^T X_l = Q_l^T (U_l^T X_l): U_l = E P_l as two bf16 parts (2^-17 of
+ *   each entry) against X on the tensor cores with fp32 accumulation, the r-long product with
+ *   Q_l in fp32.  T is not rounded to bf16 here (loca_gram_cross with a T from loca_targets is),
+ *   so the two cross products differ by that rounding.  X: L x N x d bf16 only (dtype LOCA_BF16),
  *   E, P, Q as loca_targets_sq, 1 <= r <= 32, C <= 64.  Workspace:
- *   loca_gram_cross_fused_workspace_size(L, N, r) bytes (launch-local flags and U_l = E P_l as
- *   bf16 hi / lo parts, 4 L N rp bytes with rp = 16 for r <= 16, else 32).  Other arguments,
- *   layouts and determinism as loca_gram_cross.
- *   Cost: the cross tiles take one accumulator each (the T generation needs the other TMEM
- *   half), so this kernel does more passes over X than loca_gram_cross; it saves the write of
- *   T and its reads.
+ *   loca_gram_cross_fused_workspace_size(L, N, r) bytes (launch-local flags, the parts of U_l, 4 L N
+ *   rp bytes with rp = 16 for r <= 16, else 32, and U_l^T X_l for 8192 columns, 65536 L rp bytes;
+ *   wider X takes one column range after the other).  Other arguments, layouts and determinism
+ *   as loca_gram_cross; the Gram matrix is the same bit for bit.
+ *   Cost: d (d + 1) + 2 d * 256 flops per token and block instead of 3 d^2 + d, and no T in memory.
  */
 int loca_targets_sq_workspace_size(int64_t N, int32_t C, size_t* bytes /* host */);
 int loca_targets_sq(const float* E, int64_t N, int32_t C, const float* P, const float* Q, int32_t L, int32_t r,

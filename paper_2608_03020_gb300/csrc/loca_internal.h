@@ -66,8 +66,8 @@ cudaError_t launch_gram_cross_tc(const void* X, const void* T, int L, int64_t N,
                                  const float* alpha, int zero_first, float* gram, float* cross,
                                  int32_t* status, int32_t* abort_flag, cudaStream_t s);
 
-// Gram / cross with the targets generated in the kernel from E, P, Q (bf16 X only); r <= 32.
-// Workspace: launch-local flags (256 bytes), then U_l = E P_l as bf16 hi / lo parts.
+// Gram / cross from the factors E P_l and Q_l of the targets (bf16 X only); r <= 32.
+// Workspace: launch-local flags (256 bytes), U_l = E P_l as bf16 hi / lo parts, S_l = U_l^T X_l.
 int gram_fused_max_r();
 size_t gram_fused_workspace_bytes(int L, int64_t N, int r);
 cudaError_t launch_gram_cross_fused_tc(const void* X, const float* E, int C, const float* P, const float* Q,

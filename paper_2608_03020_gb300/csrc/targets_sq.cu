@@ -3,18 +3,22 @@
 //             = < P_l (Q_l Q_l^T) P_l^T , E^T E >   (Frobenius inner product of two C x C matrices).
 // The step of Eq. 10 needs it when the statistics kernel generates T itself (fused targets).
 //
-// k_tsq_ete    partial E^T E over chunks of TSQ_CHUNK tokens (fp32 products summed in fp64), one
-//              C x C slot per chunk.
-// k_tsq_block  one CTA per block l: the chunks' slots summed in a fixed order, M_l = Q_l Q_l^T
-//              (fp32 products over runs of 32 channels, runs summed in fp64), K = P_l M_l P_l^T and
-//              <K, E^T E> in fp64.  Deterministic.
+// k_tsq_ete    partial E^T E over chunks of TSQ_CHUNK tokens (products and sums in fp64), one C x C
+//              slot per chunk.  Up to C = 16 the CTA's threads are split over entries and token
+//              groups (summed in a fixed order): with one thread per entry, 16 threads walked
+//              2048 tokens each (275 us at C = 4, N = 32768; 11 us now).
+// k_tsq_block  one CTA of 32 warps per block l: the chunks' slots summed in a fixed order, M_l =
+//              Q_l Q_l^T (fp32 products over runs of 32 channels, runs summed in fp64), K = P_l M_l
+//              P_l^T and <K, E^T E> in fp64.  Latency-bound: 4 to 5 of M's 136 entries per warp at
+//              r = 16.  Deterministic.
 #include "loca_internal.h"
 
 namespace loca {
 namespace {
 
 constexpr int TSQ_THREADS = 256;
-constexpr int TSQ_CHUNK = 2048;  // tokens per E^T E partial
+constexpr int TSQ_BLOCK_THREADS = 1024;
+constexpr int TSQ_CHUNK = 512;  // tokens per E^T E partial
 constexpr int kMaxC = 64;
 constexpr int kMaxR = 32;
 
@@ -23,39 +27,69 @@ __global__ void __launch_bounds__(TSQ_THREADS) k_tsq_ete(const float* __restrict
   const int64_t n0 = int64_t(blockIdx.x) * TSQ_CHUNK;
   const int64_t n1 = n0 + TSQ_CHUNK < N ? n0 + TSQ_CHUNK : N;
   double* out = part + int64_t(blockIdx.x) * C * C;
-  for (int e = threadIdx.x; e < C * C; e += TSQ_THREADS) {
-    const int a = e / C, b = e % C;
+  const int C2 = C * C;
+  const int groups = C2 <= TSQ_THREADS ? TSQ_THREADS / C2 : 1;  // token groups per entry
+  __shared__ double red[TSQ_THREADS];
+  for (int e0 = 0; e0 < C2; e0 += TSQ_THREADS) {
+    const int e = groups > 1 ? int(threadIdx.x) % C2 : e0 + int(threadIdx.x);
+    const int grp = groups > 1 ? int(threadIdx.x) / C2 : 0;
     double acc = 0.0;
-    for (int64_t n = n0; n < n1; ++n)
-      if (LOCA_CHECK(n * C + a, N * C) && LOCA_CHECK(n * C + b, N * C)) acc += double(E[n * C + a]) * double(E[n * C + b]);
-    if (LOCA_CHECK(int64_t(blockIdx.x) * C * C + e, int64_t(gridDim.x) * C * C)) out[e] = acc;
+    if (e < C2 && grp < groups) {
+      const int a = e / C, b = e % C;
+#pragma unroll 8
+      for (int64_t n = n0 + grp; n < n1; n += groups)
+        if (LOCA_CHECK(n * C + a, N * C) && LOCA_CHECK(n * C + b, N * C)) acc = fma(double(E[n * C + a]), double(E[n * C + b]), acc);
+    }
+    if (groups > 1) {
+      red[threadIdx.x] = acc;
+      __syncthreads();
+      if (threadIdx.x < C2)
+        for (int q = 1; q < groups; ++q) acc += red[q * C2 + threadIdx.x];
+    }
+    if (grp == 0 && e < C2 && LOCA_CHECK(int64_t(blockIdx.x) * C2 + e, int64_t(gridDim.x) * C2)) out[e] = acc;
   }
 }
 
-__global__ void __launch_bounds__(TSQ_THREADS) k_tsq_block(const double* __restrict__ part, int nchunks, int C,
+__global__ void __launch_bounds__(TSQ_BLOCK_THREADS) k_tsq_block(const double* __restrict__ part, int nchunks, int C,
                                                             const float* __restrict__ P, const float* __restrict__ Q,
                                                             int r, int64_t d, double* __restrict__ tsq) {
   __shared__ double ete[kMaxC * kMaxC];
   __shared__ double M[kMaxR * kMaxR];
   __shared__ double PM[kMaxC * kMaxR];
-  __shared__ double red[TSQ_THREADS];
+  __shared__ double red[TSQ_BLOCK_THREADS];
+  constexpr int TT = TSQ_BLOCK_THREADS;
   const int l = blockIdx.x;
-  for (int e = threadIdx.x; e < C * C; e += TSQ_THREADS) {
+  const int C2 = C * C;
+  const int groups = C2 <= TT ? TT / C2 : 1;  // groups of chunks per entry
+  for (int e0 = 0; e0 < C2; e0 += TT) {
+    const int e = groups > 1 ? int(threadIdx.x) % C2 : e0 + int(threadIdx.x);
+    const int grp = groups > 1 ? int(threadIdx.x) / C2 : 0;
     double acc = 0.0;
-    for (int c = 0; c < nchunks; ++c) acc += part[int64_t(c) * C * C + e];  // e < C * C
-    ete[e] = acc;
+    if (e < C2 && grp < groups) {
+#pragma unroll 4
+      for (int c = grp; c < nchunks; c += groups) acc += part[int64_t(c) * C2 + e];  // e < C * C
+    }
+    if (groups > 1) {
+      red[threadIdx.x] = acc;
+      __syncthreads();
+      if (threadIdx.x < C2)
+        for (int q = 1; q < groups; ++q) acc += red[q * C2 + threadIdx.x];
+    }
+    if (grp == 0 && e < C2) ete[e] = acc;
   }
   // M = Q_l Q_l^T: one warp per entry (s, t), lanes over channels, fp32 runs of 32 products
   const float* Ql = Q + int64_t(l) * r * d;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int e = warp; e < r * r; e += TSQ_THREADS / 32) {
-    const int si = e / r, ti = e % r;
-    if (ti < si) continue;
+  for (int e = warp; e < r * (r + 1) / 2; e += TT / 32) {
+    int si = 0, ti = e;  // e-th entry of the upper triangle
+    while (ti >= r - si) ti -= r - si++;
+    ti += si;
     const float* qs = Ql + int64_t(si) * d;
     const float* qt = Ql + int64_t(ti) * d;
     double acc = 0.0;
     for (int64_t c0 = 0; c0 < d; c0 += 32 * 32) {
       float run = 0.f;
+#pragma unroll 8
       for (int64_t c = c0 + lane; c < c0 + 32 * 32 && c < d; c += 32) run = fmaf(qs[c], qt[c], run);
       acc += double(run);
     }
@@ -68,7 +102,7 @@ __global__ void __launch_bounds__(TSQ_THREADS) k_tsq_block(const double* __restr
   __syncthreads();
   // PM = P_l M (C x r)
   const float* Pl = P + int64_t(l) * C * r;
-  for (int e = threadIdx.x; e < C * r; e += TSQ_THREADS) {
+  for (int e = threadIdx.x; e < C * r; e += TT) {
     const int a = e / r, t = e % r;
     double acc = 0.0;
     for (int s = 0; s < r; ++s) acc += double(Pl[a * r + s]) * M[s * r + t];
@@ -77,7 +111,7 @@ __global__ void __launch_bounds__(TSQ_THREADS) k_tsq_block(const double* __restr
   __syncthreads();
   // <P M P^T, E^T E> = sum_ab (sum_t PM[a, t] P[b, t]) ete[a, b]
   double acc = 0.0;
-  for (int e = threadIdx.x; e < C * C; e += TSQ_THREADS) {
+  for (int e = threadIdx.x; e < C * C; e += TT) {
     const int a = e / C, b = e % C;
     double k = 0.0;
     for (int t = 0; t < r; ++t) k += PM[a * r + t] * double(Pl[b * r + t]);
@@ -85,7 +119,7 @@ __global__ void __launch_bounds__(TSQ_THREADS) k_tsq_block(const double* __restr
   }
   red[threadIdx.x] = acc;
   __syncthreads();
-  for (int w = TSQ_THREADS / 2; w > 0; w >>= 1) {
+  for (int w = TT / 2; w > 0; w >>= 1) {
     if (threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
     __syncthreads();
   }
@@ -109,7 +143,7 @@ cudaError_t launch_targets_sq(const float* E, int64_t N, int C, const float* P, 
   if (nchunks > 0) k_tsq_ete<<<unsigned(nchunks), TSQ_THREADS, 0, s>>>(E, N, C, part);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  k_tsq_block<<<unsigned(L), TSQ_THREADS, 0, s>>>(part, int(nchunks), C, P, Q, r, d, tsq);
+  k_tsq_block<<<unsigned(L), TSQ_BLOCK_THREADS, 0, s>>>(part, int(nchunks), C, P, Q, r, d, tsq);
   return cudaGetLastError();
 }
 

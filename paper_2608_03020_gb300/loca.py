@@ -506,7 +506,8 @@ def gram_cross_fused_workspace_size(L, N, r) -> int:
 
 
 def loca_gram_cross_fused(X, E, P, Q, alpha, gram, cross, zero_first, workspace=None, stream=None):
-    """loca_gram_cross with each block's targets ``T_l = (E P_l) Q_l`` generated inside the kernel."""
+    """loca_gram_cross from the factors of the targets ``T_l = (E P_l) Q_l``, which are never formed:
+    ``T_l^T X_l = Q_l^T ((E P_l)^T X_l)``."""
     _dev(X, "X", torch.bfloat16, 3)
     _dev(E, "E", torch.float32, 2)
     _dev(P, "P", torch.float32, 3)

@@ -1,0 +1,79 @@
+"""Edges of the size-dependent kernel paths, against the fp64 oracle: the smallest and largest of
+each path's range, remainders of its tiles, and both sides of each dispatch rule."""
+
+import numpy as np
+import pytest
+import torch
+
+from oracle import loca_oracle as O
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def lc():
+    assert torch.cuda.is_available(), "GPU tests need a CUDA device"
+    from paper_2608_03020_gb300 import _build
+
+    _build.build()
+    from paper_2608_03020_gb300 import loca
+
+    loca.lib()
+    return loca
+
+
+def _np(t):
+    return t.detach().double().cpu().numpy()
+
+
+def _rel(a, b):
+    a, b = np.asarray(a, dtype=np.float64), np.asarray(b, dtype=np.float64)
+    return float(np.linalg.norm(a - b) / max(np.linalg.norm(b), 1e-300))
+
+
+def _dev(a, dtype=torch.float32):
+    return torch.from_numpy(np.ascontiguousarray(a)).to(device="cuda", dtype=dtype)
+
+
+@pytest.mark.parametrize("L,N,d,C,r,batches", [
+    (2, 65, 40, 2, 3, 2),       # one partial tile in every direction, U columns padded to 32
+    (1, 130, 8456, 4, 5, 1),    # two column ranges of S, the second ragged and without 4-D loads
+    (2, 70, 264, 8, 17, 2),     # U columns padded to 64, an 8-column last tile
+])
+def test_factored_cross_product(lc, L, N, d, C, r, batches):
+    """cross = Q^T ((E P)^T X): U's two bf16 parts carry 2^-17 = 7.6e-6 of each entry, the sums
+    over a few hundred tokens and over r are fp32, so 2e-5 of the exact product."""
+    rng = np.random.default_rng(d)
+    gram, cross = (torch.full((L, d, d), float("nan"), device="cuda") for _ in range(2))
+    P = rng.normal(0, 1, (L, C, r)).astype(np.float32)
+    Q = rng.normal(0, 1, (L, r, d)).astype(np.float32)
+    alpha = np.linspace(0.5, -1.0, L).astype(np.float32)
+    ref = np.zeros((L, d, d))
+    gref = np.zeros((L, d, d))
+    for b in range(batches):
+        X = torch.from_numpy(rng.standard_normal((L, N, d)).astype(np.float32)).to(torch.bfloat16)
+        E = rng.standard_normal((N, C)).astype(np.float32)
+        lc.loca_gram_cross_fused(X.to("cuda"), _dev(E), _dev(P), _dev(Q), _dev(alpha), gram, cross, zero_first=b == 0)
+        Xn = X.double().numpy()
+        T, _ = O.feedback_targets(E, P, Q)
+        for l in range(L):
+            ref[l] += float(alpha[l]) * (T[l].T @ Xn[l])
+            gref[l] += Xn[l].T @ Xn[l]
+    torch.cuda.synchronize()
+    assert lc.loca_device_status() == 0
+    assert _rel(_np(cross), ref) <= 2e-5
+    assert _rel(_np(gram), gref) <= 2e-5
+
+
+@pytest.mark.parametrize("N,C", [(1, 1), (513, 16), (1500, 17), (700, 64)])
+def test_targets_sq_entry_groups(lc, N, C):
+    """One thread group per E^T E entry up to C = 16, several entries per thread above: fp64 sums of
+    fp64 products, M = Q Q^T from fp32 runs of 32 products (32 * 2^-24 = 2e-6)."""
+    rng = np.random.default_rng(N)
+    E = rng.standard_normal((N, C)).astype(np.float32)
+    P = rng.standard_normal((2, C, 7)).astype(np.float32)
+    Q = rng.standard_normal((2, 7, 100)).astype(np.float32)
+    tsq = torch.empty((2,), dtype=torch.float64, device="cuda")
+    lc.loca_targets_sq(_dev(E), _dev(P), _dev(Q), tsq)
+    _, ref = O.feedback_targets(E, P, Q)
+    assert np.allclose(_np(tsq), ref, rtol=2e-6, atol=0)
