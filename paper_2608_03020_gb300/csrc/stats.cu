@@ -12,6 +12,7 @@
 // k_gram_cross_f32: Gram_l (+)= X^T X (upper tiles, mirrored) and Cross_l (+)= alpha T^T X for
 //               fp32 inputs with fp64 accumulation: the exact-input path used for tight parity
 //               on small shapes; the bf16 path runs on the tensor cores (gram_tc.cu).
+#include <cooperative_groups.h>
 #include <cuda_bf16.h>
 
 #include "loca_internal.h"
@@ -88,13 +89,19 @@ __global__ void __launch_bounds__(256) k_sumsq(const void* __restrict__ Xv, int6
   }
 }
 
-__global__ void k_step(const double* __restrict__ partials, int G, int L, const double* __restrict__ tsq,
-                       float eta, int zero_first, double* __restrict__ xsq_total,
-                       float* __restrict__ alpha) {
-  const int l = blockIdx.x * blockDim.x + threadIdx.x;
+// One warp per block l: lanes over the partials, then a fixed butterfly (one thread walking them took
+// 7-10 us a call).
+__global__ void __launch_bounds__(128) k_step(const double* __restrict__ partials, int G, int L,
+                                              const double* __restrict__ tsq, float eta, int zero_first,
+                                              double* __restrict__ xsq_total, float* __restrict__ alpha) {
+  const int l = blockIdx.x * 4 + int(threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (l >= L || !LOCA_CHECK(G, kMaxPartials + 1)) return;
   double xb = 0.0;
-  for (int g = 0; g < G; ++g) xb += partials[int64_t(l) * kMaxPartials + g];
+#pragma unroll 4
+  for (int g = lane; g < G; g += 32) xb += partials[int64_t(l) * kMaxPartials + g];
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) xb += __shfl_xor_sync(0xffffffffu, xb, off);
+  if (lane != 0) return;
   const double ts = tsq[l];
   alpha[l] = ts > 0.0 ? float(-double(eta) * sqrt(xb / ts)) : 0.f;
   xsq_total[l] = (zero_first ? 0.0 : xsq_total[l]) + xb;
@@ -123,69 +130,108 @@ __global__ void __launch_bounds__(256) k_step_from_gram(const float* __restrict_
   }
 }
 
-// 64 x 64 output tile per thread block, 4 x 4 per thread, fp64 accumulators.
-constexpr int FT = 64;
-constexpr int FK = 16;
+// 32 x 32 output tile per cluster, 2 x 2 fp64 accumulators per thread.  The fp64 pipe (2 FMAs per clock
+// and SM) bounds it, so what counts is that all SMs have work: the cluster's CTAs take equal ranges
+// of the tokens and their partial tiles are added through distributed shared memory in rank order
+// (fixed: deterministic; no workspace).  Operands are converted to fp64 once, when staged: a
+// conversion per use shares the fp64 pipe with the FMAs.  The 64 x 64 tiles without a token split that this
+// replaces put 4 CTAs on the chip at L = 2, d = 64.
+constexpr int FT = 32;
+constexpr int FK = 32;           // tokens per staged slab
+constexpr int kMaxSplit = 8;     // token ranges (CTAs per cluster; 8 is the portable limit)
 
 __global__ void __launch_bounds__(256) k_gram_cross_f32(const float* __restrict__ X,
                                                         const float* __restrict__ T, int64_t N,
-                                                        int64_t d, const float* __restrict__ alpha,
+                                                        int64_t d, int nt, int ntri, int per_block,
+                                                        const float* __restrict__ alpha,
                                                         int zero_first, float* __restrict__ gram,
                                                         float* __restrict__ cross) {
-  const int l = blockIdx.z >> 1;
-  const bool is_gram = (blockIdx.z & 1) == 0;
-  const int mt = blockIdx.y, nt = blockIdx.x;
-  if (is_gram && nt < mt) return;  // tile strictly below the diagonal: written by the mirror
-  __shared__ float As[FK][FT];
-  __shared__ float Bs[FK][FT];
+  namespace cg = cooperative_groups;
+  cg::cluster_group cl = cg::this_cluster();
+  const int split = int(cl.num_blocks()), rank = int(cl.block_rank());
+  const int64_t tile = int64_t(blockIdx.x) / split;
+  const int l = int(tile / per_block);
+  const int t = int(tile - int64_t(l) * per_block);
+  // the first ntri tiles are the Gram's, row tile mt <= column tile nt_ (column-major over the
+  // triangle), the others the cross product's
+  const bool is_gram = t < ntri;
+  int mt, nc;
+  if (is_gram) {
+    nc = int((sqrtf(8.f * float(t) + 1.f) - 1.f) * 0.5f);
+    while ((nc + 1) * (nc + 2) / 2 <= t) ++nc;
+    while (nc * (nc + 1) / 2 > t) --nc;
+    mt = t - nc * (nc + 1) / 2;
+  } else {
+    mt = (t - ntri) / nt;
+    nc = (t - ntri) - mt * nt;
+  }
+  __shared__ __align__(16) double As[FK][FT];
+  __shared__ __align__(16) double Bs[FK][FT];
+  __shared__ double part[FT * FT];
   const float* Xl = X + int64_t(l) * N * d;
   const float* Rl = (is_gram ? X : T) + int64_t(l) * N * d;
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  const int64_t i0 = int64_t(mt) * FT, j0 = int64_t(nt) * FT;
-  double acc[4][4] = {};
-  for (int64_t n0 = 0; n0 < N; n0 += FK) {
-    for (int e = threadIdx.x; e < FK * FT; e += 256) {
-      const int kk = e / FT, c = e % FT;
+  const int64_t i0 = int64_t(mt) * FT, j0 = int64_t(nc) * FT;
+  const int64_t per = (N + split - 1) / split;
+  const int64_t nb = per * rank, ne = nb + per < N ? nb + per : N;
+  double acc[2][2] = {};
+  // next slab's elements in registers while this one is multiplied
+  constexpr int LD = FK * FT / 256;
+  float pa[LD], pb[LD];
+  auto load = [&](int64_t n0) {
+#pragma unroll
+    for (int i = 0; i < LD; ++i) {
+      const int e = int(threadIdx.x) + 256 * i, kk = e / FT, c = e % FT;
       const int64_t n = n0 + kk;
-      As[kk][c] = (n < N && i0 + c < d && LOCA_CHECK(n * d + i0 + c, N * d)) ? Rl[n * d + i0 + c] : 0.f;
-      Bs[kk][c] = (n < N && j0 + c < d && LOCA_CHECK(n * d + j0 + c, N * d)) ? Xl[n * d + j0 + c] : 0.f;
+      pa[i] = (n < ne && i0 + c < d && LOCA_CHECK(n * d + i0 + c, N * d)) ? Rl[n * d + i0 + c] : 0.f;
+      pb[i] = (n < ne && j0 + c < d && LOCA_CHECK(n * d + j0 + c, N * d)) ? Xl[n * d + j0 + c] : 0.f;
     }
+  };
+  if (nb < ne) load(nb);
+  for (int64_t n0 = nb; n0 < ne; n0 += FK) {
     __syncthreads();
 #pragma unroll
-    for (int kk = 0; kk < FK; ++kk) {
-      double a[4], b[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) a[i] = As[kk][ty * 4 + i];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) b[j] = Bs[kk][tx * 4 + j];
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
+    for (int i = 0; i < LD; ++i) {
+      const int e = int(threadIdx.x) + 256 * i;
+      As[e / FT][e % FT] = double(pa[i]);
+      Bs[e / FT][e % FT] = double(pb[i]);
     }
     __syncthreads();
+    if (n0 + FK < ne) load(n0 + FK);
+    const int kn = ne - n0 < FK ? int(ne - n0) : FK;
+#pragma unroll 8
+    for (int kk = 0; kk < kn; ++kk) {
+      const double2 a = *reinterpret_cast<const double2*>(&As[kk][ty * 2]);
+      const double2 b = *reinterpret_cast<const double2*>(&Bs[kk][tx * 2]);
+      acc[0][0] = fma(a.x, b.x, acc[0][0]);
+      acc[0][1] = fma(a.x, b.y, acc[0][1]);
+      acc[1][0] = fma(a.y, b.x, acc[1][0]);
+      acc[1][1] = fma(a.y, b.y, acc[1][1]);
+    }
   }
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+#pragma unroll
+    for (int j = 0; j < 2; ++j) part[(ty * 2 + i) * FT + tx * 2 + j] = acc[i][j];
+  cl.sync();
   const double al = is_gram ? 1.0 : double(alpha[l]);
   float* out = (is_gram ? gram : cross) + int64_t(l) * d * d;
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int64_t r = i0 + ty * 4 + i;
-    if (r >= d) continue;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int64_t c = j0 + tx * 4 + j;
-      if (c >= d) continue;
-      if (is_gram && r > c) continue;
-      if (!LOCA_CHECK(r * d + c, d * d) || !LOCA_CHECK(c * d + r, d * d)) continue;
-      const double v = al * acc[i][j];
-      float* p = out + r * d + c;
-      *p = zero_first ? float(v) : float(double(*p) + v);
-      if (is_gram && r < c) {
-        float* q = out + c * d + r;
-        *q = zero_first ? float(v) : float(double(*q) + v);
-      }
+  // this CTA's share of the tile: the ranks' partial sums in rank order
+  for (int e = rank * 256 + int(threadIdx.x); e < FT * FT; e += 256 * split) {
+    double v = 0.0;
+    for (int q = 0; q < split; ++q) v += *cl.map_shared_rank(&part[e], q);
+    const int64_t r = i0 + e / FT, c = j0 + e % FT;
+    if (r >= d || c >= d || (is_gram && r > c)) continue;
+    if (!LOCA_CHECK(r * d + c, d * d) || !LOCA_CHECK(c * d + r, d * d)) continue;
+    v *= al;
+    float* p = out + r * d + c;
+    *p = zero_first ? float(v) : float(double(*p) + v);
+    if (is_gram && r < c) {
+      float* q = out + c * d + r;
+      *q = zero_first ? float(v) : float(double(*q) + v);
     }
   }
+  cl.sync();  // no CTA leaves while its partial tile may still be read
 }
 
 }  // namespace
@@ -214,17 +260,33 @@ cudaError_t launch_sumsq_and_step(const void* X, int dtype, int L, int64_t N, in
   } else {
     G = 0;
   }
-  k_step<<<(L + 127) / 128, 128, 0, s>>>(partials, int(G), L, tsq, eta, zero_first, xsq_total, alpha);
+  k_step<<<(L + 3) / 4, 128, 0, s>>>(partials, int(G), L, tsq, eta, zero_first, xsq_total, alpha);
   return cudaGetLastError();
 }
 
 cudaError_t launch_gram_cross_f32(const float* X, const float* T, int L, int64_t N, int64_t d,
                                   const float* alpha, int zero_first, float* gram, float* cross,
                                   cudaStream_t s) {
-  const unsigned nt = unsigned((d + FT - 1) / FT);
-  const dim3 grid = dim3(nt, nt, unsigned(2 * L));
-  k_gram_cross_f32<<<grid, 256, 0, s>>>(X, T, N, d, alpha, zero_first, gram, cross);
-  return cudaGetLastError();
+  const int64_t nt = (d + FT - 1) / FT;
+  const int64_t ntri = nt * (nt + 1) / 2, per_block = ntri + nt * nt;
+  // split the tokens until the tiles fill the chip (one CTA per SM: the fp64 pipe is full with one),
+  // but not below a slab per CTA
+  int split = 1;
+  while (split < kMaxSplit && per_block * L * split * 2 <= int64_t(sm_count()) + sm_count() / 2 && N >= int64_t(2) * split * FK)
+    split *= 2;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(unsigned(per_block * L * split));
+  cfg.blockDim = dim3(256);
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = unsigned(split);
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k_gram_cross_f32, X, T, N, d, int(nt), int(ntri), int(per_block), alpha, zero_first,
+                            gram, cross);
 }
 
 cudaError_t launch_step_from_gram(const float* gram, int L, int64_t d, const double* tsq, float eta,

@@ -77,3 +77,23 @@ def test_targets_sq_entry_groups(lc, N, C):
     lc.loca_targets_sq(_dev(E), _dev(P), _dev(Q), tsq)
     _, ref = O.feedback_targets(E, P, Q)
     assert np.allclose(_np(tsq), ref, rtol=2e-6, atol=0)
+
+
+@pytest.mark.parametrize("L,N,d", [(1, 1, 1), (2, 63, 33), (1, 64, 32), (3, 257, 65), (1, 2000, 31), (2, 300, 250)])
+def test_fp32_statistics_token_split(lc, L, N, d):
+    """The fp32-input statistics at every cluster size (1 to 8 token ranges, ragged and empty ones) and
+    tile remainders: fp64 sums, so the fp32 rounding of the exact result (2^-24 = 6e-8 of each entry)
+    and, accumulated over two batches, one more."""
+    rng = np.random.default_rng(N * 7 + d)
+    gram, cross = (torch.full((L, d, d), float("nan"), device="cuda") for _ in range(2))
+    alpha = np.linspace(0.5, -1.0, L).astype(np.float32)
+    g_ref, c_ref = np.zeros((L, d, d)), np.zeros((L, d, d))
+    for b in range(2):
+        X, T = (rng.standard_normal((L, N, d)).astype(np.float32) for _ in range(2))
+        lc.loca_gram_cross(_dev(X), _dev(T), _dev(alpha), gram, cross, zero_first=b == 0)
+        for l in range(L):
+            x, t = X[l].astype(np.float64), T[l].astype(np.float64)
+            g_ref[l] += x.T @ x
+            c_ref[l] += float(alpha[l]) * (t.T @ x)
+    assert _rel(_np(gram), g_ref) <= 1.2e-7 and _rel(_np(cross), c_ref) <= 1.2e-7
+    assert torch.equal(gram, gram.transpose(1, 2))
