@@ -209,14 +209,17 @@ __global__ void __launch_bounds__(256) k_factor_u(const float* __restrict__ E, i
 }
 
 // cross_l[:, c0 .. c0 + cw) (+)= alpha_l Q_l^T S_l, S_l = its hi rows + its lo rows (2 rp x ldS).  One
-// 64-row x 256-column tile per CTA; a thread owns 4 columns x 16 rows, so a step of the r-long sum
-// is 5 shared-memory vector loads for 64 FMAs.  Bound by the write of cross (4 d^2 bytes a block).
-constexpr int EX_ROWS = 64, EX_COLS = 256;
+// tile of 256 columns x ex_rows rows per CTA, so that staging S and Q is a small part of its work; a
+// thread owns 4 columns x 16 rows at a time, so a step of the r-long sum is 5 shared-memory vector
+// loads for 64 FMAs.  Bound by the write of cross (4 d^2 bytes a block).
+constexpr int EX_COLS = 256;
+__host__ __device__ constexpr int ex_rows(int rp) { return rp <= 16 ? 256 : 128; }
 
 template <int RP>
 __global__ void __launch_bounds__(256) k_expand_cross(const float* __restrict__ S, int64_t ldS, const float* __restrict__ Q,
                                                       int r, int d, int c0, int cw, const float* __restrict__ alpha,
                                                       int zero_first, float* __restrict__ cross) {
+  constexpr int EX_ROWS = ex_rows(RP);
   __shared__ __align__(16) float Ss[RP][EX_COLS];
   __shared__ __align__(16) float Qs[RP][EX_ROWS];
   const int l = blockIdx.z;
@@ -237,40 +240,45 @@ __global__ void __launch_bounds__(256) k_expand_cross(const float* __restrict__ 
                    : 0.f;
   }
   __syncthreads();
-  const int tj = (threadIdx.x & 63) * 4, ti = (threadIdx.x >> 6) * 16;
-  float acc[16][4];
-#pragma unroll
-  for (int i = 0; i < 16; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
-  for (int s = 0; s < r; ++s) {
-    const float4 x = *reinterpret_cast<const float4*>(&Ss[s][tj]);
-#pragma unroll
-    for (int v = 0; v < 4; ++v) {
-      const float4 q = *reinterpret_cast<const float4*>(&Qs[s][ti + 4 * v]);
-      const float qq[4] = {q.x, q.y, q.z, q.w};
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        acc[4 * v + i][0] = fmaf(qq[i], x.x, acc[4 * v + i][0]);
-        acc[4 * v + i][1] = fmaf(qq[i], x.y, acc[4 * v + i][1]);
-        acc[4 * v + i][2] = fmaf(qq[i], x.z, acc[4 * v + i][2]);
-        acc[4 * v + i][3] = fmaf(qq[i], x.w, acc[4 * v + i][3]);
-      }
-    }
-  }
+  const int tj = (threadIdx.x & 63) * 4;
   if (j0 + tj >= cw) return;  // cw and d are multiples of 8: the 4 columns are all inside or all outside
   float* out = cross + int64_t(l) * d * d + c0 + j0 + tj;
+#pragma unroll 1
+  for (int ti = (threadIdx.x >> 6) * 16; ti < EX_ROWS; ti += 64) {
+    if (i0 + ti >= d) break;
+    float acc[16][4];
 #pragma unroll
-  for (int i = 0; i < 16; ++i) {
-    const int64_t row = i0 + ti + i;
-    if (row >= d || !LOCA_CHECK_SPAN(row * d + c0 + j0 + tj, 4, int64_t(d) * d)) continue;
-    float4* o = reinterpret_cast<float4*>(out + row * d);
-    float4 v = make_float4(al * acc[i][0], al * acc[i][1], al * acc[i][2], al * acc[i][3]);
-    if (!zero_first) {
-      const float4 p = *o;
-      v = make_float4(p.x + v.x, p.y + v.y, p.z + v.z, p.w + v.w);
+    for (int i = 0; i < 16; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
+#pragma unroll 2
+    for (int s = 0; s < r; ++s) {
+      const float4 x = *reinterpret_cast<const float4*>(&Ss[s][tj]);
+#pragma unroll
+      for (int v = 0; v < 4; ++v) {
+        const float4 q = *reinterpret_cast<const float4*>(&Qs[s][ti + 4 * v]);
+        const float qq[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          acc[4 * v + i][0] = fmaf(qq[i], x.x, acc[4 * v + i][0]);
+          acc[4 * v + i][1] = fmaf(qq[i], x.y, acc[4 * v + i][1]);
+          acc[4 * v + i][2] = fmaf(qq[i], x.z, acc[4 * v + i][2]);
+          acc[4 * v + i][3] = fmaf(qq[i], x.w, acc[4 * v + i][3]);
+        }
+      }
     }
-    *o = v;
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+      const int64_t row = i0 + ti + i;
+      if (row >= d || !LOCA_CHECK_SPAN(row * d + c0 + j0 + tj, 4, int64_t(d) * d)) continue;
+      float4* o = reinterpret_cast<float4*>(out + row * d);
+      float4 v = make_float4(al * acc[i][0], al * acc[i][1], al * acc[i][2], al * acc[i][3]);
+      if (!zero_first) {
+        const float4 p = *o;
+        v = make_float4(p.x + v.x, p.y + v.y, p.z + v.z, p.w + v.w);
+      }
+      *o = v;
+    }
   }
 }
 
@@ -803,7 +811,7 @@ cudaError_t gram_cross_factored(const void* X, const float* E, int C, const floa
     const Factored f{2 * RP, int(c0 / BN), int((c0 + cw + BN - 1) / BN), c0 == 0 ? 1 : 0};
     e = launch_stats(X, U, L, N, d, alpha, zero_first, gram, S, status, reinterpret_cast<int32_t*>(ws), f, s);
     if (e != cudaSuccess) return e;
-    const dim3 grid(unsigned((cw + EX_COLS - 1) / EX_COLS), unsigned((d + EX_ROWS - 1) / EX_ROWS), unsigned(L));
+    const dim3 grid(unsigned((cw + EX_COLS - 1) / EX_COLS), unsigned((d + ex_rows(RP) - 1) / ex_rows(RP)), unsigned(L));
     k_expand_cross<RP><<<grid, 256, 0, s>>>(S, cw, Q, r, int(d), int(c0), int(cw), alpha, zero_first, cross);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
