@@ -3,30 +3,29 @@
 // with G_l the exact hidden-state gradients at the probe positions.  T is formed element by
 // element in registers (r FMAs each) and never written.
 //
-// k_align_part   grid (token chunk, 256-channel tile, block): each thread owns one channel of the
-//                tile; per 32-token sub-chunk the CTA forms U = E P_l for those tokens in shared
-//                memory, then every thread walks the tokens: t = U[n] . Q_l[:, j], g = G[n][j],
-//                and sums g t, g g, t t (fp32 over the chunk; fp64 block reduction in a fixed
-//                order), one partial triple per CTA.
+// k_align_u      U_l = E P_l (Np x RP per block, fp32, rows padded with zeros), tiled over 64 tokens x 64
+//                error channels in shared memory.
+// k_align_part   grid (token chunk x channel tile, block): a lane owns 32 / RP channels, whose Q_l
+//                entries stay in 32 registers; every warp streams its tokens' rows of G and U through
+//                its own ring (row_stream.cuh) and sums g t, g g, t t with t = U[n] . Q_l[:, j] (fp32 over
+//                the chunk; fp64 block reduction in a fixed order), one partial triple per CTA.  Bound
+//                by the read of G: 1.41 GB at L = 28, Np = 8192, d = 1536 (0.71 ms with Q_l re-read from
+//                shared memory for every token, two shared loads per FMA).
 // k_align_final  per block, the partial triples in a fixed order -> alpha_l (0 if a norm is 0).
-// k_align_u      for error spaces wider than kMaxM (the paper's d-wide e): U_l = E P_l (Np x r per
-//                block, fp32) first, tiled over 64 tokens x 64 error channels in shared memory;
-//                k_align_part then reads U_l instead of forming E P_l itself.
 #include "loca_internal.h"
+#include "row_stream.cuh"
 
 namespace loca {
 namespace {
 
-constexpr int AL_THREADS = 256;  // channels per tile
-constexpr int AL_SUB = 32;       // tokens staged at a time
+constexpr int AL_THREADS = 256;
 constexpr int AL_CHUNK = 1024;   // tokens per CTA
-constexpr int kMaxM = 64;      // error width formed in k_align_part itself
 constexpr int kMaxWideM = 16384;
 constexpr int kMaxR = 32;
 constexpr int AU_TOK = 64;     // tokens per CTA of k_align_u
 constexpr int AU_CH = 64;      // error channels staged per step
 
-// U[l][n][s] = sum_c E[n][c] P_l[c][s] (fp32), U laid out L x Np x r.
+// U[l][n][s] = sum_c E[n][c] P_l[c][s] (fp32), U laid out L x Np x RP, zero for s >= r.
 template <int RP>
 __global__ void __launch_bounds__(AL_THREADS) k_align_u(const float* __restrict__ E, const float* __restrict__ P,
                                                       int64_t Np, int m, int r, float* __restrict__ U) {
@@ -64,85 +63,120 @@ __global__ void __launch_bounds__(AL_THREADS) k_align_u(const float* __restrict_
 #pragma unroll
   for (int i = 0; i < SPT; ++i) {
     const int s = sg + SG * i;
-    if (s < r && LOCA_CHECK((int64_t(l) * Np + n) * r + s, int64_t(gridDim.y) * Np * r)) U[(int64_t(l) * Np + n) * r + s] = acc[i];
+    if (LOCA_CHECK((int64_t(l) * Np + n) * RP + s, int64_t(gridDim.y) * Np * RP)) U[(int64_t(l) * Np + n) * RP + s] = acc[i];
   }
 }
 
-// kU: E holds U (L x Np x r) and P is not used: the predictions' r-dimensional codes are read,
-// not formed.
-template <int RP, bool kU>
-__global__ void __launch_bounds__(AL_THREADS) k_align_part(const float* __restrict__ E, const float* __restrict__ P,
-                                                         const float* __restrict__ Q, const float* __restrict__ G,
-                                                         int64_t Np, int m, int64_t d, int r, int nch, int ntile,
-                                                         double* __restrict__ part) {
-  __shared__ float Qs[RP][AL_THREADS];
-  __shared__ float Ps[kMaxM][RP];
-  __shared__ float Us[AL_SUB][RP];
-  __shared__ double red[3][AL_THREADS / 32];
-  const int ch = blockIdx.x, tile = blockIdx.y, l = blockIdx.z, tid = threadIdx.x;
-  const int64_t j = int64_t(tile) * AL_THREADS + tid;
-  const bool jv = j < d;
-  for (int s = 0; s < RP; ++s) Qs[s][tid] = (s < r && jv) ? Q[(int64_t(l) * r + s) * d + j] : 0.f;
-  if (!kU)
-    for (int e = tid; e < kMaxM * RP; e += AL_THREADS) {
-      const int c = e / RP, s = e % RP;
-      Ps[c][s] = (c < m && s < r) ? P[(int64_t(l) * m + c) * r + s] : 0.f;
+__host__ __device__ constexpr int align_rp(int r) { return r <= 8 ? 8 : (r <= 16 ? 16 : 32); }
+// channels per tile: 32 / RP a lane
+__host__ __device__ constexpr int align_cols(int rp) { return 32 * (32 / rp); }
+
+template <int RP>
+__global__ void __launch_bounds__(AL_THREADS, 2) k_align_part(const float* __restrict__ U, const float* __restrict__ Q,
+                                                            const float* __restrict__ G, int64_t Np, int64_t d, int r,
+                                                            int nch, int ntile, double* __restrict__ part) {
+  constexpr int CPT = 32 / RP;
+  using Ring = RowRing<RP, CPT>;
+  constexpr int WARPS = AL_THREADS / 32;
+  extern __shared__ __align__(16) float al_smem[];
+  __shared__ double red[3][WARPS];
+  const int ch = int(blockIdx.x % unsigned(nch)), tile = int(blockIdx.x / unsigned(nch)), l = blockIdx.y, tid = threadIdx.x;
+  const int warp = tid >> 5, lane = tid & 31;
+  const int64_t j0 = int64_t(tile) * align_cols(RP), j = j0 + lane * CPT;
+  uint64_t q[RP / 2][CPT];
+#pragma unroll
+  for (int s = 0; s < RP / 2; ++s)
+#pragma unroll
+    for (int c = 0; c < CPT; ++c) {
+      const bool in = j + c < d;
+      q[s][c] = f32x2(in && 2 * s < r ? Q[(int64_t(l) * r + 2 * s) * d + j + c] : 0.f,
+                      in && 2 * s + 1 < r ? Q[(int64_t(l) * r + 2 * s + 1) * d + j + c] : 0.f);
     }
   const int64_t n0 = int64_t(ch) * AL_CHUNK;
   const int64_t n1 = (n0 + AL_CHUNK < Np) ? n0 + AL_CHUNK : Np;
   const float* Gl = G + int64_t(l) * Np * d;
-  float gt = 0.f, gg = 0.f, tt = 0.f;
-  for (int64_t s0 = n0; s0 < n1; s0 += AL_SUB) {
-    __syncthreads();
-    for (int e = tid; e < AL_SUB * RP; e += AL_THREADS) {
-      const int t = e / RP, s = e % RP;
-      float acc = 0.f;
-      if (kU) {
-        if (s0 + t < n1 && s < r) acc = E[(int64_t(l) * Np + s0 + t) * r + s];
-      } else if (s0 + t < n1) {
-        for (int c = 0; c < m; ++c) acc = fmaf(E[(s0 + t) * m + c], Ps[c][s], acc);
+  const float* Ul = U + int64_t(l) * Np * RP;
+  const bool vec = d % 4 == 0 && (reinterpret_cast<uintptr_t>(G) & 15) == 0;
+  float* ring = al_smem + warp * (2 * Ring::SLOT);
+  const int total = int((n1 - n0 + Ring::TOK - 1) / Ring::TOK);  // slots of the chunk, warp by warp in turn
+  const int mine = total > warp ? (total - warp - 1) / WARPS + 1 : 0;
+  auto issue = [&](int i) {
+    row_issue<RP, CPT>(ring + (i & 1) * Ring::SLOT, Gl, d, j0, Ul, RP, n0 + int64_t(warp + i * WARPS) * Ring::TOK, n1, vec,
+                       lane);
+  };
+  float gt[CPT], gg[CPT], tt[CPT];
+#pragma unroll
+  for (int c = 0; c < CPT; ++c) gt[c] = gg[c] = tt[c] = 0.f;
+  if (mine > 0) issue(0);
+  for (int i = 0; i < mine; ++i) {
+    if (i + 1 < mine) {
+      issue(i + 1);
+      cp_async_wait<1>();
+    } else {
+      cp_async_wait<0>();
+    }
+    __syncwarp();
+    const float* slot = ring + (i & 1) * Ring::SLOT;
+#pragma unroll 4
+    for (int t = 0; t < Ring::TOK; ++t) {  // tokens and channels out of range hold zeros
+      float g[CPT];
+      row_cols<RP, CPT>(slot, t, lane, g);
+      uint64_t tv[CPT];
+#pragma unroll
+      for (int c = 0; c < CPT; ++c) tv[c] = 0ull;
+      const ulonglong2* ur = reinterpret_cast<const ulonglong2*>(slot + Ring::Y_FLOATS + t * RP);
+#pragma unroll
+      for (int s4 = 0; s4 < RP / 4; ++s4) {
+        const ulonglong2 uv = ur[s4];
+#pragma unroll
+        for (int c = 0; c < CPT; ++c) tv[c] = fma2(uv.y, q[2 * s4 + 1][c], fma2(uv.x, q[2 * s4][c], tv[c]));
       }
-      Us[t][s] = acc;
-    }
-    __syncthreads();
-    const int nt = int((n1 - s0) < AL_SUB ? (n1 - s0) : AL_SUB);
-    for (int t = 0; t < nt; ++t) {
-      float tv = 0.f;
 #pragma unroll
-      for (int s = 0; s < RP; ++s) tv = fmaf(Us[t][s], Qs[s][tid], tv);
-      const float g = (jv && LOCA_CHECK((s0 + t) * d + j, Np * d)) ? Gl[(s0 + t) * d + j] : 0.f;
-      gt = fmaf(g, tv, gt);
-      gg = fmaf(g, g, gg);
-      tt = fmaf(tv, tv, tt);
+      for (int c = 0; c < CPT; ++c) {
+        const float2 h = f32x2_parts(tv[c]);
+        const float v = h.x + h.y;
+        gt[c] = fmaf(g[c], v, gt[c]);
+        gg[c] = fmaf(g[c], g[c], gg[c]);
+        tt[c] = fmaf(v, v, tt[c]);
+      }
     }
+    __syncwarp();  // the slot is refilled by the next issue
   }
-  double v[3] = {double(gt), double(gg), double(tt)};
+  double v[3] = {0.0, 0.0, 0.0};
 #pragma unroll
-  for (int q = 0; q < 3; ++q)
+  for (int c = 0; c < CPT; ++c) {
+    v[0] += double(gt[c]);
+    v[1] += double(gg[c]);
+    v[2] += double(tt[c]);
+  }
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) v[q] += __shfl_xor_sync(0xffffffffu, v[q], off);
-  if ((tid & 31) == 0)
-    for (int q = 0; q < 3; ++q) red[q][tid >> 5] = v[q];
+  for (int k = 0; k < 3; ++k)
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) v[k] += __shfl_xor_sync(0xffffffffu, v[k], off);
+  if (lane == 0)
+    for (int k = 0; k < 3; ++k) red[k][warp] = v[k];
   __syncthreads();
   if (tid < 3) {
     double a = 0.0;
-    for (int w = 0; w < AL_THREADS / 32; ++w) a += red[tid][w];
-    if (LOCA_CHECK(((int64_t(l) * ntile + tile) * nch + ch) * 3 + tid, int64_t(gridDim.z) * ntile * nch * 3))
+    for (int w = 0; w < WARPS; ++w) a += red[tid][w];
+    if (LOCA_CHECK(((int64_t(l) * ntile + tile) * nch + ch) * 3 + tid, int64_t(gridDim.y) * ntile * nch * 3))
       part[((int64_t(l) * ntile + tile) * nch + ch) * 3 + tid] = a;
   }
 }
 
+// One warp per block: lanes over the partial triples, then a fixed butterfly.
 __global__ void k_align_final(const double* __restrict__ part, int nparts, double* __restrict__ alpha) {
-  const int l = blockIdx.x;
-  if (threadIdx.x != 0) return;
-  double gt = 0.0, gg = 0.0, tt = 0.0;
-  for (int i = 0; i < nparts; ++i) {
+  const int l = blockIdx.x, lane = threadIdx.x;
+  double v[3] = {0.0, 0.0, 0.0};
+  for (int i = lane; i < nparts; i += 32) {
     const double* p = part + (int64_t(l) * nparts + i) * 3;
-    gt += p[0];
-    gg += p[1];
-    tt += p[2];
+    for (int k = 0; k < 3; ++k) v[k] += p[k];
   }
-  if (LOCA_CHECK(l, gridDim.x)) alpha[l] = (gg > 0.0 && tt > 0.0) ? gt / sqrt(gg * tt) : 0.0;
+#pragma unroll
+  for (int k = 0; k < 3; ++k)
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) v[k] += __shfl_xor_sync(0xffffffffu, v[k], off);
+  if (lane == 0 && LOCA_CHECK(l, gridDim.x)) alpha[l] = (v[1] > 0.0 && v[2] > 0.0) ? v[0] / sqrt(v[1] * v[2]) : 0.0;
 }
 
 }  // namespace
@@ -150,34 +184,31 @@ __global__ void k_align_final(const double* __restrict__ part, int nparts, doubl
 int align_max_m() { return kMaxWideM; }
 int align_max_r() { return kMaxR; }
 
-static size_t part_bytes(int64_t Np, int64_t d, int L) {
+static size_t part_bytes(int64_t Np, int64_t d, int L, int r) {
   const int64_t nch = (Np + AL_CHUNK - 1) / AL_CHUNK;
-  const int64_t ntile = (d + AL_THREADS - 1) / AL_THREADS;
+  const int64_t ntile = (d + align_cols(align_rp(r)) - 1) / align_cols(align_rp(r));
   return align256(sizeof(double) * 3 * size_t(L) * size_t(nch) * size_t(ntile));
 }
 
 size_t align_workspace_bytes(int64_t Np, int m, int64_t d, int L, int r) {
-  const size_t u = m > kMaxM ? align256(sizeof(float) * size_t(L) * size_t(Np) * size_t(r)) : 0;
-  return part_bytes(Np, d, L) + u;
+  (void)m;
+  return part_bytes(Np, d, L, r) + align256(sizeof(float) * size_t(L) * size_t(Np) * size_t(align_rp(r)));
 }
 
 template <int RP>
 static cudaError_t align_t(const float* E, const float* G, int64_t Np, int m, int64_t d, int L, const float* P,
                            const float* Q, int r, double* alpha, void* workspace, cudaStream_t s) {
   const int nch = int((Np + AL_CHUNK - 1) / AL_CHUNK);
-  const int ntile = int((d + AL_THREADS - 1) / AL_THREADS);
+  const int ntile = int((d + align_cols(RP) - 1) / align_cols(RP));
   double* part = static_cast<double*>(workspace);
-  const dim3 grid = dim3(unsigned(nch), unsigned(ntile), unsigned(L));
-  if (m > kMaxM) {
-    float* U = reinterpret_cast<float*>(static_cast<char*>(workspace) + part_bytes(Np, d, L));
-    k_align_u<RP><<<dim3(unsigned((Np + AU_TOK - 1) / AU_TOK), unsigned(L)), AL_THREADS, 0, s>>>(E, P, Np, m, r, U);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    k_align_part<RP, true><<<grid, AL_THREADS, 0, s>>>(U, P, Q, G, Np, r, d, r, nch, ntile, part);
-  } else {
-    k_align_part<RP, false><<<grid, AL_THREADS, 0, s>>>(E, P, Q, G, Np, m, d, r, nch, ntile, part);
-  }
-  cudaError_t e = cudaGetLastError();
+  float* U = reinterpret_cast<float*>(static_cast<char*>(workspace) + part_bytes(Np, d, L, r));
+  k_align_u<RP><<<dim3(unsigned((Np + AU_TOK - 1) / AU_TOK), unsigned(L)), AL_THREADS, 0, s>>>(E, P, Np, m, r, U);
+  constexpr int smem = AL_THREADS / 32 * RowRing<RP, 32 / RP>::BYTES;
+  cudaError_t e = cudaFuncSetAttribute(k_align_part<RP>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return e;
+  k_align_part<RP><<<dim3(unsigned(nch) * unsigned(ntile), unsigned(L)), AL_THREADS, smem, s>>>(U, Q, G, Np, d, r, nch,
+                                                                                              ntile, part);
+  e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   k_align_final<<<L, 32, 0, s>>>(part, nch * ntile, alpha);
   return cudaGetLastError();

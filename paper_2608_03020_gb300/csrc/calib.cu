@@ -1,274 +1,526 @@
 // One-shot reduced-rank fit of every block's feedback map from probe-backward pairs (Eq. 5;
-// Theorem "Feedback ridge solution" and Lemma "Rank-truncation error", S5).  Untimed: it
-// runs once, before Stage II.
+// Theorem "Feedback ridge solution" and Lemma "Rank-truncation error", S5).  It runs once, before
+// Stage II.
 //
 // Token-major probe pairs: E_probe (Np x m) and G_probe_l (Np x d).
-//   k_calib_xty    K = E^T E (m x m) and R_l = E^T G_l (m x d): fp32 products summed over
-//                  32-token chunks, chunks accumulated in fp64.
-//   k_calib_solve  per block l: Cholesky of K + beta I (fp64), F_l^T = (K + beta I)^-1 R_l by
-//                  two triangular substitutions per column (no inverse), then the m x m matrix
-//                  M = F^T F^T^T, its eigen-decomposition by cyclic Jacobi rotations (fp64),
-//                  which gives the left singular vectors U and sigma = sqrt(eig) of F^T, and
-//                  P_l = U_r S_r, Q_l = S_r^-1 U_r^T F^T = V_r^T.  Signs: the largest-magnitude
-//                  entry of each Q row is made positive.  Singular values below 1e-12 sigma_1
-//                  are treated as zero (zero Q row, zero P column).
+//   k_calib_pad    E with rows padded to 8, 16, 32 or 64 values (16-byte rows for every m).
+//   k_calib_xty    K = E^T E (m x m) and R_l = E^T G_l (m x d) in one launch, as partial sums over
+//                  token ranges: fp32 products summed over 32-token runs, the runs in pairs of fp32
+//                  values (sum and its rounding error, ~2^-48), warps and ranges in fp64.
+//   k_calib_chol   Cholesky of K + beta I (fp64), shared by all blocks.
+//   k_calib_fwd    F_l^T = (K + beta I)^-1 R_l by two triangular substitutions per column (no
+//                  inverse), one thread per column, and the partial sums of M = F^T F^T^T over the
+//                  CTA's columns.
+//   k_calib_eig    per block: M, its eigen-decomposition by Jacobi rotations (fp64), which gives
+//                  the left singular vectors U and sigma = sqrt(eig) of F^T.  Singular values below
+//                  1e-12 sigma_1 are treated as zero (zero Q row, zero P column).
+//   k_calib_q      Q_l = S_r^-1 U_r^T F^T = V_r^T, one thread per column, and the entry of largest
+//                  magnitude of each row over the CTA's columns.
+//   k_calib_sign   signs: the largest-magnitude entry of each Q row is made positive; P_l = U_r S_r.
+// The first version kept everything after R_l in one CTA per block (1.14 ms at L = 28, d = 1536, m = 16)
+// and summed E^T E in a single CTA (~1 ms).
 #include <cuda_runtime.h>
 
 #include "jacobi.cuh"
 #include "loca_internal.h"
+#include "row_stream.cuh"
 
 namespace loca {
 namespace {
 
-constexpr int XT_COLS = 64;
-constexpr int XT_TOK = 32;
+constexpr int XT_RUN = 32;       // tokens per fp32 run
+constexpr int CF_COLS = 128;     // columns per CTA of k_calib_fwd and k_calib_q
 
-// out[b][s][j] = sum_n E[n][s] Y_b[n][j]   (s < m, j < w); Y_b = Y + b * Np * w
+// s values and columns per thread: 32 sums, whatever m
 template <int KM>
-__global__ void __launch_bounds__(256) k_calib_xty(const float* __restrict__ E, const float* __restrict__ Y,
-                                                  int64_t Np, int m, int64_t w, double* __restrict__ out) {
-  constexpr int SPT = KM / 4;  // s values per thread
-  __shared__ float Es[XT_TOK][KM];
-  __shared__ float Ys[XT_TOK][XT_COLS];
-  const int b = blockIdx.y;
-  const int jj = threadIdx.x % XT_COLS, grp = threadIdx.x / XT_COLS;
-  const int64_t j = int64_t(blockIdx.x) * XT_COLS + jj;
-  const float* Yb = Y + int64_t(b) * Np * w;
-  double acc[SPT];
+struct Xty {
+  static constexpr int SV = KM < 32 ? KM : 32;
+  static constexpr int CPT = 32 / SV;
+  static constexpr int SG = KM / SV;   // groups of s values (warps)
+  static constexpr int TW = 8 / SG;    // warps over the tokens
+  static constexpr int COLS = 32 * CPT;
+  using Ring = RowRing<SV, CPT>;
+  static constexpr int SMEM = 8 * Ring::BYTES > SG * 32 * 33 * 8 ? 8 * Ring::BYTES : SG * 32 * 33 * 8;
+};
+
+__host__ __device__ constexpr int calib_cols(int m) { return m <= 8 ? 128 : (m <= 16 ? 64 : 32); }
+
+// Token ranges (grid.y): enough CTAs for several waves on the 152 SMs, at least 1024 tokens each.
+int64_t calib_splits(int64_t Np, int m, int64_t d, int L) {
+  const int64_t tiles = (d + calib_cols(m) - 1) / calib_cols(m) * L;
+  int64_t s = (16 * 152 + tiles - 1) / tiles;
+  const int64_t most = (Np + 1023) / 1024;
+  if (s > most) s = most;
+  if (s > 16) s = 16;
+  return s < 1 ? 1 : s;
+}
+
+__global__ void __launch_bounds__(256) k_calib_pad(const float* __restrict__ E, int64_t Np, int m, int km,
+                                                  float* __restrict__ Ep) {
+  const int64_t e = int64_t(blockIdx.x) * 256 + threadIdx.x;
+  if (e >= Np * km) return;
+  const int64_t n = e / km;
+  const int s = int(e - n * km);
+  Ep[e] = s < m ? E[n * m + s] : 0.f;
+}
+
+// part[split][b][s][j] = sum over the split's tokens of E[n][s] Y_b[n][j]; the first `tiles`
+// CTAs of grid.x take Y = E (K, width m), the next ones block after block of G (width d).  A lane owns
+// CPT columns and SV values of s (32 sums, in pairs along s); each warp streams every TW-th run of
+// 32 tokens through its own ring (row_stream.cuh).  Bound by the read of G: 1.41 GB at L = 28, Np = 8192,
+// d = 1536.  (A thread per column and 4 values of s over CTA-staged tiles, with an fp64 addition per
+// run and sum, took 1.0 ms for G and 1.0 ms more for E^T E in one CTA; fp64 adds run at 2 per clock and
+// SM.)
+template <int KM>
+__global__ void __launch_bounds__(256, 2) k_calib_xty(const float* __restrict__ E, const float* __restrict__ Ep,
+                                                     const float* __restrict__ G, int64_t Np, int m, int64_t d,
+                                                     int64_t per, int L, int tiles, double* __restrict__ Kp,
+                                                     double* __restrict__ Rp) {
+  using T = Xty<KM>;
+  using Ring = typename T::Ring;
+  extern __shared__ __align__(16) float xt_smem[];
+  const int b = int(blockIdx.x / unsigned(tiles)) - 1;
+  const int tile = int(blockIdx.x % unsigned(tiles));
+  const bool isK = b < 0;
+  const int64_t w = isK ? m : d;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int sg = warp / T::TW, tw = warp % T::TW;
+  const int64_t j0 = int64_t(tile) * T::COLS;
+  if (j0 >= w) return;  // K has fewer column tiles
+  const float* Y = isK ? E : G + int64_t(b) * Np * d;
+  const int64_t n0 = per * blockIdx.y, n1 = n0 + per < Np ? n0 + per : Np;
+  const bool vec = w % 4 == 0 && (reinterpret_cast<uintptr_t>(Y) & 15) == 0;
+  float* ring = xt_smem + warp * (2 * Ring::SLOT);
+  uint64_t part[T::SV / 2][T::CPT], hi[T::SV / 2][T::CPT], lo[T::SV / 2][T::CPT];
 #pragma unroll
-  for (int i = 0; i < SPT; ++i) acc[i] = 0.0;
-  for (int64_t n0 = 0; n0 < Np; n0 += XT_TOK) {
-    __syncthreads();
-    for (int e = threadIdx.x; e < XT_TOK * KM; e += 256) {
-      const int nn = e / KM, s = e % KM;
-      Es[nn][s] = (n0 + nn < Np && s < m) ? E[(n0 + nn) * m + s] : 0.f;
-    }
-    for (int e = threadIdx.x; e < XT_TOK * XT_COLS; e += 256) {
-      const int nn = e / XT_COLS, c = e % XT_COLS;
-      const int64_t jc = int64_t(blockIdx.x) * XT_COLS + c;
-      Ys[nn][c] = (n0 + nn < Np && jc < w && LOCA_CHECK((n0 + nn) * w + jc, Np * w)) ? Yb[(n0 + nn) * w + jc] : 0.f;
-    }
-    __syncthreads();
-    float part[SPT];
+  for (int s = 0; s < T::SV / 2; ++s)
 #pragma unroll
-    for (int i = 0; i < SPT; ++i) part[i] = 0.f;
+    for (int c = 0; c < T::CPT; ++c) part[s][c] = hi[s][c] = lo[s][c] = 0ull;
+  constexpr int PER_RUN = XT_RUN / Ring::TOK;
+  const int64_t runs = (n1 - n0 + XT_RUN - 1) / XT_RUN;  // <= 0: an empty range
+  const int64_t slots = runs > tw ? ((runs - tw - 1) / T::TW + 1) * PER_RUN : 0;
+  auto issue = [&](int64_t i) {
+    const int64_t n = n0 + (tw + (i / PER_RUN) * T::TW) * XT_RUN + (i % PER_RUN) * Ring::TOK;
+    (void)LOCA_CHECK(j0, w);
+    row_issue<T::SV, T::CPT>(ring + (i & 1) * Ring::SLOT, Y, w, j0, Ep + sg * T::SV, KM, n, n1, vec, lane);
+  };
+  if (slots > 0) issue(0);
+  for (int64_t i = 0; i < slots; ++i) {
+    if (i + 1 < slots) {
+      issue(i + 1);
+      cp_async_wait<1>();
+    } else {
+      cp_async_wait<0>();
+    }
+    __syncwarp();
+    const float* slot = ring + (i & 1) * Ring::SLOT;
 #pragma unroll 4
-    for (int nn = 0; nn < XT_TOK; ++nn) {
-      const float yv = Ys[nn][jj];
+    for (int t = 0; t < Ring::TOK; ++t) {
+      float y[T::CPT];
+      row_cols<T::SV, T::CPT>(slot, t, lane, y);
+      uint64_t yy[T::CPT];
 #pragma unroll
-      for (int i = 0; i < SPT; ++i) part[i] = fmaf(Es[nn][grp + 4 * i], yv, part[i]);
+      for (int c = 0; c < T::CPT; ++c) yy[c] = f32x2(y[c], y[c]);
+      const ulonglong2* er = reinterpret_cast<const ulonglong2*>(slot + Ring::Y_FLOATS + t * T::SV);
+#pragma unroll
+      for (int s4 = 0; s4 < T::SV / 4; ++s4) {
+        const ulonglong2 ev = er[s4];
+#pragma unroll
+        for (int c = 0; c < T::CPT; ++c) {
+          part[2 * s4][c] = fma2(ev.x, yy[c], part[2 * s4][c]);
+          part[2 * s4 + 1][c] = fma2(ev.y, yy[c], part[2 * s4 + 1][c]);
+        }
+      }
     }
+    __syncwarp();  // the slot is refilled by the next issue
+    if (i % PER_RUN == PER_RUN - 1) {
+      // hi + lo += part: the sum and its rounding error (Knuth's two-sum), the errors summed in lo
 #pragma unroll
-    for (int i = 0; i < SPT; ++i) acc[i] += double(part[i]);
+      for (int s = 0; s < T::SV / 2; ++s)
+#pragma unroll
+        for (int c = 0; c < T::CPT; ++c) {
+          const uint64_t a = hi[s][c], p = part[s][c];
+          const uint64_t t = add2(a, p), bb = sub2(t, a);
+          lo[s][c] = add2(lo[s][c], add2(sub2(a, sub2(t, bb)), sub2(p, bb)));
+          hi[s][c] = t;
+          part[s][c] = 0ull;
+        }
+    }
   }
-  if (j >= w) return;
+  // warps in order, fp64 (the ring's memory is free)
+  double(*sum)[32][33] = reinterpret_cast<double(*)[32][33]>(xt_smem);
+  for (int q = 0; q < T::TW; ++q) {
+    __syncthreads();
+    if (tw == q) {
 #pragma unroll
-  for (int i = 0; i < SPT; ++i) {
-    const int s = grp + 4 * i;
-    if (s < m && LOCA_CHECK((int64_t(b) * m + s) * w + j, int64_t(gridDim.y) * m * w)) out[(int64_t(b) * m + s) * w + j] = acc[i];
+      for (int s = 0; s < T::SV / 2; ++s)
+#pragma unroll
+        for (int c = 0; c < T::CPT; ++c) {
+          const float2 h = f32x2_parts(hi[s][c]), e = f32x2_parts(lo[s][c]);
+          const double v0 = isfinite(h.x) ? double(h.x) + double(e.x) : double(h.x);
+          const double v1 = isfinite(h.y) ? double(h.y) + double(e.y) : double(h.y);
+          double& o0 = sum[sg][2 * s * T::CPT + c][lane];
+          double& o1 = sum[sg][(2 * s + 1) * T::CPT + c][lane];
+          o0 = q == 0 ? v0 : o0 + v0;
+          o1 = q == 0 ? v1 : o1 + v1;
+        }
+    }
+  }
+  __syncthreads();
+  double* out = isK ? Kp + int64_t(blockIdx.y) * m * m : Rp + (int64_t(blockIdx.y) * L + b) * m * d;
+  for (int e = threadIdx.x; e < T::SG * 32 * 32; e += 256) {
+    const int col = e % T::COLS, sl = (e / T::COLS) % T::SV, g = e / (T::COLS * T::SV);
+    const int s = g * T::SV + sl;
+    const int64_t jc = j0 + col;
+    if (s < m && jc < w && LOCA_CHECK(int64_t(s) * w + jc, int64_t(m) * w))
+      out[int64_t(s) * w + jc] = sum[g][sl * T::CPT + col % T::CPT][col / T::CPT];
   }
 }
 
+// K + beta I = L L^T (padded to KM with an identity block): fac = L (lower, row-major) and the
+// reciprocals of its diagonal.  Positive definite for beta > 0 in exact arithmetic; a pivot that is
+// not positive means beta is below the rounding level of E^T E: reported, outputs zeroed.
 template <int KM>
-struct CalibSmem {
-  double Kc[KM][KM];  // K + beta I, then its Cholesky factor (lower)
-  double A[KM][KM];   // F^T F^T^T, rotated towards diagonal
-  double V[KM][KM];   // accumulated rotations (eigenvectors in columns)
-  double red[256];
-  int order[KM];
-  int arg[256];
-};
-
-template <int KM>
-__global__ void __launch_bounds__(256) k_calib_solve(const double* __restrict__ K, double* __restrict__ R,
-                                                    int m, int64_t d, float beta, int r,
-                                                    float* __restrict__ P, float* __restrict__ Q,
-                                                    float* __restrict__ sigma, int32_t* status) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  CalibSmem<KM>& sm = *reinterpret_cast<CalibSmem<KM>*>(smem_raw);
-  __shared__ int s_bad;
-  const int l = blockIdx.x;
+__global__ void __launch_bounds__(256) k_calib_chol(const double* __restrict__ Kp, int splits, int m, float beta,
+                                                   double* __restrict__ fac, int32_t* __restrict__ bad,
+                                                   int32_t* status) {
+  __shared__ double S[KM][KM + 1];
+  __shared__ double rinv[KM];
   const int t = threadIdx.x;
-  double* F = R + int64_t(l) * m * d;  // R_l, overwritten with F_hat^T (m x d)
-
   for (int e = t; e < KM * KM; e += 256) {
     const int a = e / KM, b = e % KM;
-    double v;
+    double v = (a == b) ? 1.0 : 0.0;
     if (a < m && b < m) {
-      v = K[a * m + b];
+      v = 0.0;
+      for (int q = 0; q < splits; ++q) v += Kp[int64_t(q) * m * m + a * m + b];
       if (a == b) v += double(beta);
-    } else {
-      v = (a == b) ? 1.0 : 0.0;
     }
-    sm.Kc[a][b] = v;
+    S[a][b] = v;
   }
   __syncthreads();
-  // Cholesky of K + beta I (positive definite for beta > 0 in exact arithmetic; a pivot that is
-  // not positive means beta is below the rounding level of E^T E: reported, outputs zeroed)
-  if (t == 0) s_bad = 0;
-  __syncthreads();
-  if (t < 32) {
-    for (int c = 0; c < KM; ++c) {
-      double diag = sm.Kc[c][c];
-      for (int u = 0; u < c; ++u) diag -= sm.Kc[c][u] * sm.Kc[c][u];
-      if (!(diag > 0.0)) {
-        if (t == 0) s_bad = 1;
-        break;
-      }
-      const double lcc = sqrt(diag);
-      __syncwarp();
-      for (int rr = c + 1 + t; rr < KM; rr += 32) {
-        double v = sm.Kc[rr][c];
-        for (int u = 0; u < c; ++u) v -= sm.Kc[rr][u] * sm.Kc[c][u];
-        sm.Kc[rr][c] = v / lcc;
-      }
-      __syncwarp();
-      if (t == 0) sm.Kc[c][c] = lcc;
-      __syncwarp();
+  int failed = 0;
+  for (int c = 0; c < KM; ++c) {
+    const double diag = S[c][c];
+    if (!(diag > 0.0)) {  // the same value in every thread
+      failed = 1;
+      break;
     }
+    const double inv = rsqrt(diag), lcc = diag * inv;
+    __syncthreads();
+    if (t > c && t < KM) S[t][c] *= inv;
+    if (t == c) {
+      S[c][c] = lcc;
+      rinv[c] = inv;
+    }
+    __syncthreads();
+    const int rem = KM - 1 - c;
+    for (int e = t; e < rem * rem; e += 256) {
+      const int a = c + 1 + e / rem, b = c + 1 + e % rem;
+      if (b <= a) S[a][b] = fma(-S[a][c], S[b][c], S[a][b]);
+    }
+    __syncthreads();
   }
+  if (t == 0) {
+    *bad = failed;
+    if (failed) atomicExch(status, int32_t(LOCA_ERR_NUMERIC));
+  }
+  if (failed) return;
+  for (int e = t; e < KM * KM; e += 256) fac[e] = S[e / KM][e % KM];
+  for (int e = t; e < KM; e += 256) fac[KM * KM + e] = rinv[e];
+}
+
+// One thread per column j of block l: x = (K + beta I)^-1 R_l[:, j], R_l the sum of its token ranges in
+// order.  F overwrites the first range.  Then M's partial sums over the CTA's columns (upper
+// triangle).  The columns stay in shared memory (one per thread): the fp64 pipe is the limit, not the
+// shared loads, and with x in registers the unrolled factor spilled (up to 18 KB a thread).
+template <int KM>
+__global__ void __launch_bounds__(CF_COLS) k_calib_fwd(const double* __restrict__ fac, const int32_t* __restrict__ bad,
+                                                      double* __restrict__ R, int splits, int m, int64_t d,
+                                                      int64_t range, double* __restrict__ Mp) {
+  extern __shared__ __align__(16) double cf_smem[];
+  double* Lf = cf_smem;                 // KM x KM
+  double* rinv = Lf + KM * KM;          // KM
+  double* Fs = rinv + KM;               // KM x (CF_COLS + 1)
+  if (*bad) return;
+  const int l = blockIdx.y, t = threadIdx.x;
+  for (int e = t; e < KM * KM + KM; e += CF_COLS) Lf[e] = fac[e];
   __syncthreads();
-  if (s_bad) {
-    if (t == 0) atomicExch(status, int32_t(LOCA_ERR_NUMERIC));
-    if (!LOCA_CHECK_SPAN(int64_t(l) * r * d, int64_t(r) * d, int64_t(gridDim.x) * r * d)) return;
-    for (int64_t e = t; e < int64_t(r) * d; e += 256) Q[int64_t(l) * r * d + e] = 0.f;
-    for (int e = t; e < m * r; e += 256) P[int64_t(l) * m * r + e] = 0.f;
-    if (sigma != nullptr)
-      for (int e = t; e < r; e += 256) sigma[int64_t(l) * r + e] = 0.f;
+  const int64_t j = int64_t(blockIdx.x) * CF_COLS + t;
+  const bool in = j < d && LOCA_CHECK((int64_t(l) * m + m - 1) * d + j, range);
+  double* F = R + int64_t(l) * m * d + j;
+  double* x = Fs + t;  // x[s] at x[s * XS]
+  constexpr int XS = CF_COLS + 1;
+  for (int s = 0; s < m; ++s) {
+    double v = 0.0;
+    if (in)
+      for (int q = 0; q < splits; ++q) v += F[int64_t(q) * range + int64_t(s) * d];
+    x[s * XS] = v;
+  }
+  auto dot = [&](double a, int s, int u0, int u1, int step) {  // a - sum_u L(s, u) x[u], L read with `step`
+    double a1 = 0.0, a2 = 0.0, a3 = 0.0;
+    int u = u0;
+    const double* lp = Lf + s;
+    for (; u + 3 < u1; u += 4) {
+      a = fma(-lp[u * step], x[u * XS], a);
+      a1 = fma(-lp[(u + 1) * step], x[(u + 1) * XS], a1);
+      a2 = fma(-lp[(u + 2) * step], x[(u + 2) * XS], a2);
+      a3 = fma(-lp[(u + 3) * step], x[(u + 3) * XS], a3);
+    }
+    for (; u < u1; ++u) a = fma(-lp[u * step], x[u * XS], a);
+    return (a + a1) + (a2 + a3);
+  };
+  for (int s = 0; s < m; ++s) x[s * XS] = dot(x[s * XS], s * KM, 0, s, 1) * rinv[s];
+  for (int s = m - 1; s >= 0; --s) x[s * XS] = dot(x[s * XS], s, s + 1, m, KM) * rinv[s];
+  if (in)
+    for (int s = 0; s < m; ++s) F[int64_t(s) * d] = x[s * XS];
+  __syncthreads();
+  const int nt = m * (m + 1) / 2;
+  double* out = Mp + (int64_t(l) * gridDim.x + blockIdx.x) * nt;
+  for (int e = t; e < nt; e += CF_COLS) {
+    int a = 0, b = e;  // e-th entry of the upper triangle
+    while (b >= m - a) b -= m - a++;
+    b += a;
+    const double *fa = Fs + a * (CF_COLS + 1), *fb = Fs + b * (CF_COLS + 1);
+    double v0 = 0.0, v1 = 0.0, v2 = 0.0, v3 = 0.0;
+#pragma unroll 4
+    for (int c = 0; c < CF_COLS; c += 4) {
+      v0 = fma(fa[c], fb[c], v0);
+      v1 = fma(fa[c + 1], fb[c + 1], v1);
+      v2 = fma(fa[c + 2], fb[c + 2], v2);
+      v3 = fma(fa[c + 3], fb[c + 3], v3);
+    }
+    out[e] = (v0 + v1) + (v2 + v3);
+  }
+}
+
+// Per block: M = F^T F^T^T from its partial sums in order, its eigenpairs; the leading r: vectors to
+// Ur[l] (m x r) and singular values to sg[l] (r).
+template <int KM>
+__global__ void __launch_bounds__(256) k_calib_eig(const double* __restrict__ Mp, int ntile, int m, int r,
+                                                  const int32_t* __restrict__ bad, double* __restrict__ Ur,
+                                                  double* __restrict__ sg, float* __restrict__ sigma) {
+  extern __shared__ __align__(16) unsigned char ce_smem[];
+  double(*A)[KM] = reinterpret_cast<double(*)[KM]>(ce_smem);
+  double(*V)[KM] = reinterpret_cast<double(*)[KM]>(ce_smem + sizeof(double) * KM * KM);
+  __shared__ int order[KM];
+  const int l = blockIdx.x, t = threadIdx.x;
+  if (*bad) {
+    for (int i = t; i < r; i += 256) {
+      sg[int64_t(l) * r + i] = 0.0;
+      if (sigma != nullptr) sigma[int64_t(l) * r + i] = 0.f;
+    }
+    for (int e = t; e < m * r; e += 256) Ur[int64_t(l) * m * r + e] = 0.0;
     return;
   }
-  // F^T[:, j] = (K + beta I)^-1 R[:, j]
-  for (int64_t j = t; j < d; j += 256) {
-    double x[KM];
-#pragma unroll
-    for (int s = 0; s < KM; ++s) x[s] = (s < m) ? F[int64_t(s) * d + j] : 0.0;
-#pragma unroll
-    for (int s = 0; s < KM; ++s) {
-      double a = x[s];
-#pragma unroll
-      for (int u = 0; u < s; ++u) a -= sm.Kc[s][u] * x[u];
-      x[s] = a / sm.Kc[s][s];
-    }
-#pragma unroll
-    for (int s = KM - 1; s >= 0; --s) {
-      double a = x[s];
-#pragma unroll
-      for (int u = s + 1; u < KM; ++u) a -= sm.Kc[u][s] * x[u];
-      x[s] = a / sm.Kc[s][s];
-    }
-#pragma unroll
-    for (int s = 0; s < KM; ++s)
-      if (s < m) F[int64_t(s) * d + j] = x[s];
+  for (int e = t; e < KM * KM; e += 256) {
+    A[e / KM][e % KM] = 0.0;
+    V[e / KM][e % KM] = (e / KM == e % KM) ? 1.0 : 0.0;
   }
   __syncthreads();
-  // A = F^T (F^T)^T  (m x m), V = I
-  for (int e = t; e < KM * KM; e += 256) {
-    const int a = e / KM, b = e % KM;
+  const int nt = m * (m + 1) / 2;
+  for (int e = t; e < nt; e += 256) {
+    int a = 0, b = e;
+    while (b >= m - a) b -= m - a++;
+    b += a;
+    const double* p = Mp + int64_t(l) * ntile * nt + e;
     double v = 0.0;
-    if (a < m && b < m && a <= b) {
-      const double* fa = F + int64_t(a) * d;
-      const double* fb = F + int64_t(b) * d;
-      for (int64_t j = 0; j < d; ++j) v += fa[j] * fb[j];
-    }
-    sm.A[a][b] = v;
-    sm.V[a][b] = (a == b) ? 1.0 : 0.0;
+#pragma unroll 4
+    for (int q = 0; q < ntile; ++q) v += p[int64_t(q) * nt];
+    A[a][b] = v;
+    A[b][a] = v;
   }
   __syncthreads();
-  for (int e = t; e < KM * KM; e += 256) {
-    const int a = e / KM, b = e % KM;
-    if (a > b) sm.A[a][b] = sm.A[b][a];
-  }
-  __syncthreads();
-  // eigen-decomposition of F^T F^T^T by Jacobi rotations (whole block)
-  jacobi_eig_block<KM>(sm.A, sm.V, sm.order, m);
-  __syncthreads();
-  const double lam1 = sm.A[sm.order[0]][sm.order[0]];
+  jacobi_eig_block<KM>(A, V, order, m);
+  const double lam1 = A[order[0]][order[0]];
   const double s1 = lam1 > 0.0 ? sqrt(lam1) : 0.0;
-  for (int i = 0; i < r; ++i) {
-    const int col = sm.order[i];
-    const double lam = (i < m) ? sm.A[col][col] : 0.0;
-    double sg = lam > 0.0 ? sqrt(lam) : 0.0;
-    if (!(sg > 1e-12 * s1)) sg = 0.0;
-    float* qrow = Q + (int64_t(l) * r + i) * d;
-    if (!LOCA_CHECK_SPAN((int64_t(l) * r + i) * d, d, int64_t(gridDim.x) * r * d)) break;
-    // Q row = U_i^T F^T / sigma_i ; track the entry of largest magnitude (lowest index on ties)
-    double best = -1.0;
-    int64_t bj = 0;
-    for (int64_t j = t; j < d; j += 256) {
-      double v = 0.0;
-      if (sg > 0.0) {
-        for (int a = 0; a < m; ++a) v += sm.V[a][col] * F[int64_t(a) * d + j];
-        v /= sg;
-      }
-      qrow[j] = float(v);
-      if (fabs(v) > best) {
-        best = fabs(v);
-        bj = j;
-      }
-    }
-    sm.red[t] = best;
-    sm.arg[t] = int(bj);
-    __syncthreads();
-    for (int wdt = 128; wdt > 0; wdt >>= 1) {
-      if (t < wdt) {
-        const double o = sm.red[t + wdt];
-        const int oa = sm.arg[t + wdt];
-        if (o > sm.red[t] || (o == sm.red[t] && oa < sm.arg[t])) {
-          sm.red[t] = o;
-          sm.arg[t] = oa;
-        }
-      }
-      __syncthreads();
-    }
-    const int64_t jmax = sm.arg[0];
-    __syncthreads();
-    const float sign = (qrow[jmax] < 0.f) ? -1.f : 1.f;
-    __syncthreads();
-    if (sign < 0.f)
-      for (int64_t j = t; j < d; j += 256) qrow[j] = -qrow[j];
-    for (int a = t; a < m; a += 256)
-      if (LOCA_CHECK((int64_t(l) * m + a) * r + i, int64_t(gridDim.x) * m * r)) P[(int64_t(l) * m + a) * r + i] = float(sign * sm.V[a][col] * sg);
-    if (sigma != nullptr && t == 0) sigma[int64_t(l) * r + i] = float(sg);
-    __syncthreads();
+  for (int i = t; i < r; i += 256) {
+    const double lam = A[order[i]][order[i]];
+    double v = lam > 0.0 ? sqrt(lam) : 0.0;
+    if (!(v > 1e-12 * s1)) v = 0.0;
+    sg[int64_t(l) * r + i] = v;
+    if (sigma != nullptr) sigma[int64_t(l) * r + i] = float(v);
   }
+  for (int e = t; e < m * r; e += 256) Ur[int64_t(l) * m * r + e] = V[e / r][order[e % r]];
+}
+
+// Q_l[i][j] = U_i^T F^T[:, j] / sigma_i for the CTA's columns, and each row's entry of largest
+// magnitude among them (lowest index on ties; NaN never wins).
+template <int KM>
+__global__ void __launch_bounds__(CF_COLS) k_calib_q(const double* __restrict__ R, const double* __restrict__ Ur,
+                                                    const double* __restrict__ sg, int m, int64_t d, int r,
+                                                    float* __restrict__ Q, double* __restrict__ amax_v,
+                                                    int64_t* __restrict__ amax_i) {
+  __shared__ double Us[KM * KM];
+  __shared__ double si[KM];  // 1 / sigma_i, 0 where sigma_i is 0
+  __shared__ double bv[KM][CF_COLS / 32];
+  __shared__ int64_t bi[KM][CF_COLS / 32];
+  const int l = blockIdx.y, t = threadIdx.x, lane = t & 31, wid = t >> 5;
+  for (int e = t; e < m * r; e += CF_COLS) Us[e] = Ur[int64_t(l) * m * r + e];
+  for (int e = t; e < r; e += CF_COLS) si[e] = sg[int64_t(l) * r + e] > 0.0 ? 1.0 / sg[int64_t(l) * r + e] : 0.0;
+  __syncthreads();
+  const int64_t j = int64_t(blockIdx.x) * CF_COLS + t;
+  const bool in = j < d;
+  double x[KM];
+#pragma unroll
+  for (int s = 0; s < KM; ++s) x[s] = (in && s < m) ? R[(int64_t(l) * m + s) * d + j] : 0.0;
+  for (int i = 0; i < r; ++i) {
+    double v = 0.0;
+    if (si[i] > 0.0) {
+#pragma unroll
+      for (int s = 0; s < KM; ++s)
+        if (s < m) v = fma(Us[s * r + i], x[s], v);
+      v *= si[i];
+    }
+    if (in && LOCA_CHECK((int64_t(l) * r + i) * d + j, int64_t(gridDim.y) * r * d)) Q[(int64_t(l) * r + i) * d + j] = float(v);
+    double best = (in && v == v) ? fabs(v) : -1.0;
+    int64_t bj = j;
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+      const double ob = __shfl_xor_sync(0xffffffffu, best, off);
+      const int64_t oj = __shfl_xor_sync(0xffffffffu, bj, off);
+      if (ob > best || (ob == best && oj < bj)) {
+        best = ob;
+        bj = oj;
+      }
+    }
+    if (lane == 0) {
+      bv[i][wid] = best;
+      bi[i][wid] = bj;
+    }
+  }
+  __syncthreads();
+  for (int i = t; i < r; i += CF_COLS) {
+    double best = bv[i][0];
+    int64_t bj = bi[i][0];
+    for (int w = 1; w < CF_COLS / 32; ++w)
+      if (bv[i][w] > best || (bv[i][w] == best && bi[i][w] < bj)) {
+        best = bv[i][w];
+        bj = bi[i][w];
+      }
+    amax_v[(int64_t(l) * r + i) * gridDim.x + blockIdx.x] = best;
+    amax_i[(int64_t(l) * r + i) * gridDim.x + blockIdx.x] = bj;
+  }
+}
+
+// grid (r, L): the sign of Q_l row i, and P_l column i.
+__global__ void __launch_bounds__(128) k_calib_sign(const double* __restrict__ amax_v, const int64_t* __restrict__ amax_i,
+                                                   int ntile, const double* __restrict__ Ur,
+                                                   const double* __restrict__ sg, int m, int64_t d, int r,
+                                                   float* __restrict__ P, float* __restrict__ Q) {
+  const int i = blockIdx.x, l = blockIdx.y, lane = threadIdx.x & 31;
+  const double* bv = amax_v + (int64_t(l) * r + i) * ntile;
+  const int64_t* bi = amax_i + (int64_t(l) * r + i) * ntile;
+  double best = -2.0;
+  int64_t bj = 0;
+  for (int q = lane; q < ntile; q += 32)
+    if (bv[q] > best) {  // ascending tiles: the lowest index wins ties
+      best = bv[q];
+      bj = bi[q];
+    }
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) {
+    const double ob = __shfl_xor_sync(0xffffffffu, best, off);
+    const int64_t oj = __shfl_xor_sync(0xffffffffu, bj, off);
+    if (ob > best || (ob == best && oj < bj)) {
+      best = ob;
+      bj = oj;
+    }
+  }
+  if (!LOCA_CHECK_SPAN((int64_t(l) * r + i) * d, d, int64_t(gridDim.y) * r * d)) return;
+  float* q = Q + (int64_t(l) * r + i) * d;
+  const bool flip = bj >= 0 && bj < d && q[bj] < 0.f;
+  __syncthreads();  // every warp has read the deciding entry
+  if (flip)
+    for (int64_t j = threadIdx.x; j < d; j += 128) q[j] = -q[j];
+  const double s = (flip ? -1.0 : 1.0) * sg[int64_t(l) * r + i];
+  for (int a = threadIdx.x; a < m; a += 128)
+    if (LOCA_CHECK((int64_t(l) * m + a) * r + i, int64_t(gridDim.y) * m * r))
+      P[(int64_t(l) * m + a) * r + i] = float(s * Ur[(int64_t(l) * m + a) * r + i]);
+}
+
+struct CalibWs {
+  size_t Ep, Kp, Rp, fac, Mp, Ur, sg, amv, ami, bad, total;
+  int64_t splits, ntile;
+};
+
+CalibWs calib_ws(int64_t Np, int m, int64_t d, int L, int r) {
+  CalibWs w{};
+  w.splits = calib_splits(Np, m, d, L);
+  w.ntile = (d + CF_COLS - 1) / CF_COLS;
+  size_t o = 0;
+  auto take = [&](size_t bytes) {
+    const size_t at = o;
+    o += align256(bytes);
+    return at;
+  };
+  const size_t md = size_t(m) * size_t(d), Ls = size_t(L), rs = size_t(r);
+  w.Ep = take(sizeof(float) * size_t(Np) * size_t(m <= 8 ? 8 : (m <= 16 ? 16 : (m <= 32 ? 32 : 64))));
+  w.Kp = take(sizeof(double) * size_t(w.splits) * size_t(m) * size_t(m));
+  w.Rp = take(sizeof(double) * size_t(w.splits) * Ls * md);
+  w.fac = take(sizeof(double) * (64 * 64 + 64));
+  w.Mp = take(sizeof(double) * Ls * size_t(w.ntile) * size_t(m) * size_t(m + 1) / 2);
+  w.Ur = take(sizeof(double) * Ls * size_t(m) * rs);
+  w.sg = take(sizeof(double) * Ls * rs);
+  w.amv = take(sizeof(double) * Ls * rs * size_t(w.ntile));
+  w.ami = take(sizeof(int64_t) * Ls * rs * size_t(w.ntile));
+  w.bad = take(sizeof(int32_t));
+  w.total = o;
+  return w;
 }
 
 template <int KM>
 cudaError_t calib_t(const float* E, const float* G, int64_t Np, int m, int64_t d, int L, float beta,
-                    int r, float* P, float* Q, float* sigma, double* Kw, double* Rw, int32_t* status,
-                    cudaStream_t s) {
-  k_calib_xty<KM><<<dim3(unsigned((m + XT_COLS - 1) / XT_COLS), 1), 256, 0, s>>>(E, E, Np, m, m, Kw);
-  cudaError_t e = cudaGetLastError();
+                    int r, float* P, float* Q, float* sigma, char* ws, int32_t* status, cudaStream_t s) {
+  const CalibWs w = calib_ws(Np, m, d, L, r);
+  float* Ep = reinterpret_cast<float*>(ws + w.Ep);
+  double* Kp = reinterpret_cast<double*>(ws + w.Kp);
+  double* Rp = reinterpret_cast<double*>(ws + w.Rp);
+  double* fac = reinterpret_cast<double*>(ws + w.fac);
+  double* Mp = reinterpret_cast<double*>(ws + w.Mp);
+  double* Ur = reinterpret_cast<double*>(ws + w.Ur);
+  double* sg = reinterpret_cast<double*>(ws + w.sg);
+  double* amv = reinterpret_cast<double*>(ws + w.amv);
+  int64_t* ami = reinterpret_cast<int64_t*>(ws + w.ami);
+  int32_t* bad = reinterpret_cast<int32_t*>(ws + w.bad);
+  const int splits = int(w.splits), ntile = int(w.ntile);
+  const int64_t per = ((Np + splits - 1) / splits + XT_RUN - 1) / XT_RUN * XT_RUN;
+  const int64_t wide = d > m ? d : m;
+  static_assert(Xty<KM>::COLS == calib_cols(KM), "column tile");
+  const int tiles = int((wide + Xty<KM>::COLS - 1) / Xty<KM>::COLS);
+  const dim3 grid(unsigned(tiles) * unsigned(L + 1), unsigned(splits));
+  k_calib_pad<<<unsigned((Np * KM + 255) / 256), 256, 0, s>>>(E, Np, m, KM, Ep);
+  cudaError_t e = cudaFuncSetAttribute(k_calib_xty<KM>, cudaFuncAttributeMaxDynamicSharedMemorySize, Xty<KM>::SMEM);
   if (e != cudaSuccess) return e;
-  k_calib_xty<KM><<<dim3(unsigned((d + XT_COLS - 1) / XT_COLS), unsigned(L)), 256, 0, s>>>(E, G, Np, m, d, Rw);
+  k_calib_xty<KM><<<grid, 256, Xty<KM>::SMEM, s>>>(E, Ep, G, Np, m, d, per, L, tiles, Kp, Rp);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  const size_t shm = sizeof(CalibSmem<KM>);
-  e = cudaFuncSetAttribute(k_calib_solve<KM>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(shm));
+  k_calib_chol<KM><<<1, 256, 0, s>>>(Kp, splits, m, beta, fac, bad, status);
+  const size_t fsm = sizeof(double) * (size_t(KM) * KM + KM + size_t(KM) * (CF_COLS + 1));
+  e = cudaFuncSetAttribute(k_calib_fwd<KM>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(fsm));
   if (e != cudaSuccess) return e;
-  k_calib_solve<KM><<<L, 256, shm, s>>>(Kw, Rw, m, d, beta, r, P, Q, sigma, status);
+  k_calib_fwd<KM><<<dim3(unsigned(ntile), unsigned(L)), CF_COLS, fsm, s>>>(fac, bad, Rp, splits, m, d,
+                                                                          int64_t(L) * m * d, Mp);
+  const size_t esm = 2 * sizeof(double) * size_t(KM) * KM;
+  e = cudaFuncSetAttribute(k_calib_eig<KM>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(esm));
+  if (e != cudaSuccess) return e;
+  k_calib_eig<KM><<<L, 256, esm, s>>>(Mp, ntile, m, r, bad, Ur, sg, sigma);
+  k_calib_q<KM><<<dim3(unsigned(ntile), unsigned(L)), CF_COLS, 0, s>>>(Rp, Ur, sg, m, d, r, Q, amv, ami);
+  k_calib_sign<<<dim3(unsigned(r), unsigned(L)), 128, 0, s>>>(amv, ami, ntile, Ur, sg, m, d, r, P, Q);
   return cudaGetLastError();
 }
 
 }  // namespace
 
-size_t calib_workspace_bytes(int64_t Np, int m, int64_t d, int L, int r) {
-  (void)Np;
-  (void)r;
-  return align256(sizeof(double) * size_t(m) * size_t(m)) +
-         align256(sizeof(double) * size_t(L) * size_t(m) * size_t(d));
-}
+size_t calib_workspace_bytes(int64_t Np, int m, int64_t d, int L, int r) { return calib_ws(Np, m, d, L, r).total; }
 
 cudaError_t launch_calib_fit(const float* E_probe, const float* G_probe, int64_t Np, int m, int64_t d,
                              int L, float beta, int r, float* P, float* Q, float* sigma, void* workspace,
                              int32_t* status, cudaStream_t s) {
-  double* Kw = static_cast<double*>(workspace);
-  double* Rw = reinterpret_cast<double*>(static_cast<char*>(workspace) +
-                                         align256(sizeof(double) * size_t(m) * size_t(m)));
-  if (m <= 8) return calib_t<8>(E_probe, G_probe, Np, m, d, L, beta, r, P, Q, sigma, Kw, Rw, status, s);
-  if (m <= 16) return calib_t<16>(E_probe, G_probe, Np, m, d, L, beta, r, P, Q, sigma, Kw, Rw, status, s);
-  if (m <= 32) return calib_t<32>(E_probe, G_probe, Np, m, d, L, beta, r, P, Q, sigma, Kw, Rw, status, s);
-  return calib_t<64>(E_probe, G_probe, Np, m, d, L, beta, r, P, Q, sigma, Kw, Rw, status, s);
+  char* ws = static_cast<char*>(workspace);
+  if (m <= 8) return calib_t<8>(E_probe, G_probe, Np, m, d, L, beta, r, P, Q, sigma, ws, status, s);
+  if (m <= 16) return calib_t<16>(E_probe, G_probe, Np, m, d, L, beta, r, P, Q, sigma, ws, status, s);
+  if (m <= 32) return calib_t<32>(E_probe, G_probe, Np, m, d, L, beta, r, P, Q, sigma, ws, status, s);
+  return calib_t<64>(E_probe, G_probe, Np, m, d, L, beta, r, P, Q, sigma, ws, status, s);
 }
 
 }  // namespace loca

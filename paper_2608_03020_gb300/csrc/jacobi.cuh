@@ -13,35 +13,51 @@ namespace loca {
 //
 // Parallel ordering: a sweep is m - 1 rounds (m rounded up to even, the extra index a dummy) of
 // a round-robin tournament, so that every pair (p, q) meets once per sweep and the m / 2 pairs
-// of a round are disjoint; their rotations are applied at once, to rows (A <- J^T A), then to
-// columns (A <- A J, V <- V J).  The rotation of pair (p, q) has tan(phi) = t, the root of
-// smaller magnitude of t^2 + 2 theta t - 1 = 0 with theta = (A_qq - A_pp) / (2 A_pq), which
-// zeroes (J^T A J)_pq.  Sweeps stop when the off-diagonal mass falls below 1e-30 of the total,
-// after at most 40 sweeps.  Then order[] = eigenvalue indices in descending order (stable:
-// lower index first on ties; entries m..KM-1 stay in place).  Called by every thread of the
-// block (it synchronises the block).
+// of a round are disjoint; their rotations are applied at once (A <- J^T A J, V <- V J): the 2 x 2
+// block of A where the rows of one pair meet the columns of another depends on no other element,
+// so one thread applies both rotations to it and a round needs two barriers.  The rotation of pair
+// (p, q) has tan(phi) = t, the root of smaller magnitude of t^2 + 2 theta t - 1 = 0 with theta =
+// (A_qq - A_pp) / (2 A_pq), which would zero (J^T A J)_pq.  t is taken in fp32 (the angle only has to be
+// close: the element left is ~1e-7 of what it was and convergence stays quadratic) and c = (1 +
+// t^2)^-1/2, s = t c from it in fp64, so the rotation is orthogonal to fp64 rounding.  Sweeps stop when the off-diagonal mass
+// falls below 1e-30 of the total, after at most 40 sweeps.  Then order[] = eigenvalue indices in
+// descending order (lower index first on ties; entries m..KM-1 stay in place).  Called by every
+// thread of the block (it synchronises the block; blockDim.x a multiple of 32, at most 1024).
+// Bound by the latency of the m - 1 rotations in a row per sweep; with t in fp64 their three divisions
+// and two square roots took most of a round.
 template <int KM>
 __device__ void jacobi_eig_block(double (*A)[KM], double (*V)[KM], int* order, int m) {
   __shared__ double s_c[KM / 2], s_s[KM / 2];
   __shared__ int s_p[KM / 2], s_q[KM / 2];
-  __shared__ int s_go;
+  __shared__ double s_off[32], s_tot[32];
   const int tid = threadIdx.x, nt = blockDim.x;
   const int mm = (m + 1) & ~1;
   const int np = mm / 2;
   for (int sweep = 0; sweep < 40; ++sweep) {
     __syncthreads();
-    if (tid == 0) {
-      double off = 0.0, total = 0.0;
-      for (int a = 0; a < m; ++a)
-        for (int b = 0; b < m; ++b) {
-          const double v = A[a][b] * A[a][b];
-          total += v;
-          if (a != b) off += v;
-        }
-      s_go = (off > 1e-30 * total) ? 1 : 0;
+    double off = 0.0, total = 0.0;
+    for (int e = tid; e < m * m; e += nt) {
+      const int a = e / m, b = e % m;
+      const double v = A[a][b] * A[a][b];
+      total += v;
+      if (a != b) off += v;
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+      off += __shfl_xor_sync(0xffffffffu, off, o);
+      total += __shfl_xor_sync(0xffffffffu, total, o);
+    }
+    if ((tid & 31) == 0) {
+      s_off[tid >> 5] = off;
+      s_tot[tid >> 5] = total;
     }
     __syncthreads();
-    if (!s_go) break;
+    off = 0.0;
+    total = 0.0;
+    for (int w = 0; w < nt / 32; ++w) {
+      off += s_off[w];
+      total += s_tot[w];
+    }
+    if (!(off > 1e-30 * total)) break;  // the same sums in every thread
     for (int k = 0; k < mm - 1; ++k) {
       if (tid < np) {
         int p, q;
@@ -61,9 +77,15 @@ __device__ void jacobi_eig_block(double (*A)[KM], double (*V)[KM], int* order, i
         if (q < m) {
           const double apq = A[p][q];
           if (fabs(apq) > 1e-300) {
-            const double theta = (A[q][q] - A[p][p]) / (2.0 * apq);
-            const double t = (theta >= 0 ? 1.0 : -1.0) / (fabs(theta) + sqrt(theta * theta + 1.0));
-            c = 1.0 / sqrt(t * t + 1.0);
+            const double num = A[q][q] - A[p][p], den = 2.0 * apq;
+            // both scaled by one power of two, so that the larger is in [1, 2): fp32 holds their ratio
+            const double mx = fabs(num) > fabs(den) ? fabs(num) : fabs(den);
+            const int ex = ((__double2hiint(mx) >> 20) & 0x7ff) - 1023;
+            const float nf = float(ldexp(num, -ex)), df = float(ldexp(den, -ex));
+            const float theta = nf / df;  // infinite when df underflows: t = 0
+            const float tf = (theta >= 0.f ? 1.f : -1.f) / (fabsf(theta) + sqrtf(fmaf(theta, theta, 1.f)));
+            const double t = double(tf);
+            c = rsqrt(fma(t, t, 1.0));
             sn = t * c;
           }
         }
@@ -73,45 +95,42 @@ __device__ void jacobi_eig_block(double (*A)[KM], double (*V)[KM], int* order, i
         s_s[tid] = sn;
       }
       __syncthreads();
-      for (int e = tid; e < np * m; e += nt) {
-        const int i = e / m, col = e % m;
-        const int p = s_p[i], q = s_q[i];
-        if (q >= m) continue;
-        const double c = s_c[i], sn = s_s[i];
-        const double apk = A[p][col], aqk = A[q][col];
-        A[p][col] = c * apk - sn * aqk;
-        A[q][col] = sn * apk + c * aqk;
+      for (int e = tid; e < np * np; e += nt) {
+        const int i = e / np, j = e % np;  // rows of pair i, columns of pair j
+        const int p = s_p[i], q = s_q[i], pc = s_p[j], qc = s_q[j];
+        const bool rq = q < m, cq = qc < m;  // the dummy index has no row or column
+        const double c = s_c[i], sn = s_s[i], cc = s_c[j], sc = s_s[j];
+        const double app = A[p][pc], apq = cq ? A[p][qc] : 0.0;
+        const double aqp = rq ? A[q][pc] : 0.0, aqq = rq && cq ? A[q][qc] : 0.0;
+        // rows: J^T A, then columns: (J^T A) J
+        const double rpp = c * app - sn * aqp, rpq = c * apq - sn * aqq;
+        const double rqp = sn * app + c * aqp, rqq = sn * apq + c * aqq;
+        A[p][pc] = cc * rpp - sc * rpq;
+        if (cq) A[p][qc] = sc * rpp + cc * rpq;
+        if (rq) A[q][pc] = cc * rqp - sc * rqq;
+        if (rq && cq) A[q][qc] = sc * rqp + cc * rqq;
       }
-      __syncthreads();
       for (int e = tid; e < np * m; e += nt) {
         const int i = e / m, row = e % m;
         const int p = s_p[i], q = s_q[i];
         if (q >= m) continue;
         const double c = s_c[i], sn = s_s[i];
-        const double akp = A[row][p], akq = A[row][q];
-        A[row][p] = c * akp - sn * akq;
-        A[row][q] = sn * akp + c * akq;
         const double vkp = V[row][p], vkq = V[row][q];
         V[row][p] = c * vkp - sn * vkq;
         V[row][q] = sn * vkp + c * vkq;
       }
       __syncthreads();
-      if (tid < np && s_q[tid] < m) {
-        A[s_p[tid]][s_q[tid]] = 0.0;
-        A[s_q[tid]][s_p[tid]] = 0.0;
-      }
-      __syncthreads();
     }
   }
-  if (tid == 0) {
-    for (int i = 0; i < KM; ++i) order[i] = i;
-    for (int i = 0; i < m; ++i) {
-      int best = i;
-      for (int k = i + 1; k < m; ++k)
-        if (A[order[k]][order[k]] > A[order[best]][order[best]]) best = k;
-      const int tmp = order[i];
-      order[i] = order[best];
-      order[best] = tmp;
+  // rank of each eigenvalue: how many are larger (or equal with a lower index)
+  for (int i = tid; i < KM; i += nt) {
+    if (i >= m) {
+      order[i] = i;
+    } else {
+      int rank = 0;
+      const double v = A[i][i];
+      for (int k = 0; k < m; ++k) rank += (A[k][k] > v || (A[k][k] == v && k < i)) ? 1 : 0;
+      order[rank] = i;
     }
   }
   __syncthreads();

@@ -97,3 +97,34 @@ def test_fp32_statistics_token_split(lc, L, N, d):
             c_ref[l] += float(alpha[l]) * (t.T @ x)
     assert _rel(_np(gram), g_ref) <= 1.2e-7 and _rel(_np(cross), c_ref) <= 1.2e-7
     assert torch.equal(gram, gram.transpose(1, 2))
+
+
+@pytest.mark.parametrize("Np,m,d,L,r", [
+    (33, 1, 1, 1, 1),        # one run and a remainder, one column
+    (1025, 8, 131, 2, 3),    # 4 columns per lane, odd width (scalar loads), two token ranges
+    (2100, 9, 130, 1, 9),    # 2 columns per lane (16-byte rows fail, 8-byte rows load)
+    (1500, 17, 64, 2, 5),    # one column per lane
+    (1100, 33, 70, 1, 6),    # two groups of sums
+])
+def test_calibration_and_alignment_paths(lc, Np, m, d, L, r):
+    """The fit's sums are fp32 over 32 tokens and exact to 2^-48 beyond, its solves fp64: the product
+    P Q within 1e-5 (fp32 inputs, beta = 1e-3 of the mean eigenvalue, decaying planted spectrum); the
+    diagnostic on the fitted factors within 1e-5."""
+    rng = np.random.default_rng(Np + m)
+    E = rng.standard_normal((Np, m)).astype(np.float32)
+    planted = [(rng.standard_normal((m, r)) * 0.7 ** np.arange(r)) @ rng.standard_normal((r, d)) for _ in range(L)]
+    G = np.stack([E @ M + 0.05 * rng.standard_normal((Np, d)) for M in planted]).astype(np.float32)
+    r = min(r, m, d)
+    beta = 1e-3 * float(np.sum(E.astype(np.float64) ** 2)) / m
+    P, Q = torch.empty((L, m, r), device="cuda"), torch.empty((L, r, d), device="cuda")
+    sigma, alpha = torch.empty((L, r), device="cuda"), torch.empty((L,), dtype=torch.float64, device="cuda")
+    lc.loca_calib_fit(_dev(E), _dev(G), beta, r, P, Q, sigma=sigma)
+    lc.loca_alignment(_dev(E), _dev(G), P, Q, alpha)
+    torch.cuda.synchronize()
+    assert lc.loca_device_status() == 0
+    P_ref, Q_ref, s_ref, _ = O.calib_fit(E, G, beta, r)
+    for l in range(L):
+        assert _rel(_np(P[l]) @ _np(Q[l]), P_ref[l] @ Q_ref[l]) <= 1e-5
+    assert _rel(_np(sigma), s_ref) <= 1e-5
+    ref = O.alignment(E, _np(P), _np(Q), G)
+    assert np.max(np.abs(_np(alpha) - ref)) <= 1e-5
