@@ -3,8 +3,8 @@
 // with G_l the exact hidden-state gradients at the probe positions.  T is formed element by
 // element in registers (r FMAs each) and never written.
 //
-// k_align_u      U_l = E P_l (Np x RP per block, fp32, rows padded with zeros), tiled over 64 tokens x 64
-//                error channels in shared memory.
+// k_run_gemm     U = E [P_1 .. P_L], all blocks' r columns as one product (run_gemm.cuh), rows of RP values
+//                per block (zero beyond r).
 // k_align_part   grid (token chunk x channel tile, block): a lane owns 32 / RP channels, whose Q_l
 //                entries stay in 32 registers; every warp streams its tokens' rows of G and U through
 //                its own ring (row_stream.cuh) and sums g t, g g, t t with t = U[n] . Q_l[:, j] (fp32 over
@@ -13,7 +13,7 @@
 //                shared memory for every token, two shared loads per FMA).
 // k_align_final  per block, the partial triples in a fixed order -> alpha_l (0 if a norm is 0).
 #include "loca_internal.h"
-#include "row_stream.cuh"
+#include "run_gemm.cuh"
 
 namespace loca {
 namespace {
@@ -22,51 +22,6 @@ constexpr int AL_THREADS = 256;
 constexpr int AL_CHUNK = 1024;   // tokens per CTA
 constexpr int kMaxWideM = 16384;
 constexpr int kMaxR = 32;
-constexpr int AU_TOK = 64;     // tokens per CTA of k_align_u
-constexpr int AU_CH = 64;      // error channels staged per step
-
-// U[l][n][s] = sum_c E[n][c] P_l[c][s] (fp32), U laid out L x Np x RP, zero for s >= r.
-template <int RP>
-__global__ void __launch_bounds__(AL_THREADS) k_align_u(const float* __restrict__ E, const float* __restrict__ P,
-                                                      int64_t Np, int m, int r, float* __restrict__ U) {
-  __shared__ float Es[AU_TOK][AU_CH + 1];
-  __shared__ float Ps[AU_CH][RP];
-  constexpr int SG = AL_THREADS / AU_TOK;  // column groups
-  constexpr int SPT = RP / SG;             // product columns per thread (RP >= 8)
-  const int l = blockIdx.y, tid = threadIdx.x;
-  const int tt = tid % AU_TOK, sg = tid / AU_TOK;
-  const int64_t n0 = int64_t(blockIdx.x) * AU_TOK;
-  const float* Pl = P + int64_t(l) * m * r;
-  float acc[SPT];
-#pragma unroll
-  for (int i = 0; i < SPT; ++i) acc[i] = 0.f;
-  for (int c0 = 0; c0 < m; c0 += AU_CH) {
-    __syncthreads();
-    for (int e = tid; e < AU_TOK * AU_CH; e += AL_THREADS) {
-      const int t = e / AU_CH, c = e % AU_CH;
-      Es[t][c] = (n0 + t < Np && c0 + c < m) ? E[(n0 + t) * m + c0 + c] : 0.f;
-    }
-    for (int e = tid; e < AU_CH * RP; e += AL_THREADS) {
-      const int c = e / RP, s = e % RP;
-      Ps[c][s] = (c0 + c < m && s < r) ? Pl[int64_t(c0 + c) * r + s] : 0.f;
-    }
-    __syncthreads();
-#pragma unroll 8
-    for (int c = 0; c < AU_CH; ++c) {
-      const float ev = Es[tt][c];
-#pragma unroll
-      for (int i = 0; i < SPT; ++i) acc[i] = fmaf(ev, Ps[c][sg + SG * i], acc[i]);
-    }
-  }
-  const int64_t n = n0 + tt;
-  if (n >= Np) return;
-#pragma unroll
-  for (int i = 0; i < SPT; ++i) {
-    const int s = sg + SG * i;
-    if (LOCA_CHECK((int64_t(l) * Np + n) * RP + s, int64_t(gridDim.y) * Np * RP)) U[(int64_t(l) * Np + n) * RP + s] = acc[i];
-  }
-}
-
 __host__ __device__ constexpr int align_rp(int r) { return r <= 8 ? 8 : (r <= 16 ? 16 : 32); }
 // channels per tile: 32 / RP a lane
 __host__ __device__ constexpr int align_cols(int rp) { return 32 * (32 / rp); }
@@ -202,9 +157,17 @@ static cudaError_t align_t(const float* E, const float* G, int64_t Np, int m, in
   const int ntile = int((d + align_cols(RP) - 1) / align_cols(RP));
   double* part = static_cast<double*>(workspace);
   float* U = reinterpret_cast<float*>(static_cast<char*>(workspace) + part_bytes(Np, d, L, r));
-  k_align_u<RP><<<dim3(unsigned((Np + AU_TOK - 1) / AU_TOK), unsigned(L)), AL_THREADS, 0, s>>>(E, P, Np, m, r, U);
+  cudaError_t e = cudaSuccess;
+  if (r < RP) {
+    e = cudaMemsetAsync(U, 0, sizeof(float) * size_t(L) * size_t(Np) * RP, s);
+    if (e != cudaSuccess) return e;
+  }
+  const int64_t n = int64_t(L) * r;
+  const RunGemmArgs g{E, P, U, m, 0, r, int64_t(m) * r, RP, Np * RP, Np, n, m, r, 0};
+  e = run_gemm<false, float, 128, 64>(g, 1, s);
+  if (e != cudaSuccess) return e;
   constexpr int smem = AL_THREADS / 32 * RowRing<RP, 32 / RP>::BYTES;
-  cudaError_t e = cudaFuncSetAttribute(k_align_part<RP>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  e = cudaFuncSetAttribute(k_align_part<RP>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
   k_align_part<RP><<<dim3(unsigned(nch) * unsigned(ntile), unsigned(L)), AL_THREADS, smem, s>>>(U, Q, G, Np, d, r, nch,
                                                                                               ntile, part);

@@ -28,7 +28,6 @@
 namespace loca {
 namespace {
 
-constexpr int XT_RUN = 32;       // tokens per fp32 run
 constexpr int CF_COLS = 128;     // columns per CTA of k_calib_fwd and k_calib_q
 
 // s values and columns per thread: 32 sums, whatever m
@@ -37,10 +36,8 @@ struct Xty {
   static constexpr int SV = KM < 32 ? KM : 32;
   static constexpr int CPT = 32 / SV;
   static constexpr int SG = KM / SV;   // groups of s values (warps)
-  static constexpr int TW = 8 / SG;    // warps over the tokens
   static constexpr int COLS = 32 * CPT;
-  using Ring = RowRing<SV, CPT>;
-  static constexpr int SMEM = 8 * Ring::BYTES > SG * 32 * 33 * 8 ? 8 * Ring::BYTES : SG * 32 * 33 * 8;
+  static constexpr int SMEM = xty_smem<SV, CPT, SG>();
 };
 
 __host__ __device__ constexpr int calib_cols(int m) { return m <= 8 ? 128 : (m <= 16 ? 64 : 32); }
@@ -65,9 +62,8 @@ __global__ void __launch_bounds__(256) k_calib_pad(const float* __restrict__ E, 
 }
 
 // part[split][b][s][j] = sum over the split's tokens of E[n][s] Y_b[n][j]; the first `tiles`
-// CTAs of grid.x take Y = E (K, width m), the next ones block after block of G (width d).  A lane owns
-// CPT columns and SV values of s (32 sums, in pairs along s); each warp streams every TW-th run of
-// 32 tokens through its own ring (row_stream.cuh).  Bound by the read of G: 1.41 GB at L = 28, Np = 8192,
+// CTAs of grid.x take Y = E (K, width m), the next ones block after block of G (width d).  The rows
+// stream through the warps' rings (xty_tile in row_stream.cuh).  Bound by the read of G: 1.41 GB at L = 28, Np = 8192,
 // d = 1536.  (A thread per column and 4 values of s over CTA-staged tiles, with an fp64 addition per
 // run and sum, took 1.0 ms for G and 1.0 ms more for E^T E in one CTA; fp64 adds run at 2 per clock and
 // SM.)
@@ -77,104 +73,20 @@ __global__ void __launch_bounds__(256, 2) k_calib_xty(const float* __restrict__ 
                                                      int64_t per, int L, int tiles, double* __restrict__ Kp,
                                                      double* __restrict__ Rp) {
   using T = Xty<KM>;
-  using Ring = typename T::Ring;
   extern __shared__ __align__(16) float xt_smem[];
   const int b = int(blockIdx.x / unsigned(tiles)) - 1;
   const int tile = int(blockIdx.x % unsigned(tiles));
   const bool isK = b < 0;
   const int64_t w = isK ? m : d;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int sg = warp / T::TW, tw = warp % T::TW;
   const int64_t j0 = int64_t(tile) * T::COLS;
   if (j0 >= w) return;  // K has fewer column tiles
   const float* Y = isK ? E : G + int64_t(b) * Np * d;
   const int64_t n0 = per * blockIdx.y, n1 = n0 + per < Np ? n0 + per : Np;
   const bool vec = w % 4 == 0 && (reinterpret_cast<uintptr_t>(Y) & 15) == 0;
-  float* ring = xt_smem + warp * (2 * Ring::SLOT);
-  uint64_t part[T::SV / 2][T::CPT], hi[T::SV / 2][T::CPT], lo[T::SV / 2][T::CPT];
-#pragma unroll
-  for (int s = 0; s < T::SV / 2; ++s)
-#pragma unroll
-    for (int c = 0; c < T::CPT; ++c) part[s][c] = hi[s][c] = lo[s][c] = 0ull;
-  constexpr int PER_RUN = XT_RUN / Ring::TOK;
-  const int64_t runs = (n1 - n0 + XT_RUN - 1) / XT_RUN;  // <= 0: an empty range
-  const int64_t slots = runs > tw ? ((runs - tw - 1) / T::TW + 1) * PER_RUN : 0;
-  auto issue = [&](int64_t i) {
-    const int64_t n = n0 + (tw + (i / PER_RUN) * T::TW) * XT_RUN + (i % PER_RUN) * Ring::TOK;
-    (void)LOCA_CHECK(j0, w);
-    row_issue<T::SV, T::CPT>(ring + (i & 1) * Ring::SLOT, Y, w, j0, Ep + sg * T::SV, KM, n, n1, vec, lane);
-  };
-  if (slots > 0) issue(0);
-  for (int64_t i = 0; i < slots; ++i) {
-    if (i + 1 < slots) {
-      issue(i + 1);
-      cp_async_wait<1>();
-    } else {
-      cp_async_wait<0>();
-    }
-    __syncwarp();
-    const float* slot = ring + (i & 1) * Ring::SLOT;
-#pragma unroll 4
-    for (int t = 0; t < Ring::TOK; ++t) {
-      float y[T::CPT];
-      row_cols<T::SV, T::CPT>(slot, t, lane, y);
-      uint64_t yy[T::CPT];
-#pragma unroll
-      for (int c = 0; c < T::CPT; ++c) yy[c] = f32x2(y[c], y[c]);
-      const ulonglong2* er = reinterpret_cast<const ulonglong2*>(slot + Ring::Y_FLOATS + t * T::SV);
-#pragma unroll
-      for (int s4 = 0; s4 < T::SV / 4; ++s4) {
-        const ulonglong2 ev = er[s4];
-#pragma unroll
-        for (int c = 0; c < T::CPT; ++c) {
-          part[2 * s4][c] = fma2(ev.x, yy[c], part[2 * s4][c]);
-          part[2 * s4 + 1][c] = fma2(ev.y, yy[c], part[2 * s4 + 1][c]);
-        }
-      }
-    }
-    __syncwarp();  // the slot is refilled by the next issue
-    if (i % PER_RUN == PER_RUN - 1) {
-      // hi + lo += part: the sum and its rounding error (Knuth's two-sum), the errors summed in lo
-#pragma unroll
-      for (int s = 0; s < T::SV / 2; ++s)
-#pragma unroll
-        for (int c = 0; c < T::CPT; ++c) {
-          const uint64_t a = hi[s][c], p = part[s][c];
-          const uint64_t t = add2(a, p), bb = sub2(t, a);
-          lo[s][c] = add2(lo[s][c], add2(sub2(a, sub2(t, bb)), sub2(p, bb)));
-          hi[s][c] = t;
-          part[s][c] = 0ull;
-        }
-    }
-  }
-  // warps in order, fp64 (the ring's memory is free)
-  double(*sum)[32][33] = reinterpret_cast<double(*)[32][33]>(xt_smem);
-  for (int q = 0; q < T::TW; ++q) {
-    __syncthreads();
-    if (tw == q) {
-#pragma unroll
-      for (int s = 0; s < T::SV / 2; ++s)
-#pragma unroll
-        for (int c = 0; c < T::CPT; ++c) {
-          const float2 h = f32x2_parts(hi[s][c]), e = f32x2_parts(lo[s][c]);
-          const double v0 = isfinite(h.x) ? double(h.x) + double(e.x) : double(h.x);
-          const double v1 = isfinite(h.y) ? double(h.y) + double(e.y) : double(h.y);
-          double& o0 = sum[sg][2 * s * T::CPT + c][lane];
-          double& o1 = sum[sg][(2 * s + 1) * T::CPT + c][lane];
-          o0 = q == 0 ? v0 : o0 + v0;
-          o1 = q == 0 ? v1 : o1 + v1;
-        }
-    }
-  }
-  __syncthreads();
   double* out = isK ? Kp + int64_t(blockIdx.y) * m * m : Rp + (int64_t(blockIdx.y) * L + b) * m * d;
-  for (int e = threadIdx.x; e < T::SG * 32 * 32; e += 256) {
-    const int col = e % T::COLS, sl = (e / T::COLS) % T::SV, g = e / (T::COLS * T::SV);
-    const int s = g * T::SV + sl;
-    const int64_t jc = j0 + col;
-    if (s < m && jc < w && LOCA_CHECK(int64_t(s) * w + jc, int64_t(m) * w))
-      out[int64_t(s) * w + jc] = sum[g][sl * T::CPT + col % T::CPT][col / T::CPT];
-  }
+  xty_tile<T::SV, T::CPT, T::SG>(Y, w, j0, Ep, KM, n0, n1, vec, xt_smem, [&](int s, int64_t j, double v) {
+    if (s < m && LOCA_CHECK(int64_t(s) * w + j, int64_t(m) * w)) out[int64_t(s) * w + j] = v;
+  });
 }
 
 // K + beta I = L L^T (padded to KM with an identity block): fac = L (lower, row-major) and the

@@ -10,13 +10,14 @@
 //
 // All L blocks share K, so every solve runs on the ell columns of all blocks at once.
 //
-//   k_cr_gemm     fp32 operands, products summed in fp32 over 32 terms, those sums in fp32 over
-//                 16 and in fp64 beyond (the products with E and G_l; K itself, lower tiles only)
+//   k_run_gemm, k_cr_gtt   the products with E and G_l, and K itself (lower tiles only): fp32
+//                 operands, products summed in fp32 over 32 terms, those sums as fp32 pairs (2^-48)
 //   k_cr_pad      K + beta I, padded to a multiple of 64 with an identity block
 //   k_cr_potrf / k_cr_trsm / k_cr_syrk   right-looking blocked Cholesky (64 x 64 tiles, fp64);
 //                 the diagonal kernel also inverts its triangular tile, so the panel and the
 //                 diagonal steps of the solves are tile products
-//   k_cr_tsolve   blocked forward (L Y = W) and backward (L^T X = Y) substitution: fp64 for the
+//   k_cr_colsolve, or k_cr_tsolve for few columns
+//                 blocked forward (L Y = W) and backward (L^T X = Y) substitution: fp64 for the
 //                 last F^T (which makes the final basis Q_Y) and for the Rayleigh-Ritz product
 //                 F Q_Y; fp32 (on an fp32 copy of the fp64 factor) inside the power iterations,
 //                 which only steer the subspace: an error there moves the starting vectors of
@@ -34,130 +35,19 @@
 
 #include "jacobi.cuh"
 #include "loca_internal.h"
+#include "run_gemm.cuh"
 
 namespace loca {
 namespace {
 
 constexpr int NB = 64;        // Cholesky / solve tile
 constexpr int NBP = NB + 1;   // padded shared-memory row (fp64: conflict-free column reads)
-constexpr int GM_BM = 64, GM_BN = 64, GM_BK = 32, GM_RUN = 16;
 constexpr int RZ_CH = 256;    // rows per chunk of the Rayleigh-Ritz kernels
 constexpr int kMaxEll = 64;
 constexpr int64_t kMaxWidth = 16384;  // m and d (fp64 vectors of one column in shared memory)
 constexpr size_t kTileSmem = sizeof(double) * 2 * NB * NBP;
 
 __device__ __forceinline__ bool failed(const int32_t* flag) { return *reinterpret_cast<const volatile int32_t*>(flag) != 0; }
-
-// C_b[i][j] = sum_t A_b(i, t) B_b(t, j);  A_b(i, t) = A[t lda + i] (AT) or A[i lda + t];
-// B_b(t, j) = B[t ldb + j]; batch b = blockIdx.z with element strides sA, sB, sC.  Products are
-// summed in fp32 over 32 terms, those sums in fp32 over 16 (512 terms), and those in fp64.  The
-// next 32-term slab is loaded into registers while the current one is multiplied, then stored
-// to the other shared-memory buffer (one barrier per slab).
-template <bool AT, typename TC>
-__global__ void __launch_bounds__(256) k_cr_gemm(const float* __restrict__ A, int64_t lda, int64_t sA,
-                                                const float* __restrict__ B, int64_t ldb, int64_t sB,
-                                                TC* __restrict__ C, int64_t ldc, int64_t sC, int64_t M, int64_t N,
-                                                int64_t Kc, int lower_only) {
-  __shared__ __align__(16) float As[2][GM_BK][GM_BM + 4];
-  __shared__ __align__(16) float Bs[2][GM_BK][GM_BN + 4];
-  constexpr int LPT = GM_BK * GM_BM / 256;
-  const int64_t i0 = int64_t(blockIdx.y) * GM_BM, j0 = int64_t(blockIdx.x) * GM_BN;
-  if (lower_only && j0 > i0) return;
-  const int64_t b = blockIdx.z;
-  A += b * sA;
-  B += b * sB;
-  C += b * sC;
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  float ra[LPT], rb[LPT];
-  auto gload = [&](int64_t t0) {
-#pragma unroll
-    for (int k = 0; k < LPT; ++k) {
-      const int e = tid + 256 * k;
-      int t, i;
-      if (AT) {
-        t = e / GM_BM;
-        i = e % GM_BM;
-      } else {
-        i = e / GM_BK;
-        t = e % GM_BK;
-      }
-      const int64_t gi = i0 + i, gt = t0 + t;
-      ra[k] = (gi < M && gt < Kc) ? (AT ? A[gt * lda + gi] : A[gi * lda + gt]) : 0.f;
-      const int tb = e / GM_BN, jb = e % GM_BN;
-      const int64_t gj = j0 + jb, gtb = t0 + tb;
-      rb[k] = (gj < N && gtb < Kc) ? B[gtb * ldb + gj] : 0.f;
-    }
-  };
-  auto sstore = [&](int buf) {
-#pragma unroll
-    for (int k = 0; k < LPT; ++k) {
-      const int e = tid + 256 * k;
-      if (AT)
-        As[buf][e / GM_BM][e % GM_BM] = ra[k];
-      else
-        As[buf][e % GM_BK][e / GM_BK] = ra[k];
-      Bs[buf][e / GM_BN][e % GM_BN] = rb[k];
-    }
-  };
-  double acc[4][4];
-  float run_sum[4][4];
-#pragma unroll
-  for (int p = 0; p < 4; ++p)
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      acc[p][q] = 0.0;
-      run_sum[p][q] = 0.f;
-    }
-  gload(0);
-  sstore(0);
-  __syncthreads();
-  int run = 0, buf = 0;
-  for (int64_t t0 = 0; t0 < Kc; t0 += GM_BK) {
-    const bool more = t0 + GM_BK < Kc;
-    if (more) gload(t0 + GM_BK);
-    float part[4][4];
-#pragma unroll
-    for (int p = 0; p < 4; ++p)
-#pragma unroll
-      for (int q = 0; q < 4; ++q) part[p][q] = 0.f;
-#pragma unroll
-    for (int t = 0; t < GM_BK; ++t) {
-      const float4 a4 = *reinterpret_cast<const float4*>(&As[buf][t][ty * 4]);
-      const float4 b4 = *reinterpret_cast<const float4*>(&Bs[buf][t][tx * 4]);
-      const float av[4] = {a4.x, a4.y, a4.z, a4.w};
-      const float bv[4] = {b4.x, b4.y, b4.z, b4.w};
-#pragma unroll
-      for (int p = 0; p < 4; ++p)
-#pragma unroll
-        for (int q = 0; q < 4; ++q) part[p][q] = fmaf(av[p], bv[q], part[p][q]);
-    }
-    if (more) sstore(buf ^ 1);
-    __syncthreads();
-    buf ^= 1;
-#pragma unroll
-    for (int p = 0; p < 4; ++p)
-#pragma unroll
-      for (int q = 0; q < 4; ++q) run_sum[p][q] += part[p][q];
-    if (++run == GM_RUN) {
-      run = 0;
-#pragma unroll
-      for (int p = 0; p < 4; ++p)
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          acc[p][q] += double(run_sum[p][q]);
-          run_sum[p][q] = 0.f;
-        }
-    }
-  }
-#pragma unroll
-  for (int p = 0; p < 4; ++p)
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int64_t gi = i0 + ty * 4 + p, gj = j0 + tx * 4 + q;
-      if (gi < M && gj < N && LOCA_CHECK(gi * ldc + gj, (M - 1) * ldc + N))
-        C[gi * ldc + gj] = TC(acc[p][q] + double(run_sum[p][q]));
-    }
-}
 
 // K (mp x mp): rows / columns >= m become the identity; beta is added to the first m diagonal
 // entries.
@@ -183,14 +73,16 @@ __device__ __forceinline__ void load_tile(double (*S)[NBP], const double* __rest
 // Diagonal tile jb: factor in shared memory (unblocked, right-looking), write the factor back,
 // and write the inverse of the triangular factor to Dinv[jb].  A pivot that is not positive
 // sets the failure flag (E^T E + beta I is not positive definite in floating point).  Thread
-// (ty, tx) of the 16 x 16 grid owns entries (ty + 16 p, tx + 16 q).
+// (ty, tx) of the 16 x 16 grid owns entries (ty + 16 p, tx + 16 q).  Every thread scales the entries
+// of the pivot's column that it needs itself, so a step has one barrier; bound by the latency of the
+// 64 + 64 steps in a row (with a scaling phase of its own, a division and a square root per step,
+// 162 us; one tile per 64 columns of K, nothing else runs beside it).
 __global__ void __launch_bounds__(256) k_cr_potrf(double* __restrict__ K, int64_t mp, int jb,
                                                  double* __restrict__ Dinv, int32_t* flag) {
   extern __shared__ __align__(16) unsigned char cr_smem[];
   double(*S)[NBP] = reinterpret_cast<double(*)[NBP]>(cr_smem);
   double(*X)[NBP] = reinterpret_cast<double(*)[NBP]>(cr_smem + sizeof(double) * NB * NBP);
   __shared__ double rinv[NB];
-  __shared__ int bad;
   if (failed(flag)) return;
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
   const int64_t o = int64_t(jb) * NB;
@@ -198,132 +90,283 @@ __global__ void __launch_bounds__(256) k_cr_potrf(double* __restrict__ K, int64_
   for (int e = tid; e < NB * NB; e += 256) {
     const int r = e / NB, c = e % NB;
     S[r][c] = (c <= r) ? Kd[int64_t(r) * mp + c] : 0.0;
-    X[r][c] = (r == c) ? 1.0 : 0.0;
+    X[r][c] = 0.0;
   }
-  if (tid == 0) bad = 0;
   __syncthreads();
   for (int c = 0; c < NB; ++c) {
     const double piv = S[c][c];
-    if (!(piv > 0.0)) {
-      bad = 1;
-      break;
+    if (!(piv > 0.0)) {  // the same value in every thread
+      if (tid == 0) atomicExch(flag, 1);
+      return;
     }
-    const double lc = sqrt(piv);
-    const double inv = 1.0 / lc;
-    __syncthreads();
-    if (tid < NB) {
-      if (tid > c) S[tid][c] *= inv;
-      if (tid == c) {
-        S[c][c] = lc;
-        rinv[c] = inv;
-      }
-    }
-    __syncthreads();
+    const double inv = rsqrt(piv);
+    double lc[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) lc[q] = S[tx + 16 * q][c] * inv;
 #pragma unroll
     for (int p = 0; p < 4; ++p) {
       const int rr = ty + 16 * p;
       if (rr <= c) continue;
-      const double lrc = S[rr][c];
+      const double lrc = S[rr][c] * inv;
+      if (tx == 0) X[rr][c] = lrc;  // the factor collects in X: column c of S is still being read
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
         const int ss = tx + 16 * q;
-        if (ss > c && ss <= rr) S[rr][ss] = fma(-lrc, S[ss][c], S[rr][ss]);
+        if (ss > c && ss <= rr) S[rr][ss] = fma(-lrc, lc[q], S[rr][ss]);
       }
+    }
+    if (tid == 0) {
+      X[c][c] = piv * inv;
+      rinv[c] = inv;
     }
     __syncthreads();
   }
-  if (bad) {
-    if (tid == 0) atomicExch(flag, 1);
-    return;
-  }
   for (int e = tid; e < NB * NB; e += 256) {
     const int r = e / NB, c = e % NB;
-    if (c <= r) Kd[int64_t(r) * mp + c] = S[r][c];
+    if (c <= r) Kd[int64_t(r) * mp + c] = X[r][c];
+    S[r][c] = (r == c) ? 1.0 : 0.0;
   }
-  // X = L^-1, right-looking on the identity: row c scaled by 1 / L_cc, then removed from the rows
-  // below
+  __syncthreads();
+  // S = L^-1, right-looking on the identity: row c scaled by 1 / L_cc (by its readers; stored by the
+  // threads of its own row one step later, when nobody reads it), then removed from the rows below
   for (int c = 0; c < NB; ++c) {
-    if (tid <= c) X[c][tid] *= rinv[c];
-    __syncthreads();
+    const double rc = rinv[c];
+    double xc[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) xc[q] = S[c][tx + 16 * q] * rc;
 #pragma unroll
     for (int p = 0; p < 4; ++p) {
       const int rr = ty + 16 * p;
       if (rr <= c) continue;
-      const double lrc = S[rr][c];
+      const double lrc = X[rr][c];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int u = tx + 16 * q;
-        if (u <= c) X[rr][u] = fma(-lrc, X[c][u], X[rr][u]);
-      }
+      for (int q = 0; q < 4; ++q)
+        if (tx + 16 * q <= c) S[rr][tx + 16 * q] = fma(-lrc, xc[q], S[rr][tx + 16 * q]);
     }
     __syncthreads();
   }
   double* D = Dinv + int64_t(jb) * NB * NB;
-  for (int e = tid; e < NB * NB; e += 256) D[e] = X[e / NB][e % NB];
+  for (int e = tid; e < NB * NB; e += 256) D[e] = S[e / NB][e % NB] * rinv[e / NB];
 }
 
-// Panel: L(ib, jb) = A(ib, jb) L(jb, jb)^-T for ib = jb + 1 + blockIdx.x.
+constexpr int CT = 32;         // tile of the panel and trailing updates
+constexpr int CTP = NB + 1;    // padded row of a CT x NB operand
+
+// Panel: L(ib, jb) = A(ib, jb) L(jb, jb)^-T, 16 rows of it per CTA: rows rb = NB (jb + 1) + 16
+// blockIdx.x.  An output row needs only its own input row, so the CTA works in place.  The fp64 pipe (2
+// FMAs per clock and SM) is the bound: 64-row tiles left most SMs idle for 68 us per panel.
 __global__ void __launch_bounds__(256) k_cr_trsm(double* __restrict__ K, int64_t mp, int jb,
                                                 const double* __restrict__ Dinv, const int32_t* flag) {
+  __shared__ double At[16][CTP];
   extern __shared__ __align__(16) unsigned char cr_smem[];
-  double(*At)[NBP] = reinterpret_cast<double(*)[NBP]>(cr_smem);
-  double(*Dt)[NBP] = reinterpret_cast<double(*)[NBP]>(cr_smem + sizeof(double) * NB * NBP);
+  double(*Dt)[NBP] = reinterpret_cast<double(*)[NBP]>(cr_smem);
   if (failed(flag)) return;
-  const int ib = jb + 1 + blockIdx.x;
-  double* Ab = K + int64_t(ib) * NB * mp + int64_t(jb) * NB;
-  load_tile(At, Ab, mp);
+  double* Ab = K + (int64_t(jb + 1) * NB + 16 * int64_t(blockIdx.x)) * mp + int64_t(jb) * NB;
+  for (int e = threadIdx.x; e < 16 * NB; e += 256) At[e / NB][e % NB] = Ab[int64_t(e / NB) * mp + e % NB];
   load_tile(Dt, Dinv + int64_t(jb) * NB * NB, NB);
   __syncthreads();
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  double acc[4][4] = {};
+  double acc[4] = {};
   for (int u = 0; u < NB; ++u) {
+    const double a = At[ty][u];
 #pragma unroll
-    for (int p = 0; p < 4; ++p) {
-      const double a = At[ty + 16 * p][u];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) acc[p][q] = fma(a, Dt[tx + 16 * q][u], acc[p][q]);
-    }
+    for (int q = 0; q < 4; ++q) acc[q] = fma(a, Dt[tx + 16 * q][u], acc[q]);
   }
-  __syncthreads();
 #pragma unroll
-  for (int p = 0; p < 4; ++p)
-#pragma unroll
-    for (int q = 0; q < 4; ++q) Ab[int64_t(ty + 16 * p) * mp + tx + 16 * q] = acc[p][q];
+  for (int q = 0; q < 4; ++q) Ab[int64_t(ty) * mp + tx + 16 * q] = acc[q];
 }
 
-// Trailing update: A(ib, kb) -= L(ib, jb) L(kb, jb)^T for jb < kb <= ib (one tile per CTA).
+// Trailing update: A(i, k) -= L(i, jb) L(k, jb)^T on 32 x 32 tiles of the trailing lower triangle
+// (one per CTA; the smaller tile spreads the last panels' few tiles over more SMs).
 __global__ void __launch_bounds__(256) k_cr_syrk(double* __restrict__ K, int64_t mp, int jb, const int32_t* flag) {
-  extern __shared__ __align__(16) unsigned char cr_smem[];
-  double(*Li)[NBP] = reinterpret_cast<double(*)[NBP]>(cr_smem);
-  double(*Lk)[NBP] = reinterpret_cast<double(*)[NBP]>(cr_smem + sizeof(double) * NB * NBP);
+  __shared__ double Li[CT][CTP];
+  __shared__ double Lk[CT][CTP];
   if (failed(flag)) return;
   const int x = blockIdx.x;
   int ii = int((sqrt(8.0 * x + 1.0) - 1.0) * 0.5);
   while ((ii + 1) * (ii + 2) / 2 <= x) ++ii;
   while (ii * (ii + 1) / 2 > x) --ii;
   const int kk = x - ii * (ii + 1) / 2;
-  const int ib = jb + 1 + ii, kb = jb + 1 + kk;
-  load_tile(Li, K + int64_t(ib) * NB * mp + int64_t(jb) * NB, mp);
-  load_tile(Lk, K + int64_t(kb) * NB * mp + int64_t(jb) * NB, mp);
+  const int64_t r0 = int64_t(jb + 1) * NB;
+  const double* Lb = K + int64_t(jb) * NB;  // columns of the panel
+  for (int e = threadIdx.x; e < CT * NB; e += 256) {
+    const int r = e / NB, c = e % NB;
+    Li[r][c] = Lb[(r0 + ii * CT + r) * mp + c];
+    Lk[r][c] = Lb[(r0 + kk * CT + r) * mp + c];
+  }
   __syncthreads();
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  double acc[4][4] = {};
+  double acc[2][2] = {};
+#pragma unroll 4
   for (int u = 0; u < NB; ++u) {
+    const double a0 = Li[ty][u], a1 = Li[ty + 16][u], b0 = Lk[tx][u], b1 = Lk[tx + 16][u];
+    acc[0][0] = fma(a0, b0, acc[0][0]);
+    acc[0][1] = fma(a0, b1, acc[0][1]);
+    acc[1][0] = fma(a1, b0, acc[1][0]);
+    acc[1][1] = fma(a1, b1, acc[1][1]);
+  }
+  double* Cb = K + (r0 + ii * CT) * mp + r0 + kk * CT;
 #pragma unroll
-    for (int p = 0; p < 4; ++p) {
-      const double a = Li[ty + 16 * p][u];
+  for (int p = 0; p < 2; ++p)
 #pragma unroll
-      for (int q = 0; q < 4; ++q) acc[p][q] = fma(a, Lk[tx + 16 * q][u], acc[p][q]);
+    for (int q = 0; q < 2; ++q) {
+      double* o = Cb + int64_t(ty + 16 * p) * mp + tx + 16 * q;
+      *o -= acc[p][q];
+    }
+}
+
+// W (mp x n) <- K^-1 W for the NC columns of this CTA, forward then backward, in one launch: the columns
+// stay in shared memory (X, mp x NC) and the factor streams through two tile buffers (cp.async, the
+// next 64 x 64 tile in flight while one is used).  Columns do not depend on one another, so no CTA
+// waits for another.  With NC = ceil(n / SMs) every SM has the same work: fp64 is then bound by the fp64
+// pipe (m^2 NC FMAs at 2 per clock), fp32 by the stream of the factor from L2 (8 m^2 bytes per CTA).
+// Left-looking: row block ib of the solution is D(ib) (W_ib - sum_k L(ib, k) X_k), each thread taking one
+// row and a quarter of every tile's 64 columns.
+template <typename T>
+__device__ __forceinline__ void cs_tile(uint32_t dst, const T* src, int64_t ld, int tid) {
+  // 64 x 64 tile to rows of NB + 16 / sizeof(T) elements (16-byte aligned pieces)
+  constexpr int E = 16 / int(sizeof(T)), PER = NB / E, LD = NB + E;
+#pragma unroll
+  for (int i = 0; i < NB * PER / 256; ++i) {
+    const int e = tid + 256 * i, r = e / PER, c = (e % PER) * E;
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + uint32_t((r * LD + c) * int(sizeof(T)))),
+                 "l"(src + int64_t(r) * ld + c)
+                 : "memory");
+  }
+  cp_async_commit();
+}
+
+template <typename T>
+struct Vec16;
+template <>
+struct Vec16<float> {
+  using type = float4;
+};
+template <>
+struct Vec16<double> {
+  using type = double2;
+};
+template <typename T>
+__device__ __forceinline__ void load16(const T* p, T* v) {
+  *reinterpret_cast<typename Vec16<T>::type*>(v) = *reinterpret_cast<const typename Vec16<T>::type*>(p);
+}
+
+template <typename T, int NC>
+__global__ void __launch_bounds__(256) k_cr_colsolve(const T* __restrict__ K, int64_t mp, const T* __restrict__ Dinv,
+                                                    T* __restrict__ W, int64_t n, const int32_t* flag) {
+  constexpr int E = 16 / int(sizeof(T)), LD = NB + E;
+  extern __shared__ __align__(16) unsigned char cr_smem[];
+  T* tiles = reinterpret_cast<T*>(cr_smem);  // 2 x NB x LD
+  T* red = tiles + 2 * NB * LD;              // 4 x NC x NB partial sums
+  T* X = red + 4 * NC * NB;                  // NC x mp
+  if (failed(flag)) return;
+  const int tid = threadIdx.x, r = tid & 63, kq = tid >> 6;
+  const int64_t c0 = int64_t(blockIdx.x) * NC;
+  const int nb = int(mp / NB);
+  for (int64_t e = tid; e < mp * NC; e += 256) {
+    const int64_t i = e / NC, c = e % NC;
+    X[c * mp + i] = c0 + c < n ? W[i * n + c0 + c] : T(0);
+  }
+  const uint32_t ts = uint32_t(__cvta_generic_to_shared(tiles));
+  constexpr uint32_t TB = uint32_t(NB * LD * sizeof(T));
+  // The tiles in order of use: for every row block its off-diagonal tiles, then its inverse diagonal
+  // tile; forward over L's rows, backward over L's columns (used transposed).
+  auto fetch = [&](bool fwd, int ib, int k, int buf) {
+    const T* src;
+    int64_t ld = mp;
+    if (k == ib) {
+      src = Dinv + int64_t(ib) * NB * NB;
+      ld = NB;
+    } else {
+      src = fwd ? K + int64_t(ib) * NB * mp + int64_t(k) * NB : K + int64_t(k) * NB * mp + int64_t(ib) * NB;
+    }
+    cs_tile(ts + uint32_t(buf) * TB, src, ld, tid);
+  };
+  T acc[NC];
+  // acc[c] += sum over this thread's quarter of the tile's row r times X block `xb`
+  auto multiply = [&](bool fwd, const T* Mt, const T* xb) {
+#pragma unroll
+    for (int u = kq * 16; u < kq * 16 + 16; u += E) {
+      T a[E];
+      if (fwd) {
+        load16(Mt + r * LD + u, a);
+      } else {
+#pragma unroll
+        for (int v = 0; v < E; ++v) a[v] = Mt[(u + v) * LD + r];
+      }
+#pragma unroll
+      for (int c = 0; c < NC; ++c) {
+        T x[E];
+        load16(xb + c * mp + u, x);
+#pragma unroll
+        for (int v = 0; v < E; ++v) acc[c] = fma(a[v], x[v], acc[c]);
+      }
+    }
+  };
+  auto publish = [&]() {  // this thread's partial sums, and a fresh accumulator
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+      red[(kq * NC + c) * NB + r] = acc[c];
+      acc[c] = T(0);
+    }
+  };
+  auto total_of = [&](int e) {
+    constexpr int Q = NC * NB;
+    return (red[e] + red[Q + e]) + (red[2 * Q + e] + red[3 * Q + e]);
+  };
+  const int total = nb * (nb + 1) / 2;
+  for (int pass = 0; pass < 2; ++pass) {
+    const bool fwd = pass == 0;
+    int buf = 0;
+    int ib = fwd ? 0 : nb - 1;  // row block
+    int k = ib;                 // column block of the current tile
+    __syncthreads();
+    fetch(fwd, ib, k, 0);
+#pragma unroll
+    for (int c = 0; c < NC; ++c) acc[c] = T(0);
+    for (int step = 0; step < total; ++step) {
+      int ibn = ib, kn = fwd ? k + 1 : k - 1;  // the tile after this one
+      if (k == ib) {
+        ibn = fwd ? ib + 1 : ib - 1;
+        kn = fwd ? 0 : nb - 1;
+      }
+      if (step + 1 < total) {
+        fetch(fwd, ibn, kn, buf ^ 1);
+        cp_async_wait<1>();
+      } else {
+        cp_async_wait<0>();
+      }
+      __syncthreads();  // this tile has landed for every thread
+      const T* Mt = tiles + buf * NB * LD;
+      if (k != ib) {
+        multiply(fwd, Mt, X + int64_t(k) * NB);
+      } else {
+        // the right-hand side W_ib - sum, then times the inverse tile
+        T* Xi = X + int64_t(ib) * NB;
+        publish();
+        __syncthreads();
+        for (int e = tid; e < NC * NB; e += 256) Xi[(e / NB) * mp + e % NB] -= total_of(e);
+        __syncthreads();
+        multiply(fwd, Mt, Xi);
+        publish();
+        __syncthreads();
+        for (int e = tid; e < NC * NB; e += 256) Xi[(e / NB) * mp + e % NB] = total_of(e);
+      }
+      __syncthreads();  // the tile buffer may be refilled, X_ib is complete
+      buf ^= 1;
+      ib = ibn;
+      k = kn;
     }
   }
-  double* Cb = K + int64_t(ib) * NB * mp + int64_t(kb) * NB;
-#pragma unroll
-  for (int p = 0; p < 4; ++p)
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int64_t o = int64_t(ty + 16 * p) * mp + tx + 16 * q;
-      Cb[o] -= acc[p][q];
-    }
+  for (int64_t e = tid; e < mp * NC; e += 256) {
+    const int64_t i = e / NC, c = e % NC;
+    if (c0 + c < n && LOCA_CHECK(i * n + c0 + c, mp * n)) W[i * n + c0 + c] = X[c * mp + i];
+  }
+}
+
+template <typename T>
+size_t colsolve_smem(int64_t mp, int nc) {
+  return sizeof(T) * (size_t(2) * NB * (NB + 16 / sizeof(T)) + size_t(4) * NB * nc + size_t(mp) * nc);
 }
 
 // Blocked substitution on W (mp x n, in place; T = double or float), one step per launch, on
@@ -402,18 +445,27 @@ constexpr int QR_STAGE = 64;   // rows staged at a time by k_cr_vtv
 constexpr int QR_CHUNK = 256;  // rows per CTA of k_cr_vtv / k_cr_qr_apply
 
 // Partial Gram matrices of block l's ell columns of V (rows x n, columns l ell ..):
-// part[l][chunk] (ELLP x ELLP, zero outside ell x ell) = sum over the chunk's rows of v v^T.
+// part[l][chunk] (ELLP x ELLP, lower triangle; zero outside ell x ell) = sum over the chunk's rows of
+// v v^T.  Bound by the fp64 pipe, so only the lower triangle is formed.
 template <int ELLP>
 __global__ void __launch_bounds__(256) k_cr_vtv(const double* __restrict__ V, int64_t rows, int64_t n, int ell,
                                                int nch, double* __restrict__ part) {
   __shared__ double Vs[QR_STAGE][ELLP + 1];
-  constexpr int EPT = (ELLP * ELLP + 255) / 256;
+  constexpr int NT = ELLP * (ELLP + 1) / 2;
+  constexpr int EPT = (NT + 255) / 256;
   const int ch = blockIdx.x, l = blockIdx.y, tid = threadIdx.x;
   const int64_t r0 = int64_t(ch) * QR_CHUNK;
   const int64_t r1 = (r0 + QR_CHUNK < rows) ? r0 + QR_CHUNK : rows;
   double acc[EPT];
+  int ia[EPT], ib[EPT];
 #pragma unroll
-  for (int k = 0; k < EPT; ++k) acc[k] = 0.0;
+  for (int k = 0; k < EPT; ++k) {
+    acc[k] = 0.0;
+    int a = 0, b = tid + 256 * k;  // entry of the lower triangle, row by row
+    while (b > a) b -= ++a;
+    ia[k] = a < ELLP ? a : 0;
+    ib[k] = a < ELLP ? b : 0;
+  }
   for (int64_t rs = r0; rs < r1; rs += QR_STAGE) {
     __syncthreads();
     for (int e = tid; e < QR_STAGE * ELLP; e += 256) {
@@ -423,70 +475,59 @@ __global__ void __launch_bounds__(256) k_cr_vtv(const double* __restrict__ V, in
     __syncthreads();
 #pragma unroll
     for (int k = 0; k < EPT; ++k) {
-      const int e = tid + 256 * k;
-      if (e < ELLP * ELLP) {
-        const int a = e / ELLP, b = e % ELLP;
-        double sacc = acc[k];
-        for (int rr = 0; rr < QR_STAGE; ++rr) sacc = fma(Vs[rr][a], Vs[rr][b], sacc);
-        acc[k] = sacc;
-      }
+      if (tid + 256 * k >= NT) break;
+      double sacc = acc[k];
+#pragma unroll 8
+      for (int rr = 0; rr < QR_STAGE; ++rr) sacc = fma(Vs[rr][ia[k]], Vs[rr][ib[k]], sacc);
+      acc[k] = sacc;
     }
   }
   double* out = part + (int64_t(l) * nch + ch) * ELLP * ELLP;
 #pragma unroll
-  for (int k = 0; k < EPT; ++k) {
-    const int e = tid + 256 * k;
-    if (e < ELLP * ELLP) out[e] = acc[k];
-  }
+  for (int k = 0; k < EPT; ++k)
+    if (tid + 256 * k < NT) out[ia[k] * ELLP + ib[k]] = acc[k];
 }
 
-// Per block: S = sum of the partials (fixed order), S = Lc Lc^T by Cholesky (warp 0) with
-// dependent columns (new component below 1e-7 of the column's norm: pivot <= 1e-14 S_cc) given
-// a zero column in Lc.  Writes Lc with its diagonal replaced by the reciprocals (0 when
-// dependent) to fac[l] (ELLP x ELLP).
+// Per block: S = sum of the partials (fixed order), S = Lc Lc^T by Cholesky (right-looking, one barrier per
+// column: bound by the latency of its ell steps) with dependent columns (new component below 1e-7 of the
+// column's norm: pivot <= 1e-14 S_cc) given a zero column in Lc.  Writes Lc with its diagonal replaced by
+// the reciprocals (0 when dependent) to fac[l] (ELLP x ELLP).
 template <int ELLP>
 __global__ void __launch_bounds__(256) k_cr_qr_factor(const double* __restrict__ part, int nch, int ell,
                                                      double* __restrict__ fac) {
   extern __shared__ __align__(16) unsigned char cr_smem[];
   double(*S)[ELLP + 1] = reinterpret_cast<double(*)[ELLP + 1]>(cr_smem);
   double(*Lc)[ELLP + 1] = reinterpret_cast<double(*)[ELLP + 1]>(cr_smem + sizeof(double) * ELLP * (ELLP + 1));
+  __shared__ double diag[ELLP];
   const int l = blockIdx.x, tid = threadIdx.x;
   for (int e = tid; e < ELLP * ELLP; e += blockDim.x) {
-    double v = 0.0;
-    for (int ch = 0; ch < nch; ++ch) v += part[(int64_t(l) * nch + ch) * ELLP * ELLP + e];
-    S[e / ELLP][e % ELLP] = v;
-    Lc[e / ELLP][e % ELLP] = 0.0;
-  }
-  __syncthreads();
-  if (tid < 32) {
-    const int lane = tid;
-    for (int c = 0; c < ell; ++c) {
-      double dsum = S[c][c];
-      for (int u = 0; u < c; ++u) dsum -= Lc[c][u] * Lc[c][u];
-      const bool dep = !(S[c][c] > 0.0) || !(dsum > 1e-14 * S[c][c]);
-      const double lcc = dep ? 0.0 : sqrt(dsum);
-      __syncwarp();
-      for (int j = c + 1 + lane; j < ell; j += 32) {
-        double v = 0.0;
-        if (!dep) {
-          v = S[j][c];
-          for (int u = 0; u < c; ++u) v -= Lc[j][u] * Lc[c][u];
-          v /= lcc;
-        }
-        Lc[j][c] = v;
-      }
-      if (lane == 0) Lc[c][c] = lcc;
-      __syncwarp();
-    }
-  }
-  __syncthreads();
-  double* F = fac + int64_t(l) * ELLP * ELLP;
-  for (int e = tid; e < ELLP * ELLP; e += blockDim.x) {
     const int a = e / ELLP, b = e % ELLP;
-    double v = (b < a) ? Lc[a][b] : 0.0;
-    if (a == b) v = (Lc[a][a] > 0.0) ? 1.0 / Lc[a][a] : 0.0;
-    F[e] = v;
+    double v = 0.0;
+    if (b <= a)
+#pragma unroll 4
+      for (int ch = 0; ch < nch; ++ch) v += part[(int64_t(l) * nch + ch) * ELLP * ELLP + e];
+    S[a][b] = v;
+    Lc[a][b] = 0.0;
+    if (a == b) diag[a] = v;
   }
+  __syncthreads();
+  for (int c = 0; c < ell; ++c) {
+    const double piv = S[c][c];
+    const bool dep = !(diag[c] > 0.0) || !(piv > 1e-14 * diag[c]);
+    if (!dep) {
+      const double inv = rsqrt(piv);
+      const int rem = ell - 1 - c;
+      for (int e = tid; e < rem * rem; e += 256) {
+        const int a = c + 1 + e / rem, b = c + 1 + e % rem;
+        if (b <= a) S[a][b] = fma(-(S[a][c] * inv), S[b][c] * inv, S[a][b]);
+      }
+      for (int a = c + 1 + tid; a < ell; a += 256) Lc[a][c] = S[a][c] * inv;
+      if (tid == 0) Lc[c][c] = inv;
+    }
+    __syncthreads();
+  }
+  double* F = fac + int64_t(l) * ELLP * ELLP;
+  for (int e = tid; e < ELLP * ELLP; e += blockDim.x) F[e] = Lc[e / ELLP][e % ELLP];
 }
 
 // Per row v of block l's columns: q = v R^-1 with R = Lc^T, i.e. Lc q^T = v^T by forward
@@ -591,37 +632,54 @@ __global__ void __launch_bounds__(256) k_cr_ritz_eig(const double* __restrict__ 
 // P_l[a][i] = sigma_i (Q_Y U_B)[a][i] for the chunk's rows a < m, and Q_l[i][j] =
 // (B^T U_B)[j][i] / sigma_i for the chunk's columns j < d, with each chunk's entry of largest
 // magnitude per Q_l row (value, lowest index on ties) for the sign convention.
+// A thread reads its row (ell values) once.
+template <int ELLP>
 __global__ void __launch_bounds__(RZ_CH) k_cr_ritz_out(const double* __restrict__ QY, const double* __restrict__ Bt,
                                                       int64_t n, int64_t m, int64_t d, int ell, int r, int nch,
                                                       const double* __restrict__ Ur, const double* __restrict__ sig,
                                                       float* __restrict__ P, float* __restrict__ Q,
                                                       double* __restrict__ amax_v, int64_t* __restrict__ amax_i) {
-  __shared__ double Us[kMaxEll * kMaxEll];
-  __shared__ double ss[kMaxEll];
-  __shared__ double bv[RZ_CH / 32];
-  __shared__ int64_t bi[RZ_CH / 32];
+  __shared__ double Us[ELLP * ELLP];
+  __shared__ double ss[ELLP], si[ELLP];  // sigma_i and 1 / sigma_i (0 where it is 0)
+  __shared__ double bv[ELLP][RZ_CH / 32];
+  __shared__ int64_t bi[ELLP][RZ_CH / 32];
   const int ch = blockIdx.x, l = blockIdx.y, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   for (int e = tid; e < ell * r; e += RZ_CH) Us[e] = Ur[int64_t(l) * ell * r + e];
-  for (int e = tid; e < r; e += RZ_CH) ss[e] = sig[int64_t(l) * r + e];
+  for (int e = tid; e < r; e += RZ_CH) {
+    ss[e] = sig[int64_t(l) * r + e];
+    si[e] = ss[e] > 0.0 ? 1.0 / ss[e] : 0.0;
+  }
   __syncthreads();
   const int64_t a = int64_t(ch) * RZ_CH + tid;
+  double x[ELLP];
+  auto dot = [&](int i) {
+    double v0 = 0.0, v1 = 0.0;
+#pragma unroll
+    for (int c = 0; c < ELLP; c += 2) {
+      if (c < ell) v0 = fma(x[c], Us[c * r + i], v0);
+      if (c + 1 < ell) v1 = fma(x[c + 1], Us[(c + 1) * r + i], v1);
+    }
+    return v0 + v1;
+  };
   if (a < m) {
     const double* row = QY + a * n + int64_t(l) * ell;
+#pragma unroll
+    for (int c = 0; c < ELLP; ++c) x[c] = c < ell ? row[c] : 0.0;
     for (int i = 0; i < r; ++i) {
-      double s = 0.0;
-      for (int c = 0; c < ell; ++c) s = fma(row[c], Us[c * r + i], s);
+      const double s = dot(i);
       if (LOCA_CHECK((int64_t(l) * m + a) * r + i, int64_t(gridDim.y) * m * r))
         P[(int64_t(l) * m + a) * r + i] = (ss[i] > 0.0) ? float(ss[i] * s) : 0.f;
     }
   }
-  const int64_t j = int64_t(ch) * RZ_CH + tid;
-  const double* brow = Bt + j * n + int64_t(l) * ell;
+  const int64_t j = a;
+  if (j < d) {
+    const double* brow = Bt + j * n + int64_t(l) * ell;
+#pragma unroll
+    for (int c = 0; c < ELLP; ++c) x[c] = c < ell ? brow[c] : 0.0;
+  }
   for (int i = 0; i < r; ++i) {
     double v = 0.0;
-    if (j < d && ss[i] > 0.0) {
-      for (int c = 0; c < ell; ++c) v = fma(brow[c], Us[c * r + i], v);
-      v /= ss[i];
-    }
+    if (j < d && ss[i] > 0.0) v = dot(i) * si[i];
     if (j < d && LOCA_CHECK((int64_t(l) * r + i) * d + j, int64_t(gridDim.y) * r * d))
       Q[(int64_t(l) * r + i) * d + j] = float(v);
     double best = (j < d && v == v) ? fabs(v) : -1.0;  // NaN entries never win
@@ -636,22 +694,22 @@ __global__ void __launch_bounds__(RZ_CH) k_cr_ritz_out(const double* __restrict_
       }
     }
     if (lane == 0) {
-      bv[wid] = best;
-      bi[wid] = bj;
+      bv[i][wid] = best;
+      bi[i][wid] = bj;
     }
-    __syncthreads();
-    if (tid == 0 && LOCA_CHECK((int64_t(l) * r + i) * nch + ch, int64_t(gridDim.y) * r * nch)) {
-      double b0 = bv[0];
-      int64_t i0 = bi[0];
-      for (int w = 1; w < RZ_CH / 32; ++w)
-        if (bv[w] > b0 || (bv[w] == b0 && bi[w] < i0)) {
-          b0 = bv[w];
-          i0 = bi[w];
-        }
-      amax_v[(int64_t(l) * r + i) * nch + ch] = b0;
-      amax_i[(int64_t(l) * r + i) * nch + ch] = i0;
-    }
-    __syncthreads();
+  }
+  __syncthreads();
+  for (int i = tid; i < r; i += RZ_CH) {
+    if (!LOCA_CHECK((int64_t(l) * r + i) * nch + ch, int64_t(gridDim.y) * r * nch)) continue;
+    double b0 = bv[i][0];
+    int64_t i0 = bi[i][0];
+    for (int w = 1; w < RZ_CH / 32; ++w)
+      if (bv[i][w] > b0 || (bv[i][w] == b0 && bi[i][w] < i0)) {
+        b0 = bv[i][w];
+        i0 = bi[i][w];
+      }
+    amax_v[(int64_t(l) * r + i) * nch + ch] = b0;
+    amax_i[(int64_t(l) * r + i) * nch + ch] = i0;
   }
 }
 
@@ -708,7 +766,7 @@ RsvdWs rsvd_ws(int64_t Np, int64_t m, int64_t d, int L, int ell, int r) {
   w.Wf = take(sizeof(float) * mp * n);
   w.Zd = take(sizeof(double) * d * n);
   w.Zf = take(sizeof(float) * d * n);
-  w.Tn = take(sizeof(float) * Np * n);
+  w.Tn = take(sizeof(float) * (Np * n + 32));
   w.qrpart = take(sizeof(double) * L * nchqr * ellp * ellp);
   w.qrfac = take(sizeof(double) * L * ellp * ellp);
   w.part = take(sizeof(double) * L * nchd * ell * ell);
@@ -721,18 +779,83 @@ RsvdWs rsvd_ws(int64_t Np, int64_t m, int64_t d, int L, int ell, int r) {
   return w;
 }
 
+// C_b(i, j) = sum_t A_b(i, t) B_b(t, j) (run_gemm.cuh).  32-column tiles where N is
+// one block's ell <= 32 columns.
 template <bool AT, typename TC>
 cudaError_t gemm(const float* A, int64_t lda, int64_t sA, const float* B, int64_t ldb, int64_t sB, TC* C,
                  int64_t ldc, int64_t sC, int64_t M, int64_t N, int64_t Kc, int batch, int lower_only,
                  cudaStream_t s) {
-  const dim3 grid(unsigned((N + GM_BN - 1) / GM_BN), unsigned((M + GM_BM - 1) / GM_BM), unsigned(batch));
-  k_cr_gemm<AT, TC><<<grid, 256, 0, s>>>(A, lda, sA, B, ldb, sB, C, ldc, sC, M, N, Kc, lower_only);
+  const RunGemmArgs g{A, B, C, lda, sA, ldb, sB, ldc, sC, M, N, Kc, 0, lower_only};
+  return N <= 32 ? run_gemm<AT, TC, 128, 32>(g, batch, s) : run_gemm<AT, TC, 128, 64>(g, batch, s);
+}
+
+// Zd[j][l ell + s] = sum_n Tn[n][l ell + s] G_l[n][j] (G_l^T Tn for every block): a warp streams rows of G_l
+// and of Tn (row_stream.cuh).  Bound by the read of G.  Tn's rows are read SV values wide: a multiple of 4
+// columns per block keeps them 16-byte aligned, and Tn has room for the last row's overhang.
+template <int SV>
+__global__ void __launch_bounds__(256, 2) k_cr_gtt(const float* __restrict__ G, const float* __restrict__ Tn, int64_t Np,
+                                                  int64_t d, int64_t n, int ell, int tiles, double* __restrict__ Zd) {
+  constexpr int CPT = 32 / SV;
+  extern __shared__ __align__(16) float gt_smem[];
+  const int l = int(blockIdx.x / unsigned(tiles));
+  const int64_t j0 = int64_t(blockIdx.x % unsigned(tiles)) * (32 * CPT);
+  const float* Gl = G + int64_t(l) * Np * d;
+  const bool vec = d % 4 == 0 && (reinterpret_cast<uintptr_t>(G) & 15) == 0;
+  xty_tile<SV, CPT, 1>(Gl, d, j0, Tn + int64_t(l) * ell, n, 0, Np, vec, gt_smem, [&](int s, int64_t j, double v) {
+    if (s < ell && LOCA_CHECK(j * n + int64_t(l) * ell + s, d * n)) Zd[j * n + int64_t(l) * ell + s] = v;
+  });
+}
+
+template <int SV>
+cudaError_t gtt(const float* G, const float* Tn, int64_t Np, int64_t d, int64_t n, int ell, int L, double* Zd,
+                cudaStream_t s) {
+  constexpr int smem = xty_smem<SV, 32 / SV, 1>();
+  cudaError_t e = cudaFuncSetAttribute(k_cr_gtt<SV>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return e;
+  const int tiles = int((d + 32 * (32 / SV) - 1) / (32 * (32 / SV)));
+  k_cr_gtt<SV><<<unsigned(tiles) * unsigned(L), 256, smem, s>>>(G, Tn, Np, d, n, ell, tiles, Zd);
   return cudaGetLastError();
 }
 
-// W (mp x n) <- K^-1 W with K = L L^T (forward, then backward substitution), in T.
+template <typename T, int NC>
+cudaError_t colsolve(const T* K, int64_t mp, const T* Dinv, T* W, int64_t n, const int32_t* flag, cudaStream_t s) {
+  const size_t smem = colsolve_smem<T>(mp, NC);
+  cudaError_t e = cudaFuncSetAttribute(k_cr_colsolve<T, NC>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+  if (e != cudaSuccess) return e;
+  k_cr_colsolve<T, NC><<<unsigned((n + NC - 1) / NC), 256, smem, s>>>(K, mp, Dinv, W, n, flag);
+  return cudaGetLastError();
+}
+
+// W (mp x n) <- K^-1 W with K = L L^T (forward, then backward substitution), in T.  With at least one
+// column per two SMs, and in fp32 a factor whose triangle stays in L2 (every CTA streams all of it), the
+// columns are divided over the SMs (k_cr_colsolve).  Fewer columns leave SMs idle there, and a larger
+// fp32 factor would come from HBM once per CTA: then the step-by-step kernels, which spread each update
+// over the row blocks.  At m = 1536, n = 896: 13.2 ms step by step (two fp64 solves) against 7.6 ms.
 template <typename T>
 cudaError_t solve(const T* K, int64_t mp, const T* Dinv, T* W, int64_t n, const int32_t* flag, cudaStream_t s) {
+  constexpr size_t kMost = 232448 - 1024;
+  const bool in_l2 = sizeof(T) == 8 || mp * mp * 2 <= (int64_t(64) << 20);
+  // columns per CTA: the least time (waves x columns) over the SMs, the most columns on a tie
+  int64_t nc = 0, best = 0;
+  for (int c = 1; c <= 8 && colsolve_smem<T>(mp, c) <= kMost; ++c) {
+    const int64_t waves = ((n + c - 1) / c + sm_count() - 1) / sm_count();
+    if (nc == 0 || waves * c <= best) {
+      nc = c;
+      best = waves * c;
+    }
+  }
+  if (2 * n >= sm_count() && in_l2 && nc > 0) {
+    switch (nc) {
+      case 1: return colsolve<T, 1>(K, mp, Dinv, W, n, flag, s);
+      case 2: return colsolve<T, 2>(K, mp, Dinv, W, n, flag, s);
+      case 3: return colsolve<T, 3>(K, mp, Dinv, W, n, flag, s);
+      case 4: return colsolve<T, 4>(K, mp, Dinv, W, n, flag, s);
+      case 5: return colsolve<T, 5>(K, mp, Dinv, W, n, flag, s);
+      case 6: return colsolve<T, 6>(K, mp, Dinv, W, n, flag, s);
+      case 7: return colsolve<T, 7>(K, mp, Dinv, W, n, flag, s);
+      default: return colsolve<T, 8>(K, mp, Dinv, W, n, flag, s);
+    }
+  }
   const int nb = int(mp / NB);
   const size_t smem = sizeof(T) * 2 * NB * NBP;
   const unsigned ct16 = unsigned((n + 15) / 16), ct64 = unsigned((n + 63) / 64);
@@ -770,7 +893,7 @@ cudaError_t orth(double* V, int64_t rows, int64_t n, int ell, int L, double* qrp
 cudaError_t set_smem_attributes() {
   static const void* fns64[] = {
       reinterpret_cast<const void*>(k_cr_potrf), reinterpret_cast<const void*>(k_cr_trsm),
-      reinterpret_cast<const void*>(k_cr_syrk), reinterpret_cast<const void*>(k_cr_tsolve<double, 0, 16>),
+      reinterpret_cast<const void*>(k_cr_tsolve<double, 0, 16>),
       reinterpret_cast<const void*>(k_cr_tsolve<double, 1, 64>),
       reinterpret_cast<const void*>(k_cr_tsolve<double, 2, 16>),
       reinterpret_cast<const void*>(k_cr_tsolve<double, 3, 64>)};
@@ -827,8 +950,9 @@ cudaError_t rsvd_t(const float* E, const float* G, int64_t Np, int64_t m, int64_
     k_cr_potrf<<<1, 256, kTileSmem, s>>>(K, mp, jb, Dinv, flag);
     const int T = nb - jb - 1;
     if (T > 0) {
-      k_cr_trsm<<<T, 256, kTileSmem, s>>>(K, mp, jb, Dinv, flag);
-      k_cr_syrk<<<T * (T + 1) / 2, 256, kTileSmem, s>>>(K, mp, jb, flag);
+      k_cr_trsm<<<T * (NB / 16), 256, kTileSmem / 2, s>>>(K, mp, jb, Dinv, flag);
+      const int T2 = T * (NB / CT);
+      k_cr_syrk<<<T2 * (T2 + 1) / 2, 256, 0, s>>>(K, mp, jb, flag);
     }
     CR_TRY(cudaGetLastError());
   }
@@ -858,6 +982,9 @@ cudaError_t rsvd_t(const float* E, const float* G, int64_t Np, int64_t m, int64_
       CR_TRY(solve<float>(Kf, mp, Dinvf, Wf, n, flag, s));
     }
     CR_TRY((gemm<false, float>(E, m, 0, Wf, n, 0, Tn, n, 0, Np, n, m, 1, 0, s)));
+    if (ell % 4 == 0 && ell <= 32)
+      return ell <= 8 ? gtt<8>(G, Tn, Np, d, n, ell, L, Zd, s)
+                      : (ell <= 16 ? gtt<16>(G, Tn, Np, d, n, ell, L, Zd, s) : gtt<32>(G, Tn, Np, d, n, ell, L, Zd, s));
     return gemm<true, double>(G, d, Np * d, Tn, n, ell, Zd, n, ell, d, ell, Np, L, 0, s);
   };
   CR_TRY(apply_Ft(Omega, int64_t(ell), int64_t(0), q == 0));
@@ -885,7 +1012,7 @@ cudaError_t rsvd_t(const float* E, const float* G, int64_t Np, int64_t m, int64_
   CR_TRY(cudaFuncSetAttribute(k_cr_ritz_eig<ELLP>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(eig_smem)));
   k_cr_ritz_eig<ELLP><<<L, 256, eig_smem, s>>>(part, nchd, ell, r, flag, status, Ur, sig, sigma);
   CR_TRY(cudaGetLastError());
-  k_cr_ritz_out<<<dim3(unsigned(nchq), unsigned(L)), RZ_CH, 0, s>>>(Ym, Zd, n, m, d, ell, r, nchq, Ur, sig, P, Q, amv,
+  k_cr_ritz_out<ELLP><<<dim3(unsigned(nchq), unsigned(L)), RZ_CH, 0, s>>>(Ym, Zd, n, m, d, ell, r, nchq, Ur, sig, P, Q, amv,
                                                                       ami);
   CR_TRY(cudaGetLastError());
   k_cr_ritz_sign<<<dim3(unsigned(L), unsigned(r)), 256, 0, s>>>(P, Q, m, d, r, nchq, amv, ami);

@@ -80,8 +80,9 @@ __device__ void jacobi_eig_block(double (*A)[KM], double (*V)[KM], int* order, i
             const double num = A[q][q] - A[p][p], den = 2.0 * apq;
             // both scaled by one power of two, so that the larger is in [1, 2): fp32 holds their ratio
             const double mx = fabs(num) > fabs(den) ? fabs(num) : fabs(den);
-            const int ex = ((__double2hiint(mx) >> 20) & 0x7ff) - 1023;
-            const float nf = float(ldexp(num, -ex)), df = float(ldexp(den, -ex));
+            const int be = (__double2hiint(mx) >> 20) & 0x7ff;
+            const double scale = __hiloint2double((be < 2045 ? 2046 - be : 1) << 20, 0);
+            const float nf = float(num * scale), df = float(den * scale);
             const float theta = nf / df;  // infinite when df underflows: t = 0
             const float tf = (theta >= 0.f ? 1.f : -1.f) / (fabsf(theta) + sqrtf(fmaf(theta, theta, 1.f)));
             const double t = double(tf);

@@ -40,6 +40,18 @@ __device__ __forceinline__ uint64_t sub2(uint64_t a, uint64_t b) {  // a - b
   return fma2(b, f32x2(-1.f, -1.f), a);  // exact product: one rounding
 }
 
+// hi + lo += p, lane by lane: the sum and its rounding error (Knuth's two-sum), the errors summed in lo;
+// p is cleared.
+__device__ __forceinline__ void two_sum2(uint64_t& hi, uint64_t& lo, uint64_t& p) {
+  const uint64_t a = hi, t = add2(a, p), bb = sub2(t, a);
+  lo = add2(lo, add2(sub2(a, sub2(t, bb)), sub2(p, bb)));
+  hi = t;
+  p = 0ull;
+}
+__device__ __forceinline__ double pair_value(float hi, float lo) {
+  return isfinite(hi) ? double(hi) + double(lo) : double(hi);
+}
+
 // Tokens per slot, and floats per slot: Y then V.
 template <int RP, int CPT>
 struct RowRing {
@@ -65,36 +77,45 @@ __device__ __forceinline__ void cp_async_wait() {
 
 // Start the copies of tokens [n0, n0 + TOK) (zeros from n1 on): columns [j0, j0 + COLS) of Y (zeros from
 // w on) and V's rows, ldv floats apart.  vec: Y's rows and j0 are 16-byte aligned.  V and ldv always are.
+// A lane's pieces are a fixed column and every STEP-th row, so only pointers advance.
 template <int RP, int CPT>
 __device__ __forceinline__ void row_issue(float* slot, const float* Y, int64_t w, int64_t j0, const float* V, int64_t ldv,
                                           int64_t n0, int64_t n1, bool vec, int lane) {
   using R = RowRing<RP, CPT>;
   const uint32_t sy = uint32_t(__cvta_generic_to_shared(slot));
   const uint32_t sv = sy + R::Y_FLOATS * 4;
+  const int rows = n1 - n0 < R::TOK ? int(n1 - n0) : R::TOK;
   if (vec) {
-    constexpr int PER = R::COLS / 4;  // 16-byte pieces per row
+    constexpr int PER = R::COLS / 4, STEP = 32 / PER;  // 16-byte pieces per row, rows per instruction
+    const int t0 = lane / PER, c = (lane % PER) * 4;
+    const bool col = j0 + c < w;
+    const float* src = Y + (n0 + t0) * w + j0 + c;
+    const uint32_t dst = sy + uint32_t(t0 * R::COLS + c) * 4;
 #pragma unroll
-    for (int i = 0; i < R::TOK * PER / 32; ++i) {
-      const int e = lane + 32 * i, t = e / PER, c = (e % PER) * 4;
-      const bool in = n0 + t < n1 && j0 + c < w;
-      cp_async(sy + uint32_t(t * R::COLS + c) * 4, in ? Y + (n0 + t) * w + j0 + c : Y, 16, in);
+    for (int i = 0; i < R::TOK / STEP; ++i) {
+      const bool in = col && t0 + i * STEP < rows;
+      cp_async(dst + uint32_t(i * STEP * R::COLS) * 4, in ? src : Y, 16, in);
+      src += STEP * w;
     }
   } else {
 #pragma unroll 4
-    for (int i = 0; i < R::TOK * R::COLS / 32; ++i) {
-      const int e = lane + 32 * i, t = e / R::COLS, c = e % R::COLS;
-      const bool in = n0 + t < n1 && j0 + c < w;
-      cp_async(sy + uint32_t(e) * 4, in ? Y + (n0 + t) * w + j0 + c : Y, 4, in);
+    for (int i = 0; i < R::TOK * CPT; ++i) {
+      const int t = i / CPT, c = (i % CPT) * 32 + lane;
+      const bool in = t < rows && j0 + c < w;
+      cp_async(sy + uint32_t(t * R::COLS + c) * 4, in ? Y + (n0 + t) * w + j0 + c : Y, 4, in);
     }
   }
-  constexpr int VP = RP / 4;
+  constexpr int VP = RP / 4, VSTEP = 32 / VP;
+  const int t0 = lane / VP, c = (lane % VP) * 4;
+  const float* src = V + (n0 + t0) * ldv + c;
 #pragma unroll
-  for (int i = 0; i < (R::TOK * VP + 31) / 32; ++i) {
-    const int e = lane + 32 * i, t = e / VP, c = (e % VP) * 4;
-    if (e < R::TOK * VP) {
-      const bool in = n0 + t < n1;
-      cp_async(sv + uint32_t(e) * 16, in ? V + (n0 + t) * ldv + c : V, 16, in);
+  for (int i = 0; i < (R::TOK + VSTEP - 1) / VSTEP; ++i) {
+    const int t = t0 + i * VSTEP;
+    if (t < R::TOK) {
+      const bool in = t < rows;
+      cp_async(sv + uint32_t(t * RP + c) * 4, in ? src : V, 16, in);
     }
+    src += VSTEP * ldv;
   }
   cp_async_commit();
 }
@@ -111,6 +132,104 @@ __device__ __forceinline__ void row_cols(const float* slot, int t, int lane, flo
     y[0] = v.x, y[1] = v.y;
   } else {
     y[0] = *p;
+  }
+}
+
+// Shared memory of xty_tile: eight warps' rings, or the warps' sums (pairs).
+template <int SV, int CPT, int SG>
+constexpr int xty_smem() {
+  const int ring = 8 * RowRing<SV, CPT>::BYTES, sum = 8 * 32 * 32 * 8;
+  return ring > sum ? ring : sum;
+}
+
+// out(s, j, sum over tokens n in [n0, n1) of V[n][s] Y[n][j]) for the tile's columns j in [j0, j0 + 32 CPT),
+// j < w, and s < SG SV; called by 256 threads.  A lane owns CPT columns and SV values of s (32 sums, in
+// pairs along s); warp group sg takes s from sg SV on, and each of its warps every (8 / SG)-th run of 32
+// tokens.  Products are summed in fp32 over a run, the runs as pairs (two_sum2), and so are the warps, in
+// order (fp64 adds and conversions run at 2 per clock and SM: 8 warps of them took 6 us per CTA).
+constexpr int XT_RUN = 32;
+
+template <int SV, int CPT, int SG, typename Out>
+__device__ __forceinline__ void xty_tile(const float* Y, int64_t w, int64_t j0, const float* V, int64_t ldv, int64_t n0,
+                                         int64_t n1, bool vec, float* smem, Out out) {
+  using Ring = RowRing<SV, CPT>;
+  static_assert(SV * CPT == 32, "32 sums a lane");
+  constexpr int TW = 8 / SG, COLS = 32 * CPT;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int sg = warp / TW, tw = warp % TW;
+  float* ring = smem + warp * (2 * Ring::SLOT);
+  uint64_t part[SV / 2][CPT], hi[SV / 2][CPT], lo[SV / 2][CPT];
+#pragma unroll
+  for (int s = 0; s < SV / 2; ++s)
+#pragma unroll
+    for (int c = 0; c < CPT; ++c) part[s][c] = hi[s][c] = lo[s][c] = 0ull;
+  constexpr int PER_RUN = XT_RUN / Ring::TOK;
+  const int64_t runs = (n1 - n0 + XT_RUN - 1) / XT_RUN;  // <= 0: an empty range
+  const int64_t slots = runs > tw ? ((runs - tw - 1) / TW + 1) * PER_RUN : 0;
+  auto issue = [&](int64_t i) {
+    const int64_t n = n0 + (tw + (i / PER_RUN) * TW) * XT_RUN + (i % PER_RUN) * Ring::TOK;
+    row_issue<SV, CPT>(ring + (i & 1) * Ring::SLOT, Y, w, j0, V + sg * SV, ldv, n, n1, vec, lane);
+  };
+  if (slots > 0) issue(0);
+  for (int64_t i = 0; i < slots; ++i) {
+    if (i + 1 < slots) {
+      issue(i + 1);
+      cp_async_wait<1>();
+    } else {
+      cp_async_wait<0>();
+    }
+    __syncwarp();
+    const float* slot = ring + (i & 1) * Ring::SLOT;
+#pragma unroll 4
+    for (int t = 0; t < Ring::TOK; ++t) {
+      float y[CPT];
+      row_cols<SV, CPT>(slot, t, lane, y);
+      uint64_t yy[CPT];
+#pragma unroll
+      for (int c = 0; c < CPT; ++c) yy[c] = f32x2(y[c], y[c]);
+      const ulonglong2* er = reinterpret_cast<const ulonglong2*>(slot + Ring::Y_FLOATS + t * SV);
+#pragma unroll
+      for (int s4 = 0; s4 < SV / 4; ++s4) {
+        const ulonglong2 ev = er[s4];
+#pragma unroll
+        for (int c = 0; c < CPT; ++c) {
+          part[2 * s4][c] = fma2(ev.x, yy[c], part[2 * s4][c]);
+          part[2 * s4 + 1][c] = fma2(ev.y, yy[c], part[2 * s4 + 1][c]);
+        }
+      }
+    }
+    __syncwarp();  // the slot is refilled by the next issue
+    if (i % PER_RUN == PER_RUN - 1) {
+#pragma unroll
+      for (int s = 0; s < SV / 2; ++s)
+#pragma unroll
+        for (int c = 0; c < CPT; ++c) two_sum2(hi[s][c], lo[s][c], part[s][c]);
+    }
+  }
+  // the warps' pairs in order (the rings are free)
+  uint64_t* sum = reinterpret_cast<uint64_t*>(smem);  // [warp][sum of 32][lane]: (hi, lo)
+  __syncthreads();
+#pragma unroll
+  for (int s = 0; s < SV / 2; ++s)
+#pragma unroll
+    for (int c = 0; c < CPT; ++c) {
+      const float2 h = f32x2_parts(hi[s][c]), e = f32x2_parts(lo[s][c]);
+      sum[(warp * 32 + 2 * s * CPT + c) * 32 + lane] = f32x2(h.x, e.x);
+      sum[(warp * 32 + (2 * s + 1) * CPT + c) * 32 + lane] = f32x2(h.y, e.y);
+    }
+  __syncthreads();
+  for (int e = threadIdx.x; e < SG * 32 * 32; e += 256) {
+    const int col = e % COLS, sl = (e / COLS) % SV, g = e / (COLS * SV);
+    const int at = (sl * CPT + col % CPT) * 32 + col / CPT;
+    float h = 0.f, l = 0.f;
+#pragma unroll
+    for (int q = 0; q < TW; ++q) {
+      const float2 p = f32x2_parts(sum[(g * TW + q) * 1024 + at]);
+      const float t = __fadd_rn(h, p.x), bb = __fsub_rn(t, h);
+      l += __fadd_rn(__fadd_rn(__fsub_rn(h, __fsub_rn(t, bb)), __fsub_rn(p.x, bb)), p.y);
+      h = t;
+    }
+    if (j0 + col < w) out(g * SV + sl, j0 + col, pair_value(h, l));
   }
 }
 

@@ -1,0 +1,174 @@
+// fp32-operand matrix product of the calibration kernels, with the sums as exact as fp64 ones: products
+// are summed in fp32 over runs of 32 terms and the runs as pairs of fp32 values (sum and rounding
+// error, Knuth's two-sum: ~2^-48), converted to fp64 at the end.
+//
+//   C_b(i, j) = sum_t A_b(i, t) B_b(t, j),  A_b(i, t) = A[t lda + i] (AT) or A[i lda + t]
+//
+// One BM x BN tile per CTA of 256 threads; a thread owns BM BN / 256 outputs, pairs of rows packed
+// for fma.rn.f32x2 (a run of a pair is one register pair: the row operand comes from shared memory
+// already paired, the column operand is duplicated once for BM / 32 packed FMAs).  The next 32-term
+// slab is loaded into registers while the current one is multiplied (two shared buffers, one
+// barrier per slab).  Bound by the fp32 pipe.  At 64 x 64 tiles of 4 x 4 outputs with scalar FMAs and
+// fp64 adds the same products ran at 16 TFLOP/s, half of each tile idle where N is one block's 32
+// columns.
+#pragma once
+
+#include "row_stream.cuh"
+
+namespace loca {
+
+constexpr int RG_BK = 32;
+
+// Columns j of B and C may come in blocks of `bw` (bw > 0): column j is column j % bw of block j / bw,
+// blocks sB / sC elements apart; blockIdx.y is then 0.  Otherwise (bw = 0) the batch is blockIdx.y.
+struct RunGemmArgs {
+  const float* A;
+  const float* B;
+  void* C;
+  int64_t lda, sA, ldb, sB, ldc, sC;
+  int64_t M, N, K;
+  int bw;
+  int lower_only;  // tiles strictly above the diagonal are not computed
+};
+
+template <bool AT, typename TC, int BM, int BN>
+__global__ void __launch_bounds__(256) k_run_gemm(RunGemmArgs g) {
+  constexpr int TN = BN / 4;            // threads along the columns (4 each)
+  constexpr int RPT = BM * TN / 256;    // rows per thread
+  constexpr int NG = RPT / 4;           // groups of 4 consecutive rows
+  constexpr int LDA = BM + 4;
+  __shared__ __align__(16) float As[2][RG_BK][LDA];
+  __shared__ __align__(16) float Bs[2][RG_BK][BN];
+  const int64_t nt = (g.N + BN - 1) / BN;  // CTAs of one row tile are neighbours: its rows come from L2
+  const int64_t i0 = int64_t(blockIdx.x) / nt * BM, j0 = int64_t(blockIdx.x) % nt * BN;
+  if (g.lower_only && j0 > i0 + BM - 1) return;
+  const float* A = g.A + int64_t(blockIdx.y) * g.sA;
+  const float* B = g.B + (g.bw ? 0 : int64_t(blockIdx.y) * g.sB);
+  TC* C = static_cast<TC*>(g.C) + (g.bw ? 0 : int64_t(blockIdx.y) * g.sC);
+  const int tid = threadIdx.x, tx = tid % TN, ty = tid / TN;
+  constexpr int AV = BM * RG_BK / 4 / 256, BV = (BN * RG_BK / 4 + 255) / 256;  // float4 per thread and slab
+  const bool avec = g.lda % 4 == 0 && (reinterpret_cast<uintptr_t>(A) & 15) == 0;
+  const bool bvec = g.ldb % 4 == 0 && (reinterpret_cast<uintptr_t>(B) & 15) == 0 && (g.bw % 4 == 0) && g.sB % 4 == 0;
+  float4 ra[AV], rb[BV];
+  auto load4 = [](const float* p, int n, bool vec) {  // n valid values
+    if (vec && n >= 4) return __ldg(reinterpret_cast<const float4*>(p));
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (n > 0) v.x = __ldg(p);
+    if (n > 1) v.y = __ldg(p + 1);
+    if (n > 2) v.z = __ldg(p + 2);
+    if (n > 3) v.w = __ldg(p + 3);
+    return v;
+  };
+  auto left = [](int64_t n) { return n >= 4 ? 4 : int(n); };
+  auto gload = [&](int64_t t0) {
+#pragma unroll
+    for (int q = 0; q < AV; ++q) {
+      const int e = tid + 256 * q;
+      if constexpr (AT) {
+        const int t = e / (BM / 4), i = (e % (BM / 4)) * 4;
+        ra[q] = load4(A + (t0 + t) * g.lda + i0 + i, t0 + t < g.K ? left(g.M - i0 - i) : 0, avec);
+      } else {
+        const int i = e % BM, t = (e / BM) * 4;
+        ra[q] = load4(A + (i0 + i) * g.lda + t0 + t, i0 + i < g.M ? left(g.K - t0 - t) : 0, avec);
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < BV; ++q) {
+      const int e = tid + 256 * q;
+      const int t = e / (BN / 4);
+      const int64_t j = j0 + (e % (BN / 4)) * 4;
+      if (t >= RG_BK || t0 + t >= g.K || j >= g.N) {
+        rb[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+      } else if (g.bw == 0) {
+        rb[q] = load4(B + (t0 + t) * g.ldb + j, left(g.N - j), bvec);
+      } else if (bvec) {  // blocks of a multiple of 4 columns: 4 in one block
+        rb[q] = load4(B + (j / g.bw) * g.sB + (t0 + t) * g.ldb + j % g.bw, 4, true);
+      } else {
+        float v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          v[u] = j + u < g.N ? __ldg(B + ((j + u) / g.bw) * g.sB + (t0 + t) * g.ldb + (j + u) % g.bw) : 0.f;
+        rb[q] = make_float4(v[0], v[1], v[2], v[3]);
+      }
+    }
+  };
+  auto sstore = [&](int buf) {
+#pragma unroll
+    for (int q = 0; q < AV; ++q) {
+      const int e = tid + 256 * q;
+      if constexpr (AT) {
+        *reinterpret_cast<float4*>(&As[buf][e / (BM / 4)][(e % (BM / 4)) * 4]) = ra[q];
+      } else {
+        const int i = e % BM, t = (e / BM) * 4;
+        As[buf][t][i] = ra[q].x;
+        As[buf][t + 1][i] = ra[q].y;
+        As[buf][t + 2][i] = ra[q].z;
+        As[buf][t + 3][i] = ra[q].w;
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < BV; ++q) {
+      const int e = tid + 256 * q;
+      if (e / (BN / 4) < RG_BK) *reinterpret_cast<float4*>(&Bs[buf][e / (BN / 4)][(e % (BN / 4)) * 4]) = rb[q];
+    }
+  };
+  // rows: group v of 4 consecutive ones at v * (BM / NG) + 4 ty
+  uint64_t part[RPT / 2][4], hi[RPT / 2][4], lo[RPT / 2][4];
+#pragma unroll
+  for (int p = 0; p < RPT / 2; ++p)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) part[p][q] = hi[p][q] = lo[p][q] = 0ull;
+  gload(0);
+  sstore(0);
+  __syncthreads();
+  int buf = 0;
+  for (int64_t t0 = 0; t0 < g.K; t0 += RG_BK) {
+    const bool more = t0 + RG_BK < g.K;
+    if (more) gload(t0 + RG_BK);
+#pragma unroll 8
+    for (int t = 0; t < RG_BK; ++t) {
+      const float4 b4 = *reinterpret_cast<const float4*>(&Bs[buf][t][tx * 4]);
+      const uint64_t bb[4] = {f32x2(b4.x, b4.x), f32x2(b4.y, b4.y), f32x2(b4.z, b4.z), f32x2(b4.w, b4.w)};
+#pragma unroll
+      for (int v = 0; v < NG; ++v) {
+        const ulonglong2 a = *reinterpret_cast<const ulonglong2*>(&As[buf][t][v * (BM / NG) + ty * 4]);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          part[2 * v][q] = fma2(a.x, bb[q], part[2 * v][q]);
+          part[2 * v + 1][q] = fma2(a.y, bb[q], part[2 * v + 1][q]);
+        }
+      }
+    }
+    if (more) sstore(buf ^ 1);
+#pragma unroll
+    for (int p = 0; p < RPT / 2; ++p)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) two_sum2(hi[p][q], lo[p][q], part[p][q]);
+    __syncthreads();
+    buf ^= 1;
+  }
+#pragma unroll
+  for (int p = 0; p < RPT / 2; ++p)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const float2 h = f32x2_parts(hi[p][q]), e = f32x2_parts(lo[p][q]);
+      const float hv[2] = {h.x, h.y}, ev[2] = {e.x, e.y};
+      const int64_t j = j0 + tx * 4 + q;
+      if (j >= g.N) continue;
+      const int64_t cj = g.bw ? (j / g.bw) * g.sC + j % g.bw : j;
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const int64_t i = i0 + (p / 2) * (BM / NG) + ty * 4 + (p % 2) * 2 + u;
+        if (i < g.M && LOCA_CHECK(j, g.N)) C[i * g.ldc + cj] = TC(pair_value(hv[u], ev[u]));
+      }
+    }
+}
+
+template <bool AT, typename TC, int BM, int BN>
+cudaError_t run_gemm(const RunGemmArgs& g, int batch, cudaStream_t s) {
+  const int64_t tiles = ((g.M + BM - 1) / BM) * ((g.N + BN - 1) / BN);
+  k_run_gemm<AT, TC, BM, BN><<<dim3(unsigned(tiles), unsigned(batch)), 256, 0, s>>>(g);
+  return cudaGetLastError();
+}
+
+}  // namespace loca

@@ -128,3 +128,34 @@ def test_calibration_and_alignment_paths(lc, Np, m, d, L, r):
     assert _rel(_np(sigma), s_ref) <= 1e-5
     ref = O.alignment(E, _np(P), _np(Q), G)
     assert np.max(np.abs(_np(alpha) - ref)) <= 1e-5
+
+
+@pytest.mark.parametrize("Np,m,d,L,r,ell,q", [
+    (300, 130, 70, 10, 4, 8, 1),    # columns divided over the SMs (one each), 8-wide streams of G
+    (200, 65, 129, 26, 3, 6, 1),    # two columns a CTA; ell no multiple of 4: tiled G^T products
+    (257, 192, 101, 8, 8, 20, 0),   # 32-wide streams over 20-column blocks, scalar loads, fp64 solves only
+    (150, 70, 80, 3, 2, 4, 2),      # few columns: step-by-step solves
+    (150, 70, 80, 3, 8, 40, 1),     # 64-column tiles for one block's products
+])
+def test_wide_calibration_paths(lc, Np, m, d, L, r, ell, q):
+    """P Q against the oracle's same steps: fp32 runs of 32 products, exact to 2^-48 beyond, fp64 solves
+    where they count; planted rank r with a decaying spectrum and 1% noise, so 1e-5."""
+    rng = np.random.default_rng(Np + ell)
+    E = (rng.standard_normal((Np, m)) * rng.lognormal(0, 0.3, m)).astype(np.float32)
+    G = np.empty((L, Np, d), dtype=np.float32)
+    for l in range(L):
+        clean = (E @ (rng.standard_normal((m, r)) * 0.7 ** np.arange(r))) @ rng.standard_normal((r, d))
+        G[l] = clean + 0.01 * np.sqrt(np.mean(clean ** 2)) * rng.standard_normal((Np, d))
+    Om = rng.standard_normal((d, ell)).astype(np.float32)
+    beta = 1e-3 * float(np.sum(E.astype(np.float64) ** 2)) / m
+    P, Q = torch.empty((L, m, r), device="cuda"), torch.empty((L, r, d), device="cuda")
+    sigma, alpha = torch.empty((L, r), device="cuda"), torch.empty((L,), dtype=torch.float64, device="cuda")
+    lc.loca_calib_fit_rsvd(_dev(E), _dev(G), beta, r, _dev(Om), q, P, Q, sigma=sigma)
+    lc.loca_alignment(_dev(E), _dev(G), P, Q, alpha)
+    torch.cuda.synchronize()
+    assert lc.loca_device_status() == 0
+    P_ref, Q_ref, s_ref = O.calib_fit_rsvd(E, G, beta, r, Om, q)
+    for l in range(L):
+        assert _rel(_np(P[l]) @ _np(Q[l]), P_ref[l] @ Q_ref[l]) <= 1e-5
+    assert _rel(_np(sigma), s_ref) <= 1e-5
+    assert np.max(np.abs(_np(alpha) - O.alignment(E, _np(P), _np(Q), G))) <= 1e-5
