@@ -1,13 +1,16 @@
 // Top-layer error at the frozen head (Eq. 4; Lemma "Top-layer error", S3).
 //
-// One warp per logit row.  Each lane streams its share of the row with 16-byte loads and
+// k_head_error: one warp per logit row.  Each lane streams its share of the row with 16-byte loads and
 // keeps a running maximum and a sum of exp(z - max) rescaled whenever the maximum grows,
 // so the row is read from HBM exactly once; the 32 partial (max, sum) pairs are merged with
 // warp shuffles.  The C label columns are then gathered to form
 //   E[n, c] = w_n (exp(z[n, col_c] - lse_n) - [y_n == c]),   ce[n] = w_n (lse_n - z[n, col_{y_n}]).
 // The running maximum and sum are kept in base-2 units (t = z log2 e), so each logit costs one
 // FMA and one exp2f; lse = (m + log2 s) ln 2.
-// Bound: HBM read of the logits (N * V * elsize bytes); for V == C the kernel is launch-bound.
+// Bound: HBM read of the logits (N * V * elsize bytes).
+// k_head_error_short: one thread per row, for rows that give a warp's lanes one logit or none each
+// (V <= 32, the label-token head V == C among them): the row is read twice, the second time from L1.
+// Bound by the launch.  At N = 131072, V = C = 4 a warp per row took 54-70 us.
 #include <cuda_bf16.h>
 #include <math.h>
 
@@ -154,6 +157,50 @@ __global__ void __launch_bounds__(256) k_head_error(const Tz* __restrict__ z, in
   }
 }
 
+// Rows of at most this many logits take one thread each.
+constexpr int kShortRow = 32;
+
+template <typename Tz>
+__global__ void __launch_bounds__(256) k_head_error_short(const Tz* __restrict__ z, int64_t N, int V, int64_t ldz,
+                                                          const int32_t* __restrict__ cols, int C,
+                                                          const int32_t* __restrict__ y, const float* __restrict__ w,
+                                                          int normaliser, float* __restrict__ E,
+                                                          float* __restrict__ ce) {
+  const int64_t n = int64_t(blockIdx.x) * 256 + threadIdx.x;
+  if (n >= N || !LOCA_CHECK_SPAN(n * ldz, V, (N - 1) * ldz + V)) return;
+  const Tz* row = z + n * ldz;
+  // maximum and sum of 2^(t - m), t = z log2 e, over the row or over the label columns
+  float m = -INFINITY;
+  const int terms = normaliser == 0 ? V : C;
+  auto logit = [&](int i) {
+    const int col = normaliser == 0 ? i : cols[i];
+    return LOCA_CHECK(col, V) ? to_f(row[col]) : -INFINITY;
+  };
+  for (int i = 0; i < terms; ++i) {
+    const float t = logit(i) * kLog2e;
+    if (t > m) m = t;  // a NaN never becomes the maximum; it still reaches the sum
+  }
+  float sum = 0.f;
+  if (m != -INFINITY)
+    for (int i = 0; i < terms; ++i) sum += exp2f(fmaf(logit(i), kLog2e, -m));
+  const float lse = (m + log2f(sum)) * kLn2;
+  const int yn = y[n];
+  const float wn = (yn < 0) ? 0.f : (w ? w[n] : 1.f);
+  for (int c = 0; c < C; ++c) {
+    const int32_t col = cols[c];
+    const float zc = LOCA_CHECK(col, V) ? to_f(row[col]) : 0.f;
+    if (LOCA_CHECK(n * C + c, N * C)) E[n * C + c] = wn * (expf(zc - lse) - (c == yn ? 1.f : 0.f));
+  }
+  if (ce != nullptr) {
+    float cn = 0.f;
+    if (yn >= 0 && LOCA_CHECK(yn, C)) {
+      const int32_t cy = cols[yn];
+      if (LOCA_CHECK(cy, V)) cn = wn * (lse - to_f(row[cy]));
+    }
+    ce[n] = cn;
+  }
+}
+
 }  // namespace
 
 cudaError_t launch_head_error(const void* z, int dtype, int64_t N, int64_t V, int64_t ldz,
@@ -161,6 +208,16 @@ cudaError_t launch_head_error(const void* z, int dtype, int64_t N, int64_t V, in
                               int normaliser, float* E, float* ce, cudaStream_t s) {
   if (N == 0) return cudaSuccess;
   const int threads = 256;
+  if (V <= kShortRow) {  // C <= V
+    const unsigned grid = unsigned((N + 255) / 256);
+    if (dtype == LOCA_BF16)
+      k_head_error_short<<<grid, threads, 0, s>>>(static_cast<const __nv_bfloat16*>(z), N, int(V), ldz, cols, C, y, w,
+                                                  normaliser, E, ce);
+    else
+      k_head_error_short<<<grid, threads, 0, s>>>(static_cast<const float*>(z), N, int(V), ldz, cols, C, y, w,
+                                                  normaliser, E, ce);
+    return cudaGetLastError();
+  }
   int64_t blocks = (N + 7) / 8;
   const int64_t cap = int64_t(sm_count()) * 16;
   if (blocks > cap) blocks = cap;
