@@ -12,20 +12,20 @@
 //
 // Kernels:
 //   k_kspace_prep   per block: W_l = A_l^T split into bf16 hi / lo rows (2 kp x d, kp = 16 or
-//                   32; A_l ~= hi + lo to 2^-16), and M_l = Q_l Q_l^T (r x r), 8 CTAs per block.
+//                   32; A_l ~= hi + lo to 2^-16), and M_l = Q_l Q_l^T (r x r); E^T E of the batch (C x C),
+//                   shared by every block: ||T_l||^2 = <P_l (Q_l Q_l^T) P_l^T, E^T E>, so no
+//                   per-token work is needed for it.  One launch, CTAs of three kinds.
 //   k_kspace_xa     p = W_l x_n on tcgen05 (kind::f16, M = 128 tokens, N = 2 kp, K = 16, both
 //                   operands K-major with the 128-byte swizzle): a persistent CTA per SM streams
 //                   128-token x 64-channel tiles of X (16 KB) and the matching W tile through an
 //                   8-stage TMA ring.  Per tile, four epilogue warps take p = hi part + lo part
 //                   from TMEM (one token per thread) and add the tile's sums over their 32 tokens
-//                   (p p^T upper triangle, e p^T; fp32) to per-lane registers; each CTA's run of
-//                   tiles of a block ends in
+//                   (p p^T upper triangle, e p^T; fp32) to per-lane registers; a CTA's tiles are one
+//                   contiguous range, and its run of tiles of a block ends in
 //                   one write of its (block, CTA, warp) fp64 partial slot.  Two further warps sum
 //                   the squares of every X tile and, with the MMA commit, release the stages, so
 //                   the statistics never hold up the ring.  Nothing but X is read from HBM in
 //                   bulk, and no warp waits for another outside the mbarrier pipeline.
-//   k_kspace_ete    E^T E of the batch (C x C), shared by every block: ||T_l||^2 =
-//                   <P_l (Q_l Q_l^T) P_l^T, E^T E>, so no per-token work is needed for it.
 //   k_kspace_final  fixed-order reduction of the partial slots per block (deterministic),
 //                   ||T_l||^2, alpha_l, and the update of G, S, xsq_total.
 //   k_kspace_solve  lambda from the trace, Cholesky of G_l + lambda I, C_l rows from Q_l^T (P_l^T
@@ -47,39 +47,116 @@ using namespace tc;
 
 // ------------------------------------------------------------------ prep
 constexpr int PREP_THREADS = 256;
-constexpr int PREP_SPLIT = 8;  // CTAs per block
+constexpr int PREP_COLS = 128;    // channels per CTA of the split
+constexpr int ETE_CHUNK = 1024;   // tokens per partial of E^T E
+constexpr int kMaxCk = 16;        // C limit of the k-space path
+constexpr int kMaxRk = 32;        // r limit
 
-// grid (L, PREP_SPLIT): each CTA splits a slice of A_l^T and forms a slice of the r x r entries
-// of Q_l Q_l^T, one warp per entry (lanes over channels; fp32 lane sums, fp64 across lanes).
+// CTAs [0, nW): (block, 128-channel slab) of the split of A_l^T, transposed through shared memory.
+// CTAs [nW, nW + nM): M_l = Q_l Q_l^T, one warp per 2 x 2 block of its upper triangle of blocks: lanes over
+//   channels (fp32 lane sums, fp64 across lanes), four rows of Q_l read for four entries.
+// The rest: one 1024-token chunk of E^T E each: fp32 over a thread's 4 to 1024 / (256 / C^2) tokens, fp64
+//   across the threads, in a fixed order.
+// Every kind is bound by latency, so they share a launch (two launches and, with one warp per entry of M and
+// one thread per entry of E^T E, 100 us at L = 24, d = 2048, r = k = 32).
 __global__ void __launch_bounds__(PREP_THREADS) k_kspace_prep(const float* __restrict__ A, const float* __restrict__ Q,
-                                                             int64_t d, int k, int kp, int r,
-                                                             __nv_bfloat16* __restrict__ W, float* __restrict__ M) {
-  const int l = blockIdx.x, part = blockIdx.y;
-  const float* Al = A + int64_t(l) * d * k;
-  __nv_bfloat16* Wl = W + int64_t(l) * 2 * kp * d;
-  const int64_t tot = int64_t(kp) * d;
-  for (int64_t e = int64_t(part) * PREP_THREADS + threadIdx.x; e < tot; e += int64_t(PREP_SPLIT) * PREP_THREADS) {
-    const int s = int(e / d);
-    const int64_t j = e - int64_t(s) * d;
-    const float a = (s < k && LOCA_CHECK(j * k + s, d * k)) ? Al[j * k + s] : 0.f;
-    const __nv_bfloat16 hi = __float2bfloat16_rn(a);
-    const __nv_bfloat16 lo = __float2bfloat16_rn(a - __bfloat162float(hi));
-    if (!LOCA_CHECK(int64_t(kp + s) * d + j, int64_t(2) * kp * d)) continue;
-    Wl[int64_t(s) * d + j] = hi;
-    Wl[int64_t(kp + s) * d + j] = lo;
+                                                             const float* __restrict__ E, int64_t N, int C, int L,
+                                                             int64_t d, int k, int kp, int r, int nW,
+                                                             __nv_bfloat16* __restrict__ W, float* __restrict__ M,
+                                                             double* __restrict__ ete_part, int32_t* abort_flag) {
+  __shared__ __align__(16) float sm[PREP_COLS * 33];
+  __shared__ double red[PREP_THREADS];
+  const int tid = threadIdx.x;
+  int b = int(blockIdx.x);
+  if (b == 0 && tid == 0) *abort_flag = 0;  // the next kernel's waits
+  if (b < nW) {
+    const int slabs = int((d + PREP_COLS - 1) / PREP_COLS);
+    const int l = b / slabs;
+    const int64_t j0 = int64_t(b - l * slabs) * PREP_COLS;
+    const int nc = d - j0 < PREP_COLS ? int(d - j0) : PREP_COLS;
+    const float* Al = A + int64_t(l) * d * k + j0 * k;
+    for (int e = tid; e < nc * k; e += PREP_THREADS)
+      sm[(e / k) * 33 + e % k] = LOCA_CHECK(j0 * k + e, d * k) ? Al[e] : 0.f;
+    __syncthreads();
+    __nv_bfloat16* Wl = W + int64_t(l) * 2 * kp * d;
+    for (int e = tid; e < kp * PREP_COLS; e += PREP_THREADS) {
+      const int s = e / PREP_COLS, j = e % PREP_COLS;
+      if (j >= nc || !LOCA_CHECK(int64_t(kp + s) * d + j0 + j, int64_t(2) * kp * d)) continue;
+      const float a = s < k ? sm[j * 33 + s] : 0.f;
+      const __nv_bfloat16 hi = __float2bfloat16_rn(a);
+      Wl[int64_t(s) * d + j0 + j] = hi;
+      Wl[int64_t(kp + s) * d + j0 + j] = __float2bfloat16_rn(a - __bfloat162float(hi));
+    }
+    return;
   }
-  const float* Ql = Q + int64_t(l) * r * d;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  constexpr int kWarps = PREP_THREADS / 32;
-  for (int e = part * kWarps + warp; e < r * r; e += PREP_SPLIT * kWarps) {
-    const int a = e / r, b = e % r;
-    float acc = 0.f;
-    for (int64_t j = lane; j < d; j += 32) acc = fmaf(Ql[int64_t(a) * d + j], Ql[int64_t(b) * d + j], acc);
-    double v = double(acc);
+  b -= nW;
+  const int rb = (r + 1) / 2, nblk = rb * (rb + 1) / 2;  // 2 x 2 blocks of the upper triangle
+  constexpr int WARPS = PREP_THREADS / 32;
+  const int nM = (L * nblk + WARPS - 1) / WARPS;
+  if (b < nM) {
+    const int w = b * WARPS + (tid >> 5), lane = tid & 31;
+    if (w >= L * nblk) return;
+    const int l = w / nblk;
+    int ba = 0, bb = w - l * nblk;
+    while (bb >= rb - ba) bb -= rb - ba++;
+    bb += ba;
+    const float* Ql = Q + int64_t(l) * r * d;
+    const int a0 = 2 * ba, b0 = 2 * bb;
+    const float* qa0 = Ql + int64_t(a0) * d;
+    const float* qb0 = Ql + int64_t(b0) * d;
+    const float* qa1 = a0 + 1 < r ? qa0 + d : qa0;  // an odd r's last row stands in for the missing one
+    const float* qb1 = b0 + 1 < r ? qb0 + d : qb0;
+    float s00 = 0.f, s01 = 0.f, s10 = 0.f, s11 = 0.f;
+#pragma unroll 8
+    for (int64_t j = lane; j < d; j += 32) {
+      const float x0 = __ldg(qa0 + j), x1 = __ldg(qa1 + j), y0 = __ldg(qb0 + j), y1 = __ldg(qb1 + j);
+      s00 = fmaf(x0, y0, s00);
+      s01 = fmaf(x0, y1, s01);
+      s10 = fmaf(x1, y0, s10);
+      s11 = fmaf(x1, y1, s11);
+    }
+    double v[4] = {double(s00), double(s01), double(s10), double(s11)};
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-    if (lane == 0 && LOCA_CHECK((int64_t(l) * r + a) * r + b, int64_t(gridDim.x) * r * r))
-      M[(int64_t(l) * r + a) * r + b] = float(v);
+    for (int q = 0; q < 4; ++q)
+#pragma unroll
+      for (int off = 16; off > 0; off >>= 1) v[q] += __shfl_xor_sync(0xffffffffu, v[q], off);
+    if (lane < 4) {
+      const int ea = a0 + (lane >> 1), eb = b0 + (lane & 1);
+      const float m = float(lane == 0 ? v[0] : (lane == 1 ? v[1] : (lane == 2 ? v[2] : v[3])));
+      if (ea <= eb && eb < r && LOCA_CHECK((int64_t(l) * r + ea) * r + eb, int64_t(L) * r * r)) {
+        M[(int64_t(l) * r + ea) * r + eb] = m;
+        M[(int64_t(l) * r + eb) * r + ea] = m;
+      }
+    }
+    return;
+  }
+  b -= nM;
+  const int64_t n0 = int64_t(b) * ETE_CHUNK;
+  const int64_t n1 = n0 + ETE_CHUNK < N ? n0 + ETE_CHUNK : N;
+  const int C2 = C * C, groups = PREP_THREADS / C2;  // C <= 16
+  const int e = tid % C2, grp = tid / C2;
+  double acc = 0.0;
+  if (grp < groups) {
+    const int ca = e / C, cb = e % C;
+    float run = 0.f;
+    int cnt = 0;
+#pragma unroll 8
+    for (int64_t n = n0 + grp; n < n1; n += groups) {
+      if (LOCA_CHECK(n * C + ca, N * C) && LOCA_CHECK(n * C + cb, N * C)) run = fmaf(E[n * C + ca], E[n * C + cb], run);
+      if (++cnt == 64) {
+        acc += double(run);
+        run = 0.f;
+        cnt = 0;
+      }
+    }
+    acc += double(run);
+  }
+  red[tid] = acc;
+  __syncthreads();
+  if (tid < C2) {
+    for (int q = 1; q < groups; ++q) acc += red[q * C2 + tid];
+    if (LOCA_CHECK(int64_t(b) * kMaxCk * kMaxCk + tid, int64_t((N + ETE_CHUNK - 1) / ETE_CHUNK) * kMaxCk * kMaxCk))
+      ete_part[int64_t(b) * kMaxCk * kMaxCk + tid] = acc;
   }
 }
 
@@ -97,8 +174,6 @@ constexpr int XA_XBYTES = XA_TM * XA_BK * 2;  // 16 KB
 constexpr int XA_STAGE = 24 * 1024;           // X tile + up to 64 W rows (8 KB)
 constexpr uint32_t XA_TMEM_COLS = 128;
 constexpr int XA_MAX_GRID = 256;   // partial slots per block are sized for at most this many CTAs
-constexpr int kMaxCk = 16;         // C limit of the k-space path
-constexpr int kMaxRk = 32;         // r limit
 // per-warp p and e staging: token-major rows at kp = 16 (32 x (33 + 17) floats), channel-major
 // rows of 36 floats at kp = 32 ((32 + 16) x 36 floats)
 constexpr int XA_EPI_WARP =
@@ -109,6 +184,21 @@ constexpr int XA_EPI_SMEM = 4 * XA_EPI_WARP * 4;
 __host__ __device__ constexpr int ntri(int kp) { return kp * (kp + 1) / 2; }
 __host__ __device__ constexpr int part_stride(int kp, int C) { return ntri(kp) + C * kp + 1; }
 constexpr int XA_SMEM = XA_STAGES * XA_STAGE + 1024 + 256 + XA_EPI_SMEM;
+
+// CTA c of `grid` takes tiles [first_tile(c), first_tile(c + 1)) of all blocks' tiles in order, so a block's
+// tiles fall to total / (L grid) neighbouring CTAs and each CTA ends one or two runs: with tiles dealt out
+// in turn every CTA had a run of every block, and the partial slots (608 per block, 77 MB at L = 24, k = 32)
+// took 170 us to reduce.
+__host__ __device__ __forceinline__ int first_tile(int c, int grid, int total) { return int(int64_t(total) * c / grid); }
+__host__ __device__ __forceinline__ int tile_owner(int i, int grid, int total) {
+  return int(((int64_t(i) + 1) * grid - 1) / total);
+}
+// CTAs that may share a block of ntiles tiles: slots per block and warp.
+__host__ __device__ __forceinline__ int max_owners(int ntiles, int grid, int total) {
+  const int per = total / grid;  // >= 1: the grid is at most the number of tiles
+  const int n = (ntiles + per - 1) / per + 1;
+  return n < grid ? n : grid;
+}
 
 template <int KP>
 __global__ void __launch_bounds__(xa_threads(KP), 1)
@@ -156,13 +246,17 @@ __global__ void __launch_bounds__(xa_threads(KP), 1)
   const uint32_t tmem_base = *tmem_slot;
   const int nkc = int((d + XA_BK - 1) / XA_BK);
   const int total = L * ntiles;
+  const int it0 = first_tile(blockIdx.x, gridDim.x, total), it1 = first_tile(blockIdx.x + 1, gridDim.x, total);
+  const int64_t nslot = int64_t(max_owners(ntiles, gridDim.x, total)) * 4;
+  // this CTA's slots of block l
+  auto slot_of = [&](int l) { return 4 * (int(blockIdx.x) - tile_owner(l * ntiles, gridDim.x, total)); };
 
   if (warp == 0) {
     if (lane == 0) {
       int stage = 0;
       uint32_t phase = 0, pending = 0, pending_par = 0;
       bool ok = true;
-      for (int it = blockIdx.x; it < total && ok; it += gridDim.x) {
+      for (int it = it0; it < it1 && ok; ++it) {
         const int l = it / ntiles;
         const int t0 = (it - l * ntiles) * XA_TM;
         for (int kc = 0; kc < nkc; ++kc) {
@@ -192,7 +286,7 @@ __global__ void __launch_bounds__(xa_threads(KP), 1)
       int stage = 0;
       uint32_t phase = 0, tcount = 0;
       bool ok = true, issued = false;
-      for (int it = blockIdx.x; it < total && ok; it += gridDim.x, ++tcount) {
+      for (int it = it0; it < it1 && ok; ++it, ++tcount) {
         const int buf = int(tcount & 1u);
         const uint32_t aph = (tcount >> 1) & 1u;
         if (!mbar_try_wait(acc_empty(buf), aph ^ 1u) && !mbar_wait(acc_empty(buf), aph ^ 1u, wc)) {
@@ -231,7 +325,6 @@ __global__ void __launch_bounds__(xa_threads(KP), 1)
     // (with the MMA commit) release the stages, so the statistics below never hold up the ring
     const int w2 = warp - 6;
     const int PS = part_stride(KP, C);
-    const int64_t nslot = int64_t(gridDim.x) * 4;
     const int xe = ntri(KP) + C * KP;  // the ||x||^2 entry of slots (CTA, w2)
     double xs = 0.0;
     int cur_l = -1;
@@ -239,12 +332,11 @@ __global__ void __launch_bounds__(xa_threads(KP), 1)
       double a = xs;
 #pragma unroll
       for (int off = 16; off > 0; off >>= 1) a += __shfl_xor_sync(0xffffffffu, a, off);
-      if (lane == 0 && LOCA_CHECK((int64_t(lf) * PS + xe) * nslot + int64_t(blockIdx.x) * 4 + w2, int64_t(L) * PS * nslot))
-        part[(int64_t(lf) * PS + xe) * nslot + int64_t(blockIdx.x) * 4 + w2] = a;
+      if (lane == 0 && LOCA_CHECK(slot_of(lf) + w2, nslot)) part[(int64_t(lf) * PS + xe) * nslot + slot_of(lf) + w2] = a;
     };
     int stage = 0;
     uint32_t phase = 0;
-    for (int it = blockIdx.x; it < total; it += gridDim.x) {
+    for (int it = it0; it < it1; ++it) {
       const int l = it / ntiles;
       if (l != cur_l) {
         if (cur_l >= 0) flush(cur_l);
@@ -335,16 +427,22 @@ __global__ void __launch_bounds__(xa_threads(KP), 1)
     float* es = kBlk ? ps + 32 * TST : ps + 32 * 33;
     auto prow = [](int s2) { return (s2 >> 1) + (s2 & 1) * (KP / 2); };
     auto entry = [](int a, int b) { return a * KP - a * (a - 1) / 2 + (b - a); };
-    // this lane's sums for the current block (fp32 within one CTA's run of tiles of a block; the
-    // runs are written once, as fp64, when the block changes, and reduced in a fixed order later)
-    float accg[NACC], accs[NSM];
+    // this lane's sums for the current block: fp32 over a tile, tile sums as fp32 pairs (sum and
+    // rounding error, Knuth's two-sum); a run is written once, as fp64, when the block changes, and
+    // the runs are reduced in a fixed order later
+    float accg[NACC], accs[NSM], errg[NACC], errs[NSM];
+    auto add_tile = [](float& a, float& e, float p) {
+      const float t = __fadd_rn(a, p), bb = __fsub_rn(t, a);
+      e += __fadd_rn(__fsub_rn(a, __fsub_rn(t, bb)), __fsub_rn(p, bb));
+      a = t;
+    };
+    auto pair_sum = [](float a, float e) { return isfinite(a) ? double(a) + double(e) : double(a); };
     int cur_l = -1;
-    const int64_t nslot = int64_t(gridDim.x) * 4;
     auto flush = [&](int lf) {
       // entry-major: entry e of block lf at part[(lf * PS + e) * nslot + this slot]
-      double* slot = part + int64_t(lf) * PS * nslot + int64_t(blockIdx.x) * 4 + q;
+      double* slot = part + int64_t(lf) * PS * nslot + slot_of(lf) + q;
       // every entry index below is < PS - 1 (the last one is the ||x||^2 entry of the other warps)
-      if (!LOCA_CHECK(lf, L) || !LOCA_REQUIRE(NTRI + NS + 1 == PS)) return;
+      if (!LOCA_CHECK(lf, L) || !LOCA_CHECK(slot_of(lf) + q, nslot) || !LOCA_REQUIRE(NTRI + NS + 1 == PS)) return;
       if constexpr (kBlk) {
 #pragma unroll
         for (int i2 = 0; i2 < NG; ++i2) {
@@ -352,23 +450,23 @@ __global__ void __launch_bounds__(xa_threads(KP), 1)
             int bi, bj;
             blk_pair(i2, bi, bj);
             const int a0 = 2 * bi, b0 = 2 * bj;
-            slot[int64_t(entry(a0, b0)) * nslot] = double(accg[4 * i2]);
-            slot[int64_t(entry(a0, b0 + 1)) * nslot] = double(accg[4 * i2 + 1]);
-            if (a0 != b0) slot[int64_t(entry(a0 + 1, b0)) * nslot] = double(accg[4 * i2 + 2]);
-            slot[int64_t(entry(a0 + 1, b0 + 1)) * nslot] = double(accg[4 * i2 + 3]);
+            slot[int64_t(entry(a0, b0)) * nslot] = pair_sum(accg[4 * i2], errg[4 * i2]);
+            slot[int64_t(entry(a0, b0 + 1)) * nslot] = pair_sum(accg[4 * i2 + 1], errg[4 * i2 + 1]);
+            if (a0 != b0) slot[int64_t(entry(a0 + 1, b0)) * nslot] = pair_sum(accg[4 * i2 + 2], errg[4 * i2 + 2]);
+            slot[int64_t(entry(a0 + 1, b0 + 1)) * nslot] = pair_sum(accg[4 * i2 + 3], errg[4 * i2 + 3]);
           }
         }
       } else {
 #pragma unroll
         for (int i2 = 0; i2 < NG; ++i2)
-          if (lane + 32 * i2 < NTRI) slot[int64_t(lane + 32 * i2) * nslot] = double(accg[i2]);
+          if (lane + 32 * i2 < NTRI) slot[int64_t(lane + 32 * i2) * nslot] = pair_sum(accg[i2], errg[i2]);
       }
 #pragma unroll
       for (int i2 = 0; i2 < NSM; ++i2)
-        if (lane + 32 * i2 < NS) slot[int64_t(NTRI + lane + 32 * i2) * nslot] = double(accs[i2]);
+        if (lane + 32 * i2 < NS) slot[int64_t(NTRI + lane + 32 * i2) * nslot] = pair_sum(accs[i2], errs[i2]);
     };
     uint32_t tcount = 0;
-    for (int it = blockIdx.x; it < total; it += gridDim.x, ++tcount) {
+    for (int it = it0; it < it1; ++it, ++tcount) {
       const int l = it / ntiles;
       const int tile = it - l * ntiles;
       const int t0 = tile * XA_TM;
@@ -376,9 +474,9 @@ __global__ void __launch_bounds__(xa_threads(KP), 1)
         if (cur_l >= 0) flush(cur_l);
         cur_l = l;
 #pragma unroll
-        for (int i2 = 0; i2 < NACC; ++i2) accg[i2] = 0.f;
+        for (int i2 = 0; i2 < NACC; ++i2) accg[i2] = errg[i2] = 0.f;
 #pragma unroll
-        for (int i2 = 0; i2 < NSM; ++i2) accs[i2] = 0.f;
+        for (int i2 = 0; i2 < NSM; ++i2) accs[i2] = errs[i2] = 0.f;
       }
       const int buf = int(tcount & 1u);
       const uint32_t aph = (tcount >> 1) & 1u;
@@ -454,10 +552,10 @@ __global__ void __launch_bounds__(xa_threads(KP), 1)
               s00 = fmaf(x0.w, y0.w, s00); s01 = fmaf(x0.w, y1.w, s01);
               s10 = fmaf(x1.w, y0.w, s10); s11 = fmaf(x1.w, y1.w, s11);
             }
-            accg[4 * i2] += s00;
-            accg[4 * i2 + 1] += s01;
-            accg[4 * i2 + 2] += s10;
-            accg[4 * i2 + 3] += s11;
+            add_tile(accg[4 * i2], errg[4 * i2], s00);
+            add_tile(accg[4 * i2 + 1], errg[4 * i2 + 1], s01);
+            add_tile(accg[4 * i2 + 2], errg[4 * i2 + 2], s10);
+            add_tile(accg[4 * i2 + 3], errg[4 * i2 + 3], s11);
           }
         }
         // e p^T: this lane's channel s = lane of every label column c (eidx = c kp + lane)
@@ -477,7 +575,7 @@ __global__ void __launch_bounds__(xa_threads(KP), 1)
               sc = fmaf(ev.z, pv.z, sc);
               sc = fmaf(ev.w, pv.w, sc);
             }
-            accs[c] += sc;
+            add_tile(accs[c], errs[c], sc);
           }
         }
       } else {
@@ -488,7 +586,7 @@ __global__ void __launch_bounds__(xa_threads(KP), 1)
             float acc = 0.f;
 #pragma unroll 8
             for (int t = 0; t < 32; ++t) acc = fmaf(ps[t * PSTR + a], ps[t * PSTR + b], acc);
-            accg[i2] += acc;
+            add_tile(accg[i2], errg[i2], acc);
           }
         }
 #pragma unroll
@@ -499,7 +597,7 @@ __global__ void __launch_bounds__(xa_threads(KP), 1)
             float acc = 0.f;
 #pragma unroll 8
             for (int t = 0; t < 32; ++t) acc = fmaf(es[t * ESTR + c], ps[t * PSTR + s2], acc);
-            accs[i2] += acc;
+            add_tile(accs[i2], errs[i2], acc);
           }
         }
       }
@@ -514,47 +612,13 @@ __global__ void __launch_bounds__(xa_threads(KP), 1)
   if (warp == 1) tmem_dealloc(tmem_base, XA_TMEM_COLS);
 }
 
-// ------------------------------------------------------------------ E^T E
-// ||T_l||^2 = sum_n u_n^T (Q_l Q_l^T) u_n = <P_l (Q_l Q_l^T) P_l^T, E^T E>: the C x C matrix E^T E
-// of the batch serves every block.  Partials per chunk of tokens (fp32 over 256 tokens, fp64
-// across), reduced in a fixed order by k_kspace_final.
-constexpr int ETE_THREADS = 256;
-constexpr int ETE_SUB = 256;
-constexpr int ETE_CHUNK = 1024;
-
-__global__ void __launch_bounds__(ETE_THREADS) k_kspace_ete(const float* __restrict__ E, int64_t N, int C,
-                                                          double* __restrict__ ete_part) {
-  __shared__ float es[ETE_SUB][kMaxCk + 1];
-  const int ch = blockIdx.x, tid = threadIdx.x;
-  const int a = tid / kMaxCk, b = tid % kMaxCk;
-  const int64_t n0 = int64_t(ch) * ETE_CHUNK;
-  const int64_t n1 = (n0 + ETE_CHUNK < N) ? n0 + ETE_CHUNK : N;
-  double acc = 0.0;
-  for (int64_t s0 = n0; s0 < n1; s0 += ETE_SUB) {
-    __syncthreads();
-    for (int e = tid; e < ETE_SUB * C; e += ETE_THREADS) {
-      const int t = e / C, c = e % C;
-      es[t][c] = (s0 + t < n1 && LOCA_CHECK((s0 + t) * C + c, N * C)) ? E[(s0 + t) * C + c] : 0.f;
-    }
-    __syncthreads();
-    if (a < C && b < C) {
-      float part = 0.f;
-#pragma unroll 8
-      for (int t = 0; t < ETE_SUB; ++t) part = fmaf(es[t][a], es[t][b], part);
-      acc += double(part);
-    }
-  }
-  if (a < C && b < C && LOCA_CHECK(int64_t(ch) * kMaxCk * kMaxCk + a * kMaxCk + b, int64_t(gridDim.x) * kMaxCk * kMaxCk))
-    ete_part[int64_t(ch) * kMaxCk * kMaxCk + a * kMaxCk + b] = acc;
-}
-
 // ------------------------------------------------------------------ per-block final reduction
 constexpr int FI_THREADS = 256;
-constexpr int FI_SPLIT = 4;  // CTAs per block (entries e with e % FI_SPLIT == part)
+constexpr int FI_SPLIT = 16;  // CTAs per block (entries dealt out over their warps)
+constexpr int FI_MOST = 9;    // entries per warp at most: (32 * 33 / 2 + 16 * 32) / (16 * 8)
 
-// Sums the (CTA, warp) partial slots of block l in a fixed order (a CTA without tiles of block l,
-// possible only when blocks have fewer tiles than there are CTAs, never wrote its slot), forms
-// ||T_l||^2 = <P_l M_l P_l^T, E^T E>, the step alpha_l, and updates G, SC, xsq_total.
+// Sums the (CTA, warp) partial slots of block l in a fixed order, forms ||T_l||^2 = <P_l M_l P_l^T, E^T E>, the
+// step alpha_l, and updates G, SC, xsq_total.  Bound by latency: one warp per entry, lanes over the slots.
 __global__ void __launch_bounds__(FI_THREADS) k_kspace_final(const double* __restrict__ part,
                                                            const double* __restrict__ ete_part, int nch_e,
                                                            const float* __restrict__ P, const float* __restrict__ M,
@@ -562,85 +626,98 @@ __global__ void __launch_bounds__(FI_THREADS) k_kspace_final(const double* __res
                                                            float eta, int zero_first, float* __restrict__ G,
                                                            float* __restrict__ SC, double* __restrict__ xsq_total,
                                                            float* __restrict__ alpha_out) {
-  __shared__ unsigned char has[XA_MAX_GRID];
   __shared__ double ete[kMaxCk][kMaxCk];
   __shared__ double pm[kMaxCk][kMaxRk];  // P_l M_l
-  __shared__ double red[FI_THREADS];
+  __shared__ double red[FI_THREADS / 32];
   __shared__ double s_xsq;
   const int l = blockIdx.x, prt = blockIdx.y, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int L = int(gridDim.x), total = L * ntiles;
   const int ps = part_stride(kp, C);
-  const int64_t lo = int64_t(l) * ntiles, hi = lo + ntiles;
-  for (int c = tid; c < grid; c += FI_THREADS) has[c] = (lo + ((int64_t(c) - lo) % grid + grid) % grid) < hi;
-  for (int e = tid; e < C * C; e += FI_THREADS) {
-    const int a = e / C, b = e % C;
+  const int64_t nslot = int64_t(max_owners(ntiles, grid, total)) * 4;
+  const int owners = tile_owner((l + 1) * ntiles - 1, grid, total) - tile_owner(l * ntiles, grid, total) + 1;
+  // one warp; lanes over slots in order, then a fixed butterfly.  The ||x||^2 entry is written
+  // by the sum-of-squares warps, one slot each (slots 0..xa_sq_warps(kp)-1 of each CTA).
+  auto sum_entry = [&](int e, int nq) {
+    const double* pe = part + (int64_t(l) * ps + e) * nslot;
     double v = 0.0;
-    for (int ch = 0; ch < nch_e; ++ch) v += ete_part[int64_t(ch) * kMaxCk * kMaxCk + a * kMaxCk + b];
-    ete[a][b] = v;
+    for (int sidx = lane; sidx < owners * 4; sidx += 32)
+      if ((sidx & 3) < nq) v += pe[sidx];
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+    return v;
+  };
+  // this warp's entries: G's (the upper triangle, written on both sides), then SC's
+  const int nt = ntri(kp), ntk = k * (k + 1) / 2;
+  const int e0 = prt * (FI_THREADS / 32) + warp;
+  constexpr int STEP = FI_SPLIT * (FI_THREADS / 32);
+  double val[FI_MOST];
+#pragma unroll
+  for (int q = 0; q < FI_MOST; ++q) {
+    const int e = e0 + q * STEP;
+    val[q] = 0.0;
+    if (e >= ntk + C * k) break;
+    int src;
+    if (e < ntk) {
+      int a = 0, b = e;
+      while (b >= k - a) b -= k - a++;
+      src = a * kp - a * (a - 1) / 2 + b;  // row a of the kp-wide upper triangle
+    } else {
+      src = nt + (e - ntk) / k * kp + (e - ntk) % k;
+    }
+    val[q] = sum_entry(src, 4);
+  }
+  if (warp == 0) {
+    const double v = sum_entry(nt + C * kp, xa_sq_warps(kp));
+    if (lane == 0) s_xsq = v;
+  }
+  for (int e = warp; e < C * C; e += FI_THREADS / 32) {
+    double v = 0.0;
+    for (int ch = lane; ch < nch_e; ch += 32) v += ete_part[int64_t(ch) * kMaxCk * kMaxCk + e];
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+    if (lane == 0) ete[e / C][e % C] = v;
   }
   const float* Pl = P + int64_t(l) * C * r;
   const float* Ml = M + int64_t(l) * r * r;
   for (int e = tid; e < C * r; e += FI_THREADS) {
     const int c = e / r, b = e % r;
     double v = 0.0;
-    for (int a = 0; a < r; ++a) v += double(Pl[c * r + a]) * double(Ml[a * r + b]);
+#pragma unroll 8
+    for (int a = 0; a < r; ++a) v = fma(double(Pl[c * r + a]), double(Ml[a * r + b]), v);
     pm[c][b] = v;
   }
   __syncthreads();
-  const int nslot = grid * 4;
-  // one warp; lanes over slots in order, then a fixed butterfly.  The ||x||^2 entry is written
-  // by the sum-of-squares warps, one slot each (slots 0..xa_sq_warps(kp)-1 of each CTA).
-  auto sum_entry = [&](int e, int nq) {
-    const double* pe = part + (int64_t(l) * ps + e) * nslot;
-    double v = 0.0;
-    for (int sidx = lane; sidx < nslot; sidx += 32)
-      if (has[sidx >> 2] && (sidx & 3) < nq) v += pe[sidx];
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-    return v;
-  };
-  const int nt = ntri(kp);
-  if (warp == 0) {
-    const double v = sum_entry(nt + C * kp, xa_sq_warps(kp));
-    if (lane == 0) s_xsq = v;
-  }
-  // ||T_l||^2 = sum_{c, c'} (P M P^T)[c][c'] (E^T E)[c][c']
+  // ||T_l||^2 = sum_{c, c'} (P M P^T)[c][c'] (E^T E)[c][c'], C^2 <= 256 terms
   double t = 0.0;
-  for (int e = tid; e < C * C; e += FI_THREADS) {
-    const int a = e / C, b = e % C;
-    double kab = 0.0;
-    for (int j = 0; j < r; ++j) kab += pm[a][j] * double(Pl[b * r + j]);
-    t += kab * ete[a][b];
+  if (tid < C * C) {
+    const int a = tid / C, b = tid % C;
+#pragma unroll 8
+    for (int j = 0; j < r; ++j) t = fma(pm[a][j], double(Pl[b * r + j]), t);
+    t *= ete[a][b];
   }
-  red[tid] = t;
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) t += __shfl_xor_sync(0xffffffffu, t, off);
+  if (lane == 0) red[warp] = t;
   __syncthreads();
-  for (int w = FI_THREADS / 2; w > 0; w >>= 1) {
-    if (tid < w) red[tid] += red[tid + w];
-    __syncthreads();
-  }
-  const double xsq_b = s_xsq, tsq_b = red[0];
+  double tsq_b = 0.0;
+  for (int w = 0; w < FI_THREADS / 32; ++w) tsq_b += red[w];
+  const double xsq_b = s_xsq;
   const double al = tsq_b > 0.0 ? -double(eta) * sqrt(xsq_b / tsq_b) : 0.0;
-  // G entries (symmetric, from the upper triangle) and SC entries of this CTA's share
-  for (int e = prt * (FI_THREADS / 32) + warp; e < k * k + C * k; e += FI_SPLIT * (FI_THREADS / 32)) {
-    if (e < k * k) {
-      int a = e / k, b = e % k;
-      if (a > b) {
-        const int tmp = a;
-        a = b;
-        b = tmp;
+#pragma unroll
+  for (int q = 0; q < FI_MOST; ++q) {
+    const int e = e0 + q * STEP;
+    if (e >= ntk + C * k) break;
+    if (e < ntk) {
+      int a = 0, b = e;
+      while (b >= k - a) b -= k - a++;
+      b += a;
+      if (lane < 2 && (lane == 0 || a != b) && LOCA_CHECK(a * k + b, k * k)) {
+        float* o = G + int64_t(l) * k * k + (lane == 0 ? a * k + b : b * k + a);
+        *o = zero_first ? float(val[q]) : float(double(*o) + val[q]);
       }
-      const double v = sum_entry(a * kp - a * (a - 1) / 2 + (b - a), 4);  // row a of the upper triangle
-      if (lane == 0 && LOCA_CHECK(int64_t(l) * k * k + e, int64_t(gridDim.x) * k * k)) {
-        float* o = G + int64_t(l) * k * k + e;
-        *o = zero_first ? float(v) : float(double(*o) + v);
-      }
-    } else {
-      const int e2 = e - k * k;
-      const int cc = e2 / k, s2 = e2 % k;
-      const double v = sum_entry(nt + cc * kp + s2, 4);
-      if (lane == 0 && LOCA_CHECK(int64_t(l) * C * k + e2, int64_t(gridDim.x) * C * k)) {
-        float* o = SC + int64_t(l) * C * k + e2;
-        *o = zero_first ? float(al * v) : float(double(*o) + al * v);
-      }
+    } else if (lane == 0 && LOCA_CHECK(int64_t(l) * C * k + (e - ntk), int64_t(gridDim.x) * C * k)) {
+      float* o = SC + int64_t(l) * C * k + (e - ntk);
+      *o = zero_first ? float(al * val[q]) : float(double(*o) + al * val[q]);
     }
   }
   if (prt == 0 && tid == 0 && LOCA_CHECK(l, gridDim.x)) {
@@ -650,22 +727,26 @@ __global__ void __launch_bounds__(FI_THREADS) k_kspace_final(const double* __res
 }
 
 // ------------------------------------------------------------------ solve
-constexpr int KS_THREADS = 256;
+// CTA (row chunk, candidate j, block l): the candidate's factor, formed anew by each of the block's few row
+// chunks (no workspace to share it, and they run side by side), then the chunk's rows, NR per thread at a
+// time: C_l[i] = Q_l[:, i]^T (P_l^T S_l) (+ B_prev,l[i] G_l) and the two substitutions.  Two CTAs per SM over
+// the whole grid: more chunks only repeat the factor (14 of them at d = 3584, k = 16: 71 us).  Bound by latency; one CTA per (j, l) for all d
+// rows took 264 us at L = 24, d = 2048, k = 32 with three candidates.
+constexpr int KS_THREADS = 128;
 
-template <int KM>
+template <int KM, int NR>
 __global__ void __launch_bounds__(KS_THREADS) k_kspace_solve(
     const float* __restrict__ G, const float* __restrict__ SC, const double* __restrict__ xsq_total,
     const float* __restrict__ P, const float* __restrict__ Q, const float* __restrict__ B_prev, int64_t d,
-    int k, int C, int r, int L, float l0, float l1, float l2, float l3, float l4, float l5, float l6, float l7,
+    int k, int C, int r, int L, int vec, float l0, float l1, float l2, float l3, float l4, float l5, float l6, float l7,
     float l8, float l9, float l10, float l11, float l12, float l13, float l14, float l15, float* __restrict__ B,
     int32_t* __restrict__ info, float* __restrict__ C_out) {
-  __shared__ float Gf[KM][KM];
+  __shared__ __align__(16) float Gf[KM][KM];
   __shared__ double Md[KM][KM];
-  __shared__ float Lf[KM][KM];
+  __shared__ __align__(16) float Lf[KM][KM];
   __shared__ float Linv[KM];
-  __shared__ float W2[kMaxRk][KM];  // P_l^T S_l  (r x k)
-  __shared__ int s_info;
-  const int j = blockIdx.x, l = blockIdx.y;
+  __shared__ __align__(16) float W2[kMaxRk][KM];  // P_l^T S_l  (r x k)
+  const int j = blockIdx.y, l = blockIdx.z;
   const float lam_rel[16] = {l0, l1, l2, l3, l4, l5, l6, l7, l8, l9, l10, l11, l12, l13, l14, l15};
   for (int e = threadIdx.x; e < KM * KM; e += KS_THREADS) {
     const int a = e / KM, b = e % KM;
@@ -682,60 +763,59 @@ __global__ void __launch_bounds__(KS_THREADS) k_kspace_solve(
   const double lam = double(lam_rel[j]) * (xsq_total != nullptr ? xsq_total[l] / double(d) : 1.0);
   for (int e = threadIdx.x; e < KM * KM; e += KS_THREADS) {
     const int a = e / KM, b = e % KM;
-    double v;
-    if (a < k && b < k) {
-      v = 0.5 * (double(Gf[a][b]) + double(Gf[b][a]));
-      if (a == b) v += lam;
-    } else {
-      v = (a == b) ? 1.0 : 0.0;
-    }
-    Md[a][b] = v;
+    Md[a][b] = 0.5 * (double(Gf[a][b]) + double(Gf[b][a])) + (a == b ? lam : 0.0);
   }
   __syncthreads();
-  const int inf = chol_factor<KM>(Md, Lf, Linv, &s_info);
-  if (threadIdx.x == 0 && LOCA_CHECK(int64_t(j) * L + l, int64_t(gridDim.x) * L)) info[int64_t(j) * L + l] = inf;
+  const int inf = chol_factor<KM>(Md, Lf, Linv, k);
+  if (blockIdx.x == 0 && threadIdx.x == 0 && LOCA_CHECK(int64_t(j) * L + l, int64_t(gridDim.y) * L)) info[int64_t(j) * L + l] = inf;
   float* Bj = B + (int64_t(j) * L + l) * d * k;
-  const float* Bp = B_prev ? B_prev + int64_t(l) * d * k : nullptr;
   const float* Ql = Q + int64_t(l) * r * d;
-  for (int64_t i = threadIdx.x; i < d; i += KS_THREADS) {
-    if (!LOCA_CHECK_SPAN((int64_t(j) * L + l) * d * k + i * k, k, int64_t(gridDim.x) * L * d * k) ||
-        !LOCA_CHECK_SPAN((int64_t(l) * d + i) * k, k, int64_t(L) * d * k))
-      break;
-    float c[KM];
+  const int64_t per = (d + gridDim.x - 1) / gridDim.x;  // rows [rb, re) of this chunk
+  const int64_t rb = per * blockIdx.x, re = rb + per < d ? rb + per : d;
+#pragma unroll 1
+  for (int64_t i0 = rb + threadIdx.x; i0 < re; i0 += KS_THREADS * NR) {  // rows i0 + KS_THREADS * q
+    float c[NR][KM];
+    bool in[NR];
 #pragma unroll
-    for (int s = 0; s < KM; ++s) c[s] = 0.f;
-    for (int t = 0; t < r; ++t) {
-      const float qt = Ql[int64_t(t) * d + i];
+    for (int q = 0; q < NR; ++q) {
+      const int64_t i = i0 + KS_THREADS * q;
+      in[q] = i < re && LOCA_CHECK_SPAN((int64_t(j) * L + l) * d * k + i * k, k, int64_t(gridDim.y) * L * d * k) &&
+              LOCA_CHECK_SPAN((int64_t(l) * d + i) * k, k, int64_t(L) * d * k);
 #pragma unroll
-      for (int s = 0; s < KM; ++s) c[s] = fmaf(qt, W2[t][s], c[s]);
+      for (int s = 0; s < KM; ++s) c[q][s] = 0.f;
     }
-    if (Bp != nullptr) {
-      float b[KM];
+#pragma unroll 4
+    for (int t = 0; t < r; ++t) {
+      float qt[NR];
 #pragma unroll
-      for (int s = 0; s < KM; ++s) b[s] = (s < k) ? Bp[i * k + s] : 0.f;
+      for (int q = 0; q < NR; ++q) qt[q] = in[q] ? Ql[int64_t(t) * d + i0 + KS_THREADS * q] : 0.f;
+      add_scaled_row<KM, NR>(W2[t], qt, c);
+    }
+    if (B_prev != nullptr) {
+      const float* bp = B_prev + (int64_t(l) * d + i0) * k;
+#pragma unroll 4
+      for (int t = 0; t < k; ++t) {
+        float bt[NR];
 #pragma unroll
-      for (int s = 0; s < KM; ++s) {
-        float a = c[s];
-#pragma unroll
-        for (int t = 0; t < KM; ++t) a = fmaf(b[t], Gf[t][s], a);
-        c[s] = (s < k) ? a : 0.f;
+        for (int q = 0; q < NR; ++q) bt[q] = in[q] ? bp[int64_t(KS_THREADS) * q * k + t] : 0.f;
+        add_scaled_row<KM, NR>(Gf[t], bt, c);
       }
     }
-    if (C_out != nullptr && j == 0) {
 #pragma unroll
-      for (int s = 0; s < KM; ++s)
-        if (s < k) C_out[(int64_t(l) * d + i) * k + s] = c[s];
-    }
+    for (int q = 0; q < NR; ++q)
+      if (C_out != nullptr && j == 0 && in[q])
+        store_row<KM>(C_out + (int64_t(l) * d + i0 + KS_THREADS * q) * k, c[q], k, (vec & 2) != 0);
     if (inf != 0) {
 #pragma unroll
-      for (int s = 0; s < KM; ++s)
-        if (s < k) Bj[i * k + s] = 0.f;
-      continue;
-    }
-    chol_solve_row<KM>(Lf, Linv, c);
+      for (int q = 0; q < NR; ++q)
 #pragma unroll
-    for (int s = 0; s < KM; ++s)
-      if (s < k) Bj[i * k + s] = c[s];
+        for (int s = 0; s < KM; ++s) c[q][s] = 0.f;
+    } else {
+      chol_solve_rows<KM, NR>(Lf, Linv, c);
+    }
+#pragma unroll
+    for (int q = 0; q < NR; ++q)
+      if (in[q]) store_row<KM>(Bj + (i0 + KS_THREADS * q) * k, c[q], k, (vec & 1) != 0);
   }
 }
 
@@ -790,10 +870,13 @@ cudaError_t launch_kspace_accumulate(const void* X, int L, int64_t N, int64_t d,
   int32_t* abort_flag = reinterpret_cast<int32_t*>(ws + lay.flags);
   const int kp = kp_for(k);
   const int ntiles = int((N + XA_TM - 1) / XA_TM);
-  cudaError_t e = cudaMemsetAsync(abort_flag, 0, sizeof(int32_t), s);
-  if (e != cudaSuccess) return e;
-  k_kspace_prep<<<dim3(unsigned(L), PREP_SPLIT), PREP_THREADS, 0, s>>>(A, Q, d, k, kp, r, W, M);
-  e = cudaGetLastError();
+  const int nch_e = int((N + ETE_CHUNK - 1) / ETE_CHUNK);
+  const int nW = L * int((d + PREP_COLS - 1) / PREP_COLS);
+  const int rblk = (r + 1) / 2;
+  const int nM = (L * (rblk * (rblk + 1) / 2) + PREP_THREADS / 32 - 1) / (PREP_THREADS / 32);
+  k_kspace_prep<<<unsigned(nW + nM + nch_e), PREP_THREADS, 0, s>>>(A, Q, E, N, C, L, d, k, kp, r, nW, W, M, ete,
+                                                                  abort_flag);
+  cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   CUtensorMap tmX, tmW;
   if (!make_map3(&tmX, X, uint64_t(d), uint64_t(N), uint64_t(L), XA_TM) ||
@@ -816,10 +899,6 @@ cudaError_t launch_kspace_accumulate(const void* X, int L, int64_t N, int64_t d,
   }
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  const int nch_e = int((N + ETE_CHUNK - 1) / ETE_CHUNK);
-  k_kspace_ete<<<nch_e, ETE_THREADS, 0, s>>>(E, N, C, ete);
-  e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
   k_kspace_final<<<dim3(unsigned(L), FI_SPLIT), FI_THREADS, 0, s>>>(part, ete, nch_e, P, M, grid, ntiles, kp, k, C,
                                                                      r, eta, zero_first, G, SC, xsq_total, alpha_out);
   return cudaGetLastError();
@@ -831,16 +910,23 @@ cudaError_t launch_kspace_solve(const float* G, const float* SC, const double* x
                                 cudaStream_t s) {
   float v[16] = {};
   for (int i = 0; i < nl && i < 16; ++i) v[i] = lambda_rel[i];
-  const dim3 grid = dim3(unsigned(nl), unsigned(L));
-#define LOCA_KS(KM)                                                                                         \
-  k_kspace_solve<KM><<<grid, KS_THREADS, 0, s>>>(G, SC, xsq_total, P, Q, B_prev, d, k, C, r, L, v[0], v[1], \
-                                                 v[2], v[3], v[4], v[5], v[6], v[7], v[8], v[9], v[10], v[11], \
-                                                 v[12], v[13], v[14], v[15], B, info, C_out)
+  auto rows16 = [&](const void* p) { return k % 4 == 0 && reinterpret_cast<uintptr_t>(p) % 16 == 0; };
+  const int vec = (rows16(B) ? 1 : 0) | (rows16(C_out) ? 2 : 0);
+  int64_t chunks = (2 * int64_t(sm_count()) + int64_t(nl) * L - 1) / (int64_t(nl) * L);
+  if (chunks > (d + KS_THREADS - 1) / KS_THREADS) chunks = (d + KS_THREADS - 1) / KS_THREADS;
+  const dim3 grid = dim3(unsigned(chunks), unsigned(nl), unsigned(L));
+  const bool several = (d + chunks - 1) / chunks > KS_THREADS;  // more rows in a chunk than threads
+#define LOCA_KS1(KM, NR)                                                                                    \
+  k_kspace_solve<KM, NR><<<grid, KS_THREADS, 0, s>>>(G, SC, xsq_total, P, Q, B_prev, d, k, C, r, L, vec, v[0],   \
+                                                     v[1], v[2], v[3], v[4], v[5], v[6], v[7], v[8], v[9], v[10], \
+                                                     v[11], v[12], v[13], v[14], v[15], B, info, C_out)
+#define LOCA_KS(KM) (several ? LOCA_KS1(KM, chol_rows_per_thread(KM)) : LOCA_KS1(KM, 1))
   if (k <= 4) LOCA_KS(4);
   else if (k <= 8) LOCA_KS(8);
   else if (k <= 16) LOCA_KS(16);
   else LOCA_KS(32);
 #undef LOCA_KS
+#undef LOCA_KS1
   return cudaGetLastError();
 }
 

@@ -17,11 +17,10 @@
 //                 added in chunk order, lambda from the trace, Cholesky of G_l + lambda I in fp64
 //                 in shared memory; the fp32 factor, its diagonal reciprocals and G_l go to a
 //                 per-candidate record in the workspace.
-// k_chol_rows     one thread per row i of C_l = B_prev,l G_l + s_l CA_l (s_l = cross_scale[l], or 1),
-//                 solved by a forward and a back substitution against the staged factor:
+// k_chol_rows     two to four rows i of C_l = B_prev,l G_l + s_l CA_l (s_l = cross_scale[l], or 1) per
+//                 thread, solved by a forward and a back substitution against the staged factor:
 //                 B[j, l, i] = C_l[i] (G_l + lambda I)^-1.  k is padded to a compile-time size with
-//                 an identity block (its solution columns are zero), so each row stays in registers;
-//                 d / 128 x nl x L thread blocks keep the SMs busy.
+//                 an identity block (its solution columns are zero), so each row stays in registers.
 #include "chol.cuh"
 #include "loca_internal.h"
 
@@ -143,14 +142,16 @@ __global__ void __launch_bounds__(PR_THREADS, KM <= 16 ? 3 : 1) k_project_rows(c
 constexpr int CS_THREADS = 256;
 
 // Partial G_l = A_l^T GA_l over one chunk of rows: grid (nch, L); rows staged 128 at a time;
-// a thread owns a 2 x 2 block of entries (KM = 32) or one entry (KM <= 16), fp32 over the chunk.
+// a thread owns a 2 x 2 block of entries (KM = 32) or one entry (KM <= 16), fp32 over the chunk.  Bound by
+// the latency of staging, hence several CTAs per SM (with two and 4-byte loads, 114 us at L = 48, d = 5120,
+// k = 32, for 62 MB).
 constexpr int GP_THREADS = 256;
 constexpr int GP_ROWS = 128;
 constexpr int GP_MAX_CHUNKS = 32;
 
 template <int KM>
 __global__ void __launch_bounds__(GP_THREADS) k_chol_gram(const float* __restrict__ GA, int nsplit,
-                                                          const float* __restrict__ A, int64_t d, int k, int L,
+                                                          const float* __restrict__ A, int64_t d, int k, int L, int vec,
                                                           float* __restrict__ gpart) {
   __shared__ __align__(16) float As[GP_ROWS][KM];
   __shared__ __align__(16) float Gs[GP_ROWS][KM];
@@ -166,20 +167,38 @@ __global__ void __launch_bounds__(GP_THREADS) k_chol_gram(const float* __restric
   float g00 = 0.f, g01 = 0.f, g10 = 0.f, g11 = 0.f;
   for (int64_t i0 = r0; i0 < r1; i0 += GP_ROWS) {
     __syncthreads();
-    for (int e = tid; e < GP_ROWS * KM; e += GP_THREADS) {
-      const int ii = e / KM, s2 = e % KM;
-      const bool ok = (i0 + ii < r1) && s2 < k && LOCA_CHECK((i0 + ii) * k + s2, d * k);
-      As[ii][s2] = ok ? Al[(i0 + ii) * k + s2] : 0.f;
-      float gsum = 0.f;
-      if (ok)
-        for (int z = 0; z < nsplit; ++z) gsum += GAl[z * zs + (i0 + ii) * k + s2];
-      Gs[ii][s2] = gsum;
+    if (vec) {  // k % 4 == 0, 16-byte rows
+#pragma unroll
+      for (int e = tid; e < GP_ROWS * KM / 4; e += GP_THREADS) {
+        const int ii = e / (KM / 4), s4 = (e % (KM / 4)) * 4;
+        float4 a = make_float4(0.f, 0.f, 0.f, 0.f), g = a;
+        if (i0 + ii < r1 && s4 < k && LOCA_CHECK_SPAN((i0 + ii) * k + s4, 4, d * k)) {
+          a = __ldg(reinterpret_cast<const float4*>(Al + (i0 + ii) * k + s4));
+          for (int z = 0; z < nsplit; ++z) {
+            const float4 v = __ldg(reinterpret_cast<const float4*>(GAl + z * zs + (i0 + ii) * k + s4));
+            g.x += v.x, g.y += v.y, g.z += v.z, g.w += v.w;
+          }
+        }
+        *reinterpret_cast<float4*>(&As[ii][s4]) = a;
+        *reinterpret_cast<float4*>(&Gs[ii][s4]) = g;
+      }
+    } else {
+      for (int e = tid; e < GP_ROWS * KM; e += GP_THREADS) {
+        const int ii = e / KM, s2 = e % KM;
+        const bool ok = (i0 + ii < r1) && s2 < k && LOCA_CHECK((i0 + ii) * k + s2, d * k);
+        As[ii][s2] = ok ? Al[(i0 + ii) * k + s2] : 0.f;
+        float gsum = 0.f;
+        if (ok)
+          for (int z = 0; z < nsplit; ++z) gsum += GAl[z * zs + (i0 + ii) * k + s2];
+        Gs[ii][s2] = gsum;
+      }
     }
     __syncthreads();
     if (act) {
+      const int nr = r1 - i0 < GP_ROWS ? int(r1 - i0) : GP_ROWS;
       if constexpr (kBlk) {
 #pragma unroll 8
-        for (int ii = 0; ii < GP_ROWS; ++ii) {
+        for (int ii = 0; ii < nr; ++ii) {
           const float2 av = *reinterpret_cast<const float2*>(&As[ii][a0]);
           const float2 gv = *reinterpret_cast<const float2*>(&Gs[ii][b0]);
           g00 = fmaf(av.x, gv.x, g00);
@@ -189,7 +208,7 @@ __global__ void __launch_bounds__(GP_THREADS) k_chol_gram(const float* __restric
         }
       } else {
 #pragma unroll 8
-        for (int ii = 0; ii < GP_ROWS; ++ii) g00 = fmaf(As[ii][a0], Gs[ii][b0], g00);
+        for (int ii = 0; ii < nr; ++ii) g00 = fmaf(As[ii][a0], Gs[ii][b0], g00);
       }
     }
   }
@@ -218,15 +237,15 @@ __global__ void __launch_bounds__(CS_THREADS) k_chol_factor(
     int32_t* __restrict__ info, float* __restrict__ G_out, float* __restrict__ fac) {
   __shared__ float Gf[KM][KM];   // G_l (fp32, symmetrised), padded with identity
   __shared__ double Md[KM][KM];  // G_l + lambda I, then its Cholesky factor (lower)
-  __shared__ float Lf[KM][KM];
+  __shared__ __align__(16) float Lf[KM][KM];
   __shared__ float Linv[KM];
-  __shared__ int s_info;
   const int j = blockIdx.x, l = blockIdx.y;
   const float lam_rel[16] = {l0, l1, l2, l3, l4, l5, l6, l7, l8, l9, l10, l11, l12, l13, l14, l15};
   // G_l = A_l^T GA_l from the row chunks' partial products, summed in a fixed order in fp64
   const float* gp = gpart + int64_t(l) * nch * KM * KM;
   for (int e = threadIdx.x; e < KM * KM; e += CS_THREADS) {
     double acc = 0.0;
+#pragma unroll 8
     for (int c = 0; c < nch; ++c) acc += double(gp[int64_t(c) * KM * KM + e]);
     Gf[e / KM][e % KM] = float(acc);
   }
@@ -252,7 +271,7 @@ __global__ void __launch_bounds__(CS_THREADS) k_chol_factor(
         G_out[(int64_t(l) * k + a) * k + b] = float(0.5 * (double(Gf[a][b]) + double(Gf[b][a])));
     }
   }
-  const int inf = chol_factor<KM>(Md, Lf, Linv, &s_info);
+  const int inf = chol_factor<KM>(Md, Lf, Linv, k);
   if (threadIdx.x == 0 && LOCA_CHECK(int64_t(j) * L + l, int64_t(gridDim.x) * L)) info[int64_t(j) * L + l] = inf;
 
   float* f = fac + (int64_t(j) * L + l) * fac_floats<KM>();
@@ -264,24 +283,26 @@ __global__ void __launch_bounds__(CS_THREADS) k_chol_factor(
   for (int a = threadIdx.x; a < KM; a += CS_THREADS) f[KM * KM + a] = Linv[a];
 }
 
-// Rows of B for one (ridge candidate j, block l): thread per row i,
+// Rows of B for one (ridge candidate j, block l), NR rows per thread:
 //   c = s_l CA_l[i] (+ B_prev,l[i] G_l),  B[j, l, i] = c (L L^T)^-1
-// with the candidate's factor staged in shared memory (broadcast reads); C_out = c for j = 0.
+// with the candidate's factor staged in shared memory (broadcast reads); C_out = c for j = 0.  vec: bits
+// for 16-byte rows of CA (1), B (4) and C_out (8).  One row per thread and scalar reads of the
+// factor spilled at KM = 32 (684 us at L = 48, d = 5120, three candidates).
 constexpr int CR_THREADS = 128;
 
-template <int KM>
+template <int KM, int NR>
 __global__ void __launch_bounds__(CR_THREADS) k_chol_rows(
     const float* __restrict__ CA, int nsplit, const float* __restrict__ B_prev, const float* __restrict__ cross_scale,
-    int64_t d, int k, int L, const int32_t* __restrict__ info, const float* __restrict__ fac, float* __restrict__ B,
-    float* __restrict__ C_out) {
-  __shared__ float Lf[KM][KM];
+    int64_t d, int k, int L, int vec, const int32_t* __restrict__ info, const float* __restrict__ fac,
+    float* __restrict__ B, float* __restrict__ C_out) {
+  __shared__ __align__(16) float Lf[KM][KM];
   __shared__ float Linv[KM];
-  __shared__ float Gf[KM][KM];
+  __shared__ __align__(16) float Gf[KM][KM];
   const int j = blockIdx.y, l = blockIdx.z;
   const float* f = fac + (int64_t(j) * L + l) * fac_floats<KM>();
   for (int e = threadIdx.x; e < KM * KM; e += CR_THREADS) {
     Lf[e / KM][e % KM] = f[e];
-    Gf[e / KM][e % KM] = f[KM * KM + KM + e];
+    if (B_prev != nullptr) Gf[e / KM][e % KM] = f[KM * KM + KM + e];
   }
   for (int a = threadIdx.x; a < KM; a += CR_THREADS) Linv[a] = f[KM * KM + a];
   __syncthreads();
@@ -289,48 +310,48 @@ __global__ void __launch_bounds__(CR_THREADS) k_chol_rows(
   const int64_t zs = int64_t(L) * d * k;  // stride between the nsplit partial products
   const float cs = cross_scale != nullptr ? cross_scale[l] : 1.f;
   float* Bj = B + (int64_t(j) * L + l) * d * k;
-  const int64_t i = int64_t(blockIdx.x) * CR_THREADS + threadIdx.x;
-  if (i >= d) return;
-  if (!LOCA_CHECK_SPAN((int64_t(l) * d + i) * k, k, int64_t(L) * d * k) ||
-      !LOCA_CHECK_SPAN((int64_t(j) * L + l) * d * k + i * k, k, int64_t(gridDim.y) * L * d * k))
-    return;
-  const float* cz = CA + (int64_t(l) * d + i) * k;
-  float c[KM];
+  const int64_t i0 = int64_t(blockIdx.x) * (CR_THREADS * NR) + threadIdx.x;  // rows i0 + CR_THREADS * q
+  if (i0 >= d) return;
+  float c[NR][KM];
+  bool in[NR];
 #pragma unroll
-  for (int s2 = 0; s2 < KM; ++s2) c[s2] = 0.f;
-  for (int z = 0; z < nsplit; ++z) {
+  for (int q = 0; q < NR; ++q) {
+    const int64_t i = i0 + CR_THREADS * q;
+    in[q] = i < d && LOCA_CHECK_SPAN((int64_t(l) * d + i) * k, k, int64_t(L) * d * k) &&
+            LOCA_CHECK_SPAN((int64_t(j) * L + l) * d * k + i * k, k, int64_t(gridDim.y) * L * d * k);
 #pragma unroll
-    for (int s2 = 0; s2 < KM; ++s2)
-      if (s2 < k) c[s2] += cz[z * zs + s2];
+    for (int s2 = 0; s2 < KM; ++s2) c[q][s2] = 0.f;
+    if (in[q])
+      for (int z = 0; z < nsplit; ++z) add_row<KM>(CA + z * zs + (int64_t(l) * d + i) * k, c[q], k, (vec & 1) != 0);
+#pragma unroll
+    for (int s2 = 0; s2 < KM; ++s2) c[q][s2] *= cs;
   }
-#pragma unroll
-  for (int s2 = 0; s2 < KM; ++s2) c[s2] *= cs;
   if (B_prev != nullptr) {
-    // c += B_prev,l[i] G_l, one entry of the B_prev row at a time (only c stays in registers)
-    const float* bp = B_prev + (int64_t(l) * d + i) * k;
+    // c += B_prev,l[i] G_l, one entry of the B_prev rows at a time (only c stays in registers)
+    const float* bp = B_prev + (int64_t(l) * d + i0) * k;
 #pragma unroll 4
     for (int t = 0; t < k; ++t) {
-      const float bt = bp[t];
+      float bt[NR];
 #pragma unroll
-      for (int s2 = 0; s2 < KM; ++s2) c[s2] = fmaf(bt, Gf[t][s2], c[s2]);
+      for (int q = 0; q < NR; ++q) bt[q] = in[q] ? bp[int64_t(CR_THREADS) * q * k + t] : 0.f;
+      add_scaled_row<KM, NR>(Gf[t], bt, c);
     }
   }
-  if (C_out != nullptr && j == 0) {
 #pragma unroll
-    for (int s2 = 0; s2 < KM; ++s2)
-      if (s2 < k) C_out[(int64_t(l) * d + i) * k + s2] = c[s2];
-  }
-  float* bj = Bj + i * k;
+  for (int q = 0; q < NR; ++q)
+    if (C_out != nullptr && j == 0 && in[q])
+      store_row<KM>(C_out + (int64_t(l) * d + i0 + CR_THREADS * q) * k, c[q], k, (vec & 8) != 0);
   if (inf != 0) {
 #pragma unroll
-    for (int s2 = 0; s2 < KM; ++s2)
-      if (s2 < k) bj[s2] = 0.f;
-    return;
-  }
-  chol_solve_row<KM>(Lf, Linv, c);
+    for (int q = 0; q < NR; ++q)
 #pragma unroll
-  for (int s2 = 0; s2 < KM; ++s2)
-    if (s2 < k) bj[s2] = c[s2];
+      for (int s2 = 0; s2 < KM; ++s2) c[q][s2] = 0.f;
+  } else {
+    chol_solve_rows<KM, NR>(Lf, Linv, c);
+  }
+#pragma unroll
+  for (int q = 0; q < NR; ++q)
+    if (in[q]) store_row<KM>(Bj + (i0 + CR_THREADS * q) * k, c[q], k, (vec & 4) != 0);
 }
 
 template <int KM>
@@ -352,12 +373,14 @@ cudaError_t solve_t(const float* GA, const float* CA, int nsplit, const float* A
   float v[16] = {};
   for (int i = 0; i < nl && i < 16; ++i) v[i] = lr[i];
   float* gpart = fac + size_t(16) * size_t(L) * size_t(fac_floats<32>());
-  int64_t nch = (int64_t(sm_count()) * 2 + L - 1) / L;  // two chunk CTAs per SM over the blocks
+  int64_t nch = (int64_t(sm_count()) * 4 + L - 1) / L;  // four chunk CTAs per SM over the blocks
   const int64_t maxch = (d + GP_ROWS - 1) / GP_ROWS;
   if (nch > maxch) nch = maxch;
   if (nch > GP_MAX_CHUNKS) nch = GP_MAX_CHUNKS;
   if (nch < 1) nch = 1;
-  k_chol_gram<KM><<<dim3(unsigned(nch), unsigned(L)), GP_THREADS, 0, s>>>(GA, nsplit, A, d, k, L, gpart);
+  auto rows16 = [&](const void* p) { return k % 4 == 0 && reinterpret_cast<uintptr_t>(p) % 16 == 0; };
+  k_chol_gram<KM><<<dim3(unsigned(nch), unsigned(L)), GP_THREADS, 0, s>>>(GA, nsplit, A, d, k, L,
+                                                                         rows16(GA) && rows16(A), gpart);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   k_chol_factor<KM><<<dim3(unsigned(nl), unsigned(L)), CS_THREADS, 0, s>>>(
@@ -365,9 +388,16 @@ cudaError_t solve_t(const float* GA, const float* CA, int nsplit, const float* A
       v[12], v[13], v[14], v[15], info, G_out, fac);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  const int64_t rows_per_cta = CR_THREADS;
-  const dim3 grid = dim3(unsigned((d + rows_per_cta - 1) / rows_per_cta), unsigned(nl), unsigned(L));
-  k_chol_rows<KM><<<grid, CR_THREADS, 0, s>>>(CA, nsplit, B_prev, cross_scale, d, k, L, info, fac, B, C_out);
+  const int vec = (rows16(CA) ? 1 : 0) | (rows16(B) ? 4 : 0) | (rows16(C_out) ? 8 : 0);
+  // several rows per thread share the reads of the factor; one where that would leave SMs without a CTA
+  constexpr int NR = chol_rows_per_thread(KM);
+  auto ctas = [&](int nr) { return (d + CR_THREADS * nr - 1) / (CR_THREADS * nr); };
+  if (ctas(NR) * nl * L >= 2 * sm_count())
+    k_chol_rows<KM, NR><<<dim3(unsigned(ctas(NR)), unsigned(nl), unsigned(L)), CR_THREADS, 0, s>>>(
+        CA, nsplit, B_prev, cross_scale, d, k, L, vec, info, fac, B, C_out);
+  else
+    k_chol_rows<KM, 1><<<dim3(unsigned(ctas(1)), unsigned(nl), unsigned(L)), CR_THREADS, 0, s>>>(
+        CA, nsplit, B_prev, cross_scale, d, k, L, vec, info, fac, B, C_out);
   return cudaGetLastError();
 }
 

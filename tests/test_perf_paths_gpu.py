@@ -159,3 +159,111 @@ def test_wide_calibration_paths(lc, Np, m, d, L, r, ell, q):
         assert _rel(_np(P[l]) @ _np(Q[l]), P_ref[l] @ Q_ref[l]) <= 1e-5
     assert _rel(_np(sigma), s_ref) <= 1e-5
     assert np.max(np.abs(_np(alpha) - O.alignment(E, _np(P), _np(Q), G))) <= 1e-5
+
+
+@pytest.mark.parametrize("L,N,d,k,C,r,nl", [
+    (1, 100, 64, 1, 1, 1, 1),        # one tile on one CTA
+    (3, 130, 136, 5, 3, 7, 2),       # two tiles a block, fewer tiles than CTAs, ranks off 4
+    (2, 40000, 72, 16, 16, 32, 3),   # a block's tiles on half the CTAs each
+    (7, 5000, 264, 32, 2, 17, 16),   # runs that cross block borders, 2 x 2 entry blocks
+    (5, 3000, 520, 20, 4, 8, 1),     # k padded to 32
+])
+def test_kspace_tile_ranges(lc, L, N, d, k, C, r, nl):
+    """Statistics and solves of two mini-batches whatever the tiles' distribution over the CTAs: A in two
+    bf16 parts (2^-16 of each entry, random signs), fp32 tile sums: 3e-5; the fp32 substitutions of a
+    system with condition number up to 1 / lambda_rel: the same against their own statistics."""
+    rng = np.random.default_rng(N + k)
+    A = np.linalg.qr(rng.standard_normal((L, d, k)))[0].astype(np.float32)
+    P = rng.standard_normal((L, C, r)).astype(np.float32)
+    Q = rng.standard_normal((L, r, d)).astype(np.float32)
+    Bp = (0.1 * rng.standard_normal((L, d, k))).astype(np.float32)
+    G, SC = torch.empty((L, k, k), device="cuda"), torch.empty((L, C, k), device="cuda")
+    xsq, alpha = torch.empty((L,), dtype=torch.float64, device="cuda"), torch.empty((L,), device="cuda")
+    g_ref, s_ref, x_ref = np.zeros((L, k, k)), np.zeros((L, C, k)), np.zeros(L)
+    for b in range(2):
+        X = torch.from_numpy(rng.standard_normal((L, N, d)).astype(np.float32)).to(torch.bfloat16)
+        E = rng.standard_normal((N, C)).astype(np.float32)
+        lc.loca_kspace_accumulate(X.to("cuda"), _dev(A), _dev(E), _dev(P), _dev(Q), 0.01, G, SC, xsq, zero_first=b == 0,
+                                  alpha=alpha)
+        for l in range(L):
+            x, p = X[l].double().numpy(), X[l].double().numpy() @ A[l].astype(np.float64)
+            M = Q[l].astype(np.float64) @ Q[l].astype(np.float64).T
+            U = E.astype(np.float64) @ P[l]
+            step = -0.01 * np.sqrt(np.sum(x * x) / np.sum((U @ M) * U))
+            assert abs(float(alpha[l]) - step) <= 1e-6 * abs(step)
+            g_ref[l] += p.T @ p
+            s_ref[l] += step * (E.astype(np.float64).T @ p)
+            x_ref[l] += np.sum(x * x)
+    lam = [10.0 ** -(1 + i % 3) for i in range(nl)]
+    B, info = torch.empty((nl, L, d, k), device="cuda"), torch.empty((nl, L), dtype=torch.int32, device="cuda")
+    C_out = torch.empty((L, d, k), device="cuda")
+    lc.loca_kspace_solve(G, SC, _dev(P), _dev(Q), lam, B, info, xsq_total=xsq, B_prev=_dev(Bp), C_out=C_out)
+    torch.cuda.synchronize()
+    assert lc.loca_device_status() == 0 and int(info.abs().sum()) == 0
+    assert _rel(_np(G), g_ref) <= 3e-5 and _rel(_np(SC), s_ref) <= 3e-5
+    assert np.allclose(_np(xsq), x_ref, rtol=1e-6, atol=0)
+    assert torch.equal(G, G.transpose(1, 2))
+    for l in range(L):
+        c = Bp[l].astype(np.float64) @ _np(G[l]) + Q[l].astype(np.float64).T @ (P[l].astype(np.float64).T @ _np(SC[l]))
+        assert _rel(_np(C_out[l]), c) <= 1e-5
+        for j in range(nl):
+            m = _np(G[l]) + np.float32(lam[j]) * _np(xsq)[l] / d * np.eye(k)
+            assert _rel(_np(B[j, l]), np.linalg.solve(m, c.T).T) <= 3e-5
+
+
+@pytest.mark.parametrize("k", [1, 3, 4, 7, 8, 13, 16, 17, 24, 32])
+def test_ridge_solve_ranks(lc, k):
+    """The row solves at every padding of k (two to four rows a thread, 16-byte and scalar rows), rows
+    beyond the last whole CTA, B_prev and C_out; one system that is not positive definite."""
+    L, d, nl = 3, 308, 2
+    rng = np.random.default_rng(k)
+    gram = np.stack([(lambda x: x.T @ x)(rng.standard_normal((400, d))) for _ in range(L)]).astype(np.float32)
+    gram[2] = -gram[2]
+    cross = rng.standard_normal((L, d, d)).astype(np.float32)
+    A = np.linalg.qr(rng.standard_normal((L, d, k)))[0].astype(np.float32)
+    Bp = (0.1 * rng.standard_normal((L, d, k))).astype(np.float32)
+    B, info = torch.empty((nl, L, d, k), device="cuda"), torch.empty((nl, L), dtype=torch.int32, device="cuda")
+    G, C_out = torch.empty((L, k, k), device="cuda"), torch.empty((L, d, k), device="cuda")
+    lc.loca_ridge_solve(_dev(gram), _dev(cross), _dev(A), [1.0, 30.0], B, info, B_prev=_dev(Bp), G_out=G, C_out=C_out)
+    torch.cuda.synchronize()
+    assert lc.loca_device_status() == 0
+    assert info.cpu().tolist() == [[0, 0, 1]] * nl and float(B[:, 2].abs().sum()) == 0.0
+    for l in range(2):
+        g = A[l].astype(np.float64).T @ gram[l].astype(np.float64) @ A[l]
+        c = Bp[l].astype(np.float64) @ g + cross[l].astype(np.float64) @ A[l]
+        assert _rel(_np(G[l]), g) <= 1e-5 and _rel(_np(C_out[l]), c) <= 1e-5
+        for j, lam in enumerate((1.0, 30.0)):
+            assert _rel(_np(B[j, l]), np.linalg.solve(g + lam * np.eye(k), c.T).T) <= 1e-5
+
+
+@pytest.mark.parametrize("N,V,C,dtype", [(1, 1, 1, "f32"), (257, 32, 32, "bf16"), (1000, 33, 5, "f32"), (513, 7, 3, "f32"),
+                                         (300, 32, 4, "bf16")])
+@pytest.mark.parametrize("normaliser", [0, 1])
+def test_head_error_short_rows(lc, N, V, C, dtype, normaliser):
+    """One thread per row up to V = 32, one warp above; masked labels, weights, a row pitch beyond V and
+    spread-out logits.  z, the maximum and lse are fp32 numbers of up to zmax, each rounded a few times
+    (base-2 units and back), so z - lse and with it every exponential is off by up to 4 * 2^-24 zmax
+    relative (1.3e-5 at zmax = 54); absolute floor 2e-6 of a weight up to 2 (the label entry cancels)."""
+    rng = np.random.default_rng(V + C)
+    pitch = V + 3
+    full = (rng.standard_normal((N, pitch)) * 12).astype(np.float32)
+    if dtype == "bf16":
+        full = torch.from_numpy(full).to(torch.bfloat16).float().numpy()
+    z = _dev(full, torch.float32 if dtype == "f32" else torch.bfloat16)[:, :V]
+    cols = rng.permutation(V)[:C].astype(np.int32)
+    y = rng.integers(-1, C, N).astype(np.int32)
+    w = rng.uniform(0, 2, N).astype(np.float32)
+    E, ce = torch.empty((N, C), device="cuda"), torch.empty((N,), device="cuda")
+    lc.loca_error(z, _dev(cols, torch.int32), _dev(y, torch.int32), E, w=_dev(w), ce=ce, normaliser=normaliser)
+    zz = full[:, :V].astype(np.float64)
+    zn = zz if normaliser == 0 else zz[:, cols]
+    m = zn.max(1, keepdims=True)
+    lse = m[:, 0] + np.log(np.exp(zn - m).sum(1))
+    wn = np.where(y < 0, 0.0, w)
+    onehot = (np.arange(C)[None] == y[:, None]).astype(np.float64)
+    e_ref = wn[:, None] * (np.exp(zz[:, cols] - lse[:, None]) - onehot)
+    ce_ref = np.where(y < 0, 0.0, wn * (lse - zz[np.arange(N), cols[np.maximum(y, 0)]]))
+    rel = 4 * 2.0 ** -24 * max(1.0, float(np.abs(zz).max())) + 1e-6
+    p_ref = wn[:, None] * np.exp(zz[:, cols] - lse[:, None])  # before the label entry cancels
+    assert np.all(np.abs(_np(E) - e_ref) <= rel * p_ref + 2e-6)
+    assert np.all(np.abs(_np(ce) - ce_ref) <= rel * (1 + np.abs(ce_ref)))
