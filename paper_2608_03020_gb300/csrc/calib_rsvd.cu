@@ -72,27 +72,30 @@ __device__ __forceinline__ void load_tile(double (*S)[NBP], const double* __rest
 
 // Diagonal tile jb: factor in shared memory (unblocked, right-looking), write the factor back,
 // and write the inverse of the triangular factor to Dinv[jb].  A pivot that is not positive
-// sets the failure flag (E^T E + beta I is not positive definite in floating point).  Thread
-// (ty, tx) of the 16 x 16 grid owns entries (ty + 16 p, tx + 16 q).  Every thread scales the entries
-// of the pivot's column that it needs itself, so a step has one barrier; bound by the latency of the
-// 64 + 64 steps in a row (with a scaling phase of its own, a division and a square root per step,
-// 162 us; one tile per 64 columns of K, nothing else runs beside it).
+// sets the failure flag (E^T E + beta I is not positive definite in floating point).  One CTA, nothing
+// else beside it, so the fp64 pipe of one SM (2 FMAs per clock, predicated-off lanes included) and the
+// latency of the 64 + 64 steps bound it: the trailing entries of a step are dealt out one by one, two
+// rows of the triangle folded into one of constant length.  A 16 x 16 grid of threads that owned fixed
+// entries spent most of the pipe on entries outside the triangle (161 us a tile).
 __global__ void __launch_bounds__(256) k_cr_potrf(double* __restrict__ K, int64_t mp, int jb,
                                                  double* __restrict__ Dinv, int32_t* flag) {
   extern __shared__ __align__(16) unsigned char cr_smem[];
   double(*S)[NBP] = reinterpret_cast<double(*)[NBP]>(cr_smem);
   double(*X)[NBP] = reinterpret_cast<double(*)[NBP]>(cr_smem + sizeof(double) * NB * NBP);
-  __shared__ double rinv[NB];
+  __shared__ double rinv[NB], col[NB];
   if (failed(flag)) return;
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  const int tid = threadIdx.x;
   const int64_t o = int64_t(jb) * NB;
   double* Kd = K + o * mp + o;
   for (int e = tid; e < NB * NB; e += 256) {
     const int r = e / NB, c = e % NB;
     S[r][c] = (c <= r) ? Kd[int64_t(r) * mp + c] : 0.0;
-    X[r][c] = 0.0;
+    X[r][c] = (r == c) ? 1.0 : 0.0;
   }
   __syncthreads();
+  // e / n for e * n < 2^20
+  auto divide = [](int e, uint32_t magic) { return int((uint32_t(e) * magic) >> 20); };
+  auto magic_of = [](int n) { return ((1u << 20) + uint32_t(n) - 1u) / uint32_t(n); };
   for (int c = 0; c < NB; ++c) {
     const double piv = S[c][c];
     if (!(piv > 0.0)) {  // the same value in every thread
@@ -100,53 +103,44 @@ __global__ void __launch_bounds__(256) k_cr_potrf(double* __restrict__ K, int64_
       return;
     }
     const double inv = rsqrt(piv);
-    double lc[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) lc[q] = S[tx + 16 * q][c] * inv;
-#pragma unroll
-    for (int p = 0; p < 4; ++p) {
-      const int rr = ty + 16 * p;
-      if (rr <= c) continue;
-      const double lrc = S[rr][c] * inv;
-      if (tx == 0) X[rr][c] = lrc;  // the factor collects in X: column c of S is still being read
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int ss = tx + 16 * q;
-        if (ss > c && ss <= rr) S[rr][ss] = fma(-lrc, lc[q], S[rr][ss]);
-      }
+    if (tid < NB && tid > c) {
+      const double v = S[tid][c] * inv;
+      col[tid] = v;
+      Kd[int64_t(tid) * mp + c] = v;
     }
-    if (tid == 0) {
-      X[c][c] = piv * inv;
+    if (tid == c) {
+      Kd[int64_t(c) * mp + c] = piv * inv;
       rinv[c] = inv;
     }
     __syncthreads();
+    // rows c + 1 + i, i < rem, with i + 1 entries each: rows i and rem - 1 - i side by side
+    const int rem = NB - 1 - c, width = rem + 1;
+    const uint32_t mg = magic_of(width);
+    for (int e = tid; e < (rem + 1) / 2 * width; e += 256) {
+      int i = divide(e, mg), j = e - i * width;
+      if (j > i) {
+        if (rem - 1 - i == i) continue;  // the middle row stands alone
+        j -= i + 1;
+        i = rem - 1 - i;
+      }
+      S[c + 1 + i][c + 1 + j] = fma(-col[c + 1 + i], col[c + 1 + j], S[c + 1 + i][c + 1 + j]);
+    }
+    if (tid < rem) S[c + 1 + tid][c] = col[c + 1 + tid];  // column c of the factor
+    __syncthreads();
   }
-  for (int e = tid; e < NB * NB; e += 256) {
-    const int r = e / NB, c = e % NB;
-    if (c <= r) Kd[int64_t(r) * mp + c] = X[r][c];
-    S[r][c] = (r == c) ? 1.0 : 0.0;
-  }
-  __syncthreads();
-  // S = L^-1, right-looking on the identity: row c scaled by 1 / L_cc (by its readers; stored by the
-  // threads of its own row one step later, when nobody reads it), then removed from the rows below
+  // X = L^-1, right-looking on the identity: row c scaled by 1 / L_cc, then removed from the rows below
   for (int c = 0; c < NB; ++c) {
-    const double rc = rinv[c];
-    double xc[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) xc[q] = S[c][tx + 16 * q] * rc;
-#pragma unroll
-    for (int p = 0; p < 4; ++p) {
-      const int rr = ty + 16 * p;
-      if (rr <= c) continue;
-      const double lrc = X[rr][c];
-#pragma unroll
-      for (int q = 0; q < 4; ++q)
-        if (tx + 16 * q <= c) S[rr][tx + 16 * q] = fma(-lrc, xc[q], S[rr][tx + 16 * q]);
+    if (tid <= c) X[c][tid] *= rinv[c];
+    __syncthreads();
+    const uint32_t mg = magic_of(c + 1);
+    for (int e = tid; e < (NB - 1 - c) * (c + 1); e += 256) {
+      const int i = divide(e, mg), u = e - i * (c + 1);
+      X[c + 1 + i][u] = fma(-S[c + 1 + i][c], X[c][u], X[c + 1 + i][u]);
     }
     __syncthreads();
   }
   double* D = Dinv + int64_t(jb) * NB * NB;
-  for (int e = tid; e < NB * NB; e += 256) D[e] = S[e / NB][e % NB] * rinv[e / NB];
+  for (int e = tid; e < NB * NB; e += 256) D[e] = X[e / NB][e % NB];
 }
 
 constexpr int CT = 32;         // tile of the panel and trailing updates
@@ -779,14 +773,19 @@ RsvdWs rsvd_ws(int64_t Np, int64_t m, int64_t d, int L, int ell, int r) {
   return w;
 }
 
-// C_b(i, j) = sum_t A_b(i, t) B_b(t, j) (run_gemm.cuh).  32-column tiles where N is
-// one block's ell <= 32 columns.
+// C_b(i, j) = sum_t A_b(i, t) B_b(t, j) (run_gemm.cuh).  32-column tiles where N is one block's ell <= 32
+// columns.
 template <bool AT, typename TC>
 cudaError_t gemm(const float* A, int64_t lda, int64_t sA, const float* B, int64_t ldb, int64_t sB, TC* C,
                  int64_t ldc, int64_t sC, int64_t M, int64_t N, int64_t Kc, int batch, int lower_only,
                  cudaStream_t s) {
   const RunGemmArgs g{A, B, C, lda, sA, ldb, sB, ldc, sC, M, N, Kc, 0, lower_only};
-  return N <= 32 ? run_gemm<AT, TC, 128, 32>(g, batch, s) : run_gemm<AT, TC, 128, 64>(g, batch, s);
+  return N <= 32 ? run_gemm<AT, TC, 128, 32>(g, batch, s) : run_gemm<AT, TC, 64, 64>(g, batch, s);
+}
+
+__global__ void k_cr_add(double* __restrict__ x, const double* __restrict__ y, int64_t count) {
+  for (int64_t e = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; e < count; e += int64_t(gridDim.x) * blockDim.x)
+    x[e] += y[e];
 }
 
 // Zd[j][l ell + s] = sum_n Tn[n][l ell + s] G_l[n][j] (G_l^T Tn for every block): a warp streams rows of G_l
@@ -965,7 +964,15 @@ cudaError_t rsvd_t(const float* E, const float* G, int64_t Np, int64_t m, int64_
   // an fp32 copy)
   auto apply_Ft = [&](const float* Xf, int64_t ldx, int64_t sx, bool exact) -> cudaError_t {
     CR_TRY((gemm<false, float>(G, d, Np * d, Xf, ldx, sx, Tn, n, ell, Np, ell, d, L, 0, s)));
-    CR_TRY((gemm<true, double>(E, m, 0, Tn, n, 0, Ym, n, 0, m, n, Np, 1, 0, s)));
+    // E^T Tn: two halves of the tokens when the tiles are fewer than six a SM (a last wave of few long
+    // tiles costs more than the addition)
+    const int64_t half = (m + 63) / 64 * ((n + 63) / 64) < 6 * sm_count() && Np >= 1024 ? (Np / 2 + 31) / 32 * 32 : Np;
+    CR_TRY((gemm<true, double>(E, m, 0, Tn, n, 0, Ym, n, 0, m, n, half, 1, 0, s)));
+    if (half < Np) {
+      CR_TRY((gemm<true, double>(E + half * m, m, 0, Tn + half * n, n, 0, Wm, n, 0, m, n, Np - half, 1, 0, s)));
+      k_cr_add<<<2 * sm_count(), 256, 0, s>>>(Ym, Wm, m * n);
+      CR_TRY(cudaGetLastError());
+    }
     if (exact) return solve<double>(K, mp, Dinv, Ym, n, flag, s);
     CR_TRY((cvt<double, float>(Ym, Wf, mp * n, s)));
     CR_TRY(solve<float>(Kf, mp, Dinvf, Wf, n, flag, s));

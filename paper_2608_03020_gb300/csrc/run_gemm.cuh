@@ -4,9 +4,10 @@
 //
 //   C_b(i, j) = sum_t A_b(i, t) B_b(t, j),  A_b(i, t) = A[t lda + i] (AT) or A[i lda + t]
 //
-// One BM x BN tile per CTA of 256 threads; a thread owns BM BN / 256 outputs, pairs of rows packed
-// for fma.rn.f32x2 (a run of a pair is one register pair: the row operand comes from shared memory
-// already paired, the column operand is duplicated once for BM / 32 packed FMAs).  The next 32-term
+// One BM x BN tile per CTA; a thread owns 8 x 4 outputs, pairs of rows packed for fma.rn.f32x2 (the row
+// operand comes from shared memory already paired, the column operand is duplicated once for 4 packed
+// FMAs).  128 threads a CTA (4096-output tiles), so that three CTAs share an SM at ~160 registers: one of
+// 256 threads left the fp32 pipe idle at every barrier (29 TFLOP/s).  The next 32-term
 // slab is loaded into registers while the current one is multiplied (two shared buffers, one
 // barrier per slab).  Bound by the fp32 pipe.  At 64 x 64 tiles of 4 x 4 outputs with scalar FMAs and
 // fp64 adds the same products ran at 16 TFLOP/s, half of each tile idle where N is one block's 32
@@ -32,9 +33,10 @@ struct RunGemmArgs {
 };
 
 template <bool AT, typename TC, int BM, int BN>
-__global__ void __launch_bounds__(256) k_run_gemm(RunGemmArgs g) {
-  constexpr int TN = BN / 4;            // threads along the columns (4 each)
-  constexpr int RPT = BM * TN / 256;    // rows per thread
+__global__ void __launch_bounds__(BM * BN / 32) k_run_gemm(RunGemmArgs g) {
+  constexpr int NT = BM * BN / 32;      // threads
+  constexpr int TN = BN / 4;            // of them along the columns (4 each)
+  constexpr int RPT = 8;                // rows per thread
   constexpr int NG = RPT / 4;           // groups of 4 consecutive rows
   constexpr int LDA = BM + 4;
   __shared__ __align__(16) float As[2][RG_BK][LDA];
@@ -46,7 +48,7 @@ __global__ void __launch_bounds__(256) k_run_gemm(RunGemmArgs g) {
   const float* B = g.B + (g.bw ? 0 : int64_t(blockIdx.y) * g.sB);
   TC* C = static_cast<TC*>(g.C) + (g.bw ? 0 : int64_t(blockIdx.y) * g.sC);
   const int tid = threadIdx.x, tx = tid % TN, ty = tid / TN;
-  constexpr int AV = BM * RG_BK / 4 / 256, BV = (BN * RG_BK / 4 + 255) / 256;  // float4 per thread and slab
+  constexpr int AV = BM * RG_BK / 4 / NT, BV = BN * RG_BK / 4 / NT;  // float4 per thread and slab
   const bool avec = g.lda % 4 == 0 && (reinterpret_cast<uintptr_t>(A) & 15) == 0;
   const bool bvec = g.ldb % 4 == 0 && (reinterpret_cast<uintptr_t>(B) & 15) == 0 && (g.bw % 4 == 0) && g.sB % 4 == 0;
   float4 ra[AV], rb[BV];
@@ -63,7 +65,7 @@ __global__ void __launch_bounds__(256) k_run_gemm(RunGemmArgs g) {
   auto gload = [&](int64_t t0) {
 #pragma unroll
     for (int q = 0; q < AV; ++q) {
-      const int e = tid + 256 * q;
+      const int e = tid + NT * q;
       if constexpr (AT) {
         const int t = e / (BM / 4), i = (e % (BM / 4)) * 4;
         ra[q] = load4(A + (t0 + t) * g.lda + i0 + i, t0 + t < g.K ? left(g.M - i0 - i) : 0, avec);
@@ -74,10 +76,10 @@ __global__ void __launch_bounds__(256) k_run_gemm(RunGemmArgs g) {
     }
 #pragma unroll
     for (int q = 0; q < BV; ++q) {
-      const int e = tid + 256 * q;
+      const int e = tid + NT * q;
       const int t = e / (BN / 4);
       const int64_t j = j0 + (e % (BN / 4)) * 4;
-      if (t >= RG_BK || t0 + t >= g.K || j >= g.N) {
+      if (t0 + t >= g.K || j >= g.N) {
         rb[q] = make_float4(0.f, 0.f, 0.f, 0.f);
       } else if (g.bw == 0) {
         rb[q] = load4(B + (t0 + t) * g.ldb + j, left(g.N - j), bvec);
@@ -95,7 +97,7 @@ __global__ void __launch_bounds__(256) k_run_gemm(RunGemmArgs g) {
   auto sstore = [&](int buf) {
 #pragma unroll
     for (int q = 0; q < AV; ++q) {
-      const int e = tid + 256 * q;
+      const int e = tid + NT * q;
       if constexpr (AT) {
         *reinterpret_cast<float4*>(&As[buf][e / (BM / 4)][(e % (BM / 4)) * 4]) = ra[q];
       } else {
@@ -108,8 +110,8 @@ __global__ void __launch_bounds__(256) k_run_gemm(RunGemmArgs g) {
     }
 #pragma unroll
     for (int q = 0; q < BV; ++q) {
-      const int e = tid + 256 * q;
-      if (e / (BN / 4) < RG_BK) *reinterpret_cast<float4*>(&Bs[buf][e / (BN / 4)][(e % (BN / 4)) * 4]) = rb[q];
+      const int e = tid + NT * q;
+      *reinterpret_cast<float4*>(&Bs[buf][e / (BN / 4)][(e % (BN / 4)) * 4]) = rb[q];
     }
   };
   // rows: group v of 4 consecutive ones at v * (BM / NG) + 4 ty
@@ -167,7 +169,7 @@ __global__ void __launch_bounds__(256) k_run_gemm(RunGemmArgs g) {
 template <bool AT, typename TC, int BM, int BN>
 cudaError_t run_gemm(const RunGemmArgs& g, int batch, cudaStream_t s) {
   const int64_t tiles = ((g.M + BM - 1) / BM) * ((g.N + BN - 1) / BN);
-  k_run_gemm<AT, TC, BM, BN><<<dim3(unsigned(tiles), unsigned(batch)), 256, 0, s>>>(g);
+  k_run_gemm<AT, TC, BM, BN><<<dim3(unsigned(tiles), unsigned(batch)), BM * BN / 32, 0, s>>>(g);
   return cudaGetLastError();
 }
 
