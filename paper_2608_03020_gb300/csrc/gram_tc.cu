@@ -22,7 +22,8 @@
 //                (128-byte swizzle) and hand them to the TMA unit: a bulk store for the first
 //                segment of a zero_first launch, a bulk reduce-add into the fp32 output otherwise.
 // Work item = one 256-column tile of X (B) and up to two 256-row accumulators sharing it (Gram
-// tiles that touch the upper triangle and all cross tiles of that column, paired in order).
+// tiles that touch the upper triangle and all cross tiles of that column, paired in order); where it
+// saves rounds, the odd last cross tiles of two columns share an item and its A.
 // Factored cross product (loca_gram_cross_fused): with T_l = U_l Q_l, U_l = E P_l (N x r),
 //   T_l^T X_l = Q_l^T S_l,   S_l = U_l^T X_l  (r x d),
 // so a column tile needs one slot for S (its A operand is U_l, at most 64 rows) instead of d / 256
@@ -51,8 +52,10 @@
 // pace (about 1.25x slower at 7B size); the points within items keep the clusters' token windows
 // within ~L2 of each other (HBM re-reads 4.0x -> 2.6x of X and T, 3-4% faster under the power cap).
 // Rounds are aligned to blocks: the items are ordered so that a round holds the items of one block
-// only, each block filling whole rounds, and the few items left of every block follow at the end;
-// a round then streams one block's tiles instead of parts of two.
+// only, each block filling whole (or nine tenths of) rounds, and the few items left of every block
+// follow at the end; a round then streams one block's tiles instead of parts of two.  The items of a
+// last round that leaves half the clusters idle are cut into token ranges (L = 24, d = 896,
+// N = 16384: 4.1 rounds' worth in 4.25 instead of 5 rounds, 811 -> 762 us).
 // Every mbarrier wait is bounded: on expiry the status word gets LOCA_ERR_TIMEOUT, a launch-local
 // flag makes every other wait give up, and the roles stop, each CTA's producer at its own point.
 // At the end both CTAs meet at a cluster barrier (the odd CTA has posted how many pipeline
@@ -97,8 +100,11 @@ constexpr uint32_t IDESC_PAIR = tc::idesc(1, 1, 1, 1, BMP, BN);
 struct Geo {
   int L, d, N;
   int nM, nN;       // 256-row tiles and 256-column tiles
+  int pair;         // tiles per item: 2 (1), or 1 (0) when every tile has a cluster of its own
+  int odd_pairs;    // odd last tiles of two columns share an item
   int per_block;    // work items per block l
-  int full;         // items of each block that fill whole rounds of their own (0: plain order)
+  int rpb, main;    // rounds of a block's own and the items of it that fill them (0, 0: none)
+  int ways;         // clusters per item in a last, partial round
   int gram;         // 1: Gram tiles are computed (0: a later column range of a factored launch)
   int factored;     // 1: a cross slot is S = U^T X of its column tile, not a tile of T^T X
   int s0, s1;       // factored: column tiles with an S slot (s0 <= nt < s1)
@@ -117,52 +123,155 @@ __device__ __host__ __forceinline__ int gram_rows(const Geo& g, int nt) {
 __device__ __host__ __forceinline__ int cross_rows(const Geo& g, int nt) {
   return g.factored ? int(nt >= g.s0 && nt < g.s1) : g.nM;
 }
-// Items of column tile nt: its Gram and cross slots paired in order.
-__device__ __host__ __forceinline__ int items_of_col(const Geo& g, int nt) {
-  return (gram_rows(g, nt) + cross_rows(g, nt) + 1) / 2;
+__device__ __host__ __forceinline__ int col_tiles(const Geo& g, int nt) {
+  return gram_rows(g, nt) + cross_rows(g, nt);
+}
+// Items of a block: the tiles of each column in pairs, an odd last one by itself; or (odd_pairs) the whole
+// pairs of every column, then the columns' odd last tiles, two columns to an item where they are cross
+// tiles (their A operand, the last row tile of T or U, is the same), then what is left of columns without
+// cross tiles.
+__device__ __host__ __forceinline__ int items_of_block(const Geo& g) {
+  int n = 0, oddc = 0, oddg = 0;
+  for (int nt = 0; nt < g.nN; ++nt) {
+    const int k = col_tiles(g, nt);
+    n += g.pair ? k / 2 : k;
+    if (g.pair && (k & 1)) (cross_rows(g, nt) ? oddc : oddg) += 1;
+  }
+  return n + (g.odd_pairs ? (oddc + 1) / 2 : oddc) + oddg;
 }
 
 struct Item {
-  int l, nt;
+  int l;
   int nslots;
-  int kind[2];  // 0 = Gram (rows from X), 1 = cross (rows from T, or U when factored)
-  int mt[2];    // 256-row tile index
+  int nt0, nt1;        // column tile of each slot's output
+  int mt0, mt1;        // its 256-row tile
+  bool gram0, gram1;   // Gram (rows from X) or cross (rows from T, or U when factored)
+  bool shared_a;       // the slots share A (two columns); otherwise they share B (one column)
+  int kb0, kb1;        // k-blocks of the token axis
+  int part, split;     // part of an item that several clusters share (`split` its index, -1: not shared)
 };
 
-// Round-aligned order: a round is the items cid + round * (clusters).  The first `full` items of
-// block l (a multiple of the cluster count) fill rounds of block l alone, so a round streams the
-// tiles of one block; the per_block - full items left of every block come after all blocks.
-__device__ __forceinline__ Item decode(const Geo& g, int it) {
-  Item r;
-  int rem;
-  if (g.full > 0 && it < g.L * g.full) {
-    r.l = it / g.full;
-    rem = it - r.l * g.full;
-  } else if (g.full > 0) {
-    const int q = g.per_block - g.full;  // > 0 here: it < L * per_block
-    const int j = it - g.L * g.full;
-    r.l = j / q;
-    rem = g.full + (j - r.l * q);
-  } else {
-    r.l = it / g.per_block;
-    rem = it - r.l * g.per_block;
-  }
-  int nt = 0;
-  for (;; ++nt) {
-    const int c = items_of_col(g, nt);
-    if (rem < c) break;
-    rem -= c;
-  }
-  r.nt = nt;
+// Tile i of column nt, as slot s of r.
+__device__ __forceinline__ void set_slot(const Geo& g, Item& r, int s, int nt, int i) {
   const int ng = gram_rows(g, nt);
-  r.nslots = 0;
-  const int len = ng + cross_rows(g, nt);
-  for (int q = 2 * rem; q < 2 * rem + 2 && q < len; ++q) {
-    r.kind[r.nslots] = q < ng ? 0 : 1;
-    r.mt[r.nslots] = q < ng ? q : q - ng;
-    ++r.nslots;
+  const bool gr = i < ng;
+  if (s == 0) {
+    r.nt0 = nt;
+    r.gram0 = gr;
+    r.mt0 = gr ? i : i - ng;
+  } else {
+    r.nt1 = nt;
+    r.gram1 = gr;
+    r.mt1 = gr ? i : i - ng;
   }
-  return r;
+  r.nslots = s + 1;
+}
+
+// The idx-th item of block l.
+__device__ __forceinline__ void make_item(const Geo& g, int l, int idx, Item& r) {
+  r.l = l;
+  r.shared_a = false;
+  r.nt1 = r.mt1 = 0;
+  r.gram1 = false;
+  int oddc = 0;
+  for (int nt = 0; nt < g.nN; ++nt) {
+    const int len = col_tiles(g, nt), k = g.pair ? (g.odd_pairs ? len / 2 : (len + 1) / 2) : len;
+    if (idx < k) {
+      set_slot(g, r, 0, nt, g.pair ? 2 * idx : idx);
+      if (g.pair && 2 * idx + 1 < len) set_slot(g, r, 1, nt, 2 * idx + 1);
+      return;
+    }
+    idx -= k;
+    if (g.pair && (len & 1) && cross_rows(g, nt)) ++oddc;
+  }
+  const int two = (oddc + 1) / 2;
+  const bool cross = idx < two;
+  int skip = cross ? 2 * idx : idx - two;  // odd columns of its kind before this item's
+  int s = 0;
+  for (int nt = 0; nt < g.nN; ++nt) {
+    const int len = col_tiles(g, nt);
+    if (!(len & 1) || (cross_rows(g, nt) != 0) != cross || skip-- > 0) continue;
+    set_slot(g, r, s, nt, len - 1);
+    if (s == 1 || !cross) break;
+    s = 1;
+  }
+  r.shared_a = r.nslots == 2;
+}
+
+// A round is one item on each cluster.  Rounds aligned to blocks: where a block has at least about a
+// round of items, its first `main` items take `rpb` rounds of their own, so a round streams the tiles of
+// one block; what is left of the blocks follows in order, n items a round.  Neighbouring items
+// read the same operands: items sorted by length instead (the two-tile ones first) put tiles of
+// different blocks side by side and ran at the HBM's pace (148 us for a round of single tiles, 82
+// for one of pairs, at L = 28, d = 1536, N = 8192).
+// A last round of rem <= n / 2 items gives each to `ways` clusters, a range of the tokens each; their
+// sums are added in the order of the tokens (see the epilogue).
+struct Sched {
+  int c, n, nkb, seg_kb;
+  int P;               // sync points per item
+  int last, kc;        // clusters with an item in a block's last own round; own rounds of cluster c
+  int own;             // items of cluster c in blocks' own rounds
+  int per, R, rem;     // left-over items per block, their whole rounds, items of the last one
+};
+__device__ __forceinline__ Sched schedule(const Geo& g, int c, int n, int nkb, int seg_kb) {
+  Sched v;
+  v.c = c;
+  v.n = n;
+  v.nkb = nkb;
+  v.seg_kb = seg_kb;
+  v.P = (nkb + kSyncEvery - 1) / kSyncEvery;
+  v.last = g.main - (g.rpb - 1) * n;
+  v.kc = g.rpb == 0 ? 0 : (c < v.last ? g.rpb : g.rpb - 1);
+  v.own = g.L * v.kc;
+  v.per = g.per_block - g.main;
+  const int left = g.L * v.per;
+  v.R = left / n;
+  v.rem = left - v.R * n;
+  return v;
+}
+// The t-th item of cluster c of n; false when it has none left.  Lockstep: `before` sync counts come from
+// earlier rounds, `active` clusters take part in this one (0: not synchronised).
+__device__ __forceinline__ bool item_at(const Geo& g, const Sched& v, int t, Item& r, int& before, int& active) {
+  r.kb0 = 0;
+  r.kb1 = v.nkb;
+  r.part = 0;
+  r.split = -1;
+  if (t < v.own) {
+    const int l = t / v.kc, q = t - l * v.kc;
+    before = (l * g.main + q * v.n) * v.P;
+    active = q < g.rpb - 1 ? v.n : v.last;
+    make_item(g, l, q * v.n + v.c, r);
+    return true;
+  }
+  const int u = t - v.own;
+  before = (g.L * g.main + u * v.n) * v.P;
+  int j = u * v.n + v.c;
+  active = v.n;
+  if (u >= v.R) {
+    if (u > v.R || v.rem == 0) return false;
+    if (g.ways == 1) {
+      if (v.c >= v.rem) return false;
+      active = v.rem;
+    } else {
+      r.part = v.c / v.rem;
+      if (r.part >= g.ways) return false;
+      r.split = v.c - r.part * v.rem;
+      j = v.R * v.n + r.split;
+      active = 0;
+      const int nseg = (v.nkb + v.seg_kb - 1) / v.seg_kb;
+      if (nseg > 1) {  // at accumulation segments: the same sums as undivided
+        r.kb0 = nseg * r.part / g.ways * v.seg_kb;
+        r.kb1 = nseg * (r.part + 1) / g.ways * v.seg_kb;
+        if (r.kb1 > v.nkb) r.kb1 = v.nkb;
+      } else {
+        r.kb0 = v.nkb * r.part / g.ways;
+        r.kb1 = v.nkb * (r.part + 1) / g.ways;
+      }
+    }
+  }
+  const int l = j / v.per;
+  make_item(g, l, g.main + (j - l * v.per), r);
+  return true;
 }
 
 // ------------------------------------------------------------------ factored cross product
@@ -175,8 +284,9 @@ constexpr int kColGroup = 8192;  // columns of S held at a time (a multiple of B
 template <int RP>
 __global__ void __launch_bounds__(256) k_factor_u(const float* __restrict__ E, int64_t N, int C,
                                                   const float* __restrict__ P, int r,
-                                                  __nv_bfloat16* __restrict__ U) {
+                                                  __nv_bfloat16* __restrict__ U, int32_t* flags) {
   const int l = blockIdx.y;
+  if (l == 0 && blockIdx.x == 0 && threadIdx.x < kGramFlags) flags[threadIdx.x] = 0;  // for the statistics launch
   const int64_t n = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (n >= N) return;
   if (!LOCA_CHECK_SPAN(n * C, C, N * C) ||
@@ -296,9 +406,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     k_gram_cross_tc(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmT,
                     const __grid_constant__ CUtensorMap tmXa, const __grid_constant__ CUtensorMap tmTa,
                     const __grid_constant__ CUtensorMap tmXb, const __grid_constant__ CUtensorMap tmG,
-                    const __grid_constant__ CUtensorMap tmC, int blocked, Geo g, int total_items, int seg_kb,
+                    const __grid_constant__ CUtensorMap tmC, int blocked, Geo g, int seg_kb,
                     const float* __restrict__ alpha, int zero_first, int32_t* status, int32_t* abort_flag,
-                    uint32_t* round_ctr, unsigned long long limit_ns, unsigned long long sync_ns) {
+                    uint32_t* round_ctr, uint32_t* split_ctr, unsigned long long limit_ns, unsigned long long sync_ns) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~uintptr_t(1023));
@@ -325,10 +435,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   // rows of U (an S slot) are the even CTA's alone, the rest of that A tile is not loaded (its
   // accumulator rows are never read)
   auto item_bytes = [&](const Item& w, uint32_t rk) -> uint32_t {
-    uint32_t n = B_BYTES;
-    for (int s = 0; s < w.nslots; ++s)
-      n += (g.factored && w.kind[s] == 1) ? (rk == 0 ? uint32_t(SUB_BYTES) : 0u) : uint32_t(A_BYTES);
-    return n;
+    auto a_bytes = [&](bool gram) {
+      return g.factored && !gram ? (rk == 0 ? uint32_t(SUB_BYTES) : 0u) : uint32_t(A_BYTES);
+    };
+    return B_BYTES + a_bytes(w.gram0) + (w.nslots == 2 ? (w.shared_a ? uint32_t(B_BYTES) : a_bytes(w.gram1)) : 0u);
   };
 
   if (threadIdx.x == 0) {
@@ -345,9 +455,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       prefetch_tensormap(&tmXa);
       if (!g.factored) prefetch_tensormap(&tmTa);
       prefetch_tensormap(&tmXb);
-    } else {
-      prefetch_tensormap(&tmX);
     }
+    prefetch_tensormap(&tmX);
     if (!blocked || g.factored) prefetch_tensormap(&tmT);
     prefetch_tensormap(&tmG);
     prefetch_tensormap(&tmC);
@@ -358,7 +467,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   fence_after();
   const uint32_t tmem_base = *tmem_slot;
   const int nkb = (g.N + BK - 1) / BK;
-  const int nseg = (nkb + seg_kb - 1) / seg_kb;
+  const Sched sched = schedule(g, cid, ncl, nkb, seg_kb);
   uint32_t iters_done = 0;  // producer: pipeline iterations this CTA issued
 
   if (warp == 0) {
@@ -369,9 +478,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       uint32_t iter = 0;  // pipeline iterations issued by this CTA
       bool ok = true;
       bool sync = leader;  // dropped for the rest of the launch if a wait runs out
-      // sync points: each item counts one every kSyncEvery k-blocks and one at its end (P per item)
-      const int P = (nkb + kSyncEvery - 1) / kSyncEvery;
-      uint32_t before = 0;  // counts expected from all earlier rounds
       auto wait_for = [&](uint32_t target) {  // a hint: bounded, no error
         const uint64_t t0 = globaltimer();
         while (*reinterpret_cast<volatile uint32_t*>(round_ctr) < target) {
@@ -381,18 +487,31 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
           }
         }
       };
-      uint32_t round = 0;
-      for (int it = cid; it < total_items && ok; it += ncl, ++round) {
-        // clusters with an item in this round (the last round may be partial)
-        const int left = total_items - int(round) * ncl;
-        const uint32_t active = uint32_t(left < ncl ? left : ncl);
-        if (sync && round > 0) wait_for(before);  // every cluster finished issuing its last item
-        const Item w = decode(g, it);
+      Item w;
+      int before = 0, active = 0;
+      for (int t = 0; ok && item_at(g, sched, t, w, before, active); ++t) {
+        const bool counted = leader && active > 0;
+        if (sync && counted && t > 0) wait_for(uint32_t(before));  // every cluster finished issuing its last item
         const uint32_t bytes_both = item_bytes(w, 0) + item_bytes(w, 1);
-        for (int kb = 0; kb < nkb; ++kb) {
-          if (leader && kb > 0 && kb % kSyncEvery == 0) {
+        // the second A region holds the second slot's rows, or its columns when the slots share A
+        const bool x0 = w.gram0, x1 = w.gram1 || w.shared_a;
+        const int row_0 = w.mt0 * BMP + int(rank) * BMC;
+        const int row_1 = (w.shared_a ? w.nt1 : w.mt1) * BMP + int(rank) * BMC;
+        auto load_a = [&](uint32_t dst, bool from_x, int row0, uint32_t fb, int tok) {
+          if (g.factored && !from_x) {
+            if (leader) tma_load_3d_pair(dst, &tmT, fb, 0, tok, w.l);
+          } else if (blocked) {
+            tma_load_4d_pair(dst, from_x ? &tmXa : &tmTa, fb, 0, tok, row0 / 64, w.l);
+          } else {
+            const CUtensorMap* map = from_x ? &tmX : &tmT;
+            tma_load_3d_pair(dst, map, fb, row0, tok, w.l);
+            tma_load_3d_pair(dst + SUB_BYTES, map, fb, row0 + 64, tok, w.l);
+          }
+        };
+        for (int kb = w.kb0; kb < w.kb1; ++kb) {
+          if (counted && kb > 0 && kb % kSyncEvery == 0) {
             atomicAdd(round_ctr, 1u);
-            if (sync) wait_for(before + active * uint32_t(kb / kSyncEvery));
+            if (sync) wait_for(uint32_t(before) + uint32_t(active) * uint32_t(kb / kSyncEvery));
           }
           if (!mbar_try_wait_cluster(empty_bar(stage), phase ^ 1u) &&
               !mbar_wait_cluster(empty_bar(stage), phase ^ 1u, wc)) {
@@ -404,24 +523,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
           const uint32_t st = smem_base + uint32_t(stage) * STAGE_BYTES;
           const uint32_t bdst = st + 2u * A_BYTES;
           const int tok = kb * BK;
-          const int col0 = w.nt * BN + int(rank) * BNC;
+          const int col0 = w.nt0 * BN + int(rank) * BNC;
           // the stage is armed: a failed check is recorded, the loads (out-of-range boxes are
           // filled by the TMA unit) still run so that the barrier completes
           (void)LOCA_REQUIRE(tok >= 0 && col0 % 64 == 0);
-          for (int s = 0; s < w.nslots; ++s) {
-            const uint32_t dst = st + uint32_t(s) * A_BYTES;
-            const int row0 = w.mt[s] * BMP + int(rank) * BMC;
-            (void)LOCA_REQUIRE(row0 % 64 == 0);
-            if (g.factored && w.kind[s] == 1) {
-              if (leader) tma_load_3d_pair(dst, &tmT, fb, 0, tok, w.l);
-            } else if (blocked) {
-              tma_load_4d_pair(dst, w.kind[s] == 0 ? &tmXa : &tmTa, fb, 0, tok, row0 / 64, w.l);
-            } else {
-              const CUtensorMap* map = w.kind[s] == 0 ? &tmX : &tmT;
-              tma_load_3d_pair(dst, map, fb, row0, tok, w.l);
-              tma_load_3d_pair(dst + SUB_BYTES, map, fb, row0 + 64, tok, w.l);
-            }
-          }
+          (void)LOCA_REQUIRE(row_0 % 64 == 0 && row_1 % 64 == 0);
+          load_a(st, x0, row_0, fb, tok);
+          if (w.nslots == 2) load_a(st + A_BYTES, x1, row_1, fb, tok);
           if (blocked) {
             tma_load_4d_pair(bdst, &tmXb, fb, 0, tok, col0 / 64, w.l);
           } else {
@@ -431,8 +539,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
           ++iter;
           if (++stage == STAGES) { stage = 0; phase ^= 1u; }
         }
-        if (ok && leader) atomicAdd(round_ctr, 1u);
-        before += active * uint32_t(P);
+        if (ok && counted) atomicAdd(round_ctr, 1u);
       }
       // the odd CTA posts how many iterations it issued (read by the even CTA after the barrier)
       if (!leader) st_shared_cluster_u32(mapa_shared(smem_u32(odd_issued), 0), iter);
@@ -450,11 +557,16 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       const uint64_t b_desc0 = sdesc(smem_base + 2u * A_BYTES, SUB_BYTES, 1024u, kSwizzle128B);
       constexpr uint64_t kStageStep = STAGE_BYTES >> 4, kSlotStep = A_BYTES >> 4, kKStep = 2048 >> 4;
       const uint32_t d0 = tmem_base, d1 = tmem_base + uint32_t(BN);
-      for (int it = cid; it < total_items && ok; it += ncl) {
-        const Item w = decode(g, it);
+      Item w;
+      int before, active;
+      for (int t = 0; ok && item_at(g, sched, t, w, before, active); ++t) {
         const bool two = w.nslots == 2;
-        for (int kb = 0; kb < nkb; ++kb) {
-          const int in_seg = kb % seg_kb;
+        // the second slot's operands: its own A and the common B, or the common A and its own B, which is in
+        // the second A region (A and B tiles have one layout)
+        const uint64_t a1_off = w.shared_a ? 0 : kSlotStep;
+        const uint64_t b1_off = w.shared_a ? a_desc0 + kSlotStep - b_desc0 : 0;
+        for (int kb = w.kb0; kb < w.kb1; ++kb) {
+          const int in_seg = (kb - w.kb0) % seg_kb;
           if (in_seg == 0) {  // a new segment: the epilogue has read the sums
             if (!mbar_try_wait_cluster(acc_empty, acc_phase ^ 1u) &&
                 !mbar_wait_cluster(acc_empty, acc_phase ^ 1u, wc)) {
@@ -471,16 +583,17 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
           fence_after();
           const uint64_t so = uint64_t(stage) * kStageStep;
           const uint64_t ad = a_desc0 + so, bd = b_desc0 + so;
+          const uint64_t a1 = ad + a1_off, b1 = bd + b1_off;
 #pragma unroll
           for (int kk = 0; kk < BK / 16; ++kk) {
             const uint32_t acc = (in_seg | kk) != 0 ? 1u : 0u;
             mma_f16_pair(d0, ad + kk * kKStep, bd + kk * kKStep, IDESC_PAIR, acc);
-            if (two) mma_f16_pair(d1, ad + kSlotStep + kk * kKStep, bd + kk * kKStep, IDESC_PAIR, acc);
+            if (two) mma_f16_pair(d1, a1 + kk * kKStep, b1 + kk * kKStep, IDESC_PAIR, acc);
           }
           issued = true;
           mma_commit_pair_mc(empty_bar(stage), 0x3);  // frees the stage in both CTAs
           if (++stage == STAGES) { stage = 0; phase ^= 1u; }
-          if (in_seg == seg_kb - 1 || kb == nkb - 1) {
+          if (in_seg == seg_kb - 1 || kb == w.kb1 - 1) {
             mma_commit_pair_mc(acc_full, 0x3);  // this segment's sums complete in both CTAs
             acc_phase ^= 1u;
           }
@@ -502,9 +615,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     uint32_t acc_phase = 0;
     uint32_t nbox = 0;  // boxes this warp has handed to the TMA unit
     bool go = true;
-    for (int it = cid; it < total_items && go; it += ncl) {
-      const Item w = decode(g, it);
+    Item w;
+    int before, active;
+    for (int t = 0; go && item_at(g, sched, t, w, before, active); ++t) {
       const float al = alpha[w.l];
+      const int nseg = (w.kb1 - w.kb0 + seg_kb - 1) / seg_kb;
       for (int seg = 0; seg < nseg && go; ++seg) {
         const bool ok = mbar_wait_cluster(acc_full, acc_phase, wc);
         if (!__all_sync(0xffffffffu, ok)) {  // warp-uniform decision, warp reconverged
@@ -513,16 +628,41 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         }
         fence_after();
         // the previous segment's additions to these boxes are complete: fixed order of additions
-        if (lane == 0) bulk_wait_group0();
+        if (seg > 0 && lane == 0) bulk_wait_group0();
         __syncwarp();
+        if (w.part > 0 && seg == 0) {
+          // an item shared by clusters: the additions of the earlier parts (8 warps each) are complete
+          bool ready = true;
+          if (lane == 0) {
+            const uint64_t t0 = globaltimer();
+            while (*reinterpret_cast<const volatile uint32_t*>(split_ctr + w.split) < 8u * uint32_t(w.part) && ready) {
+              if (globaltimer() - t0 > wc.limit_ns) {
+                atomicExch(wc.status, int32_t(LOCA_ERR_TIMEOUT));
+                *wc.abort_flag = 1;
+                __threadfence();
+                ready = false;
+              } else if (*wc.abort_flag != 0) {
+                ready = false;
+              }
+            }
+            __threadfence();
+            asm volatile("fence.proxy.async;" ::: "memory");
+          }
+          if (!__shfl_sync(0xffffffffu, int(ready), 0)) {
+            go = false;
+            break;
+          }
+        }
         for (int s = 0; s < w.nslots; ++s) {
-          const bool is_gram = w.kind[s] == 0;
-          const bool store = (zero_first || (g.factored && !is_gram)) && seg == 0;  // S starts from zero
+          const bool is_gram = s == 0 ? w.gram0 : w.gram1;
+          const int nt = s == 0 ? w.nt0 : w.nt1, mt = s == 0 ? w.mt0 : w.mt1;
+          // S starts from zero
+          const bool store = (zero_first || (g.factored && !is_gram)) && seg == 0 && w.part == 0;
           const CUtensorMap* omap = is_gram ? &tmG : &tmC;
           const float sc = is_gram || g.factored ? 1.f : al;
           const int rows = is_gram ? g.d : g.rowsC;
           const int jshift = g.factored && !is_gram ? g.s0 * BN : 0;  // S holds the columns of its range only
-          const int i0 = w.mt[s] * BMP + int(rank) * BMC + q * 32;
+          const int i0 = mt * BMP + int(rank) * BMC + q * 32;
 #pragma unroll 1
           for (int c = 0; c < BN / 32; ++c) {
             float v[32];
@@ -536,7 +676,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
                 else mbar_arrive_remote(acc_empty_leader);
               }
             }
-            const int j0 = w.nt * BN + c * 32;
+            const int j0 = nt * BN + c * 32;
             if (i0 >= rows || j0 >= g.d) continue;  // warp-uniform; partial boxes are clipped by the TMA unit
             const uint32_t buf = nbox % uint32_t(kBufs);
             if (lane == 0) {  // this buffer's previous box has been read
@@ -564,6 +704,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         }
         acc_phase ^= 1u;
       }
+      if (go && w.split >= 0 && w.part + 1 < g.ways) {  // this warp's additions are complete: the next part's turn
+        if (lane == 0) {
+          bulk_wait_group0();
+          __threadfence();
+          atomicAdd(split_ctr + w.split, 1u);
+        }
+        __syncwarp();
+      }
     }
     if (lane == 0) bulk_wait_group0();  // every box written before the CTA can leave
     __syncwarp();
@@ -587,10 +735,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     const uint32_t lo = hi > uint32_t(STAGES) ? hi - uint32_t(STAGES) : 0u;
     for (uint32_t t = lo; t < hi; ++t) {
       const int s = int(t % STAGES);
-      const Item w = decode(g, cid + int(t / uint32_t(nkb)) * ncl);
-      const uint32_t odd_bytes = item_bytes(w, 1);
-      if (t >= n_odd && t < n_even) mbar_complete_tx(full_bar(s), odd_bytes);
-      else if (t >= n_even && t < n_odd) mbar_arrive_expect_tx(full_bar(s), odd_bytes);
+      if (n_even != n_odd) {
+        Item w;
+        int before, active;
+        item_at(g, sched, int(t / uint32_t(nkb)), w, before, active);
+        const uint32_t odd_bytes = item_bytes(w, 1);
+        if (t >= n_odd && t < n_even) mbar_complete_tx(full_bar(s), odd_bytes);
+        else if (t >= n_even && t < n_odd) mbar_arrive_expect_tx(full_bar(s), odd_bytes);
+      }
       mbar_drain(full_bar(s), (t / STAGES) & 1u, kDrainLimitNs);
     }
   }
@@ -718,9 +870,32 @@ struct Factored {
   int s0, s1;
   int gram;    // compute the Gram tiles in this launch
 };
+// Items to n clusters: sets per_block, rpb, main and ways; returns the launch's length in twelfths of a
+// round.
+int deal_items(Geo& g, int n, int64_t nkb) {
+  g.per_block = items_of_block(g);
+  const int64_t total = int64_t(g.per_block) * g.L;
+  // Rounds of a block's own: whole ones, and a last one at least nine tenths full.
+  g.rpb = total <= n ? 0 : g.per_block / n + (g.per_block % n * 10 >= n * 9 ? 1 : 0);
+  g.main = g.per_block < g.rpb * n ? g.per_block : g.rpb * n;
+  // A last round (or only one) that leaves at least half the clusters idle: its items in up to four token
+  // ranges.  A range costs an epilogue of its own (~9 us, one after the other) and saves its share of the
+  // ~0.57 us per k-block, so two ranges pay from 96 k-blocks on, three from 128, four from 192; items of
+  // several accumulation segments are cut between segments only, so that the sums do not depend on the ways.
+  const int64_t left = total - int64_t(g.main) * g.L;
+  const int64_t rem = total <= n ? total : left % n;
+  const int64_t nsegs = (nkb + kSegTokens / BK - 1) / (kSegTokens / BK);
+  int64_t most = nkb >= 192 ? 4 : (nkb >= 128 ? 3 : (nkb >= 96 ? 2 : 1));
+  if (nsegs > 1 && most > nsegs) most = nsegs;
+  if (rem > kGramFlags - 2) most = 1;  // a counter per shared item
+  if (rem > 0 && most > n / rem) most = n / rem;
+  g.ways = most > 1 && rem > 0 ? int(most) : 1;
+  return int((int64_t(g.rpb) * g.L + (total <= n ? 0 : left / n)) * 12 + (rem > 0 ? 12 / g.ways : 0));
+}
+
 cudaError_t launch_stats(const void* X, const void* T, int L, int64_t N, int64_t d, const float* alpha,
                          int zero_first, float* gram, float* cross, int32_t* status, int32_t* abort_flag,
-                         const Factored& f, cudaStream_t s) {
+                         bool flags_clear, const Factored& f, cudaStream_t s) {
   CUtensorMap mx, mt, mxa, mta, mxb, mg, mc;
   memset(&mta, 0, sizeof(mta));
   memset(&mxa, 0, sizeof(mxa));
@@ -742,32 +917,39 @@ cudaError_t launch_stats(const void* X, const void* T, int L, int64_t N, int64_t
   g.nM = int((d + BMP - 1) / BMP);
   g.nN = int((d + BN - 1) / BN);
   g.per_block = 0;
-  g.full = 0;
   g.gram = fac ? f.gram : 1;
   g.factored = fac ? 1 : 0;
   g.s0 = f.s0;
   g.s1 = f.s1;
   g.rowsC = fac ? f.u_cols : int(d);
-  for (int nt = 0; nt < g.nN; ++nt) g.per_block += items_of_col(g, nt);
-  const int total = g.per_block * L;
-  cudaError_t e = cudaFuncSetAttribute(k_gram_cross_tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       kSmem);
-  if (e != cudaSuccess) return e;
-  static int clusters_cached = 0;  // per process; the library drives one device type
-  if (clusters_cached == 0) clusters_cached = resident_clusters();
-  int clusters = clusters_cached;
-  if (clusters > total) clusters = total;
-  if (clusters < 1) clusters = 1;
-  g.full = (g.per_block / clusters) * clusters;
-  // abort flag and round counter (two int32 of the launch-local flag area)
-  e = cudaMemsetAsync(abort_flag, 0, 2 * sizeof(int32_t), s);
+  int tiles = 0;
+  for (int nt = 0; nt < g.nN; ++nt) tiles += col_tiles(g, nt);
+  g.pair = int64_t(tiles) * L > sm_count() / 2 ? 1 : 0;
+  // abort flag, round counter and the shared items' counters
+  cudaError_t e = flags_clear ? cudaSuccess : cudaMemsetAsync(abort_flag, 0, kGramFlags * sizeof(int32_t), s);
   if (e != cudaSuccess) return e;
   // a round takes about nkb x 1024 tensor-core cycles; wait for the slowest cluster up to ~3x that
   const int64_t nkb = (N + BK - 1) / BK;
   const unsigned long long sync_ns = 50000ull + 2000ull * (unsigned long long)nkb;
-  k_gram_cross_tc<<<2 * clusters, kThreads, kSmem, s>>>(
-      mx, mt, mxa, mta, mxb, mg, mc, blocked, g, total, kSegTokens / BK, alpha, zero_first, status, abort_flag,
-      reinterpret_cast<uint32_t*>(abort_flag + 1), wait_limit_ns(), sync_ns);
+  e = cudaFuncSetAttribute(k_gram_cross_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
+  if (e != cudaSuccess) return e;
+  static int clusters_cached = 0;  // per process; the library drives one device type
+  if (clusters_cached == 0) clusters_cached = resident_clusters();
+  const int most_clusters = clusters_cached;
+  // The columns' odd tiles pair up only where that saves rounds (d = 1536, 28 blocks: 1100 -> 1037 us at
+  // N = 8192): elsewhere a round with single tiles in it is the shorter one (d = 896, 24 blocks, five
+  // rounds either way at N = 4096: 213 us, 217 paired up).
+  g.odd_pairs = 1;
+  const int paired = deal_items(g, most_clusters, nkb);
+  Geo alone = g;
+  alone.odd_pairs = 0;
+  if (deal_items(alone, most_clusters, nkb) <= paired) g = alone;
+  const int64_t total = int64_t(g.per_block) * L;
+  const int n = total <= most_clusters ? int(total) * g.ways : most_clusters;
+  uint32_t* ctr = reinterpret_cast<uint32_t*>(abort_flag + 1);
+  k_gram_cross_tc<<<unsigned(2 * n), kThreads, kSmem, s>>>(mx, mt, mxa, mta, mxb, mg, mc, blocked, g, kSegTokens / BK,
+                                                                  alpha, zero_first, status, abort_flag, ctr, ctr + 1,
+                                                                  wait_limit_ns(), sync_ns);
   e = cudaGetLastError();
   if (e != cudaSuccess || !g.gram) return e;
   const int nt = int((d + MIR_T - 1) / MIR_T);
@@ -779,9 +961,9 @@ cudaError_t launch_stats(const void* X, const void* T, int L, int64_t N, int64_t
 
 cudaError_t launch_gram_cross_tc(const void* X, const void* T, int L, int64_t N, int64_t d,
                                  const float* alpha, int zero_first, float* gram, float* cross,
-                                 int32_t* status, int32_t* abort_flag, cudaStream_t s) {
+                                 int32_t* status, int32_t* abort_flag, bool flags_clear, cudaStream_t s) {
   const Factored none{0, 0, 0, 1};
-  return launch_stats(X, T, L, N, d, alpha, zero_first, gram, cross, status, abort_flag, none, s);
+  return launch_stats(X, T, L, N, d, alpha, zero_first, gram, cross, status, abort_flag, flags_clear, none, s);
 }
 
 int gram_fused_max_r() { return 32; }
@@ -803,13 +985,14 @@ cudaError_t gram_cross_factored(const void* X, const float* E, int C, const floa
   uint8_t* ws = static_cast<uint8_t*>(workspace);
   __nv_bfloat16* U = reinterpret_cast<__nv_bfloat16*>(ws + 256);
   float* S = reinterpret_cast<float*>(ws + 256 + align256(sizeof(__nv_bfloat16) * size_t(L) * size_t(N) * size_t(2 * RP)));
-  k_factor_u<RP><<<dim3(unsigned((N + 255) / 256), unsigned(L)), 256, 0, s>>>(E, N, C, P, r, U);
+  int32_t* flags = reinterpret_cast<int32_t*>(ws);
+  k_factor_u<RP><<<dim3(unsigned((N + 255) / 256), unsigned(L)), 256, 0, s>>>(E, N, C, P, r, U, flags);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   for (int64_t c0 = 0; c0 < d; c0 += kColGroup) {
     const int64_t cw = d - c0 < kColGroup ? d - c0 : kColGroup;
     const Factored f{2 * RP, int(c0 / BN), int((c0 + cw + BN - 1) / BN), c0 == 0 ? 1 : 0};
-    e = launch_stats(X, U, L, N, d, alpha, zero_first, gram, S, status, reinterpret_cast<int32_t*>(ws), f, s);
+    e = launch_stats(X, U, L, N, d, alpha, zero_first, gram, S, status, flags, c0 == 0, f, s);
     if (e != cudaSuccess) return e;
     const dim3 grid(unsigned((cw + EX_COLS - 1) / EX_COLS), unsigned((d + ex_rows(RP) - 1) / ex_rows(RP)), unsigned(L));
     k_expand_cross<RP><<<grid, 256, 0, s>>>(S, cw, Q, r, int(d), int(c0), int(cw), alpha, zero_first, cross);

@@ -66,7 +66,7 @@ extern "C" int loca_accumulate_noalloc(const void* X, const void* T, int dtype, 
   int32_t* abort_flag = reinterpret_cast<int32_t*>(scratch + kPartialBytes + kAlphaBytes);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   // the same launches as loca_accumulate, with the scratch array in place of the workspace
-  const int rs = run_batch_step(X, dtype, L, N, d, tsq, eta, zero_first, xsq_total, alpha, partials, s);
+  const int rs = run_batch_step(X, dtype, L, N, d, tsq, eta, zero_first, xsq_total, alpha, partials, abort_flag, s);
   if (rs != LOCA_OK) return rs;
-  return run_gram_cross(X, T, dtype, L, N, d, alpha, zero_first, gram, cross, abort_flag, s);
+  return run_gram_cross(X, T, dtype, L, N, d, alpha, zero_first, gram, cross, abort_flag, true, s);
 }

@@ -93,7 +93,9 @@ __global__ void __launch_bounds__(256) k_sumsq(const void* __restrict__ Xv, int6
 // 7-10 us a call).
 __global__ void __launch_bounds__(128) k_step(const double* __restrict__ partials, int G, int L,
                                               const double* __restrict__ tsq, float eta, int zero_first,
-                                              double* __restrict__ xsq_total, float* __restrict__ alpha) {
+                                              double* __restrict__ xsq_total, float* __restrict__ alpha,
+                                              int32_t* flags) {
+  if (flags != nullptr && blockIdx.x == 0 && threadIdx.x < kGramFlags) flags[threadIdx.x] = 0;
   const int l = blockIdx.x * 4 + int(threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (l >= L || !LOCA_CHECK(G, kMaxPartials + 1)) return;
   double xb = 0.0;
@@ -240,7 +242,7 @@ int sumsq_num_partials() { return kMaxPartials; }
 
 cudaError_t launch_sumsq_and_step(const void* X, int dtype, int L, int64_t N, int64_t d,
                                   const double* tsq, float eta, int zero_first, double* xsq_total,
-                                  double* partials, float* alpha, cudaStream_t s) {
+                                  double* partials, float* alpha, int32_t* flags, cudaStream_t s) {
   int64_t G = (int64_t(sm_count()) * 8 + L - 1) / L;
   const int64_t n_el = N * d;
   const int64_t maxg = (n_el + 4095) / 4096;  // at least 4096 elements per thread block
@@ -260,7 +262,7 @@ cudaError_t launch_sumsq_and_step(const void* X, int dtype, int L, int64_t N, in
   } else {
     G = 0;
   }
-  k_step<<<(L + 3) / 4, 128, 0, s>>>(partials, int(G), L, tsq, eta, zero_first, xsq_total, alpha);
+  k_step<<<(L + 3) / 4, 128, 0, s>>>(partials, int(G), L, tsq, eta, zero_first, xsq_total, alpha, flags);
   return cudaGetLastError();
 }
 

@@ -267,3 +267,47 @@ def test_head_error_short_rows(lc, N, V, C, dtype, normaliser):
     p_ref = wn[:, None] * np.exp(zz[:, cols] - lse[:, None])  # before the label entry cancels
     assert np.all(np.abs(_np(E) - e_ref) <= rel * p_ref + 2e-6)
     assert np.all(np.abs(_np(ce) - ce_ref) <= rel * (1 + np.abs(ce_ref)))
+
+
+@pytest.mark.parametrize("L,N,d,batches", [
+    (1, 12289, 520, 2),    # 193 k-blocks, every tile an item, four token ranges each
+    (2, 33000, 72, 1),     # three accumulation segments, cut between segments
+    (13, 8200, 328, 2),    # columns of 3 and 4 tiles
+    (5, 6200, 1400, 1),    # odd columns' last tiles by themselves
+    (13, 700, 1400, 1),    # odd columns sharing A: five rounds instead of six
+])
+def test_gram_schedules(lc, L, N, d, batches):
+    """The statistics whatever the items' distribution: fp32 accumulation in the tensor cores truncates, a
+    fraction of an ulp per step over at most 1024 steps (6e-5); every launch gives the same bits."""
+    g = torch.Generator(device="cuda")
+    g.manual_seed(d)
+    out = []
+    for rep in range(2):
+        g.manual_seed(d)
+        gram, cross = (torch.full((L, d, d), float("nan"), device="cuda") for _ in range(2))
+        gram_f, cross_f = (torch.full((L, d, d), float("nan"), device="cuda") for _ in range(2))
+        alpha = torch.linspace(0.5, -1.0, L, device="cuda")
+        g_ref, c_ref, cf_ref = (torch.zeros((L, d, d), dtype=torch.float64, device="cuda") for _ in range(3))
+        for b in range(batches):
+            X, T = (torch.randn((L, N, d), generator=g, device="cuda").to(torch.bfloat16) for _ in range(2))
+            E = torch.randn((N, 3), generator=g, device="cuda")
+            P = torch.randn((L, 3, 5), generator=g, device="cuda")
+            Q = torch.randn((L, 5, d), generator=g, device="cuda")
+            lc.loca_gram_cross(X, T, alpha, gram, cross, zero_first=b == 0)
+            lc.loca_gram_cross_fused(X, E, P, Q, alpha, gram_f, cross_f, zero_first=b == 0)
+            if rep == 0:
+                for l in range(L):
+                    x = X[l].double()
+                    g_ref[l] += x.t() @ x
+                    c_ref[l] += alpha[l].double() * (T[l].double().t() @ x)
+                    cf_ref[l] += alpha[l].double() * (Q[l].double().t() @ ((E.double() @ P[l].double()).t() @ x))
+        torch.cuda.synchronize()
+        assert lc.loca_device_status() == 0
+        out.append((gram, cross, gram_f, cross_f))
+        if rep == 0:
+            rel = lambda a, b: float((a.double() - b).norm() / b.norm())  # noqa: E731
+            assert rel(gram, g_ref) <= 6e-5 and rel(cross, c_ref) <= 6e-5
+            assert rel(gram_f, g_ref) <= 6e-5 and rel(cross_f, cf_ref) <= 6e-5
+            assert torch.equal(gram, gram.transpose(1, 2)) and torch.equal(gram_f, gram_f.transpose(1, 2))
+    for a, b in zip(*out):
+        assert torch.equal(a, b)
