@@ -156,9 +156,10 @@ __device__ __forceinline__ void split8h(const float* y, uint4& hi, uint4& lo) {
 constexpr int PP_THREADS = 128;
 template <int KN>
 __global__ void __launch_bounds__(PP_THREADS) k_project_prep(const float* __restrict__ A, int64_t d, int k,
-                                                            int nkb, uint8_t* __restrict__ rec) {
+                                                            int nkb, uint8_t* __restrict__ rec, int32_t* abort_flag) {
   constexpr int SPB = PP_THREADS / KN;  // slabs per block
   const int l = blockIdx.y;
+  if (l == 0 && blockIdx.x == 0 && threadIdx.x == 0) *abort_flag = 0;  // the projection's waits
   const int kb = blockIdx.x * SPB + int(threadIdx.x) / KN;
   const int s = int(threadIdx.x) % KN;
   if (kb >= nkb) return;
@@ -484,10 +485,8 @@ cudaError_t launch_kn(const float* gram, const float* cross, const float* A, int
   g.items = L * 2 * g.nrt;
   constexpr int SPB = PP_THREADS / KN;
   k_project_prep<KN><<<dim3(unsigned((g.nkb + SPB - 1) / SPB), unsigned(L)), PP_THREADS, 0, s>>>(
-      A, d, k, g.nkb, static_cast<uint8_t*>(arec));
+      A, d, k, g.nkb, static_cast<uint8_t*>(arec), abort_flag);
   cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  e = cudaMemsetAsync(abort_flag, 0, sizeof(int32_t), s);
   if (e != cudaSuccess) return e;
   int grid = sm_count();
   if (grid > g.items) grid = g.items;

@@ -18,7 +18,7 @@
 //               (two 128-channel boxes per tile when d % 64 == 0), so HBM sees whole lines;
 //               fp32 output uses plain stores (one row per thread).  TMEM is read 64 columns
 //               per wait.
-// Work item = (block l, 256-channel tile, 4096-token chunk); ||T_l||^2 partials are written
+// Work item = (block l, 256-channel tile, chunk of up to 4096 tokens); ||T_l||^2 partials are written
 // per item and epilogue warp and summed in a fixed order by k_reduce_partials
 // (deterministic).  All waits are bounded (see tc_ptx.cuh) and no warp waits on another
 // warp except through those bounded mbarrier waits.
@@ -36,8 +36,7 @@ using namespace tc;
 
 constexpr int TM = 128;           // tokens per tile (TMEM lanes)
 constexpr int TCH = 256;          // channels per tile (TMEM columns per accumulator)
-constexpr int CHUNK_TILES = 32;   // tiles per work item
-constexpr int CHUNK = TM * CHUNK_TILES;
+constexpr int MAX_CHUNK_TILES = 32;   // tiles per work item at most
 constexpr int kMaxC = 64;
 constexpr int kMaxRP = 32;        // padded feedback rank (multiple of 8)
 constexpr int NTHREADS = 288;
@@ -87,6 +86,7 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float a, float b) {
 
 struct Geo {
   int64_t N, d;
+  int64_t chunk;   // tokens per work item
   int C, r, rp, L;
   int64_t nd, nchunks, items;
 };
@@ -102,8 +102,7 @@ template <bool kBF16>
 __global__ void __launch_bounds__(NTHREADS, 1)
     k_targets_tc(const float* __restrict__ E, const float* __restrict__ P, const float* __restrict__ Q,
                  Geo g, void* __restrict__ Tout, const __grid_constant__ CUtensorMap tmT, int store_mode,
-                 double* __restrict__ partials, int32_t* status, int32_t* abort_flag,
-                 unsigned long long limit_ns) {
+                 double* __restrict__ partials, int32_t* status, unsigned long long limit_ns) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   // 1024-byte aligned base: the 128-byte swizzle of the TMA boxes repeats every 1024 bytes
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -120,7 +119,9 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 11);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const WaitCtl wc{status, abort_flag, limit_ns};
+  // CTAs do not wait for one another, so one that gives up tells only its own roles
+  __shared__ int32_t abort_flag;
+  const WaitCtl wc{status, &abort_flag, limit_ns};
   const int rp = g.rp, r = g.r, C = g.C;
 
   if (threadIdx.x == 0) {
@@ -130,6 +131,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       mbar_init(acc_full(b), 1);
       mbar_init(acc_empty(b), 128);
     }
+    abort_flag = 0;
     mbar_init(b_full, 128);
     mbar_init(b_empty, 1);
     mbar_init(drain_bar, 1);
@@ -151,8 +153,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       int64_t jt, ck;
       decode(g, it, l, jt, ck);
       const int64_t j0 = jt * TCH;
-      const int64_t nbeg = ck * CHUNK;
-      const int64_t nend = (nbeg + CHUNK < g.N) ? nbeg + CHUNK : g.N;
+      const int64_t nbeg = ck * g.chunk;
+      const int64_t nend = (nbeg + g.chunk < g.N) ? nbeg + g.chunk : g.N;
       // the bounded waits are calls (registers saved around them): an inline try_wait goes first
       if (!mbar_try_wait(b_empty, (icount & 1u) ^ 1u) && !mbar_wait(b_empty, (icount & 1u) ^ 1u, wc)) {
         ok = false;
@@ -233,8 +235,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         int l;
         int64_t jt, ck;
         decode(g, it, l, jt, ck);
-        const int64_t nbeg = ck * CHUNK;
-        const int64_t nend = (nbeg + CHUNK < g.N) ? nbeg + CHUNK : g.N;
+        const int64_t nbeg = ck * g.chunk;
+        const int64_t nend = (nbeg + g.chunk < g.N) ? nbeg + g.chunk : g.N;
         if (!mbar_try_wait(b_full, icount & 1u) && !mbar_wait(b_full, icount & 1u, wc)) {
           ok = false;
           break;
@@ -284,8 +286,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       int64_t jt, ck;
       decode(g, it, l, jt, ck);
       const int64_t j0 = jt * TCH;
-      const int64_t nbeg = ck * CHUNK;
-      const int64_t nend = (nbeg + CHUNK < g.N) ? nbeg + CHUNK : g.N;
+      const int64_t nbeg = ck * g.chunk;
+      const int64_t nend = (nbeg + g.chunk < g.N) ? nbeg + g.chunk : g.N;
       float sq = 0.f;
       double sqd = 0.0;
       for (int64_t n0 = nbeg; n0 < nend; n0 += TM, ++tcount) {
@@ -416,12 +418,23 @@ __global__ void __launch_bounds__(256) k_reduce_partials(const double* __restric
 
 }  // namespace
 
-int64_t targets_num_partials(int64_t N, int64_t d) {
-  return ((d + TCH - 1) / TCH) * ((N + CHUNK - 1) / CHUNK) * 4;
+// Tokens per work item: 32 tiles, which spread the split of Q_l over 4096 tokens, halved while the items
+// are fewer than two per SM (152 SMs) and so leave SMs idle (at L = 6, d = 328, N = 1501: 12 items of 12 tiles,
+// 28 us; 144 of one tile, 8 us).
+static int64_t targets_chunk(int64_t N, int L, int64_t d) {
+  int64_t tiles = MAX_CHUNK_TILES;
+  const int64_t cols = int64_t(L) * ((d + TCH - 1) / TCH), all = (N + TM - 1) / TM;
+  while (tiles > 1 && cols * ((all + tiles - 1) / tiles) < 2 * 152) tiles /= 2;
+  return tiles * TM;
+}
+
+int64_t targets_num_partials(int64_t N, int L, int64_t d) {
+  const int64_t chunk = targets_chunk(N, L, d);
+  return ((d + TCH - 1) / TCH) * ((N + chunk - 1) / chunk) * 4;
 }
 
 size_t targets_workspace_bytes(int64_t N, int L, int64_t d) {
-  return align256(sizeof(double) * size_t(L) * size_t(targets_num_partials(N, d))) + 256;
+  return align256(sizeof(double) * size_t(L) * size_t(targets_num_partials(N, L, d))) + 256;  // never 0
 }
 
 int targets_max_C() { return kMaxC; }
@@ -442,13 +455,10 @@ cudaError_t launch_targets(const float* E, int64_t N, int C, const float* P, con
   g.rp = (r + 7) / 8 * 8;
   g.L = L;
   g.nd = (d + TCH - 1) / TCH;
-  g.nchunks = (N + CHUNK - 1) / CHUNK;
+  g.chunk = targets_chunk(N, L, d);
+  g.nchunks = (N + g.chunk - 1) / g.chunk;
   g.items = int64_t(L) * g.nd * g.nchunks;
   double* partials = tsq ? static_cast<double*>(workspace) : nullptr;
-  int32_t* abort_flag = reinterpret_cast<int32_t*>(
-      static_cast<char*>(workspace) + align256(sizeof(double) * size_t(L) * size_t(targets_num_partials(N, d))));
-  cudaError_t e = cudaMemsetAsync(abort_flag, 0, sizeof(int32_t), s);
-  if (e != cudaSuccess) return e;
   int64_t grid = sm_count();
   if (grid > g.items) grid = g.items;
   // bf16 output with 16-byte rows: tiles leave through TMA stores, 128-byte swizzled boxes of 64
@@ -484,20 +494,21 @@ cudaError_t launch_targets(const float* E, int64_t N, int C, const float* P, con
   const Layout lay = layout_for(g.rp);
   const size_t shm = lay.total;
   const unsigned long long limit = wait_limit_ns();
+  cudaError_t e;
   if (t_dtype == LOCA_BF16) {
     e = cudaFuncSetAttribute(k_targets_tc<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(shm));
     if (e != cudaSuccess) return e;
     k_targets_tc<true><<<unsigned(grid), NTHREADS, shm, s>>>(E, P, Q, g, T, tmT, store_mode, partials, status,
-                                                             abort_flag, limit);
+                                                             limit);
   } else {
     e = cudaFuncSetAttribute(k_targets_tc<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(shm));
     if (e != cudaSuccess) return e;
     k_targets_tc<false><<<unsigned(grid), NTHREADS, shm, s>>>(E, P, Q, g, T, tmT, 0, partials, status,
-                                                              abort_flag, limit);
+                                                              limit);
   }
   e = cudaGetLastError();
   if (e != cudaSuccess || tsq == nullptr) return e;
-  k_reduce_partials<<<L, 256, 0, s>>>(partials, targets_num_partials(N, d), tsq);
+  k_reduce_partials<<<L, 256, 0, s>>>(partials, targets_num_partials(N, L, d), tsq);
   return cudaGetLastError();
 }
 
