@@ -105,6 +105,7 @@ struct Geo {
   int per_block;    // work items per block l
   int rpb, main;    // rounds of a block's own and the items of it that fill them (0, 0: none)
   int ways;         // clusters per item in a last, partial round
+  int clusters;     // clusters with items
   int gram;         // 1: Gram tiles are computed (0: a later column range of a factored launch)
   int factored;     // 1: a cross slot is S = U^T X of its column tile, not a tile of T^T X
   int s0, s1;       // factored: column tiles with an S slot (s0 <= nt < s1)
@@ -227,6 +228,7 @@ __device__ __forceinline__ Sched schedule(const Geo& g, int c, int n, int nkb, i
   const int left = g.L * v.per;
   v.R = left / n;
   v.rem = left - v.R * n;
+  if (c >= n) v.own = v.R = v.rem = 0;  // a cluster that only takes steps
   return v;
 }
 // The t-th item of cluster c of n; false when it has none left.  Lockstep: `before` sync counts come from
@@ -393,21 +395,125 @@ __global__ void __launch_bounds__(256) k_expand_cross(const float* __restrict__ 
 }
 
 constexpr int kThreads = 192;
+constexpr int kStepWarps = 6;   // further warps that take the step (4: 111 us at d = 256, L = 28, N = 8192; 6: 95; 8: 98)
 constexpr int kBufs = 2;  // staging boxes per epilogue warp
 constexpr int kEpiBytes = 4 * kBufs * EPI_BOX_BYTES;
 constexpr int kBars = 2 * STAGES + 3;  // full[S], empty[S], acc_full, acc_empty, drain
 constexpr int kBarBytes = 256;
 constexpr int kSmem = STAGES * STAGE_BYTES + kEpiBytes + 1024 + kBarBytes;
 static_assert(kSmem <= 232448, "shared memory per CTA");
-static_assert(kBars * 8 + 8 <= kBarBytes, "barrier area");  // + TMEM slot, odd count
+static_assert(kBars * 8 + 12 <= kBarBytes, "barrier area");  // + TMEM slot, odd count, ticket
 
 // ------------------------------------------------------------------ kernel
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
+// Bounded wait for a counter in global memory; what was written before its last addition is then visible.
+__device__ __forceinline__ bool count_wait(const uint32_t* ctr, uint32_t target, const WaitCtl& wc) {
+  const uint64_t t0 = globaltimer();
+  bool ok = true;
+  while (*reinterpret_cast<const volatile uint32_t*>(ctr) < target && ok) {
+    if (globaltimer() - t0 > wc.limit_ns) {
+      atomicExch(wc.status, int32_t(LOCA_ERR_TIMEOUT));
+      *wc.abort_flag = 1;
+      __threadfence();
+      ok = false;
+    } else if (*wc.abort_flag != 0) {
+      ok = false;
+    }
+  }
+  __threadfence();
+  return ok;
+}
+
+// ------------------------------------------------------------------ step
+// alpha_l = -eta sqrt(||X_l||^2 / tsq_l) and xsq_total, taken by warps of the statistics kernel itself
+// while the tensor cores work: the cross tiles need alpha_l in their epilogues only.  A kernel of its
+// own reads X at the HBM's pace while the tensor cores idle: with k_step it added 95 us to the 762 of the
+// statistics at L = 24, d = 896, N = 16384 (757 with the step inside), 55 to 1045 at L = 28, d = 1536,
+// N = 8192 (1012), 23 to 31 at L = 6, d = 328, N = 1501 (34).
+struct Step {
+  const uint4* X;       // NULL: alpha was written by an earlier launch
+  int64_t nvec;         // 16-byte vectors of a block of X (N d / 8)
+  int64_t chunk;        // vectors a chunk
+  int chunks;           // chunks of a block, at most kSumsqPartials - 1
+  int zero_first;
+  float eta;
+  const double* tsq;
+  double* xsq_total;
+  float* alpha;
+  double* partials;     // L x chunks
+  uint32_t* claim;      // chunks handed out
+  uint32_t* done;       // per block: chunks summed, one more when alpha_l is there
+};
+
+// Chunks are handed out in order of the blocks, by a counter: a warp that has one waits for nothing, so every
+// block's step is taken however few CTAs are resident.  The partial sums of a block are added in the
+// order of its chunks, whoever summed them.
+__device__ __forceinline__ void take_step(const Step& p, int L, int lane) {
+  const int64_t all = int64_t(L) * p.chunks;
+  for (;;) {
+    uint32_t c = 0;
+    if (lane == 0) c = atomicAdd(p.claim, 1u);
+    c = __shfl_sync(0xffffffffu, c, 0);
+    if (int64_t(c) >= all) break;
+    const int l = int(c) / p.chunks;
+    const int64_t v0 = int64_t(int(c) - l * p.chunks) * p.chunk;
+    const int64_t v1 = v0 + p.chunk < p.nvec ? v0 + p.chunk : p.nvec;
+    const uint4* x = p.X + int64_t(l) * p.nvec;
+    double acc = 0.0;
+    for (int64_t v = v0 + lane; v < v1; v += 32 * 8) {
+      uint4 q[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const int64_t vi = v + 32 * i;
+        q[i] = vi < v1 && LOCA_CHECK(vi, p.nvec) ? __ldg(x + vi) : make_uint4(0u, 0u, 0u, 0u);
+      }
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        float part = 0.f;
+#pragma unroll
+        for (int i = 4 * h; i < 4 * h + 4; ++i) {
+          const uint32_t w[4] = {q[i].x, q[i].y, q[i].z, q[i].w};
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const float a = __uint_as_float(w[j] << 16), b = __uint_as_float(w[j] & 0xffff0000u);
+            part = fmaf(a, a, part);
+            part = fmaf(b, b, part);
+          }
+        }
+        acc += part;
+      }
+    }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
+    uint32_t before = 0;
+    if (lane == 0) {
+      if (LOCA_CHECK(c, all)) p.partials[c] = acc;
+      __threadfence();
+      before = atomicAdd(p.done + l, 1u);
+    }
+    before = __shfl_sync(0xffffffffu, before, 0);
+    if (before != uint32_t(p.chunks) - 1u) continue;
+    __threadfence();  // every partial sum of the block is visible
+    double xb = 0.0;
+#pragma unroll 4
+    for (int i = lane; i < p.chunks; i += 32) xb += __ldcg(p.partials + int64_t(l) * p.chunks + i);
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) xb += __shfl_xor_sync(0xffffffffu, xb, off);
+    if (lane == 0) {
+      const double ts = p.tsq[l];
+      p.alpha[l] = ts > 0.0 ? float(-double(p.eta) * sqrt(xb / ts)) : 0.f;
+      p.xsq_total[l] = (p.zero_first ? 0.0 : p.xsq_total[l]) + xb;
+      __threadfence();
+      atomicAdd(p.done + l, 1u);
+    }
+  }
+}
+
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads + 32 * kStepWarps, 1)
     k_gram_cross_tc(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmT,
                     const __grid_constant__ CUtensorMap tmXa, const __grid_constant__ CUtensorMap tmTa,
                     const __grid_constant__ CUtensorMap tmXb, const __grid_constant__ CUtensorMap tmG,
                     const __grid_constant__ CUtensorMap tmC, int blocked, Geo g, int seg_kb,
-                    const float* __restrict__ alpha, int zero_first, int32_t* status, int32_t* abort_flag,
+                    const float* alpha, int zero_first, Step step, int32_t* status, int32_t* abort_flag,
                     uint32_t* round_ctr, uint32_t* split_ctr, unsigned long long limit_ns, unsigned long long sync_ns) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
@@ -416,6 +522,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   uint64_t* bars = reinterpret_cast<uint64_t*>(epi + kEpiBytes);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + kBars);
   uint32_t* odd_issued = tmem_slot + 1;  // even CTA: pipeline iterations the odd CTA issued
+  uint32_t* ticket = tmem_slot + 2;      // even CTA: the cluster's number (shared items)
   const uint32_t smem_base = smem_u32(smem);
   const uint32_t bar_base = smem_u32(bars);
   auto full_bar = [&](int s) { return bar_base + 8u * s; };
@@ -428,8 +535,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   const int lane = threadIdx.x & 31;
   const uint32_t rank = cluster_ctarank();
   const bool leader = rank == 0;
-  const int cid = int(cluster_id_x());
-  const int ncl = int(ncluster_x());
   const WaitCtl wc{status, abort_flag, limit_ns};
   // bytes CTA `rk` loads per stage of an item: its half of B and of every A tile; the at most 64
   // rows of U (an S slot) are the even CTA's alone, the rest of that A tile is not loaded (its
@@ -450,6 +555,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     mbar_init(acc_empty, 8);  // lane 0 of the 4 epilogue warps of each CTA
     mbar_init(drain_bar, 1);
     *odd_issued = 0;
+    // Shared items: a cluster waits for those with the earlier tokens, so clusters are numbered in the
+    // order in which they start, and only ones that are running are waited for.
+    if (leader && g.ways > 1) *ticket = atomicAdd(round_ctr + kGramFlags - 3, 1u);
     mbar_init_fence();
     if (blocked) {
       prefetch_tensormap(&tmXa);
@@ -466,8 +574,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   cluster_sync();  // barriers of both CTAs initialised, TMEM allocated
   fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  const int cid = g.ways > 1 ? int(ld_shared_cluster_u32(mapa_shared(smem_u32(ticket), 0))) : int(cluster_id_x());
   const int nkb = (g.N + BK - 1) / BK;
-  const Sched sched = schedule(g, cid, ncl, nkb, seg_kb);
+  const Sched sched = schedule(g, cid, g.clusters, nkb, seg_kb);
   uint32_t iters_done = 0;  // producer: pipeline iterations this CTA issued
 
   if (warp == 0) {
@@ -606,6 +715,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       }
     }
     __syncwarp();
+  } else if (warp >= 2 + 4) {
+    take_step(step, g.L, lane);
   } else {
     // ---------------- epilogue: warps 2..5, TMEM lane quarter = warp % 4
     const int q = warp & 3;
@@ -618,7 +729,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     Item w;
     int before, active;
     for (int t = 0; go && item_at(g, sched, t, w, before, active); ++t) {
-      const float al = alpha[w.l];
+      float al = 1.f;
+      const bool cross = !g.factored && !(w.gram0 && (w.nslots == 1 || w.gram1));
       const int nseg = (w.kb1 - w.kb0 + seg_kb - 1) / seg_kb;
       for (int seg = 0; seg < nseg && go; ++seg) {
         const bool ok = mbar_wait_cluster(acc_full, acc_phase, wc);
@@ -630,22 +742,23 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         // the previous segment's additions to these boxes are complete: fixed order of additions
         if (seg > 0 && lane == 0) bulk_wait_group0();
         __syncwarp();
+        if (cross && seg == 0) {  // alpha_l, of this launch's step warps or of an earlier launch
+          bool ready = true;
+          if (lane == 0) {
+            if (step.X != nullptr) ready = count_wait(step.done + w.l, uint32_t(step.chunks) + 1u, wc);
+            al = __ldcg(alpha + w.l);
+          }
+          al = __shfl_sync(0xffffffffu, al, 0);
+          if (!__shfl_sync(0xffffffffu, int(ready), 0)) {
+            go = false;
+            break;
+          }
+        }
         if (w.part > 0 && seg == 0) {
           // an item shared by clusters: the additions of the earlier parts (8 warps each) are complete
           bool ready = true;
           if (lane == 0) {
-            const uint64_t t0 = globaltimer();
-            while (*reinterpret_cast<const volatile uint32_t*>(split_ctr + w.split) < 8u * uint32_t(w.part) && ready) {
-              if (globaltimer() - t0 > wc.limit_ns) {
-                atomicExch(wc.status, int32_t(LOCA_ERR_TIMEOUT));
-                *wc.abort_flag = 1;
-                __threadfence();
-                ready = false;
-              } else if (*wc.abort_flag != 0) {
-                ready = false;
-              }
-            }
-            __threadfence();
+            ready = count_wait(split_ctr + w.split, 8u * uint32_t(w.part), wc);
             asm volatile("fence.proxy.async;" ::: "memory");
           }
           if (!__shfl_sync(0xffffffffu, int(ready), 0)) {
@@ -847,7 +960,7 @@ int resident_clusters() {
   int clusters = sm_count() / 2;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(unsigned(2 * clusters));
-  cfg.blockDim = dim3(kThreads);
+  cfg.blockDim = dim3(kThreads + 32 * kStepWarps);
   cfg.dynamicSmemBytes = kSmem;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeClusterDimension;
@@ -878,24 +991,25 @@ int deal_items(Geo& g, int n, int64_t nkb) {
   // Rounds of a block's own: whole ones, and a last one at least nine tenths full.
   g.rpb = total <= n ? 0 : g.per_block / n + (g.per_block % n * 10 >= n * 9 ? 1 : 0);
   g.main = g.per_block < g.rpb * n ? g.per_block : g.rpb * n;
-  // A last round (or only one) that leaves at least half the clusters idle: its items in up to four token
+  // A last round (or only one) that leaves at least half the clusters idle: its items in token
   // ranges.  A range costs an epilogue of its own (~9 us, one after the other) and saves its share of the
   // ~0.57 us per k-block, so two ranges pay from 96 k-blocks on, three from 128, four from 192; items of
   // several accumulation segments are cut between segments only, so that the sums do not depend on the ways.
   const int64_t left = total - int64_t(g.main) * g.L;
   const int64_t rem = total <= n ? total : left % n;
   const int64_t nsegs = (nkb + kSegTokens / BK - 1) / (kSegTokens / BK);
-  int64_t most = nkb >= 192 ? 4 : (nkb >= 128 ? 3 : (nkb >= 96 ? 2 : 1));
-  if (nsegs > 1 && most > nsegs) most = nsegs;
-  if (rem > kGramFlags - 2) most = 1;  // a counter per shared item
+  // A range's later segments wait for the ranges before it, so `ways` ranges save ways - 1 segments.
+  int64_t most = nsegs > 1 ? nsegs : (nkb >= 192 ? 4 : (nkb >= 128 ? 3 : (nkb >= 96 ? 2 : 1)));
+  if (rem > kGramFlags - 4) most = 1;  // a counter per shared item
   if (rem > 0 && most > n / rem) most = n / rem;
   g.ways = most > 1 && rem > 0 ? int(most) : 1;
-  return int((int64_t(g.rpb) * g.L + (total <= n ? 0 : left / n)) * 12 + (rem > 0 ? 12 / g.ways : 0));
+  const int64_t last = rem == 0 ? 0 : (nsegs > 1 ? 12 * (nsegs - g.ways + 1) / nsegs : 12 / g.ways);
+  return int((int64_t(g.rpb) * g.L + (total <= n ? 0 : left / n)) * 12 + last);
 }
 
 cudaError_t launch_stats(const void* X, const void* T, int L, int64_t N, int64_t d, const float* alpha,
                          int zero_first, float* gram, float* cross, int32_t* status, int32_t* abort_flag,
-                         bool flags_clear, const Factored& f, cudaStream_t s) {
+                         bool flags_clear, const Factored& f, const Step& step, cudaStream_t s) {
   CUtensorMap mx, mt, mxa, mta, mxb, mg, mc;
   memset(&mta, 0, sizeof(mta));
   memset(&mxa, 0, sizeof(mxa));
@@ -945,11 +1059,13 @@ cudaError_t launch_stats(const void* X, const void* T, int L, int64_t N, int64_t
   alone.odd_pairs = 0;
   if (deal_items(alone, most_clusters, nkb) <= paired) g = alone;
   const int64_t total = int64_t(g.per_block) * L;
-  const int n = total <= most_clusters ? int(total) * g.ways : most_clusters;
+  g.clusters = total <= most_clusters ? int(total) * g.ways : most_clusters;
   uint32_t* ctr = reinterpret_cast<uint32_t*>(abort_flag + 1);
-  k_gram_cross_tc<<<unsigned(2 * n), kThreads, kSmem, s>>>(mx, mt, mxa, mta, mxb, mg, mc, blocked, g, kSegTokens / BK,
-                                                                  alpha, zero_first, status, abort_flag, ctr, ctr + 1,
-                                                                  wait_limit_ns(), sync_ns);
+  const int n = step.X ? most_clusters : g.clusters;  // clusters without items take steps
+  const unsigned threads = kThreads + (step.X ? 32 * kStepWarps : 0);
+  k_gram_cross_tc<<<unsigned(2 * n), threads, kSmem, s>>>(mx, mt, mxa, mta, mxb, mg, mc, blocked, g, kSegTokens / BK,
+                                                          alpha, zero_first, step, status, abort_flag, ctr, ctr + 1,
+                                                          wait_limit_ns(), sync_ns);
   e = cudaGetLastError();
   if (e != cudaSuccess || !g.gram) return e;
   const int nt = int((d + MIR_T - 1) / MIR_T);
@@ -961,9 +1077,36 @@ cudaError_t launch_stats(const void* X, const void* T, int L, int64_t N, int64_t
 
 cudaError_t launch_gram_cross_tc(const void* X, const void* T, int L, int64_t N, int64_t d,
                                  const float* alpha, int zero_first, float* gram, float* cross,
-                                 int32_t* status, int32_t* abort_flag, bool flags_clear, cudaStream_t s) {
+                                 int32_t* status, int32_t* abort_flag, cudaStream_t s) {
   const Factored none{0, 0, 0, 1};
-  return launch_stats(X, T, L, N, d, alpha, zero_first, gram, cross, status, abort_flag, flags_clear, none, s);
+  return launch_stats(X, T, L, N, d, alpha, zero_first, gram, cross, status, abort_flag, false, none, Step{}, s);
+}
+
+cudaError_t launch_accumulate_tc(const void* X, const void* T, int L, int64_t N, int64_t d, const double* tsq,
+                                 float eta, int zero_first, float* gram, float* cross, double* xsq_total,
+                                 float* alpha, int32_t* status, int32_t* abort_flag, cudaStream_t s) {
+  Step p;
+  p.X = static_cast<const uint4*>(X);
+  p.nvec = N * d / 8;  // d % 8 == 0 on this path
+  // chunks of at least 8 KB; a block's row of partial sums but one word, which holds its counter
+  p.chunk = (p.nvec + kSumsqPartials - 2) / (kSumsqPartials - 1);
+  if (p.chunk < 512) p.chunk = 512;
+  p.chunk = (p.chunk + 255) / 256 * 256;  // whole trips of the warp's loop
+  p.chunks = int((p.nvec + p.chunk - 1) / p.chunk);
+  p.zero_first = zero_first;
+  p.eta = eta;
+  p.tsq = tsq;
+  p.xsq_total = xsq_total;
+  p.alpha = alpha;
+  p.partials = reinterpret_cast<double*>(alpha) - int64_t(L) * kSumsqPartials;
+  p.done = reinterpret_cast<uint32_t*>(alpha) - L;
+  p.claim = reinterpret_cast<uint32_t*>(abort_flag) + kGramFlags - 1;
+  // the counters, alpha and the launch's flags lie side by side: one memset
+  const size_t bytes = size_t(reinterpret_cast<char*>(abort_flag + kGramFlags) - reinterpret_cast<char*>(p.done));
+  const cudaError_t e = cudaMemsetAsync(p.done, 0, bytes, s);
+  if (e != cudaSuccess) return e;
+  const Factored none{0, 0, 0, 1};
+  return launch_stats(X, T, L, N, d, alpha, zero_first, gram, cross, status, abort_flag, true, none, p, s);
 }
 
 int gram_fused_max_r() { return 32; }
@@ -992,7 +1135,7 @@ cudaError_t gram_cross_factored(const void* X, const float* E, int C, const floa
   for (int64_t c0 = 0; c0 < d; c0 += kColGroup) {
     const int64_t cw = d - c0 < kColGroup ? d - c0 : kColGroup;
     const Factored f{2 * RP, int(c0 / BN), int((c0 + cw + BN - 1) / BN), c0 == 0 ? 1 : 0};
-    e = launch_stats(X, U, L, N, d, alpha, zero_first, gram, S, status, flags, c0 == 0, f, s);
+    e = launch_stats(X, U, L, N, d, alpha, zero_first, gram, S, status, flags, c0 == 0, f, Step{}, s);
     if (e != cudaSuccess) return e;
     const dim3 grid(unsigned((cw + EX_COLS - 1) / EX_COLS), unsigned((d + ex_rows(RP) - 1) / ex_rows(RP)), unsigned(L));
     k_expand_cross<RP><<<grid, 256, 0, s>>>(S, cw, Q, r, int(d), int(c0), int(cw), alpha, zero_first, cross);

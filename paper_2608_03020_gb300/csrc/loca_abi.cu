@@ -139,7 +139,7 @@ struct AccumWs {
 AccumWs accum_ws(int32_t L) {
   AccumWs w{};
   w.partials = 0;
-  w.alpha = align256(sizeof(double) * size_t(L) * size_t(sumsq_num_partials()));
+  w.alpha = align256(sizeof(double) * size_t(L) * size_t(kSumsqPartials));
   w.abort_flag = w.alpha + align256(sizeof(float) * size_t(L));
   w.total = w.abort_flag + 256;
   return w;
@@ -339,15 +339,15 @@ int validate_accumulate(const void* X, const void* T, int dtype, int32_t L, int6
 
 int run_batch_step(const void* X, int dtype, int32_t L, int64_t N, int64_t d, const double* tsq,
                    float eta, int zero_first, double* xsq_total, float* alpha, double* partials,
-                   int32_t* flags, cudaStream_t s) {
-  cudaError_t e = launch_sumsq_and_step(X, dtype, L, N, d, tsq, eta, zero_first, xsq_total, partials, alpha, flags, s);
+                   cudaStream_t s) {
+  cudaError_t e = launch_sumsq_and_step(X, dtype, L, N, d, tsq, eta, zero_first, xsq_total, partials, alpha, s);
   if (e != cudaSuccess) return cuda_fail(e, "batch step: sum of squares");
   return LOCA_OK;
 }
 
 int run_gram_cross(const void* X, const void* T, int dtype, int32_t L, int64_t N, int64_t d,
                    const float* alpha, int zero_first, float* gram, float* cross, int32_t* abort_flag,
-                   bool flags_clear, cudaStream_t s) {
+                   cudaStream_t s) {
   cudaError_t e = cudaSuccess;
   if (N == 0) {
     if (zero_first) {
@@ -360,7 +360,7 @@ int run_gram_cross(const void* X, const void* T, int dtype, int32_t L, int64_t N
   if (dtype == LOCA_BF16) {
     int32_t* status = device_status_word();
     if (!status) return fail(LOCA_ERR_CUDA, "cannot resolve the device status word");
-    e = launch_gram_cross_tc(X, T, L, N, d, alpha, zero_first, gram, cross, status, abort_flag, flags_clear, s);
+    e = launch_gram_cross_tc(X, T, L, N, d, alpha, zero_first, gram, cross, status, abort_flag, s);
   } else {
     e = launch_gram_cross_f32(static_cast<const float*>(X), static_cast<const float*>(T), L, N, d,
                               alpha, zero_first, gram, cross, s);
@@ -369,11 +369,28 @@ int run_gram_cross(const void* X, const void* T, int dtype, int32_t L, int64_t N
   return LOCA_OK;
 }
 
+int run_accumulate(const void* X, const void* T, int dtype, int32_t L, int64_t N, int64_t d, const double* tsq,
+                   float eta, int zero_first, float* gram, float* cross, double* xsq_total, float* alpha,
+                   int32_t* abort_flag, cudaStream_t s) {
+  if (dtype == LOCA_BF16 && N > 0) {
+    int32_t* status = device_status_word();
+    if (!status) return fail(LOCA_ERR_CUDA, "cannot resolve the device status word");
+    const cudaError_t e = launch_accumulate_tc(X, T, L, N, d, tsq, eta, zero_first, gram, cross, xsq_total, alpha,
+                                               status, abort_flag, s);
+    if (e != cudaSuccess) return cuda_fail(e, "loca_accumulate launch");
+    return LOCA_OK;
+  }
+  double* partials = reinterpret_cast<double*>(alpha) - int64_t(L) * kSumsqPartials;
+  const int rc = run_batch_step(X, dtype, L, N, d, tsq, eta, zero_first, xsq_total, alpha, partials, s);
+  if (rc != LOCA_OK) return rc;
+  return run_gram_cross(X, T, dtype, L, N, d, alpha, zero_first, gram, cross, abort_flag, s);
+}
+
 }  // namespace loca
 
 namespace {
 
-size_t batch_step_ws(int32_t L) { return align256(sizeof(double) * size_t(L) * size_t(sumsq_num_partials())); }
+size_t batch_step_ws(int32_t L) { return align256(sizeof(double) * size_t(L) * size_t(kSumsqPartials)); }
 constexpr size_t kGramCrossWs = 256;
 
 }  // namespace
@@ -400,7 +417,7 @@ int loca_batch_step(const void* X, int dtype, int32_t L, int64_t N, int64_t d, c
   rc = check_ws(workspace, workspace_bytes, batch_step_ws(L));
   if (rc != LOCA_OK) return rc;
   return run_batch_step(X, dtype, L, N, d, tsq, eta, zero_first, xsq_total, alpha,
-                        reinterpret_cast<double*>(workspace), nullptr, static_cast<cudaStream_t>(stream));
+                        reinterpret_cast<double*>(workspace), static_cast<cudaStream_t>(stream));
 }
 
 int loca_gram_cross_workspace_size(size_t* bytes) {
@@ -421,7 +438,7 @@ int loca_gram_cross(const void* X, const void* T, int dtype, int32_t L, int64_t 
   rc = check_ws(workspace, workspace_bytes, kGramCrossWs);
   if (rc != LOCA_OK) return rc;
   return run_gram_cross(X, T, dtype, L, N, d, alpha, zero_first, gram, cross,
-                        reinterpret_cast<int32_t*>(workspace), false, static_cast<cudaStream_t>(stream));
+                        reinterpret_cast<int32_t*>(workspace), static_cast<cudaStream_t>(stream));
 }
 
 int loca_targets_sq_workspace_size(int64_t N, int32_t C, size_t* bytes) {
@@ -473,7 +490,7 @@ int loca_gram_cross_fused(const void* X, int dtype, int32_t L, int64_t N, int64_
   rc = check_ws(workspace, workspace_bytes, gram_fused_workspace_bytes(L, N, r));
   if (rc != LOCA_OK) return rc;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  if (N == 0) return run_gram_cross(X, X, dtype, L, N, d, alpha, zero_first, gram, cross, nullptr, false, s);
+  if (N == 0) return run_gram_cross(X, X, dtype, L, N, d, alpha, zero_first, gram, cross, nullptr, s);
   int32_t* status = device_status_word();
   if (!status) return fail(LOCA_ERR_CUDA, "cannot resolve the device status word");
   const cudaError_t e = launch_gram_cross_fused_tc(X, E, C, P, Q, r, L, N, d, alpha, zero_first, gram, cross, status,
@@ -502,12 +519,9 @@ int loca_accumulate(const void* X, const void* T, int dtype, int32_t L, int64_t 
   rc = check_ws(workspace, workspace_bytes, lay.total);
   if (rc != LOCA_OK) return rc;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  float* alpha = reinterpret_cast<float*>(ws_at(workspace, lay.alpha));
-  int32_t* flags = reinterpret_cast<int32_t*>(ws_at(workspace, lay.abort_flag));
-  rc = run_batch_step(X, dtype, L, N, d, tsq, eta, zero_first, xsq_total, alpha,
-                      reinterpret_cast<double*>(ws_at(workspace, lay.partials)), flags, s);
-  if (rc != LOCA_OK) return rc;
-  return run_gram_cross(X, T, dtype, L, N, d, alpha, zero_first, gram, cross, flags, true, s);
+  return run_accumulate(X, T, dtype, L, N, d, tsq, eta, zero_first, gram, cross, xsq_total,
+                        reinterpret_cast<float*>(ws_at(workspace, lay.alpha)),
+                        reinterpret_cast<int32_t*>(ws_at(workspace, lay.abort_flag)), s);
 }
 
 int loca_accumulate_streamed(const void* X_host, void* staging, const void* T, int dtype, int32_t L,
@@ -530,7 +544,6 @@ int loca_accumulate_streamed(const void* X_host, void* staging, const void* T, i
   if (rc != LOCA_OK) return rc;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   float* alpha = reinterpret_cast<float*>(ws_at(workspace, lay.alpha));
-  double* partials = reinterpret_cast<double*>(ws_at(workspace, lay.partials));
   int32_t* flags = reinterpret_cast<int32_t*>(ws_at(workspace, lay.abort_flag));
   if (N == 0)  // nothing to copy: the statistics of an empty batch
     return loca_accumulate(staging, T, dtype, L, N, d, tsq, eta, zero_first, gram, cross, xsq_total,
@@ -552,11 +565,9 @@ int loca_accumulate_streamed(const void* X_host, void* staging, const void* T, i
     if (e == cudaSuccess) e = cudaStreamWaitEvent(s, lane->copied[slot], 0);
     if (e != cudaSuccess) return cuda_fail(e, "streamed accumulate: copy");
     const char* Tg = static_cast<const char*>(T) + size_t(l0) * block_bytes;
-    rc = run_batch_step(dst, dtype, nb, N, d, tsq + l0, eta, zero_first, xsq_total + l0, alpha + l0,
-                        partials + size_t(l0) * size_t(sumsq_num_partials()), flags, s);
-    if (rc != LOCA_OK) return rc;
-    rc = run_gram_cross(dst, Tg, dtype, nb, N, d, alpha + l0, zero_first, gram + size_t(l0) * dd,
-                        cross + size_t(l0) * dd, flags, true, s);
+    // the groups follow one another on s, so each has the whole workspace
+    rc = run_accumulate(dst, Tg, dtype, nb, N, d, tsq + l0, eta, zero_first, gram + size_t(l0) * dd,
+                        cross + size_t(l0) * dd, xsq_total + l0, alpha, flags, s);
     if (rc != LOCA_OK) return rc;
     e = cudaEventRecord(lane->consumed[slot], s);
     if (e != cudaSuccess) return cuda_fail(e, "streamed accumulate: event");

@@ -48,13 +48,12 @@ cudaError_t launch_targets(const float* E, int64_t N, int C, const float* P, con
                            void* workspace, int32_t* status, cudaStream_t s);
 
 // ---- statistics (stats.cu, gram_tc.cu)
-constexpr int kGramFlags = 64;  // 256 bytes
-// Sum of squares of X (per block) and the step alpha_l; partials: L x sumsq_num_partials().  flags (or
-// NULL): the kGramFlags int32 of launch_gram_cross_tc, reset for a statistics launch that follows.
-int sumsq_num_partials();
+constexpr int kGramFlags = 64;        // launch-local flags of the tensor-core statistics (256 bytes)
+constexpr int kSumsqPartials = 1024;  // partial sums of ||X_l||^2, per block
+// Sum of squares of X (per block) and the step alpha_l; partials: L x kSumsqPartials.
 cudaError_t launch_sumsq_and_step(const void* X, int dtype, int L, int64_t N, int64_t d,
                                   const double* tsq, float eta, int zero_first, double* xsq_total,
-                                  double* partials, float* alpha, int32_t* flags, cudaStream_t s);
+                                  double* partials, float* alpha, cudaStream_t s);
 // alpha_l and xsq_total[l] from tr(Gram_l) of a pass with one mini-batch (no read of X).
 cudaError_t launch_step_from_gram(const float* gram, int L, int64_t d, const double* tsq, float eta,
                                   double* xsq_total, float* alpha, cudaStream_t s);
@@ -63,11 +62,16 @@ cudaError_t launch_gram_cross_f32(const float* X, const float* T, int L, int64_t
                                   const float* alpha, int zero_first, float* gram, float* cross,
                                   cudaStream_t s);
 // bf16-input Gram / cross on tcgen05 tensor cores.  abort_flag points to kGramFlags int32 of
-// launch-local device memory (abort flag, round counter, shared items' counters), reset on stream s by
-// the launcher unless flags_clear says that the work before it on s has done so.
+// launch-local device memory (abort flag, round counter, shared items' counters), reset on stream s.
 cudaError_t launch_gram_cross_tc(const void* X, const void* T, int L, int64_t N, int64_t d,
                                  const float* alpha, int zero_first, float* gram, float* cross,
-                                 int32_t* status, int32_t* abort_flag, bool flags_clear, cudaStream_t s);
+                                 int32_t* status, int32_t* abort_flag, cudaStream_t s);
+// The same with the step of launch_sumsq_and_step (written to alpha and xsq_total) taken inside the
+// launch; N > 0.  The L x kSumsqPartials doubles that end at alpha are scratch, and so is what lies
+// between alpha's L floats and abort_flag, which follows them.
+cudaError_t launch_accumulate_tc(const void* X, const void* T, int L, int64_t N, int64_t d, const double* tsq,
+                                 float eta, int zero_first, float* gram, float* cross, double* xsq_total,
+                                 float* alpha, int32_t* status, int32_t* abort_flag, cudaStream_t s);
 
 // Gram / cross from the factors E P_l and Q_l of the targets (bf16 X only); r <= 32.
 // Workspace: launch-local flags (256 bytes), U_l = E P_l as bf16 hi / lo parts, S_l = U_l^T X_l.
@@ -91,12 +95,10 @@ int validate_stats_inputs(const void* X, const void* T, int dtype, int32_t L, in
 int validate_accumulate(const void* X, const void* T, int dtype, int32_t L, int64_t N, int64_t d,
                         const double* tsq, float eta, const float* gram, const float* cross,
                         const double* xsq_total);
-int run_batch_step(const void* X, int dtype, int32_t L, int64_t N, int64_t d, const double* tsq,
-                   float eta, int zero_first, double* xsq_total, float* alpha, double* partials,
-                   int32_t* flags, cudaStream_t s);
-int run_gram_cross(const void* X, const void* T, int dtype, int32_t L, int64_t N, int64_t d,
-                   const float* alpha, int zero_first, float* gram, float* cross, int32_t* abort_flag,
-                   bool flags_clear, cudaStream_t s);
+// One mini-batch into the statistics; alpha and abort_flag as for launch_accumulate_tc.
+int run_accumulate(const void* X, const void* T, int dtype, int32_t L, int64_t N, int64_t d, const double* tsq,
+                   float eta, int zero_first, float* gram, float* cross, double* xsq_total, float* alpha,
+                   int32_t* abort_flag, cudaStream_t s);
 
 // Limit of the bounded device waits of the tensor-core kernels (targets, k-space statistics,
 // Gram / cross): 4 s unless loca_set_wait_limit changed it.

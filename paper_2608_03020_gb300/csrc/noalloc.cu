@@ -61,12 +61,9 @@ extern "C" int loca_accumulate_noalloc(const void* X, const void* T, int dtype, 
   unsigned char* scratch = scratch_on_current_device(&e);
   if (scratch == nullptr)
     return set_error_message(LOCA_ERR_CUDA, "cannot resolve the scratch array's device address: %s", cudaGetErrorString(e));
-  double* partials = reinterpret_cast<double*>(scratch);
   float* alpha = reinterpret_cast<float*>(scratch + kPartialBytes);
   int32_t* abort_flag = reinterpret_cast<int32_t*>(scratch + kPartialBytes + kAlphaBytes);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   // the same launches as loca_accumulate, with the scratch array in place of the workspace
-  const int rs = run_batch_step(X, dtype, L, N, d, tsq, eta, zero_first, xsq_total, alpha, partials, abort_flag, s);
-  if (rs != LOCA_OK) return rs;
-  return run_gram_cross(X, T, dtype, L, N, d, alpha, zero_first, gram, cross, abort_flag, true, s);
+  return run_accumulate(X, T, dtype, L, N, d, tsq, eta, zero_first, gram, cross, xsq_total, alpha, abort_flag, s);
 }

@@ -1,6 +1,8 @@
 // Per-batch sum of squares, the scale-normalised step, and the exact-input (fp32) Gram /
 // cross-product path.
 //
+// (bf16 accumulation takes the step inside its statistics launch, gram_tc.cu; k_sumsq and k_step serve
+// loca_batch_step and the fp32 path.)
 // k_sumsq:      xsq_b[l] = ||X_l||_F^2 for this mini-batch (RMS of S8; trace of the batch Gram).
 //               Grid (G, L): each thread block reduces a contiguous share of X_l with 16-byte
 //               loads into one fp64 partial; k_step sums the G partials in a fixed order.
@@ -20,7 +22,7 @@
 namespace loca {
 namespace {
 
-constexpr int kMaxPartials = 1024;
+constexpr int kMaxPartials = kSumsqPartials;
 
 template <bool kBF16>
 __global__ void __launch_bounds__(256) k_sumsq(const void* __restrict__ Xv, int64_t N, int64_t d,
@@ -93,9 +95,7 @@ __global__ void __launch_bounds__(256) k_sumsq(const void* __restrict__ Xv, int6
 // 7-10 us a call).
 __global__ void __launch_bounds__(128) k_step(const double* __restrict__ partials, int G, int L,
                                               const double* __restrict__ tsq, float eta, int zero_first,
-                                              double* __restrict__ xsq_total, float* __restrict__ alpha,
-                                              int32_t* flags) {
-  if (flags != nullptr && blockIdx.x == 0 && threadIdx.x < kGramFlags) flags[threadIdx.x] = 0;
+                                              double* __restrict__ xsq_total, float* __restrict__ alpha) {
   const int l = blockIdx.x * 4 + int(threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (l >= L || !LOCA_CHECK(G, kMaxPartials + 1)) return;
   double xb = 0.0;
@@ -238,11 +238,9 @@ __global__ void __launch_bounds__(256) k_gram_cross_f32(const float* __restrict_
 
 }  // namespace
 
-int sumsq_num_partials() { return kMaxPartials; }
-
 cudaError_t launch_sumsq_and_step(const void* X, int dtype, int L, int64_t N, int64_t d,
                                   const double* tsq, float eta, int zero_first, double* xsq_total,
-                                  double* partials, float* alpha, int32_t* flags, cudaStream_t s) {
+                                  double* partials, float* alpha, cudaStream_t s) {
   int64_t G = (int64_t(sm_count()) * 8 + L - 1) / L;
   const int64_t n_el = N * d;
   const int64_t maxg = (n_el + 4095) / 4096;  // at least 4096 elements per thread block
@@ -262,7 +260,7 @@ cudaError_t launch_sumsq_and_step(const void* X, int dtype, int L, int64_t N, in
   } else {
     G = 0;
   }
-  k_step<<<(L + 3) / 4, 128, 0, s>>>(partials, int(G), L, tsq, eta, zero_first, xsq_total, alpha, flags);
+  k_step<<<(L + 3) / 4, 128, 0, s>>>(partials, int(G), L, tsq, eta, zero_first, xsq_total, alpha);
   return cudaGetLastError();
 }
 

@@ -272,6 +272,7 @@ def test_head_error_short_rows(lc, N, V, C, dtype, normaliser):
 @pytest.mark.parametrize("L,N,d,batches", [
     (1, 12289, 520, 2),    # 193 k-blocks, every tile an item, four token ranges each
     (2, 33000, 72, 1),     # three accumulation segments, cut between segments
+    (17, 66000, 40, 1),    # five, 34 items in two ranges each
     (13, 8200, 328, 2),    # columns of 3 and 4 tiles
     (5, 6200, 1400, 1),    # odd columns' last tiles by themselves
     (13, 700, 1400, 1),    # odd columns sharing A: five rounds instead of six
@@ -311,3 +312,35 @@ def test_gram_schedules(lc, L, N, d, batches):
             assert torch.equal(gram, gram.transpose(1, 2)) and torch.equal(gram_f, gram_f.transpose(1, 2))
     for a, b in zip(*out):
         assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("L,N,d", [
+    (1, 1, 8),           # one vector
+    (3, 1501, 328),      # a short last chunk
+    (2, 40000, 64),      # few tiles: clusters that only take steps; shared items
+    (9, 700, 1096),      # several rounds
+])
+def test_step_inside_the_statistics_launch(lc, L, N, d):
+    """loca_accumulate on bf16 against loca_batch_step + loca_gram_cross over two batches.  Sums of 32
+    squares are taken in fp32, in different groups: ||X||^2 agrees to 2 * 32 * 2^-24, alpha to half of it."""
+    g = torch.Generator(device="cuda")
+    g.manual_seed(N)
+    kw = dict(device="cuda")
+    gram, cross, gram2, cross2 = (torch.full((L, d, d), float("nan"), **kw) for _ in range(4))
+    xsq, xsq2 = (torch.full((L,), float("nan"), dtype=torch.float64, **kw) for _ in range(2))
+    alpha = torch.empty((L,), **kw)
+    ref = torch.zeros((L,), dtype=torch.float64, **kw)
+    for b in range(2):
+        X, T = (torch.randn((L, N, d), generator=g, **kw).to(torch.bfloat16) for _ in range(2))
+        tsq = T.double().square().sum((1, 2))
+        tsq[L // 2] *= float(L == 1)  # a block without a target: alpha = 0
+        ref += X.double().square().sum((1, 2))
+        lc.loca_accumulate(X, T, tsq, 0.01, gram, cross, xsq, zero_first=b == 0)
+        lc.loca_batch_step(X, tsq, 0.01, xsq2, alpha, zero_first=b == 0)
+        lc.loca_gram_cross(X, T, alpha, gram2, cross2, zero_first=b == 0)
+    torch.cuda.synchronize()
+    assert lc.loca_device_status() == 0
+    tol = 2 * 32 * 2.0 ** -24
+    assert torch.equal(gram, gram2)
+    assert torch.allclose(xsq, ref, rtol=tol, atol=0) and torch.allclose(xsq, xsq2, rtol=tol, atol=0)
+    assert float((cross - cross2).abs().max()) <= tol * float(cross2.abs().max())
