@@ -17,8 +17,8 @@
 //                 the diagonal kernel also inverts its triangular tile, so the panel and the
 //                 diagonal steps of the solves are tile products
 //   k_cr_colsolve, or k_cr_tsolve for few columns
-//                 blocked forward (L Y = W) and backward (L^T X = Y) substitution: fp64 for the
-//                 last F^T (which makes the final basis Q_Y) and for the Rayleigh-Ritz product
+//                 blocked forward (L Y = W) and backward (L^T X = Y) substitution: pairs of fp32 (2^-48;
+//                 fp64 for few columns) for the last F^T (which makes the final basis Q_Y) and for the Rayleigh-Ritz product
 //                 F Q_Y; fp32 (on an fp32 copy of the fp64 factor) inside the power iterations,
 //                 which only steer the subspace: an error there moves the starting vectors of
 //                 the next step, and the exact last F^T damps it by sigma_{ell+1} / sigma_r
@@ -32,6 +32,8 @@
 //                 P_l = Q_Y U_B,r S_r, Q_l = S_r^-1 U_B,r^T B; the entry of largest magnitude of
 //                 each Q_l row is made positive; singular values <= 1e-12 sigma_1 count as zero.
 #include <cuda_runtime.h>
+
+#include <type_traits>
 
 #include "jacobi.cuh"
 #include "loca_internal.h"
@@ -212,101 +214,160 @@ __global__ void __launch_bounds__(256) k_cr_syrk(double* __restrict__ K, int64_t
 // W (mp x n) <- K^-1 W for the NC columns of this CTA, forward then backward, in one launch: the columns
 // stay in shared memory (X, mp x NC) and the factor streams through two tile buffers (cp.async, the
 // next 64 x 64 tile in flight while one is used).  Columns do not depend on one another, so no CTA
-// waits for another.  With NC = ceil(n / SMs) every SM has the same work: fp64 is then bound by the fp64
-// pipe (m^2 NC FMAs at 2 per clock), fp32 by the stream of the factor from L2 (8 m^2 bytes per CTA).
-// Left-looking: row block ib of the solution is D(ib) (W_ib - sum_k L(ib, k) X_k), each thread taking one
-// row and a quarter of every tile's 64 columns.
-template <typename T>
-__device__ __forceinline__ void cs_tile(uint32_t dst, const T* src, int64_t ld, int tid) {
-  // 64 x 64 tile to rows of NB + 16 / sizeof(T) elements (16-byte aligned pieces)
-  constexpr int E = 16 / int(sizeof(T)), PER = NB / E, LD = NB + E;
+// waits for another.  With NC = ceil(n / SMs) every SM has the same work.  Left-looking: row block ib of
+// the solution is D(ib) (W_ib - sum_k L(ib, k) X_k), each thread taking one row and a quarter of every
+// tile's 64 columns, two of them to a packed instruction.
+// PL = 2: W is fp64, and the factor, the solution and the sums are pairs of fp32 (value and rest, 2^-48):
+// the product of the values as a two-product, the cross products of values and rests, and a two-sum, 12
+// packed instructions per two terms.  The fp64 pipe takes 2 FMAs per clock and SM, the fp32 pipe 128:
+// fp64 arithmetic took 3.97 ms a solve at m = 1536, n = 896.  The factor's own entries are sums of fp32
+// products (2^-24 each), so 2^-48 in the substitutions does not show in the result.
+// PL = 1: W and the arithmetic are fp32, bound by the stream of the factor from L2 (8 m^2 bytes per CTA).
+constexpr int CSLD = NB + 4;                // tile rows of 16-byte pieces, conflict-free by rows
+constexpr int CSTILE = NB * CSLD;           // floats of a tile
+
+__device__ __forceinline__ void cs_tile(uint32_t dst, const float* src, int64_t ld, int tid) {
+  constexpr int PER = NB / 4;
 #pragma unroll
   for (int i = 0; i < NB * PER / 256; ++i) {
-    const int e = tid + 256 * i, r = e / PER, c = (e % PER) * E;
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + uint32_t((r * LD + c) * int(sizeof(T)))),
+    const int e = tid + 256 * i, r = e / PER, c = (e % PER) * 4;
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + uint32_t((r * CSLD + c) * 4)),
                  "l"(src + int64_t(r) * ld + c)
                  : "memory");
   }
-  cp_async_commit();
 }
 
-template <typename T>
-struct Vec16;
-template <>
-struct Vec16<float> {
-  using type = float4;
-};
-template <>
-struct Vec16<double> {
-  using type = double2;
-};
-template <typename T>
-__device__ __forceinline__ void load16(const T* p, T* v) {
-  *reinterpret_cast<typename Vec16<T>::type*>(v) = *reinterpret_cast<const typename Vec16<T>::type*>(p);
+// a + b for pairs (value, rest), renormalised.
+__device__ __forceinline__ float2 pair_add(float2 a, float2 b) {
+  const float t = a.x + b.x, bb = t - a.x;
+  const float e = (a.x - (t - bb)) + (b.x - bb) + (a.y + b.y);
+  const float h = t + e;
+  return make_float2(h, e - (h - t));
 }
 
-template <typename T, int NC>
-__global__ void __launch_bounds__(256) k_cr_colsolve(const T* __restrict__ K, int64_t mp, const T* __restrict__ Dinv,
-                                                    T* __restrict__ W, int64_t n, const int32_t* flag) {
-  constexpr int E = 16 / int(sizeof(T)), LD = NB + E;
+template <int PL>
+struct Acc2 {  // sums over even and odd columns of the tile
+  uint64_t v[PL];
+  __device__ __forceinline__ void clear() {
+#pragma unroll
+    for (int p = 0; p < PL; ++p) v[p] = 0ull;
+  }
+  // += a x; na = -a where PL == 2
+  __device__ __forceinline__ void mac(const uint64_t (&a)[PL], const uint64_t (&na)[PL], const uint64_t (&x)[PL]) {
+    if constexpr (PL == 1) {
+      v[0] = fma2(a[0], x[0], v[0]);
+    } else {
+      const uint64_t p = mul2(a[0], x[0]);
+      uint64_t q = fma2(na[0], x[0], p);  // minus the product's rounding error, exactly
+      q = fma2(na[0], x[1], q);
+      q = fma2(na[1], x[0], q);
+      const uint64_t t = add2(v[0], p), bb = sub2(t, v[0]);
+      const uint64_t err = add2(sub2(v[0], sub2(t, bb)), sub2(p, bb));
+      v[1] = add2(v[1], sub2(err, q));
+      v[0] = t;
+    }
+  }
+  __device__ __forceinline__ float2 total() const {
+    const float2 h = f32x2_parts(v[0]);
+    if constexpr (PL == 1) {
+      return make_float2(h.x + h.y, 0.f);
+    } else {
+      const float2 l = f32x2_parts(v[1]);
+      return pair_add(make_float2(h.x, l.x), make_float2(h.y, l.y));
+    }
+  }
+};
+
+template <int PL, int NC>
+__global__ void __launch_bounds__(256)
+    k_cr_colsolve(const float* __restrict__ K, const float* __restrict__ Krest, int64_t mp, const float* __restrict__ Dinv,
+                  const float* __restrict__ Drest, void* __restrict__ Wv, int64_t n, const int32_t* flag) {
+  using TW = typename std::conditional<PL == 2, double, float>::type;
   extern __shared__ __align__(16) unsigned char cr_smem[];
-  T* tiles = reinterpret_cast<T*>(cr_smem);  // 2 x NB x LD
-  T* red = tiles + 2 * NB * LD;              // 4 x NC x NB partial sums
-  T* X = red + 4 * NC * NB;                  // NC x mp
+  float* tiles = reinterpret_cast<float*>(cr_smem);  // 2 x PL x CSTILE
+  float* red = tiles + 2 * PL * CSTILE;              // PL x 4 x NC x NB partial sums
+  float* X = red + PL * 4 * NC * NB;                 // PL x NC x mp
+  TW* W = static_cast<TW*>(Wv);
   if (failed(flag)) return;
   const int tid = threadIdx.x, r = tid & 63, kq = tid >> 6;
-  const int64_t c0 = int64_t(blockIdx.x) * NC;
+  const int64_t c0 = int64_t(blockIdx.x) * NC, XP = NC * mp;  // XP: floats of a plane of X
   const int nb = int(mp / NB);
   for (int64_t e = tid; e < mp * NC; e += 256) {
     const int64_t i = e / NC, c = e % NC;
-    X[c * mp + i] = c0 + c < n ? W[i * n + c0 + c] : T(0);
+    const TW w = c0 + c < n ? W[i * n + c0 + c] : TW(0);
+    X[c * mp + i] = float(w);
+    if constexpr (PL == 2) X[XP + c * mp + i] = isfinite(float(w)) ? float(w - double(float(w))) : 0.f;
   }
   const uint32_t ts = uint32_t(__cvta_generic_to_shared(tiles));
-  constexpr uint32_t TB = uint32_t(NB * LD * sizeof(T));
   // The tiles in order of use: for every row block its off-diagonal tiles, then its inverse diagonal
   // tile; forward over L's rows, backward over L's columns (used transposed).
   auto fetch = [&](bool fwd, int ib, int k, int buf) {
-    const T* src;
-    int64_t ld = mp;
-    if (k == ib) {
-      src = Dinv + int64_t(ib) * NB * NB;
-      ld = NB;
-    } else {
-      src = fwd ? K + int64_t(ib) * NB * mp + int64_t(k) * NB : K + int64_t(k) * NB * mp + int64_t(ib) * NB;
-    }
-    cs_tile(ts + uint32_t(buf) * TB, src, ld, tid);
-  };
-  T acc[NC];
-  // acc[c] += sum over this thread's quarter of the tile's row r times X block `xb`
-  auto multiply = [&](bool fwd, const T* Mt, const T* xb) {
 #pragma unroll
-    for (int u = kq * 16; u < kq * 16 + 16; u += E) {
-      T a[E];
-      if (fwd) {
-        load16(Mt + r * LD + u, a);
+    for (int p = 0; p < PL; ++p) {
+      const float* src;
+      int64_t ld = mp;
+      if (k == ib) {
+        src = (p == 0 ? Dinv : Drest) + int64_t(ib) * NB * NB;
+        ld = NB;
       } else {
+        src = (p == 0 ? K : Krest) +
+              (fwd ? int64_t(ib) * NB * mp + int64_t(k) * NB : int64_t(k) * NB * mp + int64_t(ib) * NB);
+      }
+      cs_tile(ts + uint32_t((buf * PL + p) * CSTILE) * 4u, src, ld, tid);
+    }
+    cp_async_commit();
+  };
+  Acc2<PL> acc[NC];
+  // acc[c] += sum over this thread's quarter of the tile's row r times X block `xb`
+  auto multiply = [&](bool fwd, const float* Mt, const float* xb) {
 #pragma unroll
-        for (int v = 0; v < E; ++v) a[v] = Mt[(u + v) * LD + r];
+    for (int u = kq * 16; u < kq * 16 + 16; u += 4) {
+      uint64_t a[2][PL], na[2][PL];
+#pragma unroll
+      for (int p = 0; p < PL; ++p) {
+        const float* M = Mt + p * CSTILE;
+        if (fwd) {
+          const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(M + r * CSLD + u);
+          a[0][p] = t.x;
+          a[1][p] = t.y;
+        } else {
+          a[0][p] = f32x2(M[u * CSLD + r], M[(u + 1) * CSLD + r]);
+          a[1][p] = f32x2(M[(u + 2) * CSLD + r], M[(u + 3) * CSLD + r]);
+        }
+#pragma unroll
+        for (int v = 0; v < 2; ++v) na[v][p] = a[v][p] ^ 0x8000000080000000ull;
       }
 #pragma unroll
       for (int c = 0; c < NC; ++c) {
-        T x[E];
-        load16(xb + c * mp + u, x);
+        uint64_t x[2][PL];
 #pragma unroll
-        for (int v = 0; v < E; ++v) acc[c] = fma(a[v], x[v], acc[c]);
+        for (int p = 0; p < PL; ++p) {
+          const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(xb + p * XP + c * mp + u);
+          x[0][p] = t.x;
+          x[1][p] = t.y;
+        }
+#pragma unroll
+        for (int v = 0; v < 2; ++v) acc[c].mac(a[v], na[v], x[v]);
       }
     }
   };
   auto publish = [&]() {  // this thread's partial sums, and a fresh accumulator
 #pragma unroll
     for (int c = 0; c < NC; ++c) {
-      red[(kq * NC + c) * NB + r] = acc[c];
-      acc[c] = T(0);
+      const float2 t = acc[c].total();
+      red[(kq * NC + c) * NB + r] = t.x;
+      if constexpr (PL == 2) red[4 * NC * NB + (kq * NC + c) * NB + r] = t.y;
+      acc[c].clear();
     }
   };
   auto total_of = [&](int e) {
     constexpr int Q = NC * NB;
-    return (red[e] + red[Q + e]) + (red[2 * Q + e] + red[3 * Q + e]);
+    if constexpr (PL == 1) {
+      return make_float2((red[e] + red[Q + e]) + (red[2 * Q + e] + red[3 * Q + e]), 0.f);
+    } else {
+      auto part = [&](int i) { return make_float2(red[i * Q + e], red[(4 + i) * Q + e]); };
+      return pair_add(pair_add(part(0), part(1)), pair_add(part(2), part(3)));
+    }
   };
   const int total = nb * (nb + 1) / 2;
   for (int pass = 0; pass < 2; ++pass) {
@@ -317,7 +378,7 @@ __global__ void __launch_bounds__(256) k_cr_colsolve(const T* __restrict__ K, in
     __syncthreads();
     fetch(fwd, ib, k, 0);
 #pragma unroll
-    for (int c = 0; c < NC; ++c) acc[c] = T(0);
+    for (int c = 0; c < NC; ++c) acc[c].clear();
     for (int step = 0; step < total; ++step) {
       int ibn = ib, kn = fwd ? k + 1 : k - 1;  // the tile after this one
       if (k == ib) {
@@ -331,20 +392,35 @@ __global__ void __launch_bounds__(256) k_cr_colsolve(const T* __restrict__ K, in
         cp_async_wait<0>();
       }
       __syncthreads();  // this tile has landed for every thread
-      const T* Mt = tiles + buf * NB * LD;
+      const float* Mt = tiles + buf * PL * CSTILE;
       if (k != ib) {
         multiply(fwd, Mt, X + int64_t(k) * NB);
       } else {
         // the right-hand side W_ib - sum, then times the inverse tile
-        T* Xi = X + int64_t(ib) * NB;
+        float* Xi = X + int64_t(ib) * NB;
         publish();
         __syncthreads();
-        for (int e = tid; e < NC * NB; e += 256) Xi[(e / NB) * mp + e % NB] -= total_of(e);
+        for (int e = tid; e < NC * NB; e += 256) {
+          float* xe = Xi + (e / NB) * mp + e % NB;
+          const float2 t = total_of(e);
+          if constexpr (PL == 1) {
+            *xe -= t.x;
+          } else {
+            const float2 v = pair_add(make_float2(xe[0], xe[XP]), make_float2(-t.x, -t.y));
+            xe[0] = v.x;
+            xe[XP] = v.y;
+          }
+        }
         __syncthreads();
         multiply(fwd, Mt, Xi);
         publish();
         __syncthreads();
-        for (int e = tid; e < NC * NB; e += 256) Xi[(e / NB) * mp + e % NB] = total_of(e);
+        for (int e = tid; e < NC * NB; e += 256) {
+          float* xe = Xi + (e / NB) * mp + e % NB;
+          const float2 t = total_of(e);
+          xe[0] = t.x;
+          if constexpr (PL == 2) xe[XP] = t.y;
+        }
       }
       __syncthreads();  // the tile buffer may be refilled, X_ib is complete
       buf ^= 1;
@@ -354,13 +430,17 @@ __global__ void __launch_bounds__(256) k_cr_colsolve(const T* __restrict__ K, in
   }
   for (int64_t e = tid; e < mp * NC; e += 256) {
     const int64_t i = e / NC, c = e % NC;
-    if (c0 + c < n && LOCA_CHECK(i * n + c0 + c, mp * n)) W[i * n + c0 + c] = X[c * mp + i];
+    if (c0 + c >= n || !LOCA_CHECK(i * n + c0 + c, mp * n)) continue;
+    if constexpr (PL == 1) {
+      W[i * n + c0 + c] = X[c * mp + i];
+    } else {
+      W[i * n + c0 + c] = pair_value(X[c * mp + i], X[XP + c * mp + i]);
+    }
   }
 }
 
-template <typename T>
-size_t colsolve_smem(int64_t mp, int nc) {
-  return sizeof(T) * (size_t(2) * NB * (NB + 16 / sizeof(T)) + size_t(4) * NB * nc + size_t(mp) * nc);
+constexpr size_t colsolve_smem(int planes, int64_t mp, int nc) {
+  return sizeof(float) * planes * (size_t(2) * CSTILE + size_t(4) * NB * nc + size_t(mp) * nc);
 }
 
 // Blocked substitution on W (mp x n, in place; T = double or float), one step per launch, on
@@ -433,6 +513,16 @@ template <typename TI, typename TO>
 __global__ void k_cr_cvt(const TI* __restrict__ x, TO* __restrict__ y, int64_t count) {
   for (int64_t e = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; e < count; e += int64_t(gridDim.x) * blockDim.x)
     y[e] = TO(x[e]);
+}
+
+// y + rest = x to 2^-48
+__global__ void k_cr_split(const double* __restrict__ x, float* __restrict__ y, float* __restrict__ rest, int64_t count) {
+  for (int64_t e = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; e < count; e += int64_t(gridDim.x) * blockDim.x) {
+    const double v = x[e];
+    const float h = float(v);
+    y[e] = h;
+    rest[e] = isfinite(h) ? float(v - double(h)) : 0.f;
+  }
 }
 
 constexpr int QR_STAGE = 64;   // rows staged at a time by k_cr_vtv
@@ -733,7 +823,7 @@ __global__ void __launch_bounds__(256) k_cr_ritz_sign(float* __restrict__ P, flo
 }
 
 struct RsvdWs {
-  size_t K, Dinv, Kf, Dinvf, Ym, Wm, Wf, Zd, Zf, Tn, qrpart, qrfac, part, Ur, sig, amv, ami, flag, total;
+  size_t K, Dinv, Kf, Dinvf, Krest, Drest, Ym, Wm, Wf, Zd, Zf, Tn, qrpart, qrfac, part, Ur, sig, amv, ami, flag, total;
 };
 
 RsvdWs rsvd_ws(int64_t Np, int64_t m, int64_t d, int L, int ell, int r) {
@@ -755,6 +845,8 @@ RsvdWs rsvd_ws(int64_t Np, int64_t m, int64_t d, int L, int ell, int r) {
   w.Dinv = take(sizeof(double) * nb * NB * NB);
   w.Kf = take(sizeof(float) * mp * mp);
   w.Dinvf = take(sizeof(float) * nb * NB * NB);
+  w.Krest = take(sizeof(float) * mp * mp);
+  w.Drest = take(sizeof(float) * nb * NB * NB);
   w.Ym = take(sizeof(double) * mp * n);
   w.Wm = take(sizeof(double) * mp * n);
   w.Wf = take(sizeof(float) * mp * n);
@@ -816,44 +908,64 @@ cudaError_t gtt(const float* G, const float* Tn, int64_t Np, int64_t d, int64_t 
   return cudaGetLastError();
 }
 
-template <typename T, int NC>
-cudaError_t colsolve(const T* K, int64_t mp, const T* Dinv, T* W, int64_t n, const int32_t* flag, cudaStream_t s) {
-  const size_t smem = colsolve_smem<T>(mp, NC);
-  cudaError_t e = cudaFuncSetAttribute(k_cr_colsolve<T, NC>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+// The Cholesky factor: fp64, its fp32 value and what that leaves.
+struct Factor {
+  const double *K, *Dinv;
+  const float *Kf, *Dinvf, *Krest, *Drest;
+};
+
+template <int PL, int NC>
+cudaError_t colsolve(const Factor& f, int64_t mp, void* W, int64_t n, const int32_t* flag, cudaStream_t s) {
+  const size_t smem = colsolve_smem(PL, mp, NC);
+  cudaError_t e = cudaFuncSetAttribute(k_cr_colsolve<PL, NC>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
   if (e != cudaSuccess) return e;
-  k_cr_colsolve<T, NC><<<unsigned((n + NC - 1) / NC), 256, smem, s>>>(K, mp, Dinv, W, n, flag);
+  k_cr_colsolve<PL, NC><<<unsigned((n + NC - 1) / NC), 256, smem, s>>>(f.Kf, f.Krest, mp, f.Dinvf, f.Drest, W, n, flag);
   return cudaGetLastError();
 }
 
-// W (mp x n) <- K^-1 W with K = L L^T (forward, then backward substitution), in T.  With at least one
+// Columns per CTA of k_cr_colsolve with `planes` fp32 planes, 0: k_cr_tsolve.  With at least one
 // column per two SMs, and in fp32 a factor whose triangle stays in L2 (every CTA streams all of it), the
-// columns are divided over the SMs (k_cr_colsolve).  Fewer columns leave SMs idle there, and a larger
+// columns are divided over the SMs.  Fewer columns leave SMs idle there, and a larger
 // fp32 factor would come from HBM once per CTA: then the step-by-step kernels, which spread each update
-// over the row blocks.  At m = 1536, n = 896: 13.2 ms step by step (two fp64 solves) against 7.6 ms.
-template <typename T>
-cudaError_t solve(const T* K, int64_t mp, const T* Dinv, T* W, int64_t n, const int32_t* flag, cudaStream_t s) {
+// over the row blocks.  At m = 1536, n = 896, two fp64 solves: 13.2 ms step by step, 2.4 ms in pairs.
+int colsolve_columns(int planes, int64_t mp, int64_t n) {
   constexpr size_t kMost = 232448 - 1024;
-  const bool in_l2 = sizeof(T) == 8 || mp * mp * 2 <= (int64_t(64) << 20);
-  // columns per CTA: the least time (waves x columns) over the SMs, the most columns on a tie
+  if (2 * n < sm_count() || (planes == 1 && mp * mp * 2 > (int64_t(64) << 20))) return 0;
+  // the least time (waves x columns) over the SMs, the most columns on a tie
   int64_t nc = 0, best = 0;
-  for (int c = 1; c <= 8 && colsolve_smem<T>(mp, c) <= kMost; ++c) {
+  for (int c = 1; c <= 8 && colsolve_smem(planes, mp, c) <= kMost; ++c) {
     const int64_t waves = ((n + c - 1) / c + sm_count() - 1) / sm_count();
     if (nc == 0 || waves * c <= best) {
       nc = c;
       best = waves * c;
     }
   }
-  if (2 * n >= sm_count() && in_l2 && nc > 0) {
-    switch (nc) {
-      case 1: return colsolve<T, 1>(K, mp, Dinv, W, n, flag, s);
-      case 2: return colsolve<T, 2>(K, mp, Dinv, W, n, flag, s);
-      case 3: return colsolve<T, 3>(K, mp, Dinv, W, n, flag, s);
-      case 4: return colsolve<T, 4>(K, mp, Dinv, W, n, flag, s);
-      case 5: return colsolve<T, 5>(K, mp, Dinv, W, n, flag, s);
-      case 6: return colsolve<T, 6>(K, mp, Dinv, W, n, flag, s);
-      case 7: return colsolve<T, 7>(K, mp, Dinv, W, n, flag, s);
-      default: return colsolve<T, 8>(K, mp, Dinv, W, n, flag, s);
-    }
+  return int(nc);
+}
+
+// W (mp x n) <- K^-1 W with K = L L^T (forward, then backward substitution), in T.
+template <typename T>
+cudaError_t solve(const Factor& f, int64_t mp, T* W, int64_t n, const int32_t* flag, cudaStream_t s) {
+  constexpr int PL = sizeof(T) == 8 ? 2 : 1;
+  switch (colsolve_columns(PL, mp, n)) {
+    case 0: break;
+    case 1: return colsolve<PL, 1>(f, mp, W, n, flag, s);
+    case 2: return colsolve<PL, 2>(f, mp, W, n, flag, s);
+    case 3: return colsolve<PL, 3>(f, mp, W, n, flag, s);
+    case 4: return colsolve<PL, 4>(f, mp, W, n, flag, s);
+    case 5: return colsolve<PL, 5>(f, mp, W, n, flag, s);
+    case 6: return colsolve<PL, 6>(f, mp, W, n, flag, s);
+    case 7: return colsolve<PL, 7>(f, mp, W, n, flag, s);
+    default: return colsolve<PL, 8>(f, mp, W, n, flag, s);
+  }
+  const T* K;
+  const T* Dinv;
+  if constexpr (PL == 2) {
+    K = f.K;
+    Dinv = f.Dinv;
+  } else {
+    K = f.Kf;
+    Dinv = f.Dinvf;
   }
   const int nb = int(mp / NB);
   const size_t smem = sizeof(T) * 2 * NB * NBP;
@@ -923,6 +1035,8 @@ cudaError_t rsvd_t(const float* E, const float* G, int64_t Np, int64_t m, int64_
   double* Dinv = reinterpret_cast<double*>(ws + w.Dinv);
   float* Kf = reinterpret_cast<float*>(ws + w.Kf);
   float* Dinvf = reinterpret_cast<float*>(ws + w.Dinvf);
+  float* Krest = reinterpret_cast<float*>(ws + w.Krest);
+  float* Drest = reinterpret_cast<float*>(ws + w.Drest);
   double* Ym = reinterpret_cast<double*>(ws + w.Ym);
   double* Wm = reinterpret_cast<double*>(ws + w.Wm);
   float* Wf = reinterpret_cast<float*>(ws + w.Wf);
@@ -955,7 +1069,12 @@ cudaError_t rsvd_t(const float* E, const float* G, int64_t Np, int64_t m, int64_
     }
     CR_TRY(cudaGetLastError());
   }
-  if (q > 0) {
+  const Factor f{K, Dinv, Kf, Dinvf, Krest, Drest};
+  if (colsolve_columns(2, mp, n) > 0) {
+    k_cr_split<<<2 * sm_count(), 256, 0, s>>>(K, Kf, Krest, mp * mp);
+    k_cr_split<<<2 * sm_count(), 256, 0, s>>>(Dinv, Dinvf, Drest, int64_t(nb) * NB * NB);
+    CR_TRY(cudaGetLastError());
+  } else if (q > 0) {
     CR_TRY((cvt<double, float>(K, Kf, mp * mp, s)));
     CR_TRY((cvt<double, float>(Dinv, Dinvf, int64_t(nb) * NB * NB, s)));
   }
@@ -973,20 +1092,20 @@ cudaError_t rsvd_t(const float* E, const float* G, int64_t Np, int64_t m, int64_
       k_cr_add<<<2 * sm_count(), 256, 0, s>>>(Ym, Wm, m * n);
       CR_TRY(cudaGetLastError());
     }
-    if (exact) return solve<double>(K, mp, Dinv, Ym, n, flag, s);
+    if (exact) return solve<double>(f, mp, Ym, n, flag, s);
     CR_TRY((cvt<double, float>(Ym, Wf, mp * n, s)));
-    CR_TRY(solve<float>(Kf, mp, Dinvf, Wf, n, flag, s));
+    CR_TRY(solve<float>(f, mp, Wf, n, flag, s));
     return cvt<float, double>(Wf, Ym, mp * n, s);
   };
   // Zd = F Y for every block, Y = Vm (mp x n, fp64; overwritten when exact): Wf = K^-1 Y in fp32,
   // Tn = E Wf, Zd = G_l^T Tn
   auto apply_F = [&](double* Vm, bool exact) -> cudaError_t {
     if (exact) {
-      CR_TRY(solve<double>(K, mp, Dinv, Vm, n, flag, s));
+      CR_TRY(solve<double>(f, mp, Vm, n, flag, s));
       CR_TRY((cvt<double, float>(Vm, Wf, mp * n, s)));
     } else {
       CR_TRY((cvt<double, float>(Vm, Wf, mp * n, s)));
-      CR_TRY(solve<float>(Kf, mp, Dinvf, Wf, n, flag, s));
+      CR_TRY(solve<float>(f, mp, Wf, n, flag, s));
     }
     CR_TRY((gemm<false, float>(E, m, 0, Wf, n, 0, Tn, n, 0, Np, n, m, 1, 0, s)));
     if (ell % 4 == 0 && ell <= 32)
