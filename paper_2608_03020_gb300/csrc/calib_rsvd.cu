@@ -12,14 +12,14 @@
 //
 //   k_run_gemm, k_cr_gtt   the products with E and G_l, and K itself (lower tiles only): fp32
 //                 operands, products summed in fp32 over 32 terms, those sums as fp32 pairs (2^-48)
-//   k_cr_pad      K + beta I, padded to a multiple of 64 with an identity block
-//   k_cr_potrf / k_cr_trsm / k_cr_syrk   right-looking blocked Cholesky (64 x 64 tiles, fp64);
+//   k_cr_pad      K + beta I as pairs of fp32, padded to a multiple of 64 with an identity block
+//   k_cr_potrf / k_cr_trsm / k_cr_syrk   right-looking blocked Cholesky (64 x 64 tiles, pairs of fp32);
 //                 the diagonal kernel also inverts its triangular tile, so the panel and the
 //                 diagonal steps of the solves are tile products
 //   k_cr_colsolve, or k_cr_tsolve for few columns
 //                 blocked forward (L Y = W) and backward (L^T X = Y) substitution: pairs of fp32 (2^-48;
 //                 fp64 for few columns) for the last F^T (which makes the final basis Q_Y) and for the Rayleigh-Ritz product
-//                 F Q_Y; fp32 (on an fp32 copy of the fp64 factor) inside the power iterations,
+//                 F Q_Y; fp32 (with the factor's fp32 values) inside the power iterations,
 //                 which only steer the subspace: an error there moves the starting vectors of
 //                 the next step, and the exact last F^T damps it by sigma_{ell+1} / sigma_r
 //   k_cr_vtv / k_cr_qr_factor / k_cr_qr_apply
@@ -51,186 +51,33 @@ constexpr size_t kTileSmem = sizeof(double) * 2 * NB * NBP;
 
 __device__ __forceinline__ bool failed(const int32_t* flag) { return *reinterpret_cast<const volatile int32_t*>(flag) != 0; }
 
-// K (mp x mp): rows / columns >= m become the identity; beta is added to the first m diagonal
-// entries.
-__global__ void k_cr_pad(double* __restrict__ K, int64_t m, int64_t mp, double beta) {
+// K (mp x mp) into its fp32 value and what that leaves (together 2^-48): rows / columns >= m become the
+// identity, beta is added to the first m diagonal entries.  Lower triangle of 64 x 64 tiles only.
+__global__ void k_cr_pad(const double* __restrict__ K, int64_t m, int64_t mp, double beta, float* __restrict__ Kf,
+                         float* __restrict__ Krest) {
   const int64_t total = mp * mp;
   for (int64_t e = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; e < total; e += int64_t(gridDim.x) * blockDim.x) {
     const int64_t i = e / mp, j = e % mp;
-    if (i >= m || j >= m)
-      K[e] = (i == j) ? 1.0 : 0.0;
-    else if (i == j)
-      K[e] += beta;
+    if (j / NB > i / NB) continue;
+    double v = 0.0;
+    if (i < m && j < m) v = K[e] + (i == j ? beta : 0.0);
+    else if (i == j) v = 1.0;
+    const float h = float(v);
+    Kf[e] = h;
+    Krest[e] = isfinite(h) ? float(v - double(h)) : 0.f;
   }
 }
 
-// Load a 64 x 64 fp64 tile (row stride ld) into shared memory (row stride NBP).
-__device__ __forceinline__ void load_tile(double (*S)[NBP], const double* __restrict__ src, int64_t ld) {
-  for (int e = threadIdx.x; e < NB * NB; e += blockDim.x) {
-    const int r = e / NB, c = e % NB;
-    S[r][c] = src[int64_t(r) * ld + c];
-  }
-}
-
-// Diagonal tile jb: factor in shared memory (unblocked, right-looking), write the factor back,
-// and write the inverse of the triangular factor to Dinv[jb].  A pivot that is not positive
-// sets the failure flag (E^T E + beta I is not positive definite in floating point).  One CTA, nothing
-// else beside it, so the fp64 pipe of one SM (2 FMAs per clock, predicated-off lanes included) and the
-// latency of the 64 + 64 steps bound it: the trailing entries of a step are dealt out one by one, two
-// rows of the triangle folded into one of constant length.  A 16 x 16 grid of threads that owned fixed
-// entries spent most of the pipe on entries outside the triangle (161 us a tile).
-__global__ void __launch_bounds__(256) k_cr_potrf(double* __restrict__ K, int64_t mp, int jb,
-                                                 double* __restrict__ Dinv, int32_t* flag) {
-  extern __shared__ __align__(16) unsigned char cr_smem[];
-  double(*S)[NBP] = reinterpret_cast<double(*)[NBP]>(cr_smem);
-  double(*X)[NBP] = reinterpret_cast<double(*)[NBP]>(cr_smem + sizeof(double) * NB * NBP);
-  __shared__ double rinv[NB], col[NB];
-  if (failed(flag)) return;
-  const int tid = threadIdx.x;
-  const int64_t o = int64_t(jb) * NB;
-  double* Kd = K + o * mp + o;
-  for (int e = tid; e < NB * NB; e += 256) {
-    const int r = e / NB, c = e % NB;
-    S[r][c] = (c <= r) ? Kd[int64_t(r) * mp + c] : 0.0;
-    X[r][c] = (r == c) ? 1.0 : 0.0;
-  }
-  __syncthreads();
-  // e / n for e * n < 2^20
-  auto divide = [](int e, uint32_t magic) { return int((uint32_t(e) * magic) >> 20); };
-  auto magic_of = [](int n) { return ((1u << 20) + uint32_t(n) - 1u) / uint32_t(n); };
-  for (int c = 0; c < NB; ++c) {
-    const double piv = S[c][c];
-    if (!(piv > 0.0)) {  // the same value in every thread
-      if (tid == 0) atomicExch(flag, 1);
-      return;
-    }
-    const double inv = rsqrt(piv);
-    if (tid < NB && tid > c) {
-      const double v = S[tid][c] * inv;
-      col[tid] = v;
-      Kd[int64_t(tid) * mp + c] = v;
-    }
-    if (tid == c) {
-      Kd[int64_t(c) * mp + c] = piv * inv;
-      rinv[c] = inv;
-    }
-    __syncthreads();
-    // rows c + 1 + i, i < rem, with i + 1 entries each: rows i and rem - 1 - i side by side
-    const int rem = NB - 1 - c, width = rem + 1;
-    const uint32_t mg = magic_of(width);
-    for (int e = tid; e < (rem + 1) / 2 * width; e += 256) {
-      int i = divide(e, mg), j = e - i * width;
-      if (j > i) {
-        if (rem - 1 - i == i) continue;  // the middle row stands alone
-        j -= i + 1;
-        i = rem - 1 - i;
-      }
-      S[c + 1 + i][c + 1 + j] = fma(-col[c + 1 + i], col[c + 1 + j], S[c + 1 + i][c + 1 + j]);
-    }
-    if (tid < rem) S[c + 1 + tid][c] = col[c + 1 + tid];  // column c of the factor
-    __syncthreads();
-  }
-  // X = L^-1, right-looking on the identity: row c scaled by 1 / L_cc, then removed from the rows below
-  for (int c = 0; c < NB; ++c) {
-    if (tid <= c) X[c][tid] *= rinv[c];
-    __syncthreads();
-    const uint32_t mg = magic_of(c + 1);
-    for (int e = tid; e < (NB - 1 - c) * (c + 1); e += 256) {
-      const int i = divide(e, mg), u = e - i * (c + 1);
-      X[c + 1 + i][u] = fma(-S[c + 1 + i][c], X[c][u], X[c + 1 + i][u]);
-    }
-    __syncthreads();
-  }
-  double* D = Dinv + int64_t(jb) * NB * NB;
-  for (int e = tid; e < NB * NB; e += 256) D[e] = X[e / NB][e % NB];
-}
-
-constexpr int CT = 32;         // tile of the panel and trailing updates
-constexpr int CTP = NB + 1;    // padded row of a CT x NB operand
-
-// Panel: L(ib, jb) = A(ib, jb) L(jb, jb)^-T, 16 rows of it per CTA: rows rb = NB (jb + 1) + 16
-// blockIdx.x.  An output row needs only its own input row, so the CTA works in place.  The fp64 pipe (2
-// FMAs per clock and SM) is the bound: 64-row tiles left most SMs idle for 68 us per panel.
-__global__ void __launch_bounds__(256) k_cr_trsm(double* __restrict__ K, int64_t mp, int jb,
-                                                const double* __restrict__ Dinv, const int32_t* flag) {
-  __shared__ double At[16][CTP];
-  extern __shared__ __align__(16) unsigned char cr_smem[];
-  double(*Dt)[NBP] = reinterpret_cast<double(*)[NBP]>(cr_smem);
-  if (failed(flag)) return;
-  double* Ab = K + (int64_t(jb + 1) * NB + 16 * int64_t(blockIdx.x)) * mp + int64_t(jb) * NB;
-  for (int e = threadIdx.x; e < 16 * NB; e += 256) At[e / NB][e % NB] = Ab[int64_t(e / NB) * mp + e % NB];
-  load_tile(Dt, Dinv + int64_t(jb) * NB * NB, NB);
-  __syncthreads();
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  double acc[4] = {};
-  for (int u = 0; u < NB; ++u) {
-    const double a = At[ty][u];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) acc[q] = fma(a, Dt[tx + 16 * q][u], acc[q]);
-  }
-#pragma unroll
-  for (int q = 0; q < 4; ++q) Ab[int64_t(ty) * mp + tx + 16 * q] = acc[q];
-}
-
-// Trailing update: A(i, k) -= L(i, jb) L(k, jb)^T on 32 x 32 tiles of the trailing lower triangle
-// (one per CTA; the smaller tile spreads the last panels' few tiles over more SMs).
-__global__ void __launch_bounds__(256) k_cr_syrk(double* __restrict__ K, int64_t mp, int jb, const int32_t* flag) {
-  __shared__ double Li[CT][CTP];
-  __shared__ double Lk[CT][CTP];
-  if (failed(flag)) return;
-  const int x = blockIdx.x;
-  int ii = int((sqrt(8.0 * x + 1.0) - 1.0) * 0.5);
-  while ((ii + 1) * (ii + 2) / 2 <= x) ++ii;
-  while (ii * (ii + 1) / 2 > x) --ii;
-  const int kk = x - ii * (ii + 1) / 2;
-  const int64_t r0 = int64_t(jb + 1) * NB;
-  const double* Lb = K + int64_t(jb) * NB;  // columns of the panel
-  for (int e = threadIdx.x; e < CT * NB; e += 256) {
-    const int r = e / NB, c = e % NB;
-    Li[r][c] = Lb[(r0 + ii * CT + r) * mp + c];
-    Lk[r][c] = Lb[(r0 + kk * CT + r) * mp + c];
-  }
-  __syncthreads();
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  double acc[2][2] = {};
-#pragma unroll 4
-  for (int u = 0; u < NB; ++u) {
-    const double a0 = Li[ty][u], a1 = Li[ty + 16][u], b0 = Lk[tx][u], b1 = Lk[tx + 16][u];
-    acc[0][0] = fma(a0, b0, acc[0][0]);
-    acc[0][1] = fma(a0, b1, acc[0][1]);
-    acc[1][0] = fma(a1, b0, acc[1][0]);
-    acc[1][1] = fma(a1, b1, acc[1][1]);
-  }
-  double* Cb = K + (r0 + ii * CT) * mp + r0 + kk * CT;
-#pragma unroll
-  for (int p = 0; p < 2; ++p)
-#pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      double* o = Cb + int64_t(ty + 16 * p) * mp + tx + 16 * q;
-      *o -= acc[p][q];
-    }
-}
-
-// W (mp x n) <- K^-1 W for the NC columns of this CTA, forward then backward, in one launch: the columns
-// stay in shared memory (X, mp x NC) and the factor streams through two tile buffers (cp.async, the
-// next 64 x 64 tile in flight while one is used).  Columns do not depend on one another, so no CTA
-// waits for another.  With NC = ceil(n / SMs) every SM has the same work.  Left-looking: row block ib of
-// the solution is D(ib) (W_ib - sum_k L(ib, k) X_k), each thread taking one row and a quarter of every
-// tile's 64 columns, two of them to a packed instruction.
-// PL = 2: W is fp64, and the factor, the solution and the sums are pairs of fp32 (value and rest, 2^-48):
-// the product of the values as a two-product, the cross products of values and rests, and a two-sum, 12
-// packed instructions per two terms.  The fp64 pipe takes 2 FMAs per clock and SM, the fp32 pipe 128:
-// fp64 arithmetic took 3.97 ms a solve at m = 1536, n = 896.  The factor's own entries are sums of fp32
-// products (2^-24 each), so 2^-48 in the substitutions does not show in the result.
-// PL = 1: W and the arithmetic are fp32, bound by the stream of the factor from L2 (8 m^2 bytes per CTA).
 constexpr int CSLD = NB + 4;                // tile rows of 16-byte pieces, conflict-free by rows
 constexpr int CSTILE = NB * CSLD;           // floats of a tile
 
-__device__ __forceinline__ void cs_tile(uint32_t dst, const float* src, int64_t ld, int tid) {
+// ROWS x 64 floats to shared-memory rows of CSLD.
+template <int ROWS, int THREADS>
+__device__ __forceinline__ void fetch_rows(uint32_t dst, const float* src, int64_t ld, int tid) {
   constexpr int PER = NB / 4;
 #pragma unroll
-  for (int i = 0; i < NB * PER / 256; ++i) {
-    const int e = tid + 256 * i, r = e / PER, c = (e % PER) * 4;
+  for (int i = 0; i < ROWS * PER / THREADS; ++i) {
+    const int e = tid + THREADS * i, r = e / PER, c = (e % PER) * 4;
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + uint32_t((r * CSLD + c) * 4)),
                  "l"(src + int64_t(r) * ld + c)
                  : "memory");
@@ -278,6 +125,236 @@ struct Acc2 {  // sums over even and odd columns of the tile
   }
 };
 
+// Scalars as pairs (value, rest): a b, and m - a b (not renormalised).
+__device__ __forceinline__ float2 pair_norm(float2 a) {
+  const float h = a.x + a.y;
+  return make_float2(h, a.y - (h - a.x));
+}
+__device__ __forceinline__ float2 pair_mul(float2 a, float2 b) {
+  const float p = a.x * b.x;
+  float e = fmaf(a.x, b.x, -p);
+  e = fmaf(a.x, b.y, e);
+  e = fmaf(a.y, b.x, e);
+  return pair_norm(make_float2(p, e));
+}
+__device__ __forceinline__ float2 pair_nmac(float2 m, float2 a, float2 b) {
+  const float p = a.x * b.x;
+  float e = fmaf(a.x, b.x, -p);
+  e = fmaf(a.x, b.y, e);
+  e = fmaf(a.y, b.x, e);
+  const float t = m.x - p, bb = t - m.x;
+  return make_float2(t, m.y + ((m.x - (t - bb)) - (p + bb) - e));
+}
+// 1 / a and 1 / sqrt(a), a > 0: the fp32 value and one step of the binomial series in what it leaves.
+__device__ __forceinline__ float2 pair_rcp(float2 a) {
+  const float y = __frcp_rn(a.x);
+  const float r = fmaf(-a.y, y, fmaf(-a.x, y, 1.f));
+  return pair_norm(make_float2(y, y * fmaf(r, r, r)));
+}
+__device__ __forceinline__ float2 pair_rsqrt(float2 a) {
+  const float y = rsqrtf(a.x), q = y * y, qe = fmaf(y, y, -q);
+  float r = fmaf(-a.x, q, 1.f);
+  r = fmaf(-a.x, qe, r);
+  r = fmaf(-a.y, q, r);
+  return pair_norm(make_float2(y, y * fmaf(0.375f * r, r, 0.5f * r)));
+}
+
+// Diagonal tile jb, in pairs: the factor and the inverse of the triangular factor, which goes to D(jb).  A
+// pivot that is not positive sets the failure flag (E^T E + beta I is not positive definite in floating
+// point).  One CTA, nothing else beside it, so the latency of the 64 steps is what counts: the triangle
+// stays in registers (16 x 16 threads, entries (ti + 16 a, tj + 16 b)), factor and inverse are taken in
+// one sweep without square roots (columns <= c of the triangle hold the unit inverse, the others what is
+// left of the tile), and a step passes its column and row through shared memory with one barrier.  In fp64,
+// factor and inverse one after the other took 106 us a tile (34 now): 2 FMAs per clock, and every thread its
+// own rsqrt.
+constexpr int PLD = NB + 1;
+constexpr size_t kPotrfSmem = sizeof(float2) * 2 * NB * PLD;
+__global__ void __launch_bounds__(256) k_cr_potrf(float* __restrict__ K, float* __restrict__ Krest, int64_t mp, int jb,
+                                                 float* __restrict__ Dinv, float* __restrict__ Drest, int32_t* flag) {
+  extern __shared__ __align__(16) unsigned char cr_smem[];
+  float2(*V)[PLD] = reinterpret_cast<float2(*)[PLD]>(cr_smem);  // V[c]: column c of the tile at step c
+  float2(*Y)[PLD] = V + NB;                                     // Y[c]: row c of the unit inverse, left of the diagonal
+  __shared__ float2 rs[NB];
+  if (failed(flag)) return;
+  const int tid = threadIdx.x, ti = tid >> 4, tj = tid & 15;
+  const int64_t o = int64_t(jb) * NB * mp + int64_t(jb) * NB;
+  float2 m[4][4];
+#pragma unroll
+  for (int a = 0; a < 4; ++a)
+#pragma unroll
+    for (int b = 0; b <= a; ++b) {
+      const int64_t e = o + int64_t(ti + 16 * a) * mp + tj + 16 * b;
+      m[a][b] = tj + 16 * b <= ti + 16 * a ? make_float2(K[e], Krest[e]) : make_float2(0.f, 0.f);
+    }
+#pragma unroll
+  for (int cb = 0; cb < 4; ++cb) {
+#pragma unroll 1
+    for (int cl = 0; cl < 16; ++cl) {
+      const int c = 16 * cb + cl;
+      if (tj == cl) {
+#pragma unroll
+        for (int a = cb; a < 4; ++a) V[c][ti + 16 * a] = pair_norm(m[a][cb]);
+      }
+      if (ti == cl) {
+#pragma unroll
+        for (int b = 0; b <= cb; ++b) Y[c][tj + 16 * b] = pair_norm(m[cb][b]);
+      }
+      __syncthreads();
+      const float2 piv = V[c][c];
+      if (!(piv.x > 0.f)) {  // the same value in every thread
+        if (tid == 0) atomicExch(flag, 1);
+        return;
+      }
+      const float2 rp = pair_rcp(piv);
+      float2 z[4];  // row c of the unit inverse, 1, and the column transposed, over the pivot
+#pragma unroll
+      for (int b = 0; b < 4; ++b) {
+        const int j = tj + 16 * b;
+        z[b] = j == c ? rp : pair_mul(j > c ? V[c][j] : Y[c][j], rp);
+      }
+#pragma unroll
+      for (int a = cb; a < 4; ++a) {
+        const int i = ti + 16 * a;
+        const float2 v = V[c][i];
+#pragma unroll
+        for (int b = 0; b <= a; ++b) {
+          float2 old = m[a][b];
+          if (b == cb && tj == cl) old = make_float2(0.f, 0.f);
+          if (i > c) m[a][b] = pair_nmac(old, v, z[b]);
+        }
+      }
+    }
+  }
+  __syncthreads();
+  if (tid < NB) rs[tid] = pair_rsqrt(V[tid][tid]);
+  __syncthreads();
+  const int64_t od = int64_t(jb) * NB * NB;
+  for (int e = tid; e < NB * NB; e += 256) {
+    const int i = e / NB, j = e % NB;
+    float2 x = make_float2(0.f, 0.f);
+    if (j <= i) {
+      const float2 f = pair_mul(V[j][i], rs[j]);
+      K[o + int64_t(i) * mp + j] = f.x;
+      Krest[o + int64_t(i) * mp + j] = f.y;
+      x = j == i ? rs[i] : pair_mul(Y[i][j], rs[i]);
+    }
+    Dinv[od + e] = x.x;
+    Drest[od + e] = x.y;
+  }
+}
+
+// C = A B^T for ROWS x 64 and COLS x 64 pairs, or what the caller makes of the sums: two rows and
+// four columns of C per thread, two of the 64 terms to a packed instruction.  128 threads.
+template <int ROWS, int COLS>
+struct PairTile {
+  static constexpr int TC = COLS / 4, TR = ROWS / 2;
+  static_assert(TC * TR == 128, "threads");
+  static constexpr int kFloats = 2 * (ROWS + COLS) * CSLD;
+  template <typename F>
+  static __device__ __forceinline__ void run(float* sm, const float* A, const float* Arest, const float* B, const float* Brest,
+                                             int64_t lda, int64_t ldb, F&& out) {
+    const int tid = threadIdx.x, tr = tid / TC, tc = tid % TC;
+    const uint32_t base = uint32_t(__cvta_generic_to_shared(sm));
+    fetch_rows<ROWS, 128>(base, A, lda, tid);
+    fetch_rows<ROWS, 128>(base + ROWS * CSLD * 4, Arest, lda, tid);
+    fetch_rows<COLS, 128>(base + 2 * ROWS * CSLD * 4, B, ldb, tid);
+    fetch_rows<COLS, 128>(base + (2 * ROWS + COLS) * CSLD * 4, Brest, ldb, tid);
+    cp_async_commit();
+    cp_async_wait<0>();
+    __syncthreads();
+    Acc2<2> acc[2][4];
+#pragma unroll
+    for (int p = 0; p < 2; ++p)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) acc[p][q].clear();
+    const float* Bs = sm + 2 * ROWS * CSLD;
+#pragma unroll 2
+    for (int u = 0; u < NB; u += 4) {
+      uint64_t a[2][2][2], na[2][2][2];
+#pragma unroll
+      for (int p = 0; p < 2; ++p)
+#pragma unroll
+        for (int pl = 0; pl < 2; ++pl) {
+          const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(sm + (pl * ROWS + tr + p * TR) * CSLD + u);
+          a[p][0][pl] = t.x;
+          a[p][1][pl] = t.y;
+#pragma unroll
+          for (int v = 0; v < 2; ++v) na[p][v][pl] = a[p][v][pl] ^ 0x8000000080000000ull;
+        }
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        uint64_t x[2][2];
+#pragma unroll
+        for (int pl = 0; pl < 2; ++pl) {
+          const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(Bs + (pl * COLS + tc + q * TC) * CSLD + u);
+          x[0][pl] = t.x;
+          x[1][pl] = t.y;
+        }
+#pragma unroll
+        for (int v = 0; v < 2; ++v)
+#pragma unroll
+          for (int p = 0; p < 2; ++p) acc[p][q].mac(a[p][v], na[p][v], x[v]);
+      }
+    }
+#pragma unroll
+    for (int p = 0; p < 2; ++p)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) out(tr + p * TR, tc + q * TC, acc[p][q].total());
+  }
+};
+
+// Panel: L(ib, jb) = A(ib, jb) L(jb, jb)^-T, 16 rows of it per CTA: rows rb = NB (jb + 1) + 16
+// blockIdx.x.  An output row needs only its own input row, so the CTA works in place.
+__global__ void __launch_bounds__(128) k_cr_trsm(float* __restrict__ K, float* __restrict__ Krest, int64_t mp, int jb,
+                                                const float* __restrict__ Dinv, const float* __restrict__ Drest,
+                                                const int32_t* flag) {
+  __shared__ __align__(16) float sm[PairTile<16, 64>::kFloats];
+  if (failed(flag)) return;
+  const int64_t o = (int64_t(jb + 1) * NB + 16 * int64_t(blockIdx.x)) * mp + int64_t(jb) * NB;
+  const int64_t od = int64_t(jb) * NB * NB;
+  PairTile<16, 64>::run(sm, K + o, Krest + o, Dinv + od, Drest + od, mp, NB, [&](int i, int j, float2 v) {
+    K[o + int64_t(i) * mp + j] = v.x;
+    Krest[o + int64_t(i) * mp + j] = v.y;
+  });
+}
+
+constexpr int CT = 32;         // tile of the trailing updates
+
+// Trailing update: A(i, k) -= L(i, jb) L(k, jb)^T on 32 x 32 tiles of the trailing lower triangle
+// (one per CTA; the smaller tile spreads the last panels' few tiles over more SMs).  Bound by the fp32 pipe
+// (12 packed instructions per two terms): 380 us for the 23 updates at m = 1536, 1290 in fp64.
+__global__ void __launch_bounds__(128) k_cr_syrk(float* __restrict__ K, float* __restrict__ Krest, int64_t mp, int jb,
+                                                const int32_t* flag) {
+  __shared__ __align__(16) float sm[PairTile<CT, CT>::kFloats];
+  if (failed(flag)) return;
+  const int x = blockIdx.x;
+  int ii = int((sqrtf(8.f * float(x) + 1.f) - 1.f) * 0.5f);
+  while ((ii + 1) * (ii + 2) / 2 <= x) ++ii;
+  while (ii * (ii + 1) / 2 > x) --ii;
+  const int kk = x - ii * (ii + 1) / 2;
+  const int64_t r0 = int64_t(jb + 1) * NB, c0 = int64_t(jb) * NB;  // the trailing rows, the panel's columns
+  const int64_t oa = (r0 + ii * CT) * mp + c0, ob = (r0 + kk * CT) * mp + c0;
+  const int64_t oc = (r0 + ii * CT) * mp + r0 + kk * CT;
+  PairTile<CT, CT>::run(sm, K + oa, Krest + oa, K + ob, Krest + ob, mp, mp, [&](int i, int j, float2 v) {
+    const int64_t e = oc + int64_t(i) * mp + j;
+    const float2 r = pair_add(make_float2(K[e], Krest[e]), make_float2(-v.x, -v.y));
+    K[e] = r.x;
+    Krest[e] = r.y;
+  });
+}
+
+// W (mp x n) <- K^-1 W for the NC columns of this CTA, forward then backward, in one launch: the columns
+// stay in shared memory (X, mp x NC) and the factor streams through two tile buffers (cp.async, the
+// next 64 x 64 tile in flight while one is used).  Columns do not depend on one another, so no CTA
+// waits for another.  With NC = ceil(n / SMs) every SM has the same work.  Left-looking: row block ib of
+// the solution is D(ib) (W_ib - sum_k L(ib, k) X_k), each thread taking one row and a quarter of every
+// tile's 64 columns, two of them to a packed instruction.
+// PL = 2: W is fp64, and the factor, the solution and the sums are pairs of fp32 (value and rest, 2^-48):
+// the product of the values as a two-product, the cross products of values and rests, and a two-sum, 12
+// packed instructions per two terms.  The fp64 pipe takes 2 FMAs per clock and SM, the fp32 pipe 128:
+// fp64 arithmetic took 3.97 ms a solve at m = 1536, n = 896.  The factor's own entries are sums of fp32
+// products (2^-24 each), so 2^-48 in the substitutions does not show in the result.
+// PL = 1: W and the arithmetic are fp32, bound by the stream of the factor from L2 (8 m^2 bytes per CTA).
 template <int PL, int NC>
 __global__ void __launch_bounds__(256)
     k_cr_colsolve(const float* __restrict__ K, const float* __restrict__ Krest, int64_t mp, const float* __restrict__ Dinv,
@@ -313,7 +390,7 @@ __global__ void __launch_bounds__(256)
         src = (p == 0 ? K : Krest) +
               (fwd ? int64_t(ib) * NB * mp + int64_t(k) * NB : int64_t(k) * NB * mp + int64_t(ib) * NB);
       }
-      cs_tile(ts + uint32_t((buf * PL + p) * CSTILE) * 4u, src, ld, tid);
+      fetch_rows<NB, 256>(ts + uint32_t((buf * PL + p) * CSTILE) * 4u, src, ld, tid);
     }
     cp_async_commit();
   };
@@ -515,14 +592,9 @@ __global__ void k_cr_cvt(const TI* __restrict__ x, TO* __restrict__ y, int64_t c
     y[e] = TO(x[e]);
 }
 
-// y + rest = x to 2^-48
-__global__ void k_cr_split(const double* __restrict__ x, float* __restrict__ y, float* __restrict__ rest, int64_t count) {
-  for (int64_t e = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; e < count; e += int64_t(gridDim.x) * blockDim.x) {
-    const double v = x[e];
-    const float h = float(v);
-    y[e] = h;
-    rest[e] = isfinite(h) ? float(v - double(h)) : 0.f;
-  }
+__global__ void k_cr_join(const float* __restrict__ x, const float* __restrict__ rest, double* __restrict__ y, int64_t count) {
+  for (int64_t e = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; e < count; e += int64_t(gridDim.x) * blockDim.x)
+    y[e] = double(x[e]) + double(rest[e]);
 }
 
 constexpr int QR_STAGE = 64;   // rows staged at a time by k_cr_vtv
@@ -908,7 +980,7 @@ cudaError_t gtt(const float* G, const float* Tn, int64_t Np, int64_t d, int64_t 
   return cudaGetLastError();
 }
 
-// The Cholesky factor: fp64, its fp32 value and what that leaves.
+// The Cholesky factor: its fp32 value and what that leaves; fp64 where k_cr_tsolve takes it.
 struct Factor {
   const double *K, *Dinv;
   const float *Kf, *Dinvf, *Krest, *Drest;
@@ -1003,7 +1075,7 @@ cudaError_t orth(double* V, int64_t rows, int64_t n, int ell, int L, double* qrp
 
 cudaError_t set_smem_attributes() {
   static const void* fns64[] = {
-      reinterpret_cast<const void*>(k_cr_potrf), reinterpret_cast<const void*>(k_cr_trsm),
+      reinterpret_cast<const void*>(k_cr_potrf),
       reinterpret_cast<const void*>(k_cr_tsolve<double, 0, 16>),
       reinterpret_cast<const void*>(k_cr_tsolve<double, 1, 64>),
       reinterpret_cast<const void*>(k_cr_tsolve<double, 2, 16>),
@@ -1057,26 +1129,23 @@ cudaError_t rsvd_t(const float* E, const float* G, int64_t Np, int64_t m, int64_
   CR_TRY(cudaMemsetAsync(Ym, 0, sizeof(double) * mp * n, s));
   // K = E^T E (lower tiles), + beta I, padded
   CR_TRY((gemm<true, double>(E, m, 0, E, m, 0, K, mp, 0, m, m, Np, 1, 1, s)));
-  k_cr_pad<<<4 * sm_count(), 256, 0, s>>>(K, m, mp, double(beta));
+  k_cr_pad<<<4 * sm_count(), 256, 0, s>>>(K, m, mp, double(beta), Kf, Krest);
   CR_TRY(cudaGetLastError());
   for (int jb = 0; jb < nb; ++jb) {
-    k_cr_potrf<<<1, 256, kTileSmem, s>>>(K, mp, jb, Dinv, flag);
+    k_cr_potrf<<<1, 256, kPotrfSmem, s>>>(Kf, Krest, mp, jb, Dinvf, Drest, flag);
     const int T = nb - jb - 1;
     if (T > 0) {
-      k_cr_trsm<<<T * (NB / 16), 256, kTileSmem / 2, s>>>(K, mp, jb, Dinv, flag);
+      k_cr_trsm<<<T * (NB / 16), 128, 0, s>>>(Kf, Krest, mp, jb, Dinvf, Drest, flag);
       const int T2 = T * (NB / CT);
-      k_cr_syrk<<<T2 * (T2 + 1) / 2, 256, 0, s>>>(K, mp, jb, flag);
+      k_cr_syrk<<<T2 * (T2 + 1) / 2, 128, 0, s>>>(Kf, Krest, mp, jb, flag);
     }
     CR_TRY(cudaGetLastError());
   }
   const Factor f{K, Dinv, Kf, Dinvf, Krest, Drest};
-  if (colsolve_columns(2, mp, n) > 0) {
-    k_cr_split<<<2 * sm_count(), 256, 0, s>>>(K, Kf, Krest, mp * mp);
-    k_cr_split<<<2 * sm_count(), 256, 0, s>>>(Dinv, Dinvf, Drest, int64_t(nb) * NB * NB);
+  if (colsolve_columns(2, mp, n) == 0) {  // the step-by-step solves take the factor in fp64
+    k_cr_join<<<2 * sm_count(), 256, 0, s>>>(Kf, Krest, K, mp * mp);
+    k_cr_join<<<2 * sm_count(), 256, 0, s>>>(Dinvf, Drest, Dinv, int64_t(nb) * NB * NB);
     CR_TRY(cudaGetLastError());
-  } else if (q > 0) {
-    CR_TRY((cvt<double, float>(K, Kf, mp * mp, s)));
-    CR_TRY((cvt<double, float>(Dinv, Dinvf, int64_t(nb) * NB * NB, s)));
   }
   // Ym = F^T X for every block, X (d x ell per block, fp32) at column offset l ell of Xf (ld ldx,
   // block stride sx): Tn = G_l X, Ym = K^-1 E^T Tn (fp64 factor when exact, else the fp32 one on
