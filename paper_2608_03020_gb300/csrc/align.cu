@@ -163,7 +163,7 @@ static cudaError_t align_t(const float* E, const float* G, int64_t Np, int m, in
     if (e != cudaSuccess) return e;
   }
   const int64_t n = int64_t(L) * r;
-  const RunGemmArgs g{E, P, U, m, 0, r, int64_t(m) * r, RP, Np * RP, Np, n, m, r, 0};
+  const RunGemmArgs g{E, P, U, m, 0, r, int64_t(m) * r, RP, Np * RP, Np, n, m, 0, r, 0};
   e = run_gemm<false, float, 64, 64>(g, 1, s);
   if (e != cudaSuccess) return e;
   constexpr int smem = AL_THREADS / 32 * RowRing<RP, 32 / RP>::BYTES;

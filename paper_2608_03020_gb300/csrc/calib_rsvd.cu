@@ -937,13 +937,13 @@ RsvdWs rsvd_ws(int64_t Np, int64_t m, int64_t d, int L, int ell, int r) {
   return w;
 }
 
-// C_b(i, j) = sum_t A_b(i, t) B_b(t, j) (run_gemm.cuh).  32-column tiles where N is one block's ell <= 32
+// C_b(i, j) = sum_t A_b(i, t) B_b(t, j) (run_gemm.cuh); Kall: the batches are ranges of Kc of Kall terms.  32-column tiles where N is one block's ell <= 32
 // columns.
 template <bool AT, typename TC>
 cudaError_t gemm(const float* A, int64_t lda, int64_t sA, const float* B, int64_t ldb, int64_t sB, TC* C,
                  int64_t ldc, int64_t sC, int64_t M, int64_t N, int64_t Kc, int batch, int lower_only,
-                 cudaStream_t s) {
-  const RunGemmArgs g{A, B, C, lda, sA, ldb, sB, ldc, sC, M, N, Kc, 0, lower_only};
+                 cudaStream_t s, int64_t Kall = 0) {
+  const RunGemmArgs g{A, B, C, lda, sA, ldb, sB, ldc, sC, M, N, Kc, Kall, 0, lower_only};
   return N <= 32 ? run_gemm<AT, TC, 128, 32>(g, batch, s) : run_gemm<AT, TC, 64, 64>(g, batch, s);
 }
 
@@ -1155,9 +1155,8 @@ cudaError_t rsvd_t(const float* E, const float* G, int64_t Np, int64_t m, int64_
     // E^T Tn: two halves of the tokens when the tiles are fewer than six a SM (a last wave of few long
     // tiles costs more than the addition)
     const int64_t half = (m + 63) / 64 * ((n + 63) / 64) < 6 * sm_count() && Np >= 1024 ? (Np / 2 + 31) / 32 * 32 : Np;
-    CR_TRY((gemm<true, double>(E, m, 0, Tn, n, 0, Ym, n, 0, m, n, half, 1, 0, s)));
+    CR_TRY((gemm<true, double>(E, m, half * m, Tn, n, half * n, Ym, n, Wm - Ym, m, n, half, half < Np ? 2 : 1, 0, s, Np)));
     if (half < Np) {
-      CR_TRY((gemm<true, double>(E + half * m, m, 0, Tn + half * n, n, 0, Wm, n, 0, m, n, Np - half, 1, 0, s)));
       k_cr_add<<<2 * sm_count(), 256, 0, s>>>(Ym, Wm, m * n);
       CR_TRY(cudaGetLastError());
     }
