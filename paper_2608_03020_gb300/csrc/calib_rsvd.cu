@@ -51,23 +51,6 @@ constexpr size_t kTileSmem = sizeof(double) * 2 * NB * NBP;
 
 __device__ __forceinline__ bool failed(const int32_t* flag) { return *reinterpret_cast<const volatile int32_t*>(flag) != 0; }
 
-// K (mp x mp) into its fp32 value and what that leaves (together 2^-48): rows / columns >= m become the
-// identity, beta is added to the first m diagonal entries.  Lower triangle of 64 x 64 tiles only.
-__global__ void k_cr_pad(const double* __restrict__ K, int64_t m, int64_t mp, double beta, float* __restrict__ Kf,
-                         float* __restrict__ Krest) {
-  const int64_t total = mp * mp;
-  for (int64_t e = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; e < total; e += int64_t(gridDim.x) * blockDim.x) {
-    const int64_t i = e / mp, j = e % mp;
-    if (j / NB > i / NB) continue;
-    double v = 0.0;
-    if (i < m && j < m) v = K[e] + (i == j ? beta : 0.0);
-    else if (i == j) v = 1.0;
-    const float h = float(v);
-    Kf[e] = h;
-    Krest[e] = isfinite(h) ? float(v - double(h)) : 0.f;
-  }
-}
-
 constexpr int CSLD = NB + 4;                // tile rows of 16-byte pieces, conflict-free by rows
 constexpr int CSTILE = NB * CSLD;           // floats of a tile
 
@@ -157,6 +140,24 @@ __device__ __forceinline__ float2 pair_rsqrt(float2 a) {
   r = fmaf(-a.x, qe, r);
   r = fmaf(-a.y, q, r);
   return pair_norm(make_float2(y, y * fmaf(0.375f * r, r, 0.5f * r)));
+}
+
+// K (mp x mp, pairs): rows / columns >= m become the identity; beta is added to the first m diagonal
+// entries.
+__global__ void k_cr_pad(float* __restrict__ K, float* __restrict__ Krest, int64_t m, int64_t mp, double beta) {
+  const float2 b = make_float2(float(beta), float(beta - double(float(beta))));
+  const int64_t total = mp * mp;
+  for (int64_t e = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; e < total; e += int64_t(gridDim.x) * blockDim.x) {
+    const int64_t i = e / mp, j = e % mp;
+    if (i >= m || j >= m) {
+      K[e] = (i == j) ? 1.f : 0.f;
+      Krest[e] = 0.f;
+    } else if (i == j) {
+      const float2 v = pair_add(make_float2(K[e], Krest[e]), b);
+      K[e] = v.x;
+      Krest[e] = v.y;
+    }
+  }
 }
 
 // Diagonal tile jb, in pairs: the factor and the inverse of the triangular factor, which goes to D(jb).  A
@@ -592,9 +593,27 @@ __global__ void k_cr_cvt(const TI* __restrict__ x, TO* __restrict__ y, int64_t c
     y[e] = TO(x[e]);
 }
 
-__global__ void k_cr_join(const float* __restrict__ x, const float* __restrict__ rest, double* __restrict__ y, int64_t count) {
-  for (int64_t e = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; e < count; e += int64_t(gridDim.x) * blockDim.x)
+// y[e] = x[e] + rest[e] for beg <= e < end, where rest may be the upper half of y's memory: the entries that a
+// range of this launch overwrites are ones that earlier launches have read (see join_in_place).
+__global__ void k_cr_join(const float* __restrict__ x, const float* rest, double* y, int64_t beg, int64_t end) {
+  for (int64_t e = beg + int64_t(blockIdx.x) * blockDim.x + threadIdx.x; e < end; e += int64_t(gridDim.x) * blockDim.x)
     y[e] = double(x[e]) + double(rest[e]);
+}
+constexpr int JOIN_LAST = 4096;
+__global__ void __launch_bounds__(256) k_cr_join_last(const float* __restrict__ x, const float* rest, double* y,
+                                                     int64_t beg, int64_t end) {
+  double v[JOIN_LAST / 256];
+#pragma unroll
+  for (int i = 0; i < JOIN_LAST / 256; ++i) {
+    const int64_t e = beg + threadIdx.x + 256 * i;
+    v[i] = e < end ? double(x[e]) + double(rest[e]) : 0.0;
+  }
+  __syncthreads();  // everything is read
+#pragma unroll
+  for (int i = 0; i < JOIN_LAST / 256; ++i) {
+    const int64_t e = beg + threadIdx.x + 256 * i;
+    if (e < end) y[e] = v[i];
+  }
 }
 
 constexpr int QR_STAGE = 64;   // rows staged at a time by k_cr_vtv
@@ -895,7 +914,7 @@ __global__ void __launch_bounds__(256) k_cr_ritz_sign(float* __restrict__ P, flo
 }
 
 struct RsvdWs {
-  size_t K, Dinv, Kf, Dinvf, Krest, Drest, Ym, Wm, Wf, Zd, Zf, Tn, qrpart, qrfac, part, Ur, sig, amv, ami, flag, total;
+  size_t K, Dinv, Kf, Dinvf, Drest, Ym, Wm, Wf, Zd, Zf, Tn, qrpart, qrfac, part, Ur, sig, amv, ami, flag, total;
 };
 
 RsvdWs rsvd_ws(int64_t Np, int64_t m, int64_t d, int L, int ell, int r) {
@@ -913,11 +932,10 @@ RsvdWs rsvd_ws(int64_t Np, int64_t m, int64_t d, int L, int ell, int r) {
   };
   const int64_t ellp = ell <= 16 ? 16 : (ell <= 32 ? 32 : 64);
   const int64_t nchqr = ((m > d ? m : d) + QR_CHUNK - 1) / QR_CHUNK;
-  w.K = take(sizeof(double) * mp * mp);
+  w.K = take(sizeof(double) * mp * mp);  // the factor's rest plane in the upper half, or all of it in fp64
   w.Dinv = take(sizeof(double) * nb * NB * NB);
   w.Kf = take(sizeof(float) * mp * mp);
   w.Dinvf = take(sizeof(float) * nb * NB * NB);
-  w.Krest = take(sizeof(float) * mp * mp);
   w.Drest = take(sizeof(float) * nb * NB * NB);
   w.Ym = take(sizeof(double) * mp * n);
   w.Wm = take(sizeof(double) * mp * n);
@@ -1060,6 +1078,20 @@ cudaError_t cvt(const TI* x, TO* y, int64_t count, cudaStream_t s) {
   return cudaGetLastError();
 }
 
+// y = x + rest with rest in the upper half of y's memory (so that the workspace needs no further plane): entry e
+// of y lies over entries 2 e - count, 2 e - count + 1 of rest, which come before e, so ranges that halve
+// what is left overwrite only what the launches before them have read.
+cudaError_t join_in_place(const float* x, const float* rest, double* y, int64_t count, cudaStream_t s) {
+  int64_t beg = 0;
+  while (count - beg > JOIN_LAST) {
+    const int64_t end = beg + (count - beg) / 2;
+    k_cr_join<<<2 * sm_count(), 256, 0, s>>>(x, rest, y, beg, end);
+    beg = end;
+  }
+  k_cr_join_last<<<1, 256, 0, s>>>(x, rest, y, beg, count);
+  return cudaGetLastError();
+}
+
 // Orthonormal basis of every block's ell columns of V (rows x n), in place: Cholesky QR twice.
 template <int ELLP>
 cudaError_t orth(double* V, int64_t rows, int64_t n, int ell, int L, double* qrpart, double* qrfac, cudaStream_t s) {
@@ -1107,7 +1139,7 @@ cudaError_t rsvd_t(const float* E, const float* G, int64_t Np, int64_t m, int64_
   double* Dinv = reinterpret_cast<double*>(ws + w.Dinv);
   float* Kf = reinterpret_cast<float*>(ws + w.Kf);
   float* Dinvf = reinterpret_cast<float*>(ws + w.Dinvf);
-  float* Krest = reinterpret_cast<float*>(ws + w.Krest);
+  float* Krest = reinterpret_cast<float*>(ws + w.K) + mp * mp;
   float* Drest = reinterpret_cast<float*>(ws + w.Drest);
   double* Ym = reinterpret_cast<double*>(ws + w.Ym);
   double* Wm = reinterpret_cast<double*>(ws + w.Wm);
@@ -1128,8 +1160,9 @@ cudaError_t rsvd_t(const float* E, const float* G, int64_t Np, int64_t m, int64_
   CR_TRY(cudaMemsetAsync(flag, 0, sizeof(int32_t) * 64, s));
   CR_TRY(cudaMemsetAsync(Ym, 0, sizeof(double) * mp * n, s));
   // K = E^T E (lower tiles), + beta I, padded
-  CR_TRY((gemm<true, double>(E, m, 0, E, m, 0, K, mp, 0, m, m, Np, 1, 1, s)));
-  k_cr_pad<<<4 * sm_count(), 256, 0, s>>>(K, m, mp, double(beta), Kf, Krest);
+  const RunGemmArgs ete{E, E, Kf, m, 0, m, 0, mp, 0, m, m, Np, 0, 0, 1, Krest};
+  CR_TRY((run_gemm<true, float, 64, 64>(ete, 1, s)));
+  k_cr_pad<<<4 * sm_count(), 256, 0, s>>>(Kf, Krest, m, mp, double(beta));
   CR_TRY(cudaGetLastError());
   for (int jb = 0; jb < nb; ++jb) {
     k_cr_potrf<<<1, 256, kPotrfSmem, s>>>(Kf, Krest, mp, jb, Dinvf, Drest, flag);
@@ -1143,8 +1176,8 @@ cudaError_t rsvd_t(const float* E, const float* G, int64_t Np, int64_t m, int64_
   }
   const Factor f{K, Dinv, Kf, Dinvf, Krest, Drest};
   if (colsolve_columns(2, mp, n) == 0) {  // the step-by-step solves take the factor in fp64
-    k_cr_join<<<2 * sm_count(), 256, 0, s>>>(Kf, Krest, K, mp * mp);
-    k_cr_join<<<2 * sm_count(), 256, 0, s>>>(Dinvf, Drest, Dinv, int64_t(nb) * NB * NB);
+    CR_TRY(join_in_place(Kf, Krest, K, mp * mp, s));
+    k_cr_join<<<2 * sm_count(), 256, 0, s>>>(Dinvf, Drest, Dinv, int64_t(0), int64_t(nb) * NB * NB);
     CR_TRY(cudaGetLastError());
   }
   // Ym = F^T X for every block, X (d x ell per block, fp32) at column offset l ell of Xf (ld ldx,

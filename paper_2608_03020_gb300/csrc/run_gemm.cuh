@@ -31,6 +31,7 @@ struct RunGemmArgs {
   int64_t Kall;  // > 0: batch b has terms b K .. of Kall, the last one what is left
   int bw;
   int lower_only;  // tiles strictly above the diagonal are not computed
+  float* rest = nullptr;  // fp32 C: the sums as pairs, the rests here (same layout)
 };
 
 template <bool AT, typename TC, int BM, int BN>
@@ -167,7 +168,14 @@ __global__ void __launch_bounds__(BM * BN / 32) k_run_gemm(RunGemmArgs g) {
 #pragma unroll
       for (int u = 0; u < 2; ++u) {
         const int64_t i = i0 + (p / 2) * (BM / NG) + ty * 4 + (p % 2) * 2 + u;
-        if (i < g.M && LOCA_CHECK(j, g.N)) C[i * g.ldc + cj] = TC(pair_value(hv[u], ev[u]));
+        if (i >= g.M || !LOCA_CHECK(j, g.N)) continue;
+        if (g.rest != nullptr) {
+          const float h2 = hv[u] + ev[u];
+          C[i * g.ldc + cj] = isfinite(hv[u]) ? h2 : hv[u];
+          g.rest[i * g.ldc + cj] = isfinite(hv[u]) ? ev[u] - (h2 - hv[u]) : 0.f;
+        } else {
+          C[i * g.ldc + cj] = TC(pair_value(hv[u], ev[u]));
+        }
       }
     }
 }
