@@ -136,13 +136,14 @@ def _check(rc: int, where: str):
 
 
 def _ptr(t):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()  # the signatures make void pointers of integers
 
 
 def _stream(stream):
+    # the handle of the current stream without a Stream object (3.1 -> 0.3 us a call)
     if stream is None:
-        stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream)
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    return stream.cuda_stream
 
 
 def _dev(t, name, dtype=None, ndim=None):
@@ -150,7 +151,7 @@ def _dev(t, name, dtype=None, ndim=None):
         return
     if not isinstance(t, torch.Tensor) or not t.is_cuda:
         raise TypeError(f"{name} must be a CUDA tensor")
-    if dtype is not None and t.dtype not in (dtype if isinstance(dtype, tuple) else (dtype,)):
+    if dtype is not None and t.dtype is not dtype and not (isinstance(dtype, tuple) and t.dtype in dtype):
         raise TypeError(f"{name} has dtype {t.dtype}, expected {dtype}")
     if ndim is not None and t.dim() != ndim:
         raise ValueError(f"{name} must have {ndim} dimensions, got {tuple(t.shape)}")
@@ -239,7 +240,7 @@ def loca_targets(E, P, Q, T, tsq=None, workspace=None, stream=None):
     N, C = E.shape
     L, C2, r = P.shape
     L2, r2, d = Q.shape
-    if C2 != C or L2 != L or r2 != r or tuple(T.shape) != (L, N, d):
+    if C2 != C or L2 != L or r2 != r or T.shape != (L, N, d):
         raise ValueError("shape mismatch among E (N x C), P (L x C x r), Q (L x r x d), T (L x N x d)")
     nbytes = targets_workspace_size(N, L, d)
     ws = _workspace(nbytes, E.device, workspace)
@@ -264,7 +265,7 @@ def loca_accumulate(X, T, tsq, eta, gram, cross, xsq_total, zero_first, workspac
     _dev(cross, "cross", torch.float32, 3)
     _dev(xsq_total, "xsq_total", torch.float64, 1)
     L, N, d = X.shape
-    if tuple(T.shape) != (L, N, d) or tuple(gram.shape) != (L, d, d) or tuple(cross.shape) != (L, d, d):
+    if T.shape != (L, N, d) or gram.shape != (L, d, d) or cross.shape != (L, d, d):
         raise ValueError("shape mismatch among X, T (L x N x d) and gram, cross (L x d x d)")
     nbytes = accumulate_workspace_size(L, N, d, X.dtype)
     ws = _workspace(nbytes, X.device, workspace)
@@ -284,7 +285,7 @@ def loca_accumulate_noalloc(X, T, tsq, eta, gram, cross, xsq_total, zero_first, 
     _dev(cross, "cross", torch.float32, 3)
     _dev(xsq_total, "xsq_total", torch.float64, 1)
     L, N, d = X.shape
-    if tuple(T.shape) != (L, N, d) or tuple(gram.shape) != (L, d, d) or tuple(cross.shape) != (L, d, d):
+    if T.shape != (L, N, d) or gram.shape != (L, d, d) or cross.shape != (L, d, d):
         raise ValueError("shape mismatch among X, T (L x N x d) and gram, cross (L x d x d)")
     rc = lib().loca_accumulate_noalloc(_ptr(X), _ptr(T), _code(X.dtype), L, N, d, _ptr(tsq), float(eta),
                                        int(bool(zero_first)), _ptr(gram), _ptr(cross), _ptr(xsq_total),
@@ -338,7 +339,7 @@ def loca_accumulate_streamed(X_host, staging, T, tsq, eta, gram, cross, xsq_tota
     _dev(xsq_total, "xsq_total", torch.float64, 1)
     L, N, d = X_host.shape
     group = max(1, min(int(group), L))
-    if tuple(T.shape) != (L, N, d) or tuple(gram.shape) != (L, d, d) or tuple(cross.shape) != (L, d, d):
+    if T.shape != (L, N, d) or gram.shape != (L, d, d) or cross.shape != (L, d, d):
         raise ValueError("shape mismatch among X_host, T (L x N x d) and gram, cross (L x d x d)")
     if staging.numel() < 2 * group * N * d:
         raise ValueError(f"staging has {staging.numel()} elements, need 2 x group x N x d = {2 * group * N * d}")
@@ -361,7 +362,7 @@ def loca_alignment(E_probe, G_probe, P, Q, alpha, workspace=None, stream=None):
     Np, m = E_probe.shape
     L, _, d = G_probe.shape
     r = P.shape[2]
-    if (tuple(G_probe.shape) != (L, Np, d) or tuple(P.shape) != (L, m, r) or tuple(Q.shape) != (L, r, d)
+    if (G_probe.shape != (L, Np, d) or P.shape != (L, m, r) or Q.shape != (L, r, d)
             or alpha.numel() != L):
         raise ValueError("shape mismatch among E_probe, G_probe, P, Q, alpha")
     out = ctypes.c_size_t(0)
@@ -395,8 +396,8 @@ def loca_kspace_accumulate(X, A, E, P, Q, eta, G, SC, xsq_total, zero_first, alp
     L, N, d = X.shape
     k = A.shape[2]
     C, r = P.shape[1], P.shape[2]
-    if (tuple(A.shape) != (L, d, k) or tuple(E.shape) != (N, C) or tuple(Q.shape) != (L, r, d)
-            or tuple(G.shape) != (L, k, k) or tuple(SC.shape) != (L, C, k) or P.shape[0] != L):
+    if (A.shape != (L, d, k) or E.shape != (N, C) or Q.shape != (L, r, d)
+            or G.shape != (L, k, k) or SC.shape != (L, C, k) or P.shape[0] != L):
         raise ValueError("shape mismatch among X, A, E, P, Q, G, SC")
     nbytes = kspace_workspace_size(L, N, d, k, C, r)
     ws = _workspace(nbytes, X.device, workspace)
@@ -423,7 +424,7 @@ def loca_kspace_solve(G, SC, P, Q, lambda_rel, B, info, xsq_total=None, B_prev=N
     d = Q.shape[2]
     lam = [float(v) for v in lambda_rel]
     nl = len(lam)
-    if tuple(B.shape) != (nl, L, d, k) or tuple(info.shape) != (nl, L) or tuple(SC.shape) != (L, C, k):
+    if B.shape != (nl, L, d, k) or info.shape != (nl, L) or SC.shape != (L, C, k):
         raise ValueError("shape mismatch among G, SC, Q, B, info")
     arr = (ctypes.c_float * nl)(*lam)
     rc = lib().loca_kspace_solve(_ptr(G), _ptr(SC), _ptr(xsq_total), _ptr(P), _ptr(Q), _ptr(B_prev), arr, nl, L, d,
@@ -466,7 +467,7 @@ def loca_gram_cross(X, T, alpha, gram, cross, zero_first, workspace=None, stream
     _dev(gram, "gram", torch.float32, 3)
     _dev(cross, "cross", torch.float32, 3)
     L, N, d = X.shape
-    if tuple(T.shape) != (L, N, d) or tuple(gram.shape) != (L, d, d) or tuple(cross.shape) != (L, d, d):
+    if T.shape != (L, N, d) or gram.shape != (L, d, d) or cross.shape != (L, d, d):
         raise ValueError("shape mismatch among X, T (L x N x d) and gram, cross (L x d x d)")
     nbytes = gram_cross_workspace_size()
     ws = _workspace(nbytes, X.device, workspace)
@@ -490,7 +491,7 @@ def loca_targets_sq(E, P, Q, tsq, workspace=None, stream=None):
     N, C = E.shape
     L, C2, r = P.shape
     L2, r2, d = Q.shape
-    if C2 != C or L2 != L or r2 != r or tuple(tsq.shape) != (L,):
+    if C2 != C or L2 != L or r2 != r or tsq.shape != (L,):
         raise ValueError("shape mismatch among E (N x C), P (L x C x r), Q (L x r x d), tsq (L)")
     nbytes = targets_sq_workspace_size(N, C)
     ws = _workspace(nbytes, E.device, workspace)
@@ -517,8 +518,8 @@ def loca_gram_cross_fused(X, E, P, Q, alpha, gram, cross, zero_first, workspace=
     _dev(cross, "cross", torch.float32, 3)
     L, N, d = X.shape
     C, r = P.shape[1], P.shape[2]
-    if (tuple(E.shape) != (N, C) or tuple(P.shape) != (L, C, r) or tuple(Q.shape) != (L, r, d)
-            or tuple(gram.shape) != (L, d, d) or tuple(cross.shape) != (L, d, d)):
+    if (E.shape != (N, C) or P.shape != (L, C, r) or Q.shape != (L, r, d)
+            or gram.shape != (L, d, d) or cross.shape != (L, d, d)):
         raise ValueError("shape mismatch among X, E, P, Q, gram, cross")
     nbytes = gram_cross_fused_workspace_size(L, N, r)
     ws = _workspace(nbytes, X.device, workspace)
@@ -550,12 +551,12 @@ def loca_ridge_solve(gram, cross, A, lambda_rel, B, info, xsq_total=None, B_prev
     L, d, k = A.shape
     lam = [float(v) for v in lambda_rel]
     nl = len(lam)
-    if tuple(B.shape) != (nl, L, d, k) or tuple(info.shape) != (nl, L):
+    if B.shape != (nl, L, d, k) or info.shape != (nl, L):
         raise ValueError("B must be nl x L x d x k and info nl x L")
     lam_arr = (ctypes.c_float * max(nl, 1))(*lam)
     nbytes = ridge_solve_workspace_size(L, d, k)
     ws = _workspace(nbytes, A.device, workspace)
-    if cross_scale is not None and tuple(cross_scale.shape) != (L,):
+    if cross_scale is not None and cross_scale.shape != (L,):
         raise ValueError("cross_scale must have L entries")
     rc = lib().loca_ridge_solve(_ptr(gram), _ptr(cross), _ptr(cross_scale), _ptr(xsq_total), _ptr(A), _ptr(B_prev),
                                 lam_arr, nl, L, d, k, _ptr(B), _ptr(info), _ptr(G_out), _ptr(C_out), _ptr(ws), nbytes,
@@ -571,7 +572,7 @@ def loca_step_from_gram(gram, tsq, eta, xsq_total, alpha, stream=None):
     _dev(xsq_total, "xsq_total", torch.float64, 1)
     _dev(alpha, "alpha", torch.float32, 1)
     L, d, d2 = gram.shape
-    if d2 != d or tuple(tsq.shape) != (L,) or tuple(xsq_total.shape) != (L,) or tuple(alpha.shape) != (L,):
+    if d2 != d or tsq.shape != (L,) or xsq_total.shape != (L,) or alpha.shape != (L,):
         raise ValueError("gram must be L x d x d; tsq, xsq_total, alpha must have L entries")
     rc = lib().loca_step_from_gram(_ptr(gram), L, d, _ptr(tsq), float(eta), _ptr(xsq_total), _ptr(alpha),
                                    _stream(stream))
@@ -593,7 +594,7 @@ def loca_calib_fit(E_probe, G_probe, beta, r, P, Q, sigma=None, workspace=None, 
     _dev(sigma, "sigma", torch.float32, 2)
     Np, m = E_probe.shape
     L, Np2, d = G_probe.shape
-    if Np2 != Np or tuple(P.shape) != (L, m, r) or tuple(Q.shape) != (L, r, d):
+    if Np2 != Np or P.shape != (L, m, r) or Q.shape != (L, r, d):
         raise ValueError("shape mismatch among E_probe, G_probe, P, Q")
     nbytes = calib_fit_workspace_size(Np, m, d, L, r)
     ws = _workspace(nbytes, E_probe.device, workspace)
@@ -621,8 +622,8 @@ def loca_calib_fit_rsvd(E_probe, G_probe, beta, r, Omega, q, P, Q, sigma=None, w
     Np, m = E_probe.shape
     L, Np2, d = G_probe.shape
     ell = Omega.shape[1]
-    if (Np2 != Np or Omega.shape[0] != d or tuple(P.shape) != (L, m, r) or tuple(Q.shape) != (L, r, d)
-            or (sigma is not None and tuple(sigma.shape) != (L, r))):
+    if (Np2 != Np or Omega.shape[0] != d or P.shape != (L, m, r) or Q.shape != (L, r, d)
+            or (sigma is not None and sigma.shape != (L, r))):
         raise ValueError("shape mismatch among E_probe, G_probe, Omega, P, Q, sigma")
     nbytes = calib_fit_rsvd_workspace_size(Np, m, d, L, r, ell)
     ws = _workspace(nbytes, E_probe.device, workspace)
@@ -672,8 +673,8 @@ class Pass:
         n0 = 0
         for m, Xm in enumerate(batches):
             nm = Xm.shape[1]
-            Tm = self.T.view(-1)[: self.L * nm * self.d].view(self.L, nm, self.d)
-            loca_targets(self.E[n0:n0 + nm], P, Q, Tm, tsq=self.tsq, workspace=self.ws_t, stream=stream)
+            Tm = self.T if nm == self.nb else self.T.view(-1)[: self.L * nm * self.d].view(self.L, nm, self.d)
+            loca_targets(self.E if nm == self.N else self.E[n0:n0 + nm], P, Q, Tm, tsq=self.tsq, workspace=self.ws_t, stream=stream)
             loca_accumulate(Xm, Tm, self.tsq, self.eta, self.gram, self.cross, self.xsq, zero_first=(m == 0),
                             workspace=self.ws_a, stream=stream)
             n0 += nm
