@@ -37,6 +37,7 @@
 
 #include "jacobi.cuh"
 #include "loca_internal.h"
+#include "pair32.cuh"
 #include "run_gemm.cuh"
 
 namespace loca {
@@ -65,14 +66,6 @@ __device__ __forceinline__ void fetch_rows(uint32_t dst, const float* src, int64
                  "l"(src + int64_t(r) * ld + c)
                  : "memory");
   }
-}
-
-// a + b for pairs (value, rest), renormalised.
-__device__ __forceinline__ float2 pair_add(float2 a, float2 b) {
-  const float t = a.x + b.x, bb = t - a.x;
-  const float e = (a.x - (t - bb)) + (b.x - bb) + (a.y + b.y);
-  const float h = t + e;
-  return make_float2(h, e - (h - t));
 }
 
 template <int PL>
@@ -107,40 +100,6 @@ struct Acc2 {  // sums over even and odd columns of the tile
     }
   }
 };
-
-// Scalars as pairs (value, rest): a b, and m - a b (not renormalised).
-__device__ __forceinline__ float2 pair_norm(float2 a) {
-  const float h = a.x + a.y;
-  return make_float2(h, a.y - (h - a.x));
-}
-__device__ __forceinline__ float2 pair_mul(float2 a, float2 b) {
-  const float p = a.x * b.x;
-  float e = fmaf(a.x, b.x, -p);
-  e = fmaf(a.x, b.y, e);
-  e = fmaf(a.y, b.x, e);
-  return pair_norm(make_float2(p, e));
-}
-__device__ __forceinline__ float2 pair_nmac(float2 m, float2 a, float2 b) {
-  const float p = a.x * b.x;
-  float e = fmaf(a.x, b.x, -p);
-  e = fmaf(a.x, b.y, e);
-  e = fmaf(a.y, b.x, e);
-  const float t = m.x - p, bb = t - m.x;
-  return make_float2(t, m.y + ((m.x - (t - bb)) - (p + bb) - e));
-}
-// 1 / a and 1 / sqrt(a), a > 0: the fp32 value and one step of the binomial series in what it leaves.
-__device__ __forceinline__ float2 pair_rcp(float2 a) {
-  const float y = __frcp_rn(a.x);
-  const float r = fmaf(-a.y, y, fmaf(-a.x, y, 1.f));
-  return pair_norm(make_float2(y, y * fmaf(r, r, r)));
-}
-__device__ __forceinline__ float2 pair_rsqrt(float2 a) {
-  const float y = rsqrtf(a.x), q = y * y, qe = fmaf(y, y, -q);
-  float r = fmaf(-a.x, q, 1.f);
-  r = fmaf(-a.x, qe, r);
-  r = fmaf(-a.y, q, r);
-  return pair_norm(make_float2(y, y * fmaf(0.375f * r, r, 0.5f * r)));
-}
 
 // K (mp x mp, pairs): rows / columns >= m become the identity; beta is added to the first m diagonal
 // entries.

@@ -1,42 +1,75 @@
 // Small positive-definite solves shared by the ridge-solve kernels (S7: no explicit inverse).
 //
-// The k x k system matrix (k <= KM) lives in shared memory in fp64; the whole block factors it
+// The k x k system matrix (k <= KM) lives in shared memory as pairs of fp32; the whole block factors it
 // (Cholesky, right-looking, one barrier per column); every thread then solves its own right-hand
 // side rows by a forward and a back substitution in fp32 registers.
 #pragma once
 
 #include <cuda_runtime.h>
+#include <math.h>
 #include <stdint.h>
+
+#include "pair32.cuh"
 
 namespace loca {
 
-// Factor Md = L L^T (lower triangle of the leading k x k part; overwritten) with every thread of the
-// block, filling Lf (KM x KM fp32 lower factor, rows 16-byte aligned; identity beyond k) and Linv (fp32
-// reciprocals of its diagonal).  Returns 0, or c + 1 when the leading minor of order c + 1 is not
-// positive definite.  Bound by the latency of its k steps (a reciprocal square root and two barriers
-// each) and the fp64 pipe, 2 operations per clock and SM: the trailing entries of a step are dealt
-// out one by one, two rows of the triangle folded into one of constant length.
+// lambda = lambda_rel xsq / d, or lambda_rel without a trace, as m 2^e with e even and 1 <= |m| < 4 (0 and
+// numbers that are not finite: e = kNoExp).  One thread's work: an fp64 division by every warp costs as much
+// as several steps of the factor.
+constexpr int kNoExp = -5000;
+struct RidgeLambda {
+  float2 m;
+  int e;
+};
+__device__ __forceinline__ RidgeLambda ridge_lambda(float lambda_rel, const double* xsq, int64_t d) {
+  const double v = double(lambda_rel) * (xsq != nullptr ? *xsq / double(d) : 1.0);
+  const int x = (__double2hiint(v) >> 20) & 0x7ff;
+  if (x == 0 || x == 0x7ff) return RidgeLambda{make_float2(float(v), 0.f), kNoExp};
+  const int e = (x - 1023) & ~1;
+  return RidgeLambda{pair_of(scalbn(v, -e)), e};
+}
+// (a + b) / 2 without overflow, rounded once.
+__device__ __forceinline__ float mean2(float a, float b) { return fmaf(0.5f, a, 0.5f * b); }
+
+// Factor (G + G^T) / 2 + lambda I = L L^T (the leading k x k part; G and lam in shared memory) with
+// every thread of the block, filling Lf (KM x KM fp32 lower factor, rows 16-byte aligned; identity beyond k) and
+// Linv (fp32 reciprocals of its diagonal).  Returns 0, or c + 1 when the leading minor of order c + 1
+// is not positive definite.  M: room for the sweep, in pairs of fp32, without square roots: column c keeps
+// what is left of it at step c, and the trailing entries lose its product with itself over the pivot.  The
+// matrix is scaled by a power of two (its largest diagonal entry near 1), so pairs keep their rests whatever its
+// size.  Bound by the latency of its k steps, one barrier each; the trailing entries of a step are dealt
+// out one by one, two rows of the triangle folded into one of constant length.  In fp64 every warp's
+// reciprocal square root and the updates queued for 2 operations per clock: 52 us for 48 blocks and three
+// candidates at k = 32 (with the sums of the partial products before it), 27 now.
 template <int KM>
-__device__ int chol_factor(double (*Md)[KM], float (*Lf)[KM], float* Linv, int k) {
-  __shared__ double col[KM];
+__device__ int chol_factor(const float (*G)[KM], const RidgeLambda& lam, float2 (*M)[KM + 1], float (*Lf)[KM], float* Linv,
+                           int k) {
   const int tid = threadIdx.x, nt = blockDim.x;
   for (int e = tid; e < KM * KM; e += nt) Lf[e / KM][e % KM] = (e / KM == e % KM) ? 1.f : 0.f;
   for (int a = tid; a < KM; a += nt) Linv[a] = 1.f;
+  // the even power of two
+  float mx = 0.f;
+  for (int a = 0; a < k; ++a) {
+    const float g = fabsf(G[a][a]);
+    if (g < INFINITY) mx = fmaxf(mx, g);
+  }
+  const int eg = mx > 0.f ? ilogbf(mx) : kNoExp, big = eg > lam.e ? eg : lam.e;
+  const int half = big == kNoExp ? 0 : big >> 1, el = lam.e == kNoExp ? 0 : lam.e;
+  const float2 lp = make_float2(scalbnf(lam.m.x, el - 2 * half), scalbnf(lam.m.y, el - 2 * half));
+  for (int e = tid; e < k * k; e += nt) {
+    const int a = e / k, b = e - a * k;
+    if (b > a) continue;
+    const float2 u = make_float2(scalbnf(0.5f * G[a][b], -2 * half), 0.f);
+    const float2 v = make_float2(scalbnf(0.5f * G[b][a], -2 * half), 0.f);
+    float2 m = pair_add(u, v);
+    if (a == b) m = pair_add(m, lp);
+    M[a][b] = m;
+  }
   __syncthreads();
   for (int c = 0; c < k; ++c) {
-    const double piv = Md[c][c];
-    if (!(piv > 0.0)) return c + 1;  // the same value in every thread
-    const double inv = rsqrt(piv);
-    for (int a = c + 1 + tid; a < k; a += nt) {
-      const double v = Md[a][c] * inv;
-      col[a] = v;
-      Lf[a][c] = float(v);
-    }
-    if (tid == 0) {
-      Lf[c][c] = float(piv * inv);
-      Linv[c] = float(inv);
-    }
-    __syncthreads();
+    const float2 piv = M[c][c];
+    if (!(piv.x > 0.f)) return c + 1;  // the same value in every thread
+    const float2 rp = piv.x < INFINITY ? pair_rcp(piv) : make_float2(0.f, 0.f);
     // rows c + 1 + i, i < rem, with i + 1 entries each: rows i and rem - 1 - i side by side
     const int rem = k - 1 - c, width = rem + 1;
     const uint32_t magic = (65536u + uint32_t(width) - 1u) / uint32_t(width);  // e / width for e width < 2^16
@@ -47,10 +80,20 @@ __device__ int chol_factor(double (*Md)[KM], float (*Lf)[KM], float* Linv, int k
         j -= i + 1;
         i = rem - 1 - i;
       }
-      Md[c + 1 + i][c + 1 + j] = fma(-col[c + 1 + i], col[c + 1 + j], Md[c + 1 + i][c + 1 + j]);
+      float2* m = &M[c + 1 + i][c + 1 + j];
+      *m = pair_norm(pair_nmac(*m, M[c + 1 + i][c], pair_mul(M[c + 1 + j][c], rp)));
     }
     __syncthreads();
   }
+  for (int e = tid; e < k * k; e += nt) {
+    const int a = e / k, b = e - a * k;
+    if (b > a) continue;
+    const float2 piv = M[b][b];
+    const float2 rs = piv.x < INFINITY ? pair_rsqrt(piv) : make_float2(0.f, 0.f);
+    Lf[a][b] = scalbnf(pair_mul(M[a][b], rs).x, half);
+    if (a == b) Linv[a] = scalbnf(rs.x, -half);
+  }
+  __syncthreads();
   return 0;
 }
 

@@ -742,12 +742,14 @@ __global__ void __launch_bounds__(KS_THREADS) k_kspace_solve(
     float l8, float l9, float l10, float l11, float l12, float l13, float l14, float l15, float* __restrict__ B,
     int32_t* __restrict__ info, float* __restrict__ C_out) {
   __shared__ __align__(16) float Gf[KM][KM];
-  __shared__ double Md[KM][KM];
+  __shared__ float2 Md[KM][KM + 1];
+  __shared__ RidgeLambda lam;
   __shared__ __align__(16) float Lf[KM][KM];
   __shared__ float Linv[KM];
   __shared__ __align__(16) float W2[kMaxRk][KM];  // P_l^T S_l  (r x k)
   const int j = blockIdx.y, l = blockIdx.z;
   const float lam_rel[16] = {l0, l1, l2, l3, l4, l5, l6, l7, l8, l9, l10, l11, l12, l13, l14, l15};
+  if (threadIdx.x == KS_THREADS - 1) lam = ridge_lambda(lam_rel[j], xsq_total ? xsq_total + l : nullptr, d);
   for (int e = threadIdx.x; e < KM * KM; e += KS_THREADS) {
     const int a = e / KM, b = e % KM;
     Gf[a][b] = (a < k && b < k) ? G[(int64_t(l) * k + a) * k + b] : 0.f;
@@ -760,13 +762,7 @@ __global__ void __launch_bounds__(KS_THREADS) k_kspace_solve(
     W2[t][s] = acc;
   }
   __syncthreads();
-  const double lam = double(lam_rel[j]) * (xsq_total != nullptr ? xsq_total[l] / double(d) : 1.0);
-  for (int e = threadIdx.x; e < KM * KM; e += KS_THREADS) {
-    const int a = e / KM, b = e % KM;
-    Md[a][b] = 0.5 * (double(Gf[a][b]) + double(Gf[b][a])) + (a == b ? lam : 0.0);
-  }
-  __syncthreads();
-  const int inf = chol_factor<KM>(Md, Lf, Linv, k);
+  const int inf = chol_factor<KM>(Gf, lam, Md, Lf, Linv, k);
   if (blockIdx.x == 0 && threadIdx.x == 0 && LOCA_CHECK(int64_t(j) * L + l, int64_t(gridDim.y) * L)) info[int64_t(j) * L + l] = inf;
   float* Bj = B + (int64_t(j) * L + l) * d * k;
   const float* Ql = Q + int64_t(l) * r * d;

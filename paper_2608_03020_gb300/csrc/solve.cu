@@ -14,8 +14,8 @@
 //                 (chunks, L), GA_l summed over its nsplit partial products (fixed order) as the
 //                 rows are staged; each chunk's k x k partial sum goes to the workspace.
 // k_chol_factor   one thread block per (ridge candidate j, block l): the chunks' partial sums
-//                 added in chunk order, lambda from the trace, Cholesky of G_l + lambda I in fp64
-//                 in shared memory; the fp32 factor, its diagonal reciprocals and G_l go to a
+//                 added in chunk order, lambda from the trace, Cholesky of G_l + lambda I as pairs
+//                 of fp32 in shared memory; the fp32 factor, its diagonal reciprocals and G_l go to a
 //                 per-candidate record in the workspace.
 // k_chol_rows     two to four rows i of C_l = B_prev,l G_l + s_l CA_l (s_l = cross_scale[l], or 1) per
 //                 thread, solved by a forward and a back substitution against the staged factor:
@@ -236,49 +236,41 @@ __global__ void __launch_bounds__(CS_THREADS) k_chol_factor(
     float l9, float l10, float l11, float l12, float l13, float l14, float l15,
     int32_t* __restrict__ info, float* __restrict__ G_out, float* __restrict__ fac) {
   __shared__ float Gf[KM][KM];   // G_l (fp32, symmetrised), padded with identity
-  __shared__ double Md[KM][KM];  // G_l + lambda I, then its Cholesky factor (lower)
+  __shared__ float2 Md[KM][KM + 1];  // the factor's sweep
+  __shared__ RidgeLambda lam;
   __shared__ __align__(16) float Lf[KM][KM];
   __shared__ float Linv[KM];
   const int j = blockIdx.x, l = blockIdx.y;
   const float lam_rel[16] = {l0, l1, l2, l3, l4, l5, l6, l7, l8, l9, l10, l11, l12, l13, l14, l15};
-  // G_l = A_l^T GA_l from the row chunks' partial products, summed in a fixed order in fp64
+  if (threadIdx.x == CS_THREADS - 1) lam = ridge_lambda(lam_rel[j], xsq_total ? xsq_total + l : nullptr, d);
+  // G_l = A_l^T GA_l from the row chunks' partial products, summed in a fixed order as pairs
   const float* gp = gpart + int64_t(l) * nch * KM * KM;
   for (int e = threadIdx.x; e < KM * KM; e += CS_THREADS) {
-    double acc = 0.0;
+    float h = 0.f, rest = 0.f;
 #pragma unroll 8
-    for (int c = 0; c < nch; ++c) acc += double(gp[int64_t(c) * KM * KM + e]);
-    Gf[e / KM][e % KM] = float(acc);
-  }
-  __syncthreads();
-  const double lam =
-      double(lam_rel[j]) * (xsq_total != nullptr ? xsq_total[l] / double(d) : 1.0);
-  for (int e = threadIdx.x; e < KM * KM; e += CS_THREADS) {
-    const int a = e / KM, b = e % KM;
-    double v;
-    if (a < k && b < k) {
-      v = 0.5 * (double(Gf[a][b]) + double(Gf[b][a]));
-      if (a == b) v += lam;
-    } else {
-      v = (a == b) ? 1.0 : 0.0;
+    for (int c = 0; c < nch; ++c) {
+      const float p = gp[int64_t(c) * KM * KM + e], t = h + p, bb = t - h;
+      rest += (h - (t - bb)) + (p - bb);
+      h = t;
     }
-    Md[a][b] = v;
+    Gf[e / KM][e % KM] = isfinite(h) ? h + rest : h;
   }
   __syncthreads();
   if (G_out != nullptr && j == 0) {
     for (int e = threadIdx.x; e < k * k; e += CS_THREADS) {
       const int a = e / k, b = e % k;
       if (LOCA_CHECK((int64_t(l) * k + a) * k + b, int64_t(L) * k * k))
-        G_out[(int64_t(l) * k + a) * k + b] = float(0.5 * (double(Gf[a][b]) + double(Gf[b][a])));
+        G_out[(int64_t(l) * k + a) * k + b] = mean2(Gf[a][b], Gf[b][a]);
     }
   }
-  const int inf = chol_factor<KM>(Md, Lf, Linv, k);
+  const int inf = chol_factor<KM>(Gf, lam, Md, Lf, Linv, k);
   if (threadIdx.x == 0 && LOCA_CHECK(int64_t(j) * L + l, int64_t(gridDim.x) * L)) info[int64_t(j) * L + l] = inf;
 
   float* f = fac + (int64_t(j) * L + l) * fac_floats<KM>();
   for (int e = threadIdx.x; e < KM * KM; e += CS_THREADS) {
     const int a = e / KM, b = e % KM;
     f[e] = Lf[a][b];
-    f[KM * KM + KM + e] = (a < k && b < k) ? float(0.5 * (double(Gf[a][b]) + double(Gf[b][a]))) : 0.f;
+    f[KM * KM + KM + e] = (a < k && b < k) ? mean2(Gf[a][b], Gf[b][a]) : 0.f;
   }
   for (int a = threadIdx.x; a < KM; a += CS_THREADS) f[KM * KM + a] = Linv[a];
 }

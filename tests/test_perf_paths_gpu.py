@@ -344,3 +344,30 @@ def test_step_inside_the_statistics_launch(lc, L, N, d):
     assert torch.equal(gram, gram2)
     assert torch.allclose(xsq, ref, rtol=tol, atol=0) and torch.allclose(xsq, xsq2, rtol=tol, atol=0)
     assert float((cross - cross2).abs().max()) <= tol * float(cross2.abs().max())
+
+
+@pytest.mark.parametrize("k,scale,lam", [
+    (1, 2.0 ** -80, 2.0 ** -87), (5, 2.0 ** 80, 2.0 ** 70), (8, 1.0, 2.0 ** 70), (17, 2.0 ** -80, 2.0 ** -82), (32, 1.0, 0.5),
+])
+def test_ridge_factor_scales(lc, k, scale, lam):
+    """The factor of G + lambda I in fp32 pairs whatever its size: condition numbers below 10, so the fp32
+    sums and substitutions leave k 2^-24 times as much, and a block that is not positive definite is named."""
+    g = torch.Generator(device="cuda")
+    g.manual_seed(k)
+    L, d = 3, 96
+    W = torch.randn((L, d, d), generator=g, device="cuda") * (0.3 / d ** 0.5)
+    gram = torch.eye(d, device="cuda") + W @ W.transpose(1, 2)
+    gram = 0.5 * (gram + gram.transpose(1, 2)) * scale
+    gram[2] *= -1.0
+    cross = torch.randn((L, d, d), generator=g, device="cuda") * (scale + lam)
+    A = torch.randn((L, d, k), generator=g, device="cuda") / d ** 0.5
+    B, info = torch.empty((1, L, d, k), device="cuda"), torch.empty((1, L), dtype=torch.int32, device="cuda")
+    lc.loca_ridge_solve(gram, cross, A, [lam], B, info)
+    torch.cuda.synchronize()
+    bad = lam < scale
+    assert info.tolist() == [[0, 0, 1 if bad else 0]] and lc.loca_device_status() == 0
+    for l in range(2 if bad else 3):
+        Ad = A[l].double()
+        G = Ad.t() @ gram[l].double() @ Ad + lam * torch.eye(k, dtype=torch.float64, device="cuda")
+        ref = torch.linalg.solve(G, (cross[l].double() @ Ad).t()).t()
+        assert float((B[0, l].double() - ref).norm() / ref.norm()) <= 10 * max(k, 8) * 2.0 ** -24
