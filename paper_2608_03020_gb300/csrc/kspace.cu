@@ -38,6 +38,7 @@
 
 #include "chol.cuh"
 #include "loca_internal.h"
+#include "pair32.cuh"
 #include "tc_ptx.cuh"
 
 namespace loca {
@@ -55,9 +56,10 @@ constexpr int kMaxRk = 32;        // r limit
 // CTAs [0, nW): (block, 128-channel slab) of the split of A_l^T, transposed through shared memory.
 // CTAs [nW, nW + nM): M_l = Q_l Q_l^T, one warp per 2 x 2 block of its upper triangle of blocks: lanes over
 //   channels (fp32 lane sums, fp64 across lanes), four rows of Q_l read for four entries.
-// The rest: one 1024-token chunk of E^T E each: fp32 over a thread's 4 to 1024 / (256 / C^2) tokens, fp64
-//   across the threads, in a fixed order.
-// Every kind is bound by latency, so they share a launch (two launches and, with one warp per entry of M and
+// The rest: one 1024-token chunk of E^T E each, staged in shared memory: fp32 over a thread's 4 to
+//   1024 / (256 / C^2) tokens, fp64 across the threads, in a fixed order.
+// Every kind is bound by latency, so they share a launch (5.1 us at L = 24, N = 1000, r = k = 8; 12.7 with E^T E
+// read token by token and its fp64 additions under a count; two launches and, with one warp per entry of M and
 // one thread per entry of E^T E, 100 us at L = 24, d = 2048, r = k = 32).
 __global__ void __launch_bounds__(PREP_THREADS) k_kspace_prep(const float* __restrict__ A, const float* __restrict__ Q,
                                                              const float* __restrict__ E, int64_t N, int C, int L,
@@ -115,14 +117,17 @@ __global__ void __launch_bounds__(PREP_THREADS) k_kspace_prep(const float* __res
       s10 = fmaf(x1, y0, s10);
       s11 = fmaf(x1, y1, s11);
     }
-    double v[4] = {double(s00), double(s01), double(s10), double(s11)};
+    // four sums over the lanes in six fp64 additions: halves of the warp take two of them, quarters one
+    const double v[4] = {double(s00), double(s01), double(s10), double(s11)};
+    const bool h1 = lane & 16, h2 = lane & 8;
+    const double k0 = (h1 ? v[2] : v[0]) + __shfl_xor_sync(0xffffffffu, h1 ? v[0] : v[2], 16);
+    const double k1 = (h1 ? v[3] : v[1]) + __shfl_xor_sync(0xffffffffu, h1 ? v[1] : v[3], 16);
+    double sum = (h2 ? k1 : k0) + __shfl_xor_sync(0xffffffffu, h2 ? k0 : k1, 8);
 #pragma unroll
-    for (int q = 0; q < 4; ++q)
-#pragma unroll
-      for (int off = 16; off > 0; off >>= 1) v[q] += __shfl_xor_sync(0xffffffffu, v[q], off);
-    if (lane < 4) {
-      const int ea = a0 + (lane >> 1), eb = b0 + (lane & 1);
-      const float m = float(lane == 0 ? v[0] : (lane == 1 ? v[1] : (lane == 2 ? v[2] : v[3])));
+    for (int off = 4; off > 0; off >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
+    if ((lane & 7) == 0) {
+      const int ea = a0 + (lane >> 4), eb = b0 + ((lane >> 3) & 1);
+      const float m = float(sum);
       if (ea <= eb && eb < r && LOCA_CHECK((int64_t(l) * r + ea) * r + eb, int64_t(L) * r * r)) {
         M[(int64_t(l) * r + ea) * r + eb] = m;
         M[(int64_t(l) * r + eb) * r + ea] = m;
@@ -135,26 +140,38 @@ __global__ void __launch_bounds__(PREP_THREADS) k_kspace_prep(const float* __res
   const int64_t n1 = n0 + ETE_CHUNK < N ? n0 + ETE_CHUNK : N;
   const int C2 = C * C, groups = PREP_THREADS / C2;  // C <= 16
   const int e = tid % C2, grp = tid / C2;
+  const int ca = e / C, cb = e % C;
+  const int stage = PREP_COLS * 33 / C;  // tokens staged at a time
   double acc = 0.0;
-  if (grp < groups) {
-    const int ca = e / C, cb = e % C;
-    float run = 0.f;
-    int cnt = 0;
+  for (int64_t ns = n0; ns < n1; ns += stage) {
+    const int nn = n1 - ns < stage ? int(n1 - ns) : stage;
+    if (ns > n0) __syncthreads();
 #pragma unroll 8
-    for (int64_t n = n0 + grp; n < n1; n += groups) {
-      if (LOCA_CHECK(n * C + ca, N * C) && LOCA_CHECK(n * C + cb, N * C)) run = fmaf(E[n * C + ca], E[n * C + cb], run);
-      if (++cnt == 64) {
+    for (int x = tid; x < nn * C; x += PREP_THREADS) sm[x] = LOCA_CHECK(ns * C + x, N * C) ? E[ns * C + x] : 0.f;
+    __syncthreads();
+    // runs of 64 terms in loops of their own: an fp64 addition guarded by a count in the loop occupies the
+    // fp64 pipe on every trip, taken or not
+    if (grp < groups)
+      for (int n = grp; n < nn;) {
+        const int end = n + 64 * groups < nn ? n + 64 * groups : nn;
+        float run = 0.f;
+#pragma unroll 8
+        for (; n < end; n += groups) run = fmaf(sm[n * C + ca], sm[n * C + cb], run);
         acc += double(run);
-        run = 0.f;
-        cnt = 0;
       }
-    }
-    acc += double(run);
   }
   red[tid] = acc;
   __syncthreads();
+  const int some = groups < 8 ? groups : 8;  // sums of every `some`-th group, then of those
+  if (tid < some * C2) {
+    acc = red[tid];
+    for (int q = grp + some; q < groups; q += some) acc += red[q * C2 + e];
+  }
+  __syncthreads();
+  if (tid < some * C2) red[tid] = acc;
+  __syncthreads();
   if (tid < C2) {
-    for (int q = 1; q < groups; ++q) acc += red[q * C2 + tid];
+    for (int q = 1; q < some; ++q) acc += red[q * C2 + tid];
     if (LOCA_CHECK(int64_t(b) * kMaxCk * kMaxCk + tid, int64_t((N + ETE_CHUNK - 1) / ETE_CHUNK) * kMaxCk * kMaxCk))
       ete_part[int64_t(b) * kMaxCk * kMaxCk + tid] = acc;
   }
@@ -614,11 +631,14 @@ __global__ void __launch_bounds__(xa_threads(KP), 1)
 
 // ------------------------------------------------------------------ per-block final reduction
 constexpr int FI_THREADS = 256;
-constexpr int FI_SPLIT = 16;  // CTAs per block (entries dealt out over their warps)
+constexpr int FI_SPLIT = 16;  // CTAs per block at most (entries dealt out over their warps)
 constexpr int FI_MOST = 9;    // entries per warp at most: (32 * 33 / 2 + 16 * 32) / (16 * 8)
 
 // Sums the (CTA, warp) partial slots of block l in a fixed order, forms ||T_l||^2 = <P_l M_l P_l^T, E^T E>, the
-// step alpha_l, and updates G, SC, xsq_total.  Bound by latency: one warp per entry, lanes over the slots.
+// step alpha_l, and updates G, SC, xsq_total.  Bound by latency: one warp per entry, lanes over the slots.  The
+// step is taken where an entry of SC needs it, its products as pairs of fp32 and its fp64 division
+// and root by one warp: with all of it in fp64 in every warp the pipe's 2 operations per clock took most of the
+// 15.9 us at L = 24, r = k = 8 (7.8 now) and 35.3 at r = k = 32 (27.6).
 __global__ void __launch_bounds__(FI_THREADS) k_kspace_final(const double* __restrict__ part,
                                                            const double* __restrict__ ete_part, int nch_e,
                                                            const float* __restrict__ P, const float* __restrict__ M,
@@ -627,9 +647,9 @@ __global__ void __launch_bounds__(FI_THREADS) k_kspace_final(const double* __res
                                                            float* __restrict__ SC, double* __restrict__ xsq_total,
                                                            float* __restrict__ alpha_out) {
   __shared__ double ete[kMaxCk][kMaxCk];
-  __shared__ double pm[kMaxCk][kMaxRk];  // P_l M_l
+  __shared__ float2 pm[kMaxCk][kMaxRk];  // P_l M_l
   __shared__ double red[FI_THREADS / 32];
-  __shared__ double s_xsq;
+  __shared__ double s_xsq, s_al;
   const int l = blockIdx.x, prt = blockIdx.y, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int L = int(gridDim.x), total = L * ntiles;
   const int ps = part_stride(kp, C);
@@ -649,7 +669,7 @@ __global__ void __launch_bounds__(FI_THREADS) k_kspace_final(const double* __res
   // this warp's entries: G's (the upper triangle, written on both sides), then SC's
   const int nt = ntri(kp), ntk = k * (k + 1) / 2;
   const int e0 = prt * (FI_THREADS / 32) + warp;
-  constexpr int STEP = FI_SPLIT * (FI_THREADS / 32);
+  const int STEP = int(gridDim.y) * (FI_THREADS / 32);
   double val[FI_MOST];
 #pragma unroll
   for (int q = 0; q < FI_MOST; ++q) {
@@ -666,43 +686,65 @@ __global__ void __launch_bounds__(FI_THREADS) k_kspace_final(const double* __res
     }
     val[q] = sum_entry(src, 4);
   }
-  if (warp == 0) {
-    const double v = sum_entry(nt + C * kp, xa_sq_warps(kp));
-    if (lane == 0) s_xsq = v;
-  }
-  for (int e = warp; e < C * C; e += FI_THREADS / 32) {
-    double v = 0.0;
-    for (int ch = lane; ch < nch_e; ch += 32) v += ete_part[int64_t(ch) * kMaxCk * kMaxCk + e];
+  // does the step matter here: the CTA of xsq_total and alpha, and those whose last entries are SC's
+  const int first = prt * (FI_THREADS / 32), left = ntk + C * k - 1 - first;
+  const bool step = prt == 0 || (left >= 0 && first + left / STEP * STEP + FI_THREADS / 32 - 1 >= ntk);
+  double al = 0.0, xsq_b = 0.0;
+  if (step) {  // the whole CTA
+    const int C2 = C * C;
+    if (warp == FI_THREADS / 32 - 1) {
+      const double v = sum_entry(nt + C * kp, xa_sq_warps(kp));
+      if (lane == 0) s_xsq = v;
+    }
+    if (nch_e <= 8) {
+      if (tid < C2) {
+        double v = 0.0;
+        for (int ch = 0; ch < nch_e; ++ch) v += ete_part[int64_t(ch) * kMaxCk * kMaxCk + tid];
+        ete[tid / C][tid % C] = v;
+      }
+    } else {
+      for (int e = warp; e < C2; e += FI_THREADS / 32) {
+        double v = 0.0;
+        for (int ch = lane; ch < nch_e; ch += 32) v += ete_part[int64_t(ch) * kMaxCk * kMaxCk + e];
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-    if (lane == 0) ete[e / C][e % C] = v;
-  }
-  const float* Pl = P + int64_t(l) * C * r;
-  const float* Ml = M + int64_t(l) * r * r;
-  for (int e = tid; e < C * r; e += FI_THREADS) {
-    const int c = e / r, b = e % r;
-    double v = 0.0;
+        for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+        if (lane == 0) ete[e / C][e % C] = v;
+      }
+    }
+    const float* Pl = P + int64_t(l) * C * r;
+    const float* Ml = M + int64_t(l) * r * r;
+    for (int e = tid; e < C * r; e += FI_THREADS) {
+      const int c = e / r, b = e % r;
+      float2 v = make_float2(0.f, 0.f);
 #pragma unroll 8
-    for (int a = 0; a < r; ++a) v = fma(double(Pl[c * r + a]), double(Ml[a * r + b]), v);
-    pm[c][b] = v;
-  }
-  __syncthreads();
-  // ||T_l||^2 = sum_{c, c'} (P M P^T)[c][c'] (E^T E)[c][c'], C^2 <= 256 terms
-  double t = 0.0;
-  if (tid < C * C) {
-    const int a = tid / C, b = tid % C;
+      for (int a = 0; a < r; ++a) v = pair_mac(v, Pl[c * r + a], Ml[a * r + b]);
+      pm[c][b] = pair_norm(v);
+    }
+    __syncthreads();
+    // ||T_l||^2 = sum_{c, c'} (P M P^T)[c][c'] (E^T E)[c][c'], C^2 <= 256 terms
+    if (warp * 32 < C2) {
+      double t = 0.0;
+      if (tid < C2) {
+        const int a = tid / C, b = tid % C;
+        float2 v = make_float2(0.f, 0.f);
 #pragma unroll 8
-    for (int j = 0; j < r; ++j) t = fma(pm[a][j], double(Pl[b * r + j]), t);
-    t *= ete[a][b];
-  }
+        for (int j = 0; j < r; ++j) v = pair_mac(v, pm[a][j], Pl[b * r + j]);
+        t = (double(v.x) + double(v.y)) * ete[a][b];
+      }
 #pragma unroll
-  for (int off = 16; off > 0; off >>= 1) t += __shfl_xor_sync(0xffffffffu, t, off);
-  if (lane == 0) red[warp] = t;
-  __syncthreads();
-  double tsq_b = 0.0;
-  for (int w = 0; w < FI_THREADS / 32; ++w) tsq_b += red[w];
-  const double xsq_b = s_xsq;
-  const double al = tsq_b > 0.0 ? -double(eta) * sqrt(xsq_b / tsq_b) : 0.0;
+      for (int off = 16; off > 0; off >>= 1) t += __shfl_xor_sync(0xffffffffu, t, off);
+      if (lane == 0) red[warp] = t;
+    }
+    __syncthreads();
+    if (tid == 0) {
+      double tsq_b = 0.0;
+      for (int w = 0; w * 32 < C2; ++w) tsq_b += red[w];
+      s_al = tsq_b > 0.0 ? -double(eta) * sqrt(s_xsq / tsq_b) : 0.0;
+    }
+    __syncthreads();
+    al = s_al;
+    xsq_b = s_xsq;
+  }
 #pragma unroll
   for (int q = 0; q < FI_MOST; ++q) {
     const int e = e0 + q * STEP;
@@ -895,7 +937,9 @@ cudaError_t launch_kspace_accumulate(const void* X, int L, int64_t N, int64_t d,
   }
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  k_kspace_final<<<dim3(unsigned(L), FI_SPLIT), FI_THREADS, 0, s>>>(part, ete, nch_e, P, M, grid, ntiles, kp, k, C,
+  int fi = (k * (k + 1) / 2 + C * k + FI_THREADS / 32 - 1) / (FI_THREADS / 32);
+  if (fi > FI_SPLIT) fi = FI_SPLIT;
+  k_kspace_final<<<dim3(unsigned(L), unsigned(fi)), FI_THREADS, 0, s>>>(part, ete, nch_e, P, M, grid, ntiles, kp, k, C,
                                                                      r, eta, zero_first, G, SC, xsq_total, alpha_out);
   return cudaGetLastError();
 }

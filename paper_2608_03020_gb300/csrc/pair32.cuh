@@ -29,6 +29,15 @@ __device__ __forceinline__ float2 pair_mul(float2 a, float2 b) {
   e = fmaf(a.y, b.x, e);
   return pair_norm(make_float2(p, e));
 }
+// m + a b for numbers a, b and for a pair a, not renormalised.
+__device__ __forceinline__ float2 pair_mac(float2 m, float a, float b) {
+  const float p = a * b, e = fmaf(a, b, -p), t = m.x + p, bb = t - m.x;
+  return make_float2(t, m.y + ((m.x - (t - bb)) + (p - bb) + e));
+}
+__device__ __forceinline__ float2 pair_mac(float2 m, float2 a, float b) {
+  const float2 s = pair_mac(m, a.x, b);
+  return make_float2(s.x, fmaf(a.y, b, s.y));
+}
 // m - a b, not renormalised.
 __device__ __forceinline__ float2 pair_nmac(float2 m, float2 a, float2 b) {
   const float p = a.x * b.x;

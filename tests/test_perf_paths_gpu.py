@@ -371,3 +371,33 @@ def test_ridge_factor_scales(lc, k, scale, lam):
         G = Ad.t() @ gram[l].double() @ Ad + lam * torch.eye(k, dtype=torch.float64, device="cuda")
         ref = torch.linalg.solve(G, (cross[l].double() @ Ad).t()).t()
         assert float((B[0, l].double() - ref).norm() / ref.norm()) <= 10 * max(k, 8) * 2.0 ** -24
+
+
+@pytest.mark.parametrize("N,C,r,k", [
+    (1, 1, 1, 1),        # one entry each
+    (700, 16, 3, 2),     # E^T E staged in three parts, one thread per entry
+    (9000, 2, 32, 7),    # nine chunks of E^T E: summed by warps; 64 groups of tokens
+    (3000, 3, 9, 32),    # several entries per warp, some CTAs without SC's
+])
+def test_kspace_step(lc, N, C, r, k):
+    """alpha, SC and xsq_total: fp32 sums of 64 terms of E^T E and of d / 32 terms of Q Q^T (64 2^-24 each, half
+    of it in alpha), A in two bf16 parts (2^-16 of each entry) with random signs in SC."""
+    g = torch.Generator(device="cuda")
+    g.manual_seed(N)
+    L, d = 2, 136
+    X = torch.randn((L, N, d), generator=g, device="cuda").to(torch.bfloat16)
+    A, E = torch.randn((L, d, k), generator=g, device="cuda"), torch.randn((N, C), generator=g, device="cuda")
+    P, Q = torch.randn((L, C, r), generator=g, device="cuda"), torch.randn((L, r, d), generator=g, device="cuda")
+    G, SC = torch.empty((L, k, k), device="cuda"), torch.empty((L, C, k), device="cuda")
+    xsq, alpha = torch.empty((L,), dtype=torch.float64, device="cuda"), torch.empty((L,), device="cuda")
+    lc.loca_kspace_accumulate(X, A, E, P, Q, 0.25, G, SC, xsq, zero_first=True, alpha=alpha)
+    torch.cuda.synchronize()
+    assert lc.loca_device_status() == 0
+    for l in range(L):
+        x, e = X[l].double(), E.double()
+        tsq = ((e @ P[l].double()) @ Q[l].double()).square().sum()
+        al = -0.25 * (x.square().sum() / tsq).sqrt()
+        sc = al * (e.t() @ (x @ A[l].double()))
+        assert abs(float(alpha[l].double() / al) - 1) <= 64 * 2.0 ** -24 + 2.0 ** -23
+        assert abs(float(xsq[l] / x.square().sum()) - 1) <= 64 * 2.0 ** -24
+        assert float((SC[l].double() - sc).norm() / sc.norm()) <= 2.0 ** -15
