@@ -430,7 +430,7 @@ def measure_workload(lc, name, dev, stream, steps, warmup, peak, hbm, wpeak):
         ach = flops / (stages["statistics"] / 1e3) / 1e12
         out["gram_roofline"] = {"bound": "tensor", "achieved": ach, "peak": peak, "unit": "TFLOP/s",
                                 "frac": ach / peak, "kernel": "k_gram_cross_tc (+ k_gram_mirror)"
-                                + (", k_sumsq / k_step per batch" if mb > 1 else ""),
+                                + (", the step of every batch inside the launch" if mb > 1 else ""),
                                 "flops_per_step": flops}
     else:
         out["gram_path"] = "fp32 inputs: k_gram_cross_f32 (CUDA cores, fp64 accumulation)"
@@ -671,7 +671,7 @@ def main():
                for i, n in enumerate(["error", "accumulate", "solve"])}
         xbytes = float(X.numel() * X.element_size())
         kspace = {"value": world * N * L / (ms_k / 1e3), "unit": UNIT, "ms_per_step": ms_k, "stages_ms": kst,
-                  "launches_per_step": 1 + 4 + 1,
+                  "launches_per_step": 1 + 3 + 1,
                   "roofline": {"bound": "hbm", "achieved": xbytes / (kst["accumulate"] / 1e3) / 1e9,
                                "peak": hbm_peak(), "unit": "GB/s",
                                "frac": xbytes / (kst["accumulate"] / 1e3) / 1e9 / hbm_peak(),

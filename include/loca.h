@@ -242,8 +242,8 @@ int loca_alignment(const float* E_probe, const float* G_probe, int64_t Np, int32
  *   Workspace: loca_kspace_workspace_size (the split A_l, Q_l Q_l^T, per-CTA partial sums and
  *   E^T E partials; 2 KB per 1024 tokens beyond a fixed part).
  *   Arithmetic: X A_l on the tensor cores with A_l split into two bf16 parts (A_l to 2^-16) and
- *   fp32 accumulation; the token sums in fp32 over 128 tokens, fp64 across; fixed-order
- *   reductions (deterministic).
+ *   fp32 accumulation; the token sums in fp32 over 128 tokens, fp64 across; ||T_l||^2's products as
+ *   pairs of fp32 (2^-48); fixed-order reductions (deterministic).
  *
  * loca_kspace_solve (Eq. 8; Theorem S6; S7): for every candidate j and block l,
  *   lambda_{j,l} = lambda_rel[j] * xsq_total[l] / d  (absolute lambda_rel if xsq_total == NULL),
@@ -316,7 +316,8 @@ int loca_gram_cross(const void* X, const void* T, int dtype, int32_t L, int64_t 
  *   loca_gram_cross_fused_workspace_size(L, N, r) bytes (launch-local flags, the parts of U_l, 4 L N
  *   rp bytes with rp = 16 for r <= 16, else 32, and U_l^T X_l for 8192 columns, 65536 L rp bytes;
  *   wider X takes one column range after the other).  Other arguments, layouts and determinism
- *   as loca_gram_cross; the Gram matrix is the same bit for bit.
+ *   as loca_gram_cross; the Gram matrix is the same but for the grouping of its fp32 sums (bit for bit
+ *   where neither call cuts a tile's tokens over several SMs).
  *   Cost: d (d + 1) + 2 d * 256 flops per token and block instead of 3 d^2 + d, and no T in memory.
  */
 int loca_targets_sq_workspace_size(int64_t N, int32_t C, size_t* bytes /* host */);
@@ -381,7 +382,8 @@ int loca_step_from_gram(const float* gram, int32_t L, int64_t d, const double* t
  *           accumulate cross with alpha = 1 and apply alpha_l here; see loca_step_from_gram)
  *   lam   = lambda_rel[j] * xsq_total[l] / d              (xsq_total != NULL; = tr(gram_l)/d)
  *         = lambda_rel[j]                                 (xsq_total == NULL: absolute)
- *   B[j, l] = C_l (G_l + lam I)^-1   via Cholesky (fp64) and two triangular substitutions
+ *   B[j, l] = C_l (G_l + lam I)^-1   via Cholesky (pairs of fp32, 2^-48) and two fp32 triangular
+ *                                    substitutions
  *
  * gram, cross   L x d x d float;  cross_scale  L float (device) or NULL
  * A             L x d x k float;  B_prev  L x d x k float or NULL (0)
@@ -421,8 +423,8 @@ int loca_ridge_solve(const float* gram, const float* cross, const float* cross_s
  *
  * E_probe  Np x m float; G_probe  L x Np x d float; beta > 0; 1 <= r <= m <= 64
  * P        L x m x r float; Q  L x r x d float; sigma  L x r float or NULL
- * Arithmetic: E^T E and E^T G_l from fp32 products summed in fp32 over 32-token chunks and in
- * fp64 across chunks; Cholesky solve (fp64) for F_hat^T; cyclic Jacobi eigen-decomposition
+ * Arithmetic: E^T E and E^T G_l from fp32 products summed in fp32 over 32-token chunks and as
+ * pairs of fp32 (2^-48) across chunks; Cholesky solve (fp64) for F_hat^T; cyclic Jacobi eigen-decomposition
  * (fp64) of the m x m matrix F_hat^T F_hat, whose eigenvectors are U and whose eigenvalues are
  * S^2; Q_l = S_r^-1 U_r^T F_hat^T.  Singular values below 1e-12 sigma_1 count as zero.  If
  * E^T E + beta I is not positive definite in floating point (beta below the rounding level
@@ -456,11 +458,12 @@ int loca_calib_fit(const float* E_probe, const float* G_probe, int64_t Np, int32
  * 1 <= r <= ell <= 64, ell <= m <= 16384, ell <= d <= 16384, 0 <= q <= 16, 1 <= L <= 65535,
  * 1 <= Np <= 4194240
  * P        L x m x r float; Q  L x r x d float; sigma  L x r float or NULL
- * Arithmetic: products with E and G_l from fp32 products summed in fp32 over 128-term runs
- * and in fp64 across runs; Cholesky factor, triangular solves, orthonormal bases (Gram-Schmidt
- * with re-orthogonalisation) and the Rayleigh-Ritz step in fp64.  Workspace (device, at least
- * loca_calib_fit_rsvd_workspace_size bytes, 256-byte aligned) holds E^T E (m x m fp64,
- * m rounded up to 64) and the ell-column blocks of every block; its contents are scratch.
+ * Arithmetic: products with E and G_l from fp32 products summed in fp32 over 32-term runs
+ * and as pairs of fp32 (value and rest, 2^-48) across runs; Cholesky factor and the triangular
+ * solves of the last F^T and of F Q_Y in such pairs (in fp64 for few columns), those of the power
+ * iterations in fp32; orthonormal bases (Cholesky QR, twice) and the Rayleigh-Ritz step in fp64.
+ * Workspace (device, at least loca_calib_fit_rsvd_workspace_size bytes, 256-byte aligned) holds the
+ * factor (12 bytes per entry of m x m, m rounded up to 64) and the ell-column blocks of every block; its contents are scratch.
  * If E^T E + beta I is not positive definite in floating point, LOCA_ERR_NUMERIC is written
  * to the device status word and P, Q and sigma are zero.
  */

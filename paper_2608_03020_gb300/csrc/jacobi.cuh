@@ -4,8 +4,18 @@
 #pragma once
 
 #include <cuda_runtime.h>
+#include <stdint.h>
 
 namespace loca {
+
+// Exponent field of v, and v 2^(e - (its exponent)) truncated to fp32 (0 below fp32's normal range): integer
+// work, since a conversion takes the fp64 pipe as long as an fp64 addition.
+__device__ __forceinline__ int exponent_of(double v) { return (__double2hiint(v) >> 20) & 0x7ff; }
+__device__ __forceinline__ float scaled_float(double v, int e) {
+  const uint32_t hi = uint32_t(__double2hiint(v)), lo = uint32_t(__double2loint(v));
+  const uint32_t bits = (hi & 0x80000000u) | (uint32_t(e + 127) << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29);
+  return e > -127 && exponent_of(v) > 0 ? __uint_as_float(bits) : 0.f;
+}
 
 // A (m x m, symmetric, shared memory with row stride KM) is rotated towards diagonal form and
 // V (initialised by the caller, usually to I) accumulates the rotations, so that on return the
@@ -23,14 +33,18 @@ namespace loca {
 // falls below 1e-30 of the total, after at most 40 sweeps.  Then order[] = eigenvalue indices in
 // descending order (lower index first on ties; entries m..KM-1 stay in place).  Called by every
 // thread of the block (it synchronises the block; blockDim.x a multiple of 32, at most 1024).
-// Bound by the latency of the m - 1 rotations in a row per sweep; with t in fp64 their three divisions
-// and two square roots took most of a round.
+// Bound by the latency of the m - 1 rotations in a row per sweep, and in it by the fp64 pipe, which takes an
+// instruction of a warp every 64 cycles per quarter of the SM: with t in fp64 its three divisions and two
+// square roots took most of a round, and with the scaling, the conversions and rsqrt() in fp64 a third
+// (28 blocks of m = 16: 276 us, 211 now).
 template <int KM>
 __device__ void jacobi_eig_block(double (*A)[KM], double (*V)[KM], int* order, int m) {
   __shared__ double s_c[KM / 2], s_s[KM / 2];
   __shared__ int s_p[KM / 2], s_q[KM / 2];
   __shared__ double s_off[32], s_tot[32];
   const int tid = threadIdx.x, nt = blockDim.x;
+  // V's share starts at the warps of the other half of the schedulers: A's blocks may not reach them
+  const int vt = nt % 256 != 0 ? tid : (tid & ~255) | ((((tid >> 5) & 2) ^ 2) << 6) | (((tid >> 7) & 1) << 6) | (tid & 63);
   const int mm = (m + 1) & ~1;
   const int np = mm / 2;
   for (int sweep = 0; sweep < 40; ++sweep) {
@@ -75,18 +89,17 @@ __device__ void jacobi_eig_block(double (*A)[KM], double (*V)[KM], int* order, i
         }
         double c = 1.0, sn = 0.0;
         if (q < m) {
-          const double apq = A[p][q];
-          if (fabs(apq) > 1e-300) {
-            const double num = A[q][q] - A[p][p], den = 2.0 * apq;
-            // both scaled by one power of two, so that the larger is in [1, 2): fp32 holds their ratio
-            const double mx = fabs(num) > fabs(den) ? fabs(num) : fabs(den);
-            const int be = (__double2hiint(mx) >> 20) & 0x7ff;
-            const double scale = __hiloint2double((be < 2045 ? 2046 - be : 1) << 20, 0);
-            const float nf = float(num * scale), df = float(den * scale);
+          const double apq = A[p][q], num = A[q][q] - A[p][p];
+          const int en = exponent_of(num), ed = exponent_of(apq) + 1;  // of A_qq - A_pp and 2 A_pq
+          if (ed > 27 && ed < 0x800) {  // |A_pq| >= 2^-996, and a number
+            const int e = en > ed ? en : ed;
+            const float nf = scaled_float(num, en - e), df = scaled_float(apq, ed - e);
             const float theta = nf / df;  // infinite when df underflows: t = 0
             const float tf = (theta >= 0.f ? 1.f : -1.f) / (fabsf(theta) + sqrtf(fmaf(theta, theta, 1.f)));
-            const double t = double(tf);
-            c = rsqrt(fma(t, t, 1.0));
+            // (1 + t^2)^-1/2: the fp32 value, then two terms of the binomial series in what it leaves
+            const double t = double(tf), c0 = double(rsqrtf(fmaf(tf, tf, 1.f)));
+            const double h = fma(-fma(t, t, 1.0), c0 * c0, 1.0);
+            c = fma(c0, h * fma(h, 0.375, 0.5), c0);
             sn = t * c;
           }
         }
@@ -111,7 +124,7 @@ __device__ void jacobi_eig_block(double (*A)[KM], double (*V)[KM], int* order, i
         if (rq) A[q][pc] = cc * rqp - sc * rqq;
         if (rq && cq) A[q][qc] = sc * rqp + cc * rqq;
       }
-      for (int e = tid; e < np * m; e += nt) {
+      for (int e = vt; e < np * m; e += nt) {
         const int i = e / m, row = e % m;
         const int p = s_p[i], q = s_q[i];
         if (q >= m) continue;
