@@ -372,7 +372,12 @@ int run_gram_cross(const void* X, const void* T, int dtype, int32_t L, int64_t N
 int run_accumulate(const void* X, const void* T, int dtype, int32_t L, int64_t N, int64_t d, const double* tsq,
                    float eta, int zero_first, float* gram, float* cross, double* xsq_total, float* alpha,
                    int32_t* abort_flag, cudaStream_t s) {
-  if (dtype == LOCA_BF16 && N > 0) {
+  // bf16: the step inside the statistics launch, but not for few tokens into outputs of many times the L2:
+  // those launches are bound by the outputs' traffic, in which the squares arrive late (adding to 822 MB at
+  // L = 8, d = 3584, N = 600: 428 us inside, 394 before; N = 2048: 573 and 584; to 420 MB at d = 2560, N = 256:
+  // 200 and 211; overwriting 2.1 GB at L = 28, d = 3072: N = 512 687 and 682, N = 1024 868 and 885).
+  const bool inside = 8.0 * double(L) * double(d) * double(d) < 6e8 || N >= (zero_first ? 1024 : 2048);
+  if (dtype == LOCA_BF16 && N > 0 && inside) {
     int32_t* status = device_status_word();
     if (!status) return fail(LOCA_ERR_CUDA, "cannot resolve the device status word");
     const cudaError_t e = launch_accumulate_tc(X, T, L, N, d, tsq, eta, zero_first, gram, cross, xsq_total, alpha,

@@ -319,6 +319,7 @@ def test_gram_schedules(lc, L, N, d, batches):
     (3, 1501, 328),      # a short last chunk
     (2, 40000, 64),      # few tiles: clusters that only take steps; shared items
     (9, 700, 1096),      # several rounds
+    (7, 100, 3600),      # few tokens, large outputs: the step before the launch
 ])
 def test_step_inside_the_statistics_launch(lc, L, N, d):
     """loca_accumulate on bf16 against loca_batch_step + loca_gram_cross over two batches.  Sums of 32
