@@ -48,21 +48,20 @@ FALLBACK_SUSTAINED_TFLOPS = 1700.0  # profiling recipe's sustained figure, used 
 # kernel source whose sha256 prefix is given.  Work items and rounds repeat block by block, so
 # the traffic of a launch over L blocks is the capture's times L / L_capture; any other N, d or
 # k, or another source, reports null.
-GRAM_TC_TRAFFIC = {"sha256": "81575fe3750817bb", "L_capture": 2, "N": 131072, "d": 3584,
-                   "read": 8478698496, "write": 1255207936,
+GRAM_TC_TRAFFIC = {"sha256": "04b820cfe0083734", "L_capture": 2, "N": 131072, "d": 3584,
+                   "read": 7951192576, "write": 1224957440,
                    "kernel": "k_gram_cross_tc"}
 # k_kspace_xa (the k-space statistics kernel, which reads X) at k = 16
-KSPACE_TRAFFIC = {"sha256": "3aba9c60b10e48c0", "L_capture": 2, "N": 131072, "d": 3584, "k": 16,
-                  "read": 1885266176, "write": 2223872,
+KSPACE_TRAFFIC = {"sha256": "bd6f8733935308c4", "L_capture": 2, "N": 131072, "d": 3584, "k": 16,
+                  "read": 1884494848, "write": 1325056,
                   "kernel": "k_kspace_xa"}
 # k_targets_tc (writes T) at r = 16, bf16 output
-TARGETS_TRAFFIC = {"sha256": "1796bbc513a2c2d2", "L_capture": 2, "N": 131072, "d": 3584, "r": 16,
-                   "read": 13250816, "write": 1817000448,
+TARGETS_TRAFFIC = {"sha256": "a692dc252508fbb1", "L_capture": 2, "N": 131072, "d": 3584, "r": 16,
+                   "read": 13382400, "write": 1816985088,
                    "kernel": "k_targets_tc"}
-# k_project_tc (the ridge solve's projection, which reads Gram and Cross once) at k = 16: taken
-# on the full launch (L = 28, 2.9 GB of statistics), so L_capture = 28
-PROJECT_TRAFFIC = {"sha256": "7771065c47a83799", "L_capture": 28, "d": 3584, "k": 16,
-                   "read": 2886107648, "write": 17300992,
+# k_project_tc (the ridge solve's projection, which reads Gram and Cross once) at k = 16
+PROJECT_TRAFFIC = {"sha256": "be210a42bd72adbc", "L_capture": 2, "d": 3584, "k": 16,
+                   "read": 206055424, "write": 1807616,
                    "kernel": "k_project_tc"}
 
 
