@@ -56,7 +56,7 @@ KSPACE_TRAFFIC = {"sha256": "bd6f8733935308c4", "L_capture": 2, "N": 131072, "d"
                   "read": 1884494848, "write": 1325056,
                   "kernel": "k_kspace_xa"}
 # k_targets_tc (writes T) at r = 16, bf16 output
-TARGETS_TRAFFIC = {"sha256": "a692dc252508fbb1", "L_capture": 2, "N": 131072, "d": 3584, "r": 16,
+TARGETS_TRAFFIC = {"sha256": "147365737e0bf0e4", "L_capture": 2, "N": 131072, "d": 3584, "r": 16,
                    "read": 13382400, "write": 1816985088,
                    "kernel": "k_targets_tc"}
 # k_project_tc (the ridge solve's projection, which reads Gram and Cross once) at k = 16
