@@ -57,7 +57,7 @@ KSPACE_TRAFFIC = {"sha256": "bd6f8733935308c4", "L_capture": 2, "N": 131072, "d"
                   "kernel": "k_kspace_xa"}
 # k_targets_tc (writes T) at r = 16, bf16 output
 TARGETS_TRAFFIC = {"sha256": "147365737e0bf0e4", "L_capture": 2, "N": 131072, "d": 3584, "r": 16,
-                   "read": 13382400, "write": 1816985088,
+                   "read": 13403392, "write": 1816695808,
                    "kernel": "k_targets_tc"}
 # k_project_tc (the ridge solve's projection, which reads Gram and Cross once) at k = 16
 PROJECT_TRAFFIC = {"sha256": "be210a42bd72adbc", "L_capture": 2, "d": 3584, "k": 16,
